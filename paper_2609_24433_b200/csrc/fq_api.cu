@@ -410,34 +410,38 @@ fq_status fq_fold_weights_gptq(const void* Wsrc, fq_dtype wt, int64_t N, int64_t
     st = alloc_handle(N, K, hadamard_block, bits, &w);
     if (st != FQ_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    // all temporaries in one allocation (each cudaMalloc and cudaFree of this size costs the fold tenths of a millisecond)
+    size_t at = 0;
+    auto take = [&at](size_t bytes) { const size_t p = at; at += align_up(bytes, 256); return p; };
     const size_t kk = sizeof(float) * (size_t)K * (size_t)K;
-    float *mult_w = nullptr, *Wt = nullptr, *Z = nullptr, *H = nullptr, *Mt = nullptr, *U = nullptr;
-    uint8_t* dead = nullptr;
-    int* bad = nullptr;
-    bool ok = cudaMalloc(&mult_w, sizeof(float) * (size_t)K) == cudaSuccess &&
-              cudaMalloc(&Wt, sizeof(float) * (size_t)(N > 0 ? N : 1) * (size_t)K) == cudaSuccess &&
-              cudaMalloc(&Z, sizeof(float) * (size_t)Mc * (size_t)K) == cudaSuccess &&
-              cudaMalloc(&H, kk) == cudaSuccess && cudaMalloc(&Mt, kk) == cudaSuccess && cudaMalloc(&U, kk) == cudaSuccess &&
-              cudaMalloc(&dead, (size_t)K) == cudaSuccess && cudaMalloc(&bad, sizeof(int)) == cudaSuccess;
-    auto release = [&]() {
-        cudaFree(mult_w); cudaFree(Wt); cudaFree(Z); cudaFree(H); cudaFree(Mt); cudaFree(U); cudaFree(dead); cudaFree(bad);
-    };
-    if (!ok) {
-        release();
+    const size_t o_mult = take(sizeof(float) * (size_t)K), o_wt = take(sizeof(float) * (size_t)N * (size_t)K),
+                 o_z = take(sizeof(float) * (size_t)Mc * (size_t)K), o_h = take(kk), o_u = take(kk),
+                 o_mt = take(gptq_factor_fits(K) ? 0 : kk), o_dead = take((size_t)K), o_flags = take(2 * sizeof(int));
+    uint8_t* temp = nullptr;
+    if (cudaMalloc(&temp, at) != cudaSuccess) {
+        cudaGetLastError();
         fq_weights_destroy(reinterpret_cast<fq_weights*>(w));
         return FQ_ERR_NOMEM;
     }
+    float* mult_w = reinterpret_cast<float*>(temp + o_mult);
+    float* Wt = reinterpret_cast<float*>(temp + o_wt);
+    float* Z = reinterpret_cast<float*>(temp + o_z);
+    float* H = reinterpret_cast<float*>(temp + o_h);
+    float* U = reinterpret_cast<float*>(temp + o_u);
+    float* Mt = gptq_factor_fits(K) ? nullptr : reinterpret_cast<float*>(temp + o_mt);
+    uint8_t* dead = temp + o_dead;
+    int* flags = reinterpret_cast<int*>(temp + o_flags);
     const float cn = block_norm(hadamard_block);
     const int qmax = bits == 4 ? 7 : 127;
     w->mult_const = smooth == nullptr;
-    ok = cudaMemsetAsync(bad, 0, sizeof(int), s) == cudaSuccess;
+    bool ok = cudaMemsetAsync(flags, 0, 2 * sizeof(int), s) == cudaSuccess;
     ok = ok && launch_multipliers(smooth, K, cn, mult_w, w->mult_g, s) == cudaSuccess;
     // per-output-channel steps: those of the round-to-nearest fold (its codes are overwritten by the sweep)
     ok = ok && launch_transform_quantize(Wsrc, wt, N, K, ldw, mult_w, cn, false, hadamard_block, qmax, 1.0f,
                                          bits == 4 ? StoreFmt::Nibble : StoreFmt::Int8, w->codes, w->w_scale, s) == cudaSuccess;
     ok = ok && launch_transform_rows(Wsrc, wt, N, K, ldw, mult_w, cn, hadamard_block, Wt, s) == cudaSuccess;
     ok = ok && launch_transform_rows(calib, ct, Mc, K, ldc, w->mult_g, cn, hadamard_block, Z, s) == cudaSuccess;
-    ok = ok && launch_gptq_factor(Z, Mc, K, damp, H, Mt, U, dead, bad, s) == cudaSuccess;
+    ok = ok && launch_gptq_factor(Z, Mc, K, damp, H, Mt, U, dead, flags, s) == cudaSuccess;
     ok = ok && launch_gptq_sweep(Wt, N, K, U, dead, w->w_scale, bits, w->codes, s) == cudaSuccess;
     if (N > 0) {
         if (bias)
@@ -446,13 +450,13 @@ fq_status fq_fold_weights_gptq(const void* Wsrc, fq_dtype wt, int64_t N, int64_t
             ok = ok && cudaMemsetAsync(w->bias, 0, sizeof(float) * (size_t)N, s) == cudaSuccess;
     }
     int bad_host = 0;
-    ok = ok && cudaMemcpyAsync(&bad_host, bad, sizeof(int), cudaMemcpyDeviceToHost, s) == cudaSuccess;
+    ok = ok && cudaMemcpyAsync(&bad_host, flags, sizeof(int), cudaMemcpyDeviceToHost, s) == cudaSuccess;
     ok = ok && cudaStreamSynchronize(s) == cudaSuccess;   // offline: the temporaries are freed below
-    release();
+    cudaFree(temp);
     if (ok && !bad_host) ok = build_weight_tmap(*w) == FQ_OK;
     if (!ok || bad_host) {
         fq_weights_destroy(reinterpret_cast<fq_weights*>(w));
-        return bad_host ? FQ_ERR_INVALID_ARG : FQ_ERR_CUDA;
+        return (bad_host & 2) ? FQ_ERR_TIMEOUT : (bad_host ? FQ_ERR_INVALID_ARG : FQ_ERR_CUDA);
     }
     *out = reinterpret_cast<fq_weights*>(w);
     return FQ_OK;

@@ -158,11 +158,14 @@ cudaError_t launch_composite_rotate(const void* x, fq_dtype xt, int64_t rows, in
 cudaError_t launch_perm_check(const int32_t* perm, int64_t K, int* bad_flag, cudaStream_t stream);
 
 // GPTQ rounding (offline): the transform without its quantizer, the damped second moment and the upper factor U
-// of its inverse (H, Mt: K x K scratch; *bad set if not positive definite), and the sweep that writes the codes.
+// of its inverse (H: K x K scratch; Mt: K x K scratch where gptq_factor_fits() says no, else null; flags: two zeroed
+// ints, flags[0] nonzero afterwards if H is not positive definite (1) or a wait expired (2)), and the sweep that
+// writes the codes.
 cudaError_t launch_transform_rows(const void* x, fq_dtype xt, int64_t rows, int64_t K, int64_t ldx, const float* mult,
                                   float cnorm, int block, float* z, cudaStream_t stream);
+bool gptq_factor_fits(int64_t K);
 cudaError_t launch_gptq_factor(const float* z, int64_t Mc, int64_t K, float damp, float* H, float* Mt, float* U,
-                               uint8_t* dead, int* bad, cudaStream_t stream);
+                               uint8_t* dead, int* flags, cudaStream_t stream);
 cudaError_t launch_gptq_sweep(const float* Wt, int64_t N, int64_t K, const float* U, const uint8_t* dead,
                               const float* w_scale, int bits, uint8_t* codes, cudaStream_t stream);
 
