@@ -1,9 +1,10 @@
-"""In-tree build of the CUDA library (sm_100a only): ``python -m paper_2609_24433_b200.build``."""
+"""In-tree build of the CUDA library (sm_100a only) and of its torch binding: ``python -m paper_2609_24433_b200.build``."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -12,6 +13,7 @@ LIB = os.path.join(HERE, "libfq_b200.so")
 SOURCES = ["fq_api.cu", "act_quant.cu", "act_quant_ring.cu", "gemm_simt.cu", "gemm_tcgen05.cu", "fq_static.cu", "linear_wonly.cu", "composite.cu", "gptq.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", CSRC]
+BINDING = os.path.join(HERE, "_fq_torch" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 
 def _stale(target: str, deps) -> bool:
@@ -19,6 +21,20 @@ def _stale(target: str, deps) -> bool:
         return True
     t = os.path.getmtime(target)
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def build_binding(force: bool = False) -> str:
+    """The CPython module over the library: plain C++ against torch's headers, linked to the library next to it."""
+    src = os.path.join(CSRC, "torch_binding.cpp")
+    if force or _stale(BINDING, [src, os.path.join(ROOT, "include", "fq.h")]):
+        import torch
+        t = os.path.dirname(torch.__file__)
+        inc = [os.path.join(ROOT, "include"), os.path.join(t, "include"), os.path.join(t, "include", "torch", "csrc", "api", "include"),
+               sysconfig.get_paths()["include"], "/usr/local/cuda/include"]
+        subprocess.run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared"] + [f for d in inc for f in ("-I", d)] +
+                       [src, "-o", BINDING, "-L", HERE, "-l:" + os.path.basename(LIB), "-L", os.path.join(t, "lib"), "-lc10",
+                        "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-Wl,-rpath,$ORIGIN"], check=True)
+    return BINDING
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -42,6 +58,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
                 pass
     if relink or _stale(LIB, objs):
         subprocess.run([nvcc, "-shared", "-o", LIB] + objs, check=True)
+    build_binding(force)
     return LIB
 
 

@@ -4,6 +4,9 @@ Argument marshalling only: every function below turns torch CUDA tensors into
 device pointers, calls the library on torch's current stream and wraps the
 outputs.  There is no Python, torch or CPU implementation of any step here; if
 the shared library is missing the first call raises.
+
+The calls of a forward pass go through a CPython module (csrc/torch_binding.cpp)
+that does the same marshalling natively; everything else through ctypes.
 """
 from __future__ import annotations
 
@@ -31,6 +34,7 @@ EXPORTS = [
 ]
 
 _lib = None
+_torch_binding = None
 
 
 class FqError(RuntimeError):
@@ -61,6 +65,20 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+def _native():
+    """The native marshalling of the calls of a forward pass (linked against the library next to it)."""
+    global _torch_binding
+    if _torch_binding is None:
+        lib()
+        try:
+            from . import _fq_torch
+        except ImportError as e:
+            raise RuntimeError("the native binding is missing: build it with `python -m paper_2609_24433_b200.build` "
+                               "(there is no fallback path)") from e
+        _torch_binding = _fq_torch
+    return _torch_binding
+
+
 def status_string(status: int) -> str:
     return lib().fq_status_string(int(status)).decode()
 
@@ -68,6 +86,13 @@ def status_string(status: int) -> str:
 def _check(status: int, what: str):
     if status != OK:
         raise FqError(status, what)
+
+
+def _result(r, what: str):
+    """What a native call returned: its result, or the status of a refusal."""
+    if r.__class__ is int:
+        raise FqError(r, what)
+    return r
 
 
 def _dt(t: torch.Tensor) -> int:
@@ -106,6 +131,7 @@ class Weights:
         _check(lib().fq_weights_info(self._h, ctypes.byref(n), ctypes.byref(k), ctypes.byref(blk),
                                      ctypes.byref(bits)), "fq_weights_info")
         self.N, self.K, self.block, self.bits = n.value, k.value, blk.value, bits.value
+        self._addr = self._h.value
         self.fold_after = bool(lib().fq_weights_fold_after(self._h))
 
     @property
@@ -113,6 +139,12 @@ class Weights:
         if self._h is None:
             raise RuntimeError("weights handle already destroyed")
         return self._h
+
+    @property
+    def address(self) -> int:
+        if self._addr is None:
+            raise RuntimeError("weights handle already destroyed")
+        return self._addr
 
     def multiplier_ptr(self) -> int:
         return int(lib().fq_weights_multiplier(self.handle) or 0)
@@ -140,7 +172,7 @@ class Weights:
     def destroy(self):
         if self._h is not None:
             lib().fq_weights_destroy(self._h)
-            self._h = None
+            self._h = self._addr = None
 
     def __del__(self):
         try:
@@ -205,21 +237,9 @@ def quantize_act_composite(x: torch.Tensor, mult_g, perm: torch.Tensor, blocks: 
                            delta: Optional[torch.Tensor] = None, workspace: Optional[torch.Tensor] = None):
     """Runtime prologue of a composite-rotation site: z = R ((1/s) (.) x), then Eq. 5.  ``mult_g``: device
     float tensor, a Weights (its multiplier) or None.  ``workspace``: uint8 tensor of at least 4*M*K bytes."""
-    x = _rowmajor(x)
-    M, K = x.shape
-    assert perm.dtype == torch.int32 and blocks.dtype == torch.float32 and blocks.is_contiguous()
-    if codes is None:
-        codes = torch.empty((M, K * bits // 8), dtype=torch.uint8, device=x.device)
-    if delta is None:
-        delta = torch.empty(M, dtype=torch.float32, device=x.device)
-    if workspace is None:
-        workspace = torch.empty(max(16, 4 * M * K), dtype=torch.uint8, device=x.device)
-    g = ctypes.c_void_p(mult_g.multiplier_ptr()) if isinstance(mult_g, Weights) else _ptr(mult_g)
-    _check(lib().fq_quantize_act_composite(_ptr(x), _dt(x), ctypes.c_int64(M), ctypes.c_int64(K), ctypes.c_int64(x.stride(0)),
-                                           g, _ptr(perm), _ptr(blocks), ctypes.c_int(blocks.shape[1]), ctypes.c_int(bits),
-                                           ctypes.c_float(clip_ratio), _ptr(codes), _ptr(delta), _ptr(workspace),
-                                           ctypes.c_size_t(workspace.numel()), _stream()), "fq_quantize_act_composite")
-    return codes, delta
+    g = mult_g.multiplier_ptr() if isinstance(mult_g, Weights) else (0 if mult_g is None else mult_g.data_ptr())
+    return _result(_native().quantize_act_composite(x, g, perm, blocks, bits, clip_ratio, codes, delta, workspace),
+                   "fq_quantize_act_composite")
 
 
 def weights_import(codes: torch.Tensor, w_scale: torch.Tensor, mult_g: Optional[torch.Tensor],
@@ -258,23 +278,14 @@ def quantize_act(x: torch.Tensor, mult_g, hadamard_block: int, bits: int, clip_r
                  fold_after: Optional[bool] = None):
     """Runtime prologue. ``mult_g``: device float tensor, a Weights (its multiplier) or None.
     ``fold_after``: the multiplier is the post-rotation 1/p (default: what the Weights says, else False)."""
-    x = _rowmajor(x)
-    M, K = x.shape
-    if codes is None:
-        codes = torch.empty((M, K * bits // 8), dtype=torch.uint8, device=x.device)
-    if delta is None:
-        delta = torch.empty(M, dtype=torch.float32, device=x.device)
     if isinstance(mult_g, Weights):
-        g = ctypes.c_void_p(mult_g.multiplier_ptr())
+        g = mult_g.multiplier_ptr()
         if fold_after is None:
             fold_after = mult_g.fold_after
     else:
-        g = _ptr(mult_g)
-    fn_name = "fq_quantize_act_after" if fold_after else "fq_quantize_act"
-    _check(getattr(lib(), fn_name)(_ptr(x), _dt(x), ctypes.c_int64(M), ctypes.c_int64(K), ctypes.c_int64(x.stride(0)),
-                                   g, ctypes.c_int(hadamard_block), ctypes.c_int(bits), ctypes.c_float(clip_ratio),
-                                   _ptr(codes), _ptr(delta), _stream()), fn_name)
-    return codes, delta
+        g = 0 if mult_g is None else mult_g.data_ptr()
+    return _result(_native().quantize_act(x, g, hadamard_block, bits, clip_ratio, codes, delta, 1 if fold_after else 0),
+                   "fq_quantize_act_after" if fold_after else "fq_quantize_act")
 
 
 def workspace_bytes(M: int, K: int, N: int, bits: int) -> int:
@@ -288,44 +299,20 @@ def _workspace(M: int, W: Weights, workspace: Optional[torch.Tensor], device) ->
     return workspace
 
 
-def _gemm(fn_name: str, a_codes, a_delta, W: Weights, out_dtype, y, workspace):
-    M = a_codes.shape[0]
-    if y is None:
-        y = torch.empty((M, W.N), dtype=out_dtype, device=a_codes.device)
-    ws = _workspace(M, W, workspace, a_codes.device)
-    fn = getattr(lib(), fn_name)
-    _check(fn(_ptr(a_codes), _ptr(a_delta), ctypes.c_int64(M), W.handle, _ptr(y), _out_dt(y.dtype),
-              ctypes.c_int64(y.stride(0)), _ptr(ws), ctypes.c_size_t(ws.numel()), _stream()), fn_name)
-    return y
-
-
 def gemm_w4a4(a_codes, a_delta, W: Weights, out_dtype=torch.float32, y=None, workspace=None):
-    return _gemm("fq_gemm_w4a4", a_codes, a_delta, W, out_dtype, y, workspace)
+    return _result(_native().gemm(a_codes, a_delta, W.address, W.K, W.N, W.bits, 4, out_dtype, y, workspace), "fq_gemm_w4a4")
 
 
 def gemm_w8a8(a_codes, a_delta, W: Weights, out_dtype=torch.float32, y=None, workspace=None):
-    return _gemm("fq_gemm_w8a8", a_codes, a_delta, W, out_dtype, y, workspace)
-
-
-def _linear(fn_name: str, x, W: Weights, clip_ratio, out_dtype, y, workspace):
-    x = _rowmajor(x)
-    M = x.shape[0]
-    if y is None:
-        y = torch.empty((M, W.N), dtype=out_dtype, device=x.device)
-    ws = _workspace(M, W, workspace, x.device)
-    fn = getattr(lib(), fn_name)
-    _check(fn(_ptr(x), _dt(x), ctypes.c_int64(M), ctypes.c_int64(x.stride(0)), W.handle, ctypes.c_float(clip_ratio),
-              _ptr(y), _out_dt(y.dtype), ctypes.c_int64(y.stride(0)), _ptr(ws), ctypes.c_size_t(ws.numel()),
-              _stream()), fn_name)
-    return y
+    return _result(_native().gemm(a_codes, a_delta, W.address, W.K, W.N, W.bits, 8, out_dtype, y, workspace), "fq_gemm_w8a8")
 
 
 def linear_w4a4(x, W: Weights, clip_ratio: float = 1.0, out_dtype=torch.float32, y=None, workspace=None):
-    return _linear("fq_linear_w4a4", x, W, clip_ratio, out_dtype, y, workspace)
+    return _result(_native().linear(x, W.address, W.K, W.N, W.bits, 4, clip_ratio, out_dtype, y, workspace, -1), "fq_linear_w4a4")
 
 
 def linear_w8a8(x, W: Weights, clip_ratio: float = 1.0, out_dtype=torch.float32, y=None, workspace=None):
-    return _linear("fq_linear_w8a8", x, W, clip_ratio, out_dtype, y, workspace)
+    return _result(_native().linear(x, W.address, W.K, W.N, W.bits, 8, clip_ratio, out_dtype, y, workspace, -1), "fq_linear_w8a8")
 
 
 STATIC_MAX_CODE_BYTES = 4 << 20
@@ -366,27 +353,13 @@ def quantize_act_gated(gate_up: torch.Tensor, act: int, mult_g, hadamard_block: 
 def linear_gated(gate_up: torch.Tensor, act: int, W: Weights, clip_ratio: float = 1.0, out_dtype=torch.float32, y=None,
                  workspace=None):
     """down_proj with the gate product fused into its prologue: y = linear(act(gate) * up)."""
-    gate_up = _rowmajor(gate_up)
-    M = gate_up.shape[0]
-    if y is None:
-        y = torch.empty((M, W.N), dtype=out_dtype, device=gate_up.device)
-    ws = _workspace(M, W, workspace, gate_up.device)
-    _check(lib().fq_linear_gated(_ptr(gate_up), _dt(gate_up), ctypes.c_int64(M), ctypes.c_int64(gate_up.stride(0)),
-                                 ctypes.c_int(act), W.handle, ctypes.c_float(clip_ratio), _ptr(y), _out_dt(y.dtype),
-                                 ctypes.c_int64(y.stride(0)), _ptr(ws), ctypes.c_size_t(ws.numel()), _stream()),
-           "fq_linear_gated")
-    return y
+    return _result(_native().linear(gate_up, W.address, W.K, W.N, W.bits, W.bits, clip_ratio, out_dtype, y, workspace, act),
+                   "fq_linear_gated")
 
 
 def linear_w4a16(x, W: Weights, out_dtype=torch.float32, y=None):
     """Weight-only 4-bit projection of float activations: y = s^W (qW x) + b (no quantization of x)."""
-    x = _rowmajor(x)
-    M = x.shape[0]
-    if y is None:
-        y = torch.empty((M, W.N), dtype=out_dtype, device=x.device)
-    _check(lib().fq_linear_w4a16(_ptr(x), _dt(x), ctypes.c_int64(M), ctypes.c_int64(x.stride(0)), W.handle,
-                                 _ptr(y), _out_dt(y.dtype), ctypes.c_int64(y.stride(0)), _stream()), "fq_linear_w4a16")
-    return y
+    return _result(_native().linear_w4a16(x, W.address, W.N, out_dtype, y), "fq_linear_w4a16")
 
 
 def linear(x, W: Weights, clip_ratio: float = 1.0, out_dtype=torch.float32, y=None, workspace=None):
