@@ -72,33 +72,6 @@ struct RawRow<__nv_bfloat16, E> {
     }
 };
 
-// Gate non-linearity of a gated MLP in fixed binary32 arithmetic: act(x) = x * sigmoid(k), k = x (SiLU) or
-// k = 2 sqrt(2/pi) (x + 0.044715 x^3) (GELU, tanh form).  exp(-k): argument clamped to [-87, 88], n = rint(a log2e),
-// two-step reduction by ln2, degree-6 Taylor polynomial in Horner form, times 2^n from its exponent bits.  The
-// product act(gate) * up feeds a quantizer, so every operation and its order are part of the definition.
-__device__ __forceinline__ float exp_fixed(float a) {
-    a = fminf(fmaxf(a, -87.0f), 88.0f);
-    const float n = rintf(__fmul_rn(a, 1.44269504f));
-    float r = __fmaf_rn(n, -0.693145752f, a);
-    r = __fmaf_rn(n, -1.42860677e-06f, r);
-    float p = 1.38888892e-03f;
-    p = __fmaf_rn(p, r, 8.33333377e-03f);
-    p = __fmaf_rn(p, r, 4.16666679e-02f);
-    p = __fmaf_rn(p, r, 1.66666672e-01f);
-    p = __fmaf_rn(p, r, 0.5f);
-    p = __fmaf_rn(p, r, 1.0f);
-    p = __fmaf_rn(p, r, 1.0f);
-    return __fmul_rn(p, __int_as_float(((int)n + 127) << 23));
-}
-__device__ __forceinline__ float gate_act(float x, int kind) {
-    float k = x;
-    if (kind == 1) {
-        const float x3 = __fmul_rn(__fmul_rn(x, x), x);
-        k = __fmul_rn(1.59576917f, __fmaf_rn(0.044715f, x3, x));
-    }
-    return __fdiv_rn(x, __fadd_rn(1.0f, exp_fixed(-k)));
-}
-
 // FMT: 0 = two 4-bit codes per byte, 1 = one int8 per code.  CLAMP: clip_ratio < 1.
 // GATED (lean variant only): the row is [gate | up] with 2K columns and the kernel's input is
 // act(gate) * up (the site behind a gated MLP), gate_kind 0 = SiLU, 1 = GELU-tanh.
@@ -164,7 +137,17 @@ transform_quantize_kernel(const XT* __restrict__ x, int64_t rows, int K, int64_t
                 float u[E];
                 up.widen(u);
 #pragma unroll
-                for (int i = 0; i < E; ++i) v[i] = __fmul_rn(gate_act(v[i], gate_kind), u[i]);
+                for (int i = 0; i < E; i += 8) {
+                    float2 gp[4], upp[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        gp[j] = make_float2(v[i + 2 * j], v[i + 2 * j + 1]);
+                        upp[j] = make_float2(u[i + 2 * j], u[i + 2 * j + 1]);
+                    }
+                    gate_product<4>(gp, upp, gate_kind);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) { v[i + 2 * j] = gp[j].x; v[i + 2 * j + 1] = gp[j].y; }
+                }
             }
             if (mult != nullptr && col_ok && !mult_after) {
 #pragma unroll
@@ -428,13 +411,17 @@ cudaError_t launch_transform_quantize(const void* x, fq_dtype xt, int64_t rows, 
 }
 
 // The site behind a gated MLP: x is [rows, 2K] = [gate | up], the quantizer's input is act(gate) * up.
-// Always the register kernel's lean variant (the streaming kernel has no gated form).
 cudaError_t launch_gated_transform_quantize(const void* x, fq_dtype xt, int64_t rows, int64_t K, int64_t ldx, int gate_kind,
                                             const float* mult, float cnorm, bool mult_after_rotation, int block, int qmax,
                                             float clip_ratio, StoreFmt fmt, void* codes, float* delta, cudaStream_t stream) {
     if (rows == 0) return cudaSuccess;
     const int k = (int)K;
     const int after = mult_after_rotation ? 1 : 0;
+    {
+        const cudaError_t e = launch_transform_quantize_ring(x, xt, rows, K, ldx, mult, cnorm, after != 0, block, qmax, clip_ratio,
+                                                             fmt, codes, delta, stream, gate_kind);
+        if (e != cudaErrorNotSupported) return e;
+    }
     if (xt == FQ_F32) {
         const float* p = static_cast<const float*>(x);
         if (fmt == StoreFmt::Nibble) return launch_t<float, 0>(p, rows, k, ldx, mult, cnorm, after, block, qmax, clip_ratio, codes, delta, stream, gate_kind);

@@ -104,10 +104,15 @@ struct RingParams {
     int depth;         // ring slots per group
     uint32_t slot_bytes;
     uint32_t g_bytes;  // bytes of the multiplier stage (0 if no multiplier)
+    uint32_t up_bytes; // gated sites: the row's up half starts so many bytes into its slot, and at this line of the row
+    int up_line;
+    int gate_kind;
     uint32_t* watchdog;
 };
 
-template <typename XT, int FMT, bool CLAMP, int E, int BLOCK, bool AFTER, int THREADS = kThreads>
+// GATED: a row is [gate | up], 2K bf16 channels in one slot; the transform's input is act(gate) * up, formed as the row is
+// read from shared memory.
+template <typename XT, int FMT, bool CLAMP, int E, int BLOCK, bool AFTER, bool GATED, int THREADS = kThreads>
 __global__ void __launch_bounds__(THREADS, 1)
 transform_quantize_ring_kernel(const __grid_constant__ CUtensorMap map_x, const RingParams p) {
     constexpr int H = E / 2;                       // channels per half: v[i] = (channel i, channel i + H)
@@ -142,7 +147,7 @@ transform_quantize_ring_kernel(const __grid_constant__ CUtensorMap map_x, const 
     const int first = group * (int)gridDim.x + (int)blockIdx.x;   // rows < 2^31 (checked by the launcher)
     const int step = (int)gridDim.x * ngroups;
     const int rows = (int)p.rows;
-    const uint32_t tx = (uint32_t)p.K * (uint32_t)sizeof(XT);
+    const uint32_t tx = (uint32_t)p.K * (uint32_t)sizeof(XT) * (GATED ? 2u : 1u);
     const uint32_t slot0 = base + slots_off + (uint32_t)(group * p.depth) * p.slot_bytes;
     uint64_t* full0 = &s_full[group * p.depth];
 
@@ -155,6 +160,7 @@ transform_quantize_ring_kernel(const __grid_constant__ CUtensorMap map_x, const 
             if (r < rows) {
                 mbar_arrive_expect_tx(smem_u32(&full0[d]), tx);
                 tma_load_3d(slot0 + d * p.slot_bytes, &map_x, 0, 0, r, smem_u32(&full0[d]));
+                if (GATED) tma_load_3d(slot0 + d * p.slot_bytes + p.up_bytes, &map_x, 0, p.up_line, r, smem_u32(&full0[d]));
                 ++issued;
             }
         }
@@ -199,19 +205,27 @@ transform_quantize_ring_kernel(const __grid_constant__ CUtensorMap map_x, const 
         pin_after_wait(x0);
         pin_after_wait(x1);
         auto load_row = [&]() {
-            if (sizeof(XT) == 2) {
+            auto widen = [](const uint4& lo, const uint4& hi, float2* out) {      // 8 pairs (channel of lo, channel of hi)
+                const uint32_t wl[4] = {lo.x, lo.y, lo.z, lo.w}, wh[4] = {hi.x, hi.y, hi.z, hi.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    out[2 * j + 0] = make_float2(__uint_as_float(wl[j] << 16), __uint_as_float(wh[j] << 16));
+                    out[2 * j + 1] = make_float2(__uint_as_float(wl[j] & 0xffff0000u), __uint_as_float(wh[j] & 0xffff0000u));
+                }
+            };
+            if (GATED) {
+#pragma unroll
+                for (int i = 0; i < H / 8; ++i) {
+                    float2 u[8];
+                    widen(lds128(piece(x0, x1, i)), lds128(piece(x0, x1, i + H / 8)), v + 8 * i);
+                    widen(lds128(piece(x0 + p.up_bytes, x1 + p.up_bytes, i)), lds128(piece(x0 + p.up_bytes, x1 + p.up_bytes, i + H / 8)), u);
+                    gate_product<8>(v + 8 * i, u, p.gate_kind);
+                }
+            } else if (sizeof(XT) == 2) {
                 // bf16: 8 channels per 16-byte piece; pieces [0, H/8) are the low half, the rest the high half
 #pragma unroll
                 for (int i = 0; i < H / 8; ++i) {
-                    const uint4 lo = lds128(piece(x0, x1, i));
-                    const uint4 hi = lds128(piece(x0, x1, i + H / 8));
-                    const uint32_t wl[4] = {lo.x, lo.y, lo.z, lo.w}, wh[4] = {hi.x, hi.y, hi.z, hi.w};
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        v[8 * i + 2 * j + 0] = make_float2(__uint_as_float(wl[j] << 16), __uint_as_float(wh[j] << 16));
-                        v[8 * i + 2 * j + 1] = make_float2(__uint_as_float(wl[j] & 0xffff0000u),
-                                                           __uint_as_float(wh[j] & 0xffff0000u));
-                    }
+                    widen(lds128(piece(x0, x1, i)), lds128(piece(x0, x1, i + H / 8)), v + 8 * i);
                 }
             } else {
 #pragma unroll
@@ -313,6 +327,7 @@ transform_quantize_ring_kernel(const __grid_constant__ CUtensorMap map_x, const 
                 fence_proxy_async_smem();
                 mbar_arrive_expect_tx(smem_u32(&full0[d]), tx);
                 tma_load_3d(slot0 + d * p.slot_bytes, &map_x, 0, 0, nr, smem_u32(&full0[d]));
+                if (GATED) tma_load_3d(slot0 + d * p.slot_bytes + p.up_bytes, &map_x, 0, p.up_line, nr, smem_u32(&full0[d]));
                 ++issued;
             }
         }
@@ -377,7 +392,7 @@ transform_quantize_ring_kernel(const __grid_constant__ CUtensorMap map_x, const 
     }
 }
 
-template <typename XT, int FMT, int E, int BLOCK>
+template <typename XT, int FMT, int E, int BLOCK, bool GATED = false>
 cudaError_t launch_ring(const CUtensorMap& map, const RingParams& p, int grid, size_t smem, cudaStream_t stream) {
     constexpr int THREADS = threads_for(E);
     auto go = [&](auto kern) -> cudaError_t {
@@ -385,24 +400,27 @@ cudaError_t launch_ring(const CUtensorMap& map, const RingParams& p, int grid, s
         if (e != cudaSuccess) return e;
         return launch_pdl(kern, (unsigned)grid, (unsigned)THREADS, smem, stream, 1u, map, p);
     };
-    // (the fold-after variant is its own instantiation: as a run-time branch it cost the default
-    // path registers, and spills, in the 64-channels-per-thread kernels)
-    if (p.mult_after) {
-        if (p.clip_ratio < 1.0f) return go(transform_quantize_ring_kernel<XT, FMT, true, E, BLOCK, true, THREADS>);
-        return go(transform_quantize_ring_kernel<XT, FMT, false, E, BLOCK, true, THREADS>);
+    // (the fold-after variant is its own instantiation: as a run-time branch it cost the default path registers, and spills,
+    // in the 64-channels-per-thread kernels; it has no gated form, nor one for 64 channels with shuffle stages)
+    if constexpr (!GATED && (E == 32 || BLOCK <= 64)) {
+        if (p.mult_after) {
+            if (p.clip_ratio < 1.0f) return go(transform_quantize_ring_kernel<XT, FMT, true, E, BLOCK, true, false, THREADS>);
+            return go(transform_quantize_ring_kernel<XT, FMT, false, E, BLOCK, true, false, THREADS>);
+        }
     }
-    if (p.clip_ratio < 1.0f) return go(transform_quantize_ring_kernel<XT, FMT, true, E, BLOCK, false, THREADS>);
-    return go(transform_quantize_ring_kernel<XT, FMT, false, E, BLOCK, false, THREADS>);
+    if (p.mult_after) return cudaErrorNotSupported;
+    if (p.clip_ratio < 1.0f) return go(transform_quantize_ring_kernel<XT, FMT, true, E, BLOCK, false, GATED, THREADS>);
+    return go(transform_quantize_ring_kernel<XT, FMT, false, E, BLOCK, false, GATED, THREADS>);
 }
 
-template <typename XT, int FMT, int E>
+template <typename XT, int FMT, int E, bool GATED = false>
 cudaError_t launch_ring_block(int block, const CUtensorMap& map, const RingParams& p, int grid, size_t smem,
                               cudaStream_t stream) {
     switch (block) {
-        case 32: return launch_ring<XT, FMT, E, 32>(map, p, grid, smem, stream);
-        case 64: return launch_ring<XT, FMT, E, 64>(map, p, grid, smem, stream);
-        case 128: return launch_ring<XT, FMT, E, 128>(map, p, grid, smem, stream);
-        case 256: return launch_ring<XT, FMT, E, 256>(map, p, grid, smem, stream);
+        case 32: return launch_ring<XT, FMT, E, 32, GATED>(map, p, grid, smem, stream);
+        case 64: return launch_ring<XT, FMT, E, 64, GATED>(map, p, grid, smem, stream);
+        case 128: return launch_ring<XT, FMT, E, 128, GATED>(map, p, grid, smem, stream);
+        case 256: return launch_ring<XT, FMT, E, 256, GATED>(map, p, grid, smem, stream);
         default: return cudaErrorNotSupported;
     }
 }
@@ -419,7 +437,8 @@ cudaError_t launch_ring_e(int e, int block, const CUtensorMap& map, const RingPa
 cudaError_t launch_transform_quantize_ring(const void* x, fq_dtype xt, int64_t rows, int64_t K, int64_t ldx,
                                            const float* mult, float cnorm, bool mult_after_rotation, int block,
                                            int qmax, float clip_ratio, StoreFmt fmt, void* codes, float* delta,
-                                           cudaStream_t stream) {
+                                           cudaStream_t stream, int gate_kind) {
+    const bool gated = gate_kind >= 0;
     const size_t esz = xt == FQ_BF16 ? 2 : 4;
     const size_t row_bytes = (size_t)K * esz;
     // shape gate: whole 128-byte lines, at most 256 of them per box, blocks of 32..256 channels
@@ -429,17 +448,24 @@ cudaError_t launch_transform_quantize_ring(const void* x, fq_dtype xt, int64_t r
     // Short batches are latency-bound and go to the register kernel, which spreads a row over more threads: fewer
     // than 8 rows per SM, unless the rows are long (measured at M = 816: K = 2048 6.4 us there against 7.1-7.9 us
     // here, K = 16384 24.3 us there against 21.2 us here).
-    if (rows < 2 * (int64_t)sms || (rows < 8 * (int64_t)sms && K < 8192)) return cudaErrorNotSupported;
+    if (gated) {
+        // Gated sites: from two rows per SM on, or long rows.  Prologue alone, GELU, 8-bit codes, operands from memory, here /
+        // register kernel: M = 816, K = 2048 4.6 / 5.7 us, K = 8192 14.0 / 16.0, K = 16384 25.9 / 37.7 (66 before the paired
+        // gate arithmetic); M = 148, K = 8192 4.1 / 3.9, K = 16384 7.0 / 8.5.
+        if (xt != FQ_BF16 || (mult != nullptr && mult_after_rotation) || (rows < 2 * (int64_t)sms && K <= 8192))
+            return cudaErrorNotSupported;
+    } else if (rows < 2 * (int64_t)sms || (rows < 8 * (int64_t)sms && K < 8192)) return cudaErrorNotSupported;
 
     // channels per thread (the fold-after variant with shuffle stages does not fit 64 without spills)
-    const int e = (K >= 2048 && K % 64 == 0 && !(mult != nullptr && mult_after_rotation && block >= 128)) ? 64 : 32;
+    const int e = (!gated && K >= 2048 && K % 64 == 0 && !(mult != nullptr && mult_after_rotation && block >= 128)) ? 64 : 32;
     const int threads = threads_for(e);
     int gw = 1;
     while ((int64_t)gw * 32 * e < K) gw <<= 1;
     if (gw > threads / 32) return cudaErrorNotSupported;
     const int ngroups = (threads / 32) / gw;
     if (gw > 1 && ngroups > 15) return cudaErrorNotSupported;      // one named barrier per group
-    const size_t slot = (row_bytes + 1023) / 1024 * 1024;
+    const size_t half = (row_bytes + 1023) / 1024 * 1024;
+    const size_t slot = gated ? 2 * half : half;
     const size_t g_bytes = mult ? ((size_t)K * 4 + 1023) / 1024 * 1024 : 0;
     const size_t budget = 227 * 1024 - 2048 - 1024;
     if (g_bytes + 2 * slot * ngroups > budget) return cudaErrorNotSupported;
@@ -448,7 +474,7 @@ cudaError_t launch_transform_quantize_ring(const void* x, fq_dtype xt, int64_t r
     if (depth < 2 || ngroups * depth > kMaxSlots) return cudaErrorNotSupported;
 
     CUtensorMap map;
-    const uint64_t dims[3] = {128 / esz, row_bytes / 128, (uint64_t)rows};
+    const uint64_t dims[3] = {128 / esz, row_bytes / 128 * (gated ? 2 : 1), (uint64_t)rows};
     const uint64_t strides[2] = {128, (uint64_t)ldx * esz};
     const uint32_t box[3] = {(uint32_t)(128 / esz), (uint32_t)(row_bytes / 128), 1};
     if (!encode_tiled(&map, xt == FQ_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, x,
@@ -458,6 +484,7 @@ cudaError_t launch_transform_quantize_ring(const void* x, fq_dtype xt, int64_t r
     RingParams p{};
     p.rows = rows; p.K = (int)K; p.cnorm = cnorm; p.qmax = (float)qmax; p.clip_ratio = clip_ratio;
     p.mult = mult; p.mult_after = (mult != nullptr && mult_after_rotation) ? 1 : 0; p.codes = static_cast<uint8_t*>(codes); p.delta = delta; p.gw = gw; p.depth = depth;
+    p.up_bytes = (uint32_t)half; p.up_line = (int)(row_bytes / 128); p.gate_kind = gate_kind;
     p.slot_bytes = (uint32_t)slot; p.g_bytes = (uint32_t)g_bytes;
     p.watchdog = watchdog_device_ptr();
     if (!p.watchdog) return cudaErrorUnknown;
@@ -465,6 +492,11 @@ cudaError_t launch_transform_quantize_ring(const void* x, fq_dtype xt, int64_t r
     // Rows are dealt to the CTAs first and to a CTA's row groups second (row r -> CTA r % grid),
     // so that a short batch spreads over all SMs instead of filling every group of a few CTAs.
     const int grid = (int)(rows < sms ? rows : sms);
+    if (gated) {
+        if (fmt == StoreFmt::Nibble) return launch_ring_block<__nv_bfloat16, 0, 32, true>(block, map, p, grid, smem, stream);
+        if (fmt == StoreFmt::Int8) return launch_ring_block<__nv_bfloat16, 1, 32, true>(block, map, p, grid, smem, stream);
+        return launch_ring_block<__nv_bfloat16, 2, 32, true>(block, map, p, grid, smem, stream);
+    }
     if (xt == FQ_BF16)
     {
         if (fmt == StoreFmt::Nibble) return launch_ring_e<__nv_bfloat16, 0>(e, block, map, p, grid, smem, stream);

@@ -148,7 +148,7 @@ bool encode_tiled(CUtensorMap* map, CUtensorMapDataType dt, uint32_t rank, const
 cudaError_t launch_transform_quantize_ring(const void* x, fq_dtype xt, int64_t rows, int64_t K, int64_t ldx,
                                            const float* mult, float cnorm, bool mult_after_rotation, int block,
                                            int qmax, float clip_ratio, StoreFmt fmt, void* codes, float* delta,
-                                           cudaStream_t stream);
+                                           cudaStream_t stream, int gate_kind = -1);
 
 // Stored composite rotation: u[t][b*beta + i] = sum_j B_b[i][j] * (x (.) diag)[t][perm[b*beta + j]] in binary32,
 // u [rows, K] (pitch K).  beta in {16, 32, 64, 128, 256}; diag may be null.
