@@ -46,6 +46,7 @@
 #include "fq_common.cuh"
 #include "ptx_sm100.cuh"
 #include "act_common.cuh"
+#include "tc_sm100.cuh"
 
 namespace fq {
 
@@ -139,26 +140,12 @@ struct Params {
     int split, split_shift;   // K split: a tile is `split` (power of two) work units, each on a slice of K
     int32_t* partials;   // [tile][slice][bt tokens][128 channels] int32 raw sums of the slices (K split)
     uint32_t* counters;  // [tile] slices finished so far; zeroed by the host before the launch (K split)
+    int slot_first;      // 1: the unpack sets wait for the TMEM slot ahead of the packed stage (see there)
     int delta_vec;       // a_delta is 16-byte aligned: the epilogue may read four steps per load
     uint32_t zero;       // 0, as a run-time value (see the unpack warps' release of a packed stage)
 };
 
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(bar)
-        : "memory");
-}
 // ---- CTA-pair (cta_group::2) helpers -----------------------------------------------------
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void cluster_sync_all() {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 // Arrive on the barrier at the same shared-memory offset in CTA `rank` of the cluster.
 __device__ __forceinline__ void mbar_arrive_cta(uint32_t bar, uint32_t rank) {
     asm volatile(
@@ -175,28 +162,6 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
         "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
         ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(bar & 0xFEFFFFFFu)
         : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-template <int CTAS>
-__device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t cols) {
-    if (CTAS == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(cols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    } else {   // same warp index in both CTAs of the pair, same destination offset
-        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(cols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-    }
-}
-template <int CTAS>
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t cols) {
-    if (CTAS == 1)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
-    else
-        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
 }
 // One k-block of work for the issuing warp, as ONE block of PTX so that the two barrier tests for
 // the NEXT k-block are in flight while this k-block's four MMAs and its commits are issued (their
@@ -271,50 +236,6 @@ __device__ __forceinline__ uint32_t issue_kblock_ss(uint32_t issue, uint32_t d_t
         asm volatile(FQ_ISSUE_HEAD FQ_ISSUE_MMAS("2", "", "") FQ_ISSUE_COMMITS_2 FQ_ISSUE_TAIL FQ_ISSUE_OPERANDS(FQ_CON_L));
     return ready;
 }
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t* r) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
-        "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
-        ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
-          "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]),
-          "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]),
-          "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
-        : "memory");
-}
-// Four TS-form MMAs (one K = 128 atom) from the lane elect.sync picks; no commit: the stage's last atom,
-// issued by issue_kblock_ts right after, commits for both.
-__device__ __forceinline__ void issue_mmas_ts(uint32_t d_tmem, const uint32_t* a, const uint64_t* b, uint32_t idesc,
-                                              uint32_t accumulate) {
-    asm volatile(
-        "{\n\t"
-        ".reg .pred pl, pacc, pt;\n\t"
-        "elect.sync _|pl, 0xffffffff;\n\t"
-        "setp.ne.b32 pacc, %10, 0;\n\t"
-        "setp.eq.b32 pt, %0, %0;\n\t"
-        "@pl tcgen05.mma.cta_group::1.kind::i8 [%0], [%1], %5, %9, pacc;\n\t"
-        "@pl tcgen05.mma.cta_group::1.kind::i8 [%0], [%2], %6, %9, pt;\n\t"
-        "@pl tcgen05.mma.cta_group::1.kind::i8 [%0], [%3], %7, %9, pt;\n\t"
-        "@pl tcgen05.mma.cta_group::1.kind::i8 [%0], [%4], %8, %9, pt;\n\t"
-        "}"
-        ::"r"(d_tmem), "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "l"(b[0]), "l"(b[1]), "l"(b[2]), "l"(b[3]), "r"(idesc),
-          "r"(accumulate)
-        : "memory");
-}
-__device__ __forceinline__ uint4 lds128(uint32_t addr) {
-    uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
-    return v;
-}
-__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-}
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 // 16 TMEM lanes x 16 columns in the layout of a warp-level MMA accumulator: thread T holds, for column groups n = 0, 1,
 //   r[4n + 0], r[4n + 1] = lane T/4,     columns 8n + 2(T%4), 8n + 2(T%4) + 1
 //   r[4n + 2], r[4n + 3] = lane T/4 + 8, the same two columns.
@@ -351,29 +272,6 @@ __device__ __forceinline__ uint32_t scale_pair_bf16(uint32_t a0, uint32_t a1, fl
     uint32_t w;
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(v2.y), "f"(v2.x));
     return w;
-}
-
-// Shared-memory matrix descriptor: K-major operand, 128-byte rows, 128B swizzle,
-// 8-row groups 1024 bytes apart.
-__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((addr & 0x3FFFFu) >> 4);   // start address, 16-byte units
-    d |= (uint64_t)1 << 16;                    // leading byte offset (unused for swizzled K-major)
-    d |= (uint64_t)(1024 >> 4) << 32;          // stride byte offset between 8-row groups
-    d |= (uint64_t)1 << 46;                    // descriptor version of this architecture
-    d |= (uint64_t)2 << 61;                    // 128-byte swizzle
-    return d;
-}
-// Instruction descriptor: s8 x s8 -> s32, both operands K-major, M = m (128, or 256 for a CTA pair), N = n.
-__device__ __forceinline__ uint32_t instr_desc_i8(int m, int n) {
-    return (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
-}
-
-// After an expired wait a producer lets the copies it already issued land before the CTA gives its
-// shared memory back: they complete within microseconds, so a bounded pause suffices.
-__device__ __forceinline__ void drain_after_abort() {
-    const uint64_t t0 = global_timer_ns();
-    while (global_timer_ns() - t0 < 100000ull) __nanosleep(1000);
 }
 
 enum : uint32_t {
@@ -960,17 +858,29 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         while (es >= p.stages) { es -= p.stages; eph ^= 1u; }
         for (int n = uset; n < total_kb && ok; n += kUnpackSets) {
             {
+                bool slot_free = false;
+                if (p.slot_first && m >= 0) {
+                    // A parity wait cannot tell use k of a packed stage from use k - 2.  On a ring of odd length a stage's uses
+                    // alternate between the two sets, and a set that has finished k-block n - 2 only knows that k-block
+                    // n - 2 - stages_w was multiplied, hence that it had landed.  Where the stage's previous use, k-block
+                    // n - stages_p, is later than that, its copy may still be in flight (copies land in any order), and the
+                    // wait below would return at once: stale weights, a stage given back twice, copies still under way when
+                    // the CTA ends (a launch failure with 64-token tiles on a ring of three).  With the TMEM slot free,
+                    // k-block n - stages_w was multiplied, and stages_w <= stages_p.
+                    ok = mbar_wait_all(smem_u32(&s_empty[es]), eph, abort_flag, p.watchdog, kWdUnpackEmpty);
+                    if (!ok) break;
+                    slot_free = true;
+                }
                 ok = mbar_wait_all(smem_u32(&s_full_p[ps]), pph, abort_flag, p.watchdog, kWdUnpackFull);
                 if (!ok) break;
                 const uint32_t src = smem_p + (uint32_t)ps * pk_bytes;     // shared-space address of the stage
                 const uint32_t w_tmem = tmem_base + lane_addr + (uint32_t)(kAccStages * p.bt + ws * kSlotCols);
-                bool slot_free = false;
 #pragma unroll
                 for (int h = 0; h < ATOMS; ++h) {
                     uint4 pk[4];
 #pragma unroll
                     for (int c = 0; c < 4; ++c) pk[c] = lds128(src + h * pk_atom + row_off[c]);
-                    if (h == 0) {
+                    if (h == 0 && !slot_free) {
                         // is the TMEM slot free?  (tested now, needed only after the expansion below)
                         slot_free = m < 0 || mbar_test_wait(smem_u32(&s_empty[es]), eph);
                     }
@@ -1306,6 +1216,10 @@ fq_status launch_gemm_tcgen05(const int8_t* a8, int64_t M, const Weights& W, int
         }
         p.stages = sa;
         p.stages_p = sp;
+        // (see the unpack warps; waiting for the slot first costs nothing measurable, and a ring one shorter is slower:
+        // 64 x 4096 x 8192 10.9 against 11.9 us, 128 x 4096 x 4096 10.5 against 11.4)
+        p.slot_first = sp % kUnpackSets != 0 && sp < stages_w + kUnpackSets ? 1 : 0;
+        if (p.slot_first && stages_w > sp) return FQ_ERR_UNSUPPORTED;      // (no tile comes here)
         smem = sa * a_bytes + sp * pk_bytes + epi_bytes + 1024;
     } else {
         int stages = (int)(budget / (a_bytes + w_bytes));

@@ -7,6 +7,7 @@ import torch
 import oracle
 from helpers import to_dev, to_np
 from paper_2609_24433_b200 import fq, synth
+from test_gpu_parity import assert_fused_stages, make_x
 
 pytestmark = pytest.mark.gpu
 
@@ -34,3 +35,51 @@ def test_gptq_fold_at_the_edges_of_its_kernels(N, K, Mc, block):
     hc, hs, _, _ = fq.fold_weights_gptq(to_dev(W), None, None, to_dev(calib), block, 4, 0.01).export()
     assert np.array_equal(to_np(hs).view(np.uint32), ws.view(np.uint32))
     assert np.array_equal(to_np(hc), wc)
+
+
+@pytest.mark.parametrize("M,K,block,bits,act", [
+    (296, 2048, 32, 4, oracle.SILU),                   # the shortest batch of the streamed gated rows on 148 SMs
+    (295, 2048, 128, 8, oracle.GELU_TANH),             # the longest of the register kernel
+    (3, 8448, 256, 8, oracle.GELU_TANH),               # long rows are streamed at any batch size
+])
+def test_gated_prologue_on_both_sides_of_its_rule(M, K, block, bits, act):
+    rng = np.random.default_rng(M + K)
+    gu = rng.standard_normal((M, 2 * K)).astype(np.float32)
+    gu[:, :K] *= 4.0
+    gu[:, 7:K:97] *= 40.0                              # outlier gates: the clamped ends of the exponential
+    gu[0, :6] = [0.0, -0.0, 3e38, -3e38, 9e37, -9e37]  # ... and what a quarter of the denominator would overflow
+    gu[0, K:K + 6] = [1.0, 1.0, 1e-37, 1e-37, 1e-37, 1e-37]
+    gu = synth.as_dtype(gu, "bf16")
+    want_codes, want_delta = oracle.quantize_act_gated(gu, "bf16", act, None, block, bits, 1.0)
+    codes, delta = fq.quantize_act_gated(to_dev(gu, "bf16"), act, None, block, bits, 1.0)
+    assert np.array_equal(to_np(delta).view(np.uint32), want_delta.view(np.uint32))
+    assert np.array_equal(to_np(codes), want_codes)
+
+
+@pytest.mark.parametrize("M,K,N", [
+    (64, 4096, 8192),      # 64-token tiles of four-atom stages: a packed ring of three, an odd length, for two unpack sets
+    (96, 4096, 2048),      # two-atom stages, ring of five, five TMEM slots
+    (128, 8192, 2048),     # ring of five, four TMEM slots
+])
+def test_odd_packed_rings_return_the_same_bits(M, K, N):
+    """400 launches on rotating weights (so that the copies come from memory and land out of order), all equal to the
+    CUDA-core witness."""
+    g = torch.Generator(device="cuda").manual_seed(3)
+    hs = [fq.weights_import(torch.randint(0, 255, (N, K // 2), dtype=torch.uint8, device="cuda", generator=g),
+                            torch.rand(N, device="cuda", generator=g) + 0.1, None, None, K, 64, 4) for _ in range(10)]
+    x = torch.randn(M, K, device="cuda", generator=g).to(torch.bfloat16)
+    codes, delta = fq.quantize_act(x, None, 64, 4)
+    want = [fq.gemm_simt(codes, delta, h, torch.bfloat16) for h in hs]
+    ws = torch.empty(fq.workspace_bytes(M, K, N, 4), dtype=torch.uint8, device="cuda")
+    ys = [torch.empty(M, N, dtype=torch.bfloat16, device="cuda") for _ in hs]
+    graph = torch.cuda.CUDAGraph()
+    for _ in range(2):
+        for h, y in zip(hs, ys):
+            fq.linear_w4a4(x, h, y=y, workspace=ws)
+    with torch.cuda.graph(graph):
+        for h, y in zip(hs, ys):
+            fq.linear_w4a4(x, h, y=y, workspace=ws)
+    for _ in range(40):
+        graph.replay()
+        for y, w in zip(ys, want):
+            assert torch.equal(y, w)
