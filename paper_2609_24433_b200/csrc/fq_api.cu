@@ -225,13 +225,18 @@ fq_status linear_impl(const void* x, fq_dtype xt, int64_t M, int64_t ldx, const 
     st = carve(workspace, ws_bytes, M, W->K, &ws);
     if (st != FQ_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    const int qmax = bits == 4 ? 7 : 127;
+    if (gate < 0 && g_profile_mark == nullptr) {   // short batches: one launch (a mark wants the two kernels apart)
+        const cudaError_t fe = launch_linear_fused(x, xt, M, ldx, *W, block_norm(W->block), qmax, clip_ratio, y, yt, ldy, ws.a8,
+                                                   ws.delta, s);
+        if (fe != cudaErrorNotSupported) return fe == cudaSuccess ? FQ_OK : FQ_ERR_CUDA;
+    }
     size_t scratch_bytes = 0;
     void* scratch = scratch_of(workspace, ws_bytes, M, W->K, &scratch_bytes);
     st = gemm_prepare(M, *W, scratch, scratch_bytes, s);       // ahead of the prologue: see gemm_prepare
     if (st != FQ_OK) return st;
     // Prologue writes one int8 per code into the workspace (4-bit codes stay in [-7, 7] and are laid
     // out in the channel order the GEMM's nibble unpack gives the weights).
-    const int qmax = bits == 4 ? 7 : 127;
     const StoreFmt fmt = bits == 4 ? StoreFmt::Int8Perm : StoreFmt::Int8;
     // a multiplier that is block^-1/2 in every channel is passed as "none": same products, no vector to stage
     const float* mult = W->mult_const ? nullptr : W->mult_g;

@@ -138,6 +138,12 @@ size_t gemm_scratch_bytes(int64_t M, int64_t N, int64_t K, int bits);
 // entry point ahead of the call's first kernel; a launch_gemm on the same scratch must follow on the same stream.
 fq_status gemm_prepare(int64_t M, const Weights& W, void* scratch, size_t scratch_bytes, cudaStream_t stream);
 
+// The whole runtime path of a short batch in one launch.  Returns cudaErrorNotSupported when the shape does not fit it;
+// the caller then runs prologue and GEMM.  ws_codes [M, K] and ws_delta [M] receive codes and steps (may be null).
+cudaError_t launch_linear_fused(const void* x, fq_dtype xt, int64_t M, int64_t ldx, const Weights& W, float cnorm, int qmax,
+                                float clip_ratio, void* y, fq_dtype yt, int64_t ldy, int8_t* ws_codes, float* ws_delta,
+                                cudaStream_t stream);
+
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no link-time libcuda dependency).
 // dims/box innermost first; strides_bytes has rank-1 entries (dimension 0 is contiguous).
 bool encode_tiled(CUtensorMap* map, CUtensorMapDataType dt, uint32_t rank, const void* ptr, const uint64_t* dims,

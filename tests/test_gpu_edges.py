@@ -83,3 +83,38 @@ def test_odd_packed_rings_return_the_same_bits(M, K, N):
         graph.replay()
         for y, w in zip(ys, want):
             assert torch.equal(y, w)
+
+
+@pytest.mark.parametrize("M,K,N,block,bits,dtype,smooth,clip", [
+    (1, 128, 8, 32, 4, "bf16", False, 1.0),            # one token, one slice, one CTA
+    (16, 256, 136, 256, 8, "f32", True, 0.9),          # a block as wide as a slice
+    (17, 640, 1032, 128, 4, "f32", True, 1.0),         # five units over four CTAs, a ragged channel tile
+    (32, 1024, 3072, 1, 8, "bf16", False, 1.0),        # identity rotation; the last batch of sixteen channels a thread
+    (33, 1024, 1024, 64, 4, "bf16", True, 1.0),        # the first of thirty-two
+    (50, 1792, 4104, 8, 4, "bf16", False, 0.8),        # fourteen units over eight CTAs
+    (64, 2304, 520, 128, 8, "bf16", True, 1.0),        # two rounds of channels in some slices, one in others
+    (64, 4096, 1024, 256, 4, "f32", False, 1.0),       # the longest rows
+    (50, 1024, 18944, 64, 4, "bf16", False, 1.0),      # two tiles per cluster, two CTAs per SM
+    (63, 512, 18952, 64, 8, "f32", False, 1.0),
+])
+def test_one_launch_path_equals_prologue_and_gemm(M, K, N, block, bits, dtype, smooth, clip):
+    """Codes and steps against the oracle, outputs against the two-call route, all bit for bit, three replays of a graph
+    of two calls on one workspace included."""
+    rng = np.random.default_rng(M + K + N)
+    W = torch.from_numpy(synth.draw_weights(rng, N, K)).cuda()
+    s = torch.from_numpy(np.exp(rng.uniform(-1, 1, K)).astype(np.float32)).cuda() if smooth else None
+    h = fq.fold_weights(W, s, torch.randn(N, device="cuda"), block, bits)
+    x = make_x(M, K, dtype, seed=M)
+    x_dev = to_dev(x, dtype)
+    want = oracle.quantize_act(x, dtype, to_np(h.export()[2]), block, bits, clip)
+    for ydt in (torch.float32, torch.bfloat16):
+        y = assert_fused_stages(x_dev, h, clip, ydt, *want)
+    ws = torch.zeros(fq.workspace_bytes(M, K, N, bits), dtype=torch.uint8, device="cuda")
+    x2, ya, yb = x_dev.flip(0).contiguous(), torch.empty_like(y), torch.empty_like(y)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        fq.linear(x_dev, h, clip, y=ya, workspace=ws)
+        fq.linear(x2, h, clip, y=yb, workspace=ws)
+    for _ in range(3):
+        g.replay()
+    assert torch.equal(ya, y) and torch.equal(yb, y.flip(0))
