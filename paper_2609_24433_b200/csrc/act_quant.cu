@@ -369,6 +369,8 @@ __global__ void smooth_scale_kernel(const float* __restrict__ a, const float* __
 // 16 packed bytes (32 codes) per thread -> 32 int8 holding 16*code, each group of 8 channels in the
 // (even channels, odd channels) order of StoreFmt::Int8Perm.
 __global__ void expand_nibbles_kernel(const uint4* __restrict__ packed, int64_t n_vec, uint4* __restrict__ out) {
+    griddep_wait();
+    griddep_launch_dependents();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_vec) return;
     const uint4 p = __ldg(packed + i);
@@ -473,9 +475,8 @@ cudaError_t launch_smooth_scale(const float* a, const float* w, int64_t K, doubl
 cudaError_t launch_expand_nibbles(const void* packed, int64_t rows, int64_t K, void* out, cudaStream_t stream) {
     const int64_t n_vec = rows * K / 32;
     if (n_vec == 0) return cudaSuccess;
-    expand_nibbles_kernel<<<(unsigned)((n_vec + 255) / 256), 256, 0, stream>>>(
-        static_cast<const uint4*>(packed), n_vec, static_cast<uint4*>(out));
-    return cudaGetLastError();
+    return launch_pdl(expand_nibbles_kernel, (unsigned)((n_vec + 255) / 256), 256u, 0, stream, 1u,
+                      static_cast<const uint4*>(packed), n_vec, static_cast<uint4*>(out));
 }
 
 }  // namespace fq
