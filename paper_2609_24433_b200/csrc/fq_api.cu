@@ -517,6 +517,9 @@ fq_status fq_quantize_act_composite(const void* x, fq_dtype xt, int64_t M, int64
     fq_status st = check_arch();
     if (st != FQ_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    const cudaError_t ce = launch_composite_quantize(x, xt, M, K, ldx, mult_g, perm, blocks, block, bits, clip_ratio, codes_out,
+                                                     delta_out, s);
+    if (ce != cudaErrorNotSupported) return ce == cudaSuccess ? FQ_OK : FQ_ERR_CUDA;
     float* u = static_cast<float*>(workspace);
     if (launch_composite_rotate(x, xt, M, K, ldx, mult_g, perm, blocks, block, u, s) != cudaSuccess) return FQ_ERR_CUDA;
     return launch_transform_quantize(u, FQ_F32, M, K, K, nullptr, 1.0f, false, 1, bits == 4 ? 7 : 127, clip_ratio,

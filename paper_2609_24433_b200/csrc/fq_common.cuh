@@ -160,6 +160,10 @@ cudaError_t launch_transform_quantize_ring(const void* x, fq_dtype xt, int64_t r
 // u [rows, K] (pitch K).  beta in {16, 32, 64, 128, 256}; diag may be null.
 cudaError_t launch_composite_rotate(const void* x, fq_dtype xt, int64_t rows, int64_t K, int64_t ldx, const float* diag,
                                     const int32_t* perm, const float* blocks, int beta, float* u, cudaStream_t stream);
+// The same followed by Eq. 5 (canonical codes, per-token steps) in one launch; cudaErrorNotSupported where a row is too long.
+cudaError_t launch_composite_quantize(const void* x, fq_dtype xt, int64_t rows, int64_t K, int64_t ldx, const float* diag,
+                                      const int32_t* perm, const float* blocks, int beta, int bits, float clip_ratio,
+                                      void* codes, float* delta, cudaStream_t stream);
 // *bad_flag (device int) is set to 1 if an entry of perm[K] lies outside [0, K).
 cudaError_t launch_perm_check(const int32_t* perm, int64_t K, int* bad_flag, cudaStream_t stream);
 

@@ -118,3 +118,26 @@ def test_one_launch_path_equals_prologue_and_gemm(M, K, N, block, bits, dtype, s
     for _ in range(3):
         g.replay()
     assert torch.equal(ya, y) and torch.equal(yb, y.flip(0))
+
+
+@pytest.mark.parametrize("M,K,beta,bits,dtype,smooth,lead", [
+    (1, 64, 64, 4, "bf16", False, 0),                  # one token, one item, one CTA
+    (17, 512, 16, 8, "f32", True, 0),                  # the smallest blocks, one token into the second tile
+    (33, 768, 256, 4, "bf16", True, 0),                # blocks of four items, an uneven share of them
+    (700, 1024, 32, 4, "bf16", True, 8),               # more tiles than SMs, rows with a lead
+    (20, 4096, 128, 8, "f32", False, 0),               # binary32 rows of which eight fit
+    (9, 8192, 64, 4, "f32", False, 0),                 # ... and none: the two-kernel form
+    (20, 4096, 128, 8, "bf16", False, 4),              # rows that are not 16-byte aligned
+])
+def test_composite_prologue_at_the_edges_of_its_kernels(M, K, beta, bits, dtype, smooth, lead):
+    rng = np.random.default_rng(M + K)
+    perm, blocks = synth.composite_rotation(K, beta, seed=K)
+    x = make_x(M, K, dtype, seed=M)
+    g = np.exp(rng.uniform(-1, 1, K)).astype(np.float32) if smooth else None
+    want_codes, want_delta = oracle.composite_quantize(x, dtype, g, perm, blocks, bits, 0.9)
+    big = torch.zeros((M, K + 8), dtype=torch.bfloat16 if dtype == "bf16" else torch.float32, device="cuda")
+    x_dev = big[:, lead:lead + K]
+    x_dev.copy_(to_dev(x, dtype))
+    codes, delta = fq.quantize_act_composite(x_dev, to_dev(g), to_dev(perm), to_dev(blocks), bits, 0.9)
+    assert np.array_equal(to_np(delta).view(np.uint32), want_delta.view(np.uint32))
+    assert np.array_equal(to_np(codes), want_codes)
