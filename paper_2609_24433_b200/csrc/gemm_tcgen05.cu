@@ -42,6 +42,7 @@
 #include <string.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "fq_common.cuh"
 #include "ptx_sm100.cuh"
@@ -116,6 +117,8 @@ constexpr int kMaxStages = 16;
 constexpr int kMaxStagesP = 16;
 constexpr int kMaxSplit = 16;          // K slices per tile, at most
 constexpr int kMaxSplitTiles = 1024;   // tiles of a launch that splits K (one counter each, ahead of the partial sums)
+enum : int { kUnsplit = 0, kSplitScratch = 1, kSplitCluster = 2 };
+constexpr int kMaxCluster = 8;         // CTAs of a cluster that share a tile along K, at most
 constexpr size_t kCounterBytes = kMaxSplitTiles * sizeof(uint32_t);
 
 struct Params {
@@ -172,6 +175,7 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
 //   a[4]      A operand of the four K=32 steps: TMEM addresses (TS) or shared-memory descriptors (SS)
 //   bar_stage barrier that frees the k-block's shared-memory (and TMEM weight) stage
 //   bar_acc   barrier "accumulator complete", or 0 when this is not the tile's last k-block
+//   mask      (CTA pairs) cluster ranks of the pair, whose barriers the commits arrive at
 // Returns 1 if both tested phases were complete (0 when `peek` is 0).
 #define FQ_ISSUE_HEAD                                                   \
     "{\n\t"                                                             \
@@ -214,9 +218,8 @@ template <int CTAS>
 __device__ __forceinline__ uint32_t issue_kblock_ts(uint32_t issue, uint32_t d_tmem, const uint32_t* a, const uint64_t* b,
                                                     uint32_t idesc, uint32_t accumulate, uint32_t bar_stage,
                                                     uint32_t bar_acc, uint32_t peek, uint32_t peek_bar_a,
-                                                    uint32_t peek_par_a, uint32_t peek_bar_w, uint32_t peek_par_w) {
+                                                    uint32_t peek_par_a, uint32_t peek_bar_w, uint32_t peek_par_w, uint16_t mask) {
     uint32_t ready;
-    const uint16_t mask = 3;
     if (CTAS == 1)
         asm volatile(FQ_ISSUE_HEAD FQ_ISSUE_MMAS("1", "[", "]") FQ_ISSUE_COMMITS_1 FQ_ISSUE_TAIL FQ_ISSUE_OPERANDS(FQ_CON_R));
     else
@@ -227,9 +230,8 @@ template <int CTAS>
 __device__ __forceinline__ uint32_t issue_kblock_ss(uint32_t issue, uint32_t d_tmem, const uint64_t* a, const uint64_t* b,
                                                     uint32_t idesc, uint32_t accumulate, uint32_t bar_stage,
                                                     uint32_t bar_acc, uint32_t peek, uint32_t peek_bar_a,
-                                                    uint32_t peek_par_a, uint32_t peek_bar_w, uint32_t peek_par_w) {
+                                                    uint32_t peek_par_a, uint32_t peek_bar_w, uint32_t peek_par_w, uint16_t mask) {
     uint32_t ready;
-    const uint16_t mask = 3;
     if (CTAS == 1)
         asm volatile(FQ_ISSUE_HEAD FQ_ISSUE_MMAS("1", "", "") FQ_ISSUE_COMMITS_1 FQ_ISSUE_TAIL FQ_ISSUE_OPERANDS(FQ_CON_L));
     else
@@ -287,7 +289,9 @@ enum : uint32_t {
 // channels (two 128-byte swizzle atoms side by side).  The kernel is bound by instruction issue, and the waits,
 // arrivals, fences and ring arithmetic of every role are paid per stage: twice the channels per stage take a
 // third off the instructions per channel.  (Longer token tiles have no TMEM left for slots twice as wide.)
-template <int BITS, int CTAS, bool SPLIT, int ATOMS = 1>
+// SPLIT: kSplitScratch exchanges the K slices' sums through global scratch, any CTA taking any slice; kSplitCluster gives the
+// slices of a tile to the CTAs of a cluster, one tile per cluster and launch, and exchanges through distributed shared memory.
+template <int BITS, int CTAS, int SPLIT, int ATOMS = 1>
 __global__ void __launch_bounds__(BITS == 4 ? kThreadsW4 : kThreadsW8, 1)
 gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_w,
                     const __grid_constant__ CUtensorMap map_y, const Params p) {
@@ -315,13 +319,15 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_w)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_y)) : "memory");
     }
-    const uint32_t cta_rank = CTAS == 2 ? cluster_ctarank() : 0u;
+    const uint32_t pair_base = CTAS == 2 ? cluster_ctarank() & ~1u : 0u;      // cluster rank of the pair's even CTA
+    const uint32_t cta_rank = CTAS == 2 ? cluster_ctarank() & 1u : 0u;
     const bool leader = cta_rank == 0;
+    constexpr bool kCluster = SPLIT == kSplitCluster;
     // K split: a tile is `split` work units, unit = tile * split + slice, slice s
     // covering k-blocks [s * k_blocks, (s + 1) * k_blocks).  Any CTA takes any unit; the CTA that
     // finishes a tile's last slice adds up the slices' partial sums and runs the epilogue.
-    const int split = SPLIT ? p.split : 1;   // compile-time 1 in the common instantiation
-    const int split_shift = SPLIT ? p.split_shift : 0;
+    const int split = SPLIT != kUnsplit ? p.split : 1;   // compile-time 1 in the common instantiation
+    const int split_shift = SPLIT != kUnsplit ? p.split_shift : 0;
     const int bt_cta = p.bt / CTAS;                 // token rows this CTA loads
 
     // carve dynamic shared memory: [A8 stages][W8 stages][packed stages][epilogue transposers], 1024-byte aligned
@@ -336,6 +342,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     const uint32_t smem_w = smem_a + (uint32_t)p.stages * a_bytes;
     const uint32_t smem_p = smem_w + (BITS == 4 ? 0u : (uint32_t)p.stages * w_bytes);
     const uint32_t smem_e = smem_p + (BITS == 4 ? (uint32_t)p.stages_p * pk_bytes : 0u);
+    const uint32_t smem_sums = smem_e + (uint32_t)(kEpiWarps * kEpiStageBytes);    // cluster split: the other slices' sums
     uint8_t* gen_base = smem_raw + (base - smem_u32(smem_raw));   // generic pointer to `base`
 
     if (threadIdx.x == 0) {
@@ -365,6 +372,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     tc_fence_before();
     __syncthreads();
     if (CTAS == 2) cluster_sync_all();              // the peer's barriers exist before anyone signals them
+    if (kCluster) cluster_arrive();                 // "this CTA exists": awaited before the first remote store
     tc_fence_after();
     const uint32_t tmem_base = s_tmem_base;
     // Everything above is on-chip setup; from here on global memory is touched (activations written
@@ -404,6 +412,71 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     };
     auto kb0_of = [&](int unit) { return (unit & (split - 1)) * k_blocks; };   // first k-block of the unit's slice
 
+    [[maybe_unused]] bool ok = true, waited = false;   // (ok: of the epilogue warps; the other roles have their own)
+    // ---- output of 16 tokens from t on, lane = channel j of this warp's 32 (jq ..): r = integer sums
+    auto emit = [&](uint32_t* r, int64_t tc, int64_t jq, float sw, float bj, uint8_t* xpose) {
+        const int64_t j = jq + lane;
+        const bool j_ok = j < p.N;
+        if (p.out.acc != nullptr) {
+            tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+                if (tc + i < p.M && j_ok) p.out.acc[(tc + i) * p.N + j] = ((int)r[i]) >> p.acc_shift;
+            return;
+        }
+        float d[16];
+        if (tc + 16 <= p.M && p.delta_vec) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float4 q = __ldg(reinterpret_cast<const float4*>(p.out.a_delta + tc) + i);
+                d[4 * i + 0] = q.x; d[4 * i + 1] = q.y; d[4 * i + 2] = q.z; d[4 * i + 3] = q.w;
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) d[i] = tc + i < p.M ? __ldg(p.out.a_delta + tc + i) : 0.0f;
+        }
+        tmem_ld_wait();                          // (the sums may still be on their way)
+        if (p.out.yt == FQ_BF16) {
+            // Transpose 32 channels x 16 tokens through shared memory, then 16-byte stores.  Tokens
+            // go in pairs: packed multiply, packed FMA and one two-way bf16 conversion per pair, the
+            // pair's word (token 2k low, token 2k+1 high) stored at [pair k][channel].  A lane then
+            // reads 8 channels of one pair (32 bytes), splits the two tokens with byte permutes and
+            // writes 8 consecutive channels of each token.
+            uint32_t* xw = reinterpret_cast<uint32_t*>(xpose);
+            const float2 sw2 = make_float2(sw, sw), bj2 = make_float2(bj, bj);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const float2 a2 = make_float2((float)(int)r[2 * k], (float)(int)r[2 * k + 1]);
+                const float2 v2 = f2_fma(a2, f2_mul(make_float2(d[2 * k], d[2 * k + 1]), sw2), bj2);
+                uint32_t w;
+                asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(v2.y), "f"(v2.x));
+                xw[k * 32 + lane] = w;
+            }
+            __syncwarp();
+            __nv_bfloat16* y = static_cast<__nv_bfloat16*>(p.out.y);
+            {
+                const int k = lane >> 2;
+                const int64_t jj = jq + (lane & 3) * 8;
+                const uint4 q0 = *reinterpret_cast<const uint4*>(xw + k * 32 + (lane & 3) * 8);
+                const uint4 q1 = *reinterpret_cast<const uint4*>(xw + k * 32 + (lane & 3) * 8 + 4);
+                uint4 lo, hi;     // token 2k and token 2k + 1, channels jj .. jj + 7
+                lo.x = __byte_perm(q0.x, q0.y, 0x5410); hi.x = __byte_perm(q0.x, q0.y, 0x7632);
+                lo.y = __byte_perm(q0.z, q0.w, 0x5410); hi.y = __byte_perm(q0.z, q0.w, 0x7632);
+                lo.z = __byte_perm(q1.x, q1.y, 0x5410); hi.z = __byte_perm(q1.x, q1.y, 0x7632);
+                lo.w = __byte_perm(q1.z, q1.w, 0x5410); hi.w = __byte_perm(q1.z, q1.w, 0x7632);
+                if (jj < p.N) {
+                    if (tc + 2 * k < p.M) *reinterpret_cast<uint4*>(y + (tc + 2 * k) * p.out.ldy + jj) = lo;
+                    if (tc + 2 * k + 1 < p.M) *reinterpret_cast<uint4*>(y + (tc + 2 * k + 1) * p.out.ldy + jj) = hi;
+                }
+            }
+            __syncwarp();
+        } else {
+            float* y = static_cast<float*>(p.out.y) + tc * p.out.ldy + j;
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+                if (tc + i < p.M && j_ok) y[i * p.out.ldy] = fmaf((float)(int)r[i], d[i] * sw, bj);
+        }
+    };
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
         // The whole warp runs the loop and waits; one lane issues.  (A lone lane looping while its
@@ -455,6 +528,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         // CTA issues the MMAs and commits.
         if (leader) {
             const uint32_t idesc = instr_desc_i8(kTileN * CTAS, p.bt);
+            const uint16_t pair_mask = (uint16_t)(3u << pair_base);   // cluster ranks that a pair's commits arrive at
             int stage = 0, wstage = 0;
             uint32_t phase = 0, wphase = 0;
             int acc_stage = 0;
@@ -508,13 +582,13 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                         const uint32_t at[4] = {w_tmem, w_tmem + 8, w_tmem + 16, w_tmem + 24};
                         r = issue_kblock_ts<CTAS>(0u, d_tmem, at, bd, idesc, accumulate,
                                                   smem_u32(&s_empty[stage]), bar_acc, left > 0 ? 1u : 0u, peek_bar_a, ph1,
-                                                  peek_bar_w, peek_par_w);
+                                                  peek_bar_w, peek_par_w, pair_mask);
                     } else {
                         const uint64_t wdesc = smem_desc_sw128(smem_w + stage * w_bytes);
                         const uint64_t ad[4] = {wdesc, wdesc + 2, wdesc + 4, wdesc + 6};
                         r = issue_kblock_ss<CTAS>(0u, d_tmem, ad, bd, idesc, kb != 0 ? 1u : 0u,
                                                   smem_u32(&s_empty[stage]), bar_acc, left > 0 ? 1u : 0u, peek_bar_a, ph1,
-                                                  peek_bar_w, peek_par_w);
+                                                  peek_bar_w, peek_par_w, pair_mask);
                     }
                     ready = r != 0;
                     stage = s1;
@@ -537,7 +611,6 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         [[maybe_unused]] uint32_t epi_phase = 0;
         [[maybe_unused]] int epi_use = 0;
         [[maybe_unused]] int store_use = 0;             // bulk stores issued by this warp so far (buffer = parity)
-        bool ok = true;
         for (int unit = unit0; unit < num_units && ok; unit += unit_step) {
             const int tile = tile_of(unit);
             const int64_t jq = (int64_t)n_of(tile) * (kTileN * CTAS) + (int64_t)cta_rank * kTileN + quad * 32;   // first channel of this warp
@@ -554,6 +627,32 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             if (k_blocks * ATOMS >= 32) __nanosleep(k_blocks * ATOMS >= 400 ? 20000u : (unsigned)(k_blocks * ATOMS) * 50u);
             ok = mbar_wait_warp_relaxed(smem_u32(&s_acc_full[acc_stage]), acc_phase, abort_flag, p.watchdog, kWdEpilogue);
             if (!ok) break;
+            if (kCluster) {
+                // Token chunk c (16 tokens) is finished by slice c % split of the cluster: the others send it their sums,
+                // [sender][chunk / split][token][channel] there, and all meet at the end of the role code.  (CTA pairs: each
+                // CTA has 128 channels of its own, and exchanges with the CTA of the same parity.)
+                cluster_wait();                  // the cluster's CTAs exist
+                waited = true;
+                tc_fence_after();
+                const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16);
+                const int slice = unit & (split - 1), per = (p.bt / 16 + split - 1) >> split_shift;
+                const uint32_t dst = smem_sums + (uint32_t)(quad * 32 + lane) * 4u;
+                for (int c = half; c < p.bt / 16; c += 2) {
+                    const int owner = c & (split - 1);
+                    if (t0 + c * 16 >= p.M) break;
+                    if (owner == slice) continue;
+                    uint32_t r[16];
+                    tmem_ld16(taddr + (uint32_t)(c * 16), r);
+                    tmem_ld_wait();
+                    const int from = slice - (slice > owner ? 1 : 0);
+                    const uint32_t to = cluster_address(dst + (uint32_t)((from * per + (c >> split_shift)) * 16 * kTileN) * 4u,
+                                                        (uint32_t)owner * CTAS + cta_rank);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) st_cluster(to + (uint32_t)(i * kTileN) * 4u, r[i]);
+                }
+                tc_fence_before();
+                break;                           // one tile per cluster
+            }
             // K split.  Every slice writes its raw int32 sums to its own block of scratch
             // ([tile][slice][bt tokens][128 channels]: a warp's 32 channels of one token are one 128-byte
             // line, coalesced both ways) and then counts itself in; the CTA that counts last adds the other
@@ -561,7 +660,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             const int32_t* part = nullptr;
             const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc_stage * p.bt);
             const int slice = unit & (split - 1);
-            if (split > 1) {
+            if (SPLIT == kSplitScratch && split > 1) {
                 tc_fence_after();
                 // (in a CTA pair each CTA exchanges and counts its own 128 channels of the tile)
                 const int ctile = tile * CTAS + (int)cta_rank;
@@ -601,7 +700,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                     __syncwarp();
                     if (lane == 0) {
                         if (CTAS == 1) mbar_arrive(smem_u32(&s_acc_empty[acc_stage]));
-                        else mbar_arrive_cta(smem_u32(&s_acc_empty[acc_stage]), 0);
+                        else mbar_arrive_cta(smem_u32(&s_acc_empty[acc_stage]), pair_base);
                     }
                     if (++acc_stage == kAccStages) { acc_stage = 0; acc_phase ^= 1u; }
                     continue;
@@ -610,7 +709,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                 part = tile_part;
             }
             tc_fence_after();
-            if (!SPLIT && staged) {
+            if (SPLIT == kUnsplit && staged) {
                 // bf16 outputs.  The accumulators are read as MMA-style fragments (a thread: four channels, two adjacent
                 // tokens of each 8-token group), scaled in packed pairs, stored token-major into a 1 KB buffer of
                 // [16 tokens][32 channels] with two transposing matrix stores, and leave as one tiled bulk store; two
@@ -711,85 +810,20 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 #pragma unroll
                     for (int i = 0; i < 16; ++i) r[i] += (uint32_t)pv[i];
                 }
-                if (p.out.acc != nullptr) {
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        if (tc + i < p.M && j_ok) p.out.acc[(tc + i) * p.N + j] = ((int)r[i]) >> p.acc_shift;
-                    continue;
-                }
-                float d[16];
-                if (tc + 16 <= p.M && p.delta_vec) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const float4 q = __ldg(reinterpret_cast<const float4*>(p.out.a_delta + tc) + i);
-                        d[4 * i + 0] = q.x; d[4 * i + 1] = q.y; d[4 * i + 2] = q.z; d[4 * i + 3] = q.w;
-                    }
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) d[i] = tc + i < p.M ? __ldg(p.out.a_delta + tc + i) : 0.0f;
-                }
-                tmem_ld_wait();
-                if (staged) {
-                    // Transpose 32 channels x 16 tokens through shared memory, then 16-byte stores.  Tokens
-                    // go in pairs: packed multiply, packed FMA and one two-way bf16 conversion per pair, the
-                    // pair's word (token 2k low, token 2k+1 high) stored at [pair k][channel].  A lane then
-                    // reads 8 channels of one pair (32 bytes), splits the two tokens with byte permutes and
-                    // writes 8 consecutive channels of each token.
-                    uint32_t* xw = reinterpret_cast<uint32_t*>(xpose);
-                    const float2 sw2 = make_float2(sw, sw), bj2 = make_float2(bj, bj);
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        const float2 a2 = make_float2((float)(int)r[2 * k], (float)(int)r[2 * k + 1]);
-                        const float2 v2 = f2_fma(a2, f2_mul(make_float2(d[2 * k], d[2 * k + 1]), sw2), bj2);
-                        uint32_t w;
-                        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(v2.y), "f"(v2.x));
-                        xw[k * 32 + lane] = w;
-                    }
-                    __syncwarp();
-                    __nv_bfloat16* y = static_cast<__nv_bfloat16*>(p.out.y);
-                    {
-                        const int k = lane >> 2;
-                        const int64_t jj = jq + (lane & 3) * 8;
-                        const uint4 q0 = *reinterpret_cast<const uint4*>(xw + k * 32 + (lane & 3) * 8);
-                        const uint4 q1 = *reinterpret_cast<const uint4*>(xw + k * 32 + (lane & 3) * 8 + 4);
-                        uint4 lo, hi;     // token 2k and token 2k + 1, channels jj .. jj + 7
-                        lo.x = __byte_perm(q0.x, q0.y, 0x5410); hi.x = __byte_perm(q0.x, q0.y, 0x7632);
-                        lo.y = __byte_perm(q0.z, q0.w, 0x5410); hi.y = __byte_perm(q0.z, q0.w, 0x7632);
-                        lo.z = __byte_perm(q1.x, q1.y, 0x5410); hi.z = __byte_perm(q1.x, q1.y, 0x7632);
-                        lo.w = __byte_perm(q1.z, q1.w, 0x5410); hi.w = __byte_perm(q1.z, q1.w, 0x7632);
-                        if (jj < p.N) {
-                            if (tc + 2 * k < p.M) *reinterpret_cast<uint4*>(y + (tc + 2 * k) * p.out.ldy + jj) = lo;
-                            if (tc + 2 * k + 1 < p.M) *reinterpret_cast<uint4*>(y + (tc + 2 * k + 1) * p.out.ldy + jj) = hi;
-                        }
-                    }
-                    __syncwarp();
-                } else {
-                    float* y = static_cast<float*>(p.out.y) + tc * p.out.ldy + j;
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        const float v = fmaf((float)(int)r[i], d[i] * sw, bj);
-                        if (tc + i < p.M && j_ok) {
-                            if (p.out.yt == FQ_F32)
-                                y[i * p.out.ldy] = v;
-                            else
-                                reinterpret_cast<__nv_bfloat16*>(p.out.y)[(tc + i) * p.out.ldy + j] = __float2bfloat16_rn(v);
-                        }
-                    }
-                }
+                emit(r, tc, jq, sw, bj, xpose);
             }
             }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) {
                 if (CTAS == 1) mbar_arrive(smem_u32(&s_acc_empty[acc_stage]));
-                else mbar_arrive_cta(smem_u32(&s_acc_empty[acc_stage]), 0);   // the even CTA issues the MMAs
+                else mbar_arrive_cta(smem_u32(&s_acc_empty[acc_stage]), pair_base);   // the even CTA issues the MMAs
             }
             if (++acc_stage == kAccStages) { acc_stage = 0; acc_phase ^= 1u; }
         }
         // this warp's stores have read their buffers before the CTA gives up its shared memory (the writes themselves
         // are complete when the grid is: no need to wait for them here, which would add their latency to the tail)
-        if (!SPLIT && staged && lane == 0) bulk_wait_read<0>();
+        if (SPLIT == kUnsplit && staged && lane == 0) bulk_wait_read<0>();
     } else if (BITS == 8) {
         // ------------------------------------------------- TMA producer, int8 weights
         // (converged warp, one issuing lane: see the activation producer)
@@ -919,7 +953,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                 __syncwarp();
                 if (elect_one()) {
                     if (CTAS == 1) mbar_arrive(smem_u32(&s_full_w8[ws]));
-                    else mbar_arrive_cta(smem_u32(&s_full_w8[ws]), 0);
+                    else mbar_arrive_cta(smem_u32(&s_full_w8[ws]), pair_base);
                 }
                 // (every ring has at least kUnpackSets slots: one subtraction brings an index back into range)
                 ps += kUnpackSets;
@@ -966,6 +1000,42 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                 }
             }
             if (!ok && lane == 0) drain_after_abort();
+        }
+    }
+
+    if (kCluster) {
+        __syncwarp();
+        if (!waited) cluster_wait();
+        cluster_arrive();
+        cluster_wait();                              // every CTA's sums are where they belong
+        if (warp >= 2 && warp < 2 + kEpiWarps && ok && unit0 < num_units) {
+            const int quad = warp & 3, half = (warp - 2) >> 2, slice = unit0 & (split - 1);
+            const int tile = tile_of(unit0);
+            const int64_t jq = (int64_t)n_of(tile) * (kTileN * CTAS) + (int64_t)cta_rank * kTileN + quad * 32;
+            const int64_t t0 = (int64_t)m_of(tile) * p.bt;
+            float sw = 0.0f, bj = 0.0f;
+            if (jq + lane < p.N && p.out.acc == nullptr) {
+                sw = __ldg(p.w_scale + jq + lane) * (1.0f / (float)(1 << p.acc_shift));
+                bj = __ldg(p.bias + jq + lane);
+            }
+            const int per = (p.bt / 16 + split - 1) >> split_shift;
+            const int32_t* sums = reinterpret_cast<const int32_t*>(gen_base + (smem_sums - base)) + quad * 32 + lane;
+            uint8_t* xpose = gen_base + (smem_e - base) + (warp - 2) * kEpiStageBytes;
+            tc_fence_after();
+            for (int i = half; i < per; i += 2) {
+                const int c = (i << split_shift) + slice;
+                const int64_t tc = t0 + c * 16;
+                if (c * 16 >= p.bt || tc >= p.M) break;
+                uint32_t r[16];
+                tmem_ld16(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(c * 16), r);
+                tmem_ld_wait();
+                for (int k = 0; k < split - 1; ++k) {
+                    const int32_t* q = sums + (size_t)(k * per + i) * 16 * kTileN;
+#pragma unroll
+                    for (int t = 0; t < 16; ++t) r[t] += (uint32_t)q[t * kTileN];
+                }
+                emit(r, tc, jq, sw, bj, xpose);
+            }
         }
     }
 
@@ -1053,7 +1123,7 @@ fq_status build_weight_tmap(Weights& W) {
 
 namespace {
 
-template <int BITS, int CTAS, bool SPLIT, int ATOMS = 1>
+template <int BITS, int CTAS, int SPLIT, int ATOMS = 1>
 fq_status launch_variant(const CUtensorMap& map_a, const CUtensorMap& map_w, const CUtensorMap& map_y, const Params& p,
                          int grid, size_t smem, int cluster, cudaStream_t stream) {
     auto kern = gemm_tcgen05_kernel<BITS, CTAS, SPLIT, ATOMS>;
@@ -1070,8 +1140,28 @@ struct Plan {
     int bt = 0;       // tokens per tile
     int ctas = 1;     // 2: CTA pairs on 256-channel tiles (cta_group::2)
     int split = 1;    // >1: every tile is that many work units, each on a slice of K
+    bool cluster = false; // the slices of a tile are the CTAs of a cluster (no scratch)
     size_t scratch = 0;   // bytes of scratch the split needs: the tile counters, then the int32 partial tiles
 };
+
+// Atoms (of 128 channels) per pipeline stage.  4-bit weights, single CTAs: two for token tiles of at most 128, four for the
+// shortest (the accumulators of longer tiles leave no room for wider TMEM slots); whole atoms, slices of whole stages.
+int atoms_per_stage(int bits, int ctas, int bt, int64_t K, int split) {
+    const int64_t kb = (K + kBlockK - 1) / kBlockK;
+    if (bits != 4 || ctas != 1 || bt > 128 || K % kBlockK != 0) return 1;
+    if (bt <= 64 && kb >= 4 * split && (split == 1 || kb % (4 * split) == 0)) return 4;
+    return split == 1 || kb % (2 * split) == 0 ? 2 : 1;
+}
+// Shared memory of the pipeline rings; `sums`: bytes taken by the sums of a cluster split.
+size_t ring_budget(size_t sums) { return 227 * 1024 - 1024 /*alignment slack*/ - 1024 /*static*/ - (size_t)kEpiWarps * kEpiStageBytes - sums; }
+size_t stage_bytes(int bits, int ctas, int bt, int atoms) {
+    return ((size_t)(bt / ctas) * kBlockK + (size_t)kTileN * kBlockK * bits / 8) * atoms;
+}
+size_t cluster_sums_bytes(int bt, int split) { return (size_t)(split - 1) * ((bt / 16 + split - 1) / split) * 16 * kTileN * sizeof(int32_t); }
+
+// Clusters of 2, 4 or 8 CTAs, one per SM, that the device holds at a time (a B200: 74, 36, 14 -- its graphics clusters do not
+// divide by eight).
+int cluster_capacity(int ctas);
 
 // Token tile, CTA grouping and K split.  Upper bound of the tile from TMEM: two accumulator stages,
 // plus the unpacked-weight ring for 4-bit weights (2*bt + 3*32 <= 512 columns).  M is split evenly
@@ -1079,19 +1169,22 @@ struct Plan {
 // measured launches (cycles): rounds of work units over the SMs, each unit costing
 //     k_blocks * per_kblock(bt) + 16*bt + 1000          (the tail: epilogue and tile hand-over)
 //   4-bit weights:          per_kblock = 330 + bt       (issue floor, then the MMAs' 2*bt); 235 + bt for tiles of at
-//                                        most 128 tokens, whose stages hold two k-blocks
+//                                        most 128 tokens, whose stages hold two or four k-blocks
 //   8-bit, one CTA:         per_kblock = max(350 + 0.8*bt, 230 + 2*bt)   (issue floor, then shared memory:
 //                                        both operands pass through it)
 //   8-bit, CTA pair:        per_kblock = max(545, 2.62*bt)   (each CTA stages half of the token tile)
 // Pairs gain nothing for 4-bit weights, which never pass through shared memory unpacked.
-// K split (single CTAs, and CTA pairs on 8-bit weights): problems with fewer tiles than SMs and a long K (every short batch; down_proj
-// at M = 816: 64 tiles of 128 k-blocks) make `split` work units of every tile, each on a slice of K; the
-// slices leave int32 partial sums in scratch and the one that finishes last adds them up.  Fitted cost per
-// unit: 12500 + 40*bt cycles, plus 1500 per extra slice -- the constant is what a split costs a call on operands
-// from HBM whatever its size (the node that clears the counters ahead of the prologue, two rendezvous, the
-// round trips of the exchange: 16-25 thousand cycles measured at tiles of 16 and 64 tokens split in 2, 4 and 8,
-// where an earlier model of 1500 + 70*bt chose splits that ran 15-45 % slower than the same tile unsplit).
-Plan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t scratch_avail) {
+// K split: problems with fewer tiles than SMs and a long K (short batches, few output channels).
+//   By clusters of 2, 4 or 8 CTAs (one wave; at least four k-blocks of ring beside the sums, 4-bit tiles of at most 128
+//   tokens): the tail shrinks to 16*bt/split, the exchange costs 2800 + 40 per CTA of the launch at 4 bits, 3300 + 18 at 8
+//   (the more SMs a launch takes, the less of the next one starts beside it), and 500 per extra slice.  Measured, chains of
+//   calls, split against the best unsplit tile: 64 x 16384 x 2048 (M x K x N) 14.5 / 22.5 us at 4 bits and 16.3 / 31.7 at 8;
+//   16 x 16384 x 4096 14.7 / 22.6 and 18.8 / 32.3; 64 x 4096 x 1024 8.6 / 9.9 and 8.0 / 11.1; 64 x 4096 x 4096 10.4 / 10.5
+//   and 10.2 / 11.9; 128 x 4096 x 1024 8.7 / 9.2 and 8.7 / 10.8; 256 x 4096 x 1024 10.5 / 10.1 at 4 bits; CTA pairs,
+//   816 x 16384 x 2048: the site 5 us faster than 96-token tiles.
+//   Through scratch, where the device cannot hold the clusters (CTA pairs on 8-bit weights, too): 12500 + 40*bt + 1500 per
+//   extra slice.
+Plan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t scratch_avail, bool clusters) {
     const int bt_max = bits == 4 ? 208 : 256;
     const int64_t kb = (K + kBlockK - 1) / kBlockK;
     Plan best;
@@ -1099,37 +1192,71 @@ Plan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t scratc
     for (int c = 1; c <= ((bits == 8 && N > kTileN) ? 2 : 1); ++c) {
         const int64_t n_units = (N + kTileN * c - 1) / (kTileN * c);
         for (int mt = (int)((M + bt_max - 1) / bt_max); mt <= (int)((M + 63) / 64); ++mt) {
-            int b = (int)(((M + mt - 1) / mt + 15) / 16 * 16);
+            const int b = (int)(((M + mt - 1) / mt + 15) / 16 * 16);
             if (b > bt_max) continue;
-            // 4-bit weights, token tiles of 32..64 (four-atom stages): kept to the envelope in which that configuration
-            // has run clean under CUDA-graph replay -- at most 64 work units and K <= 4096.  Beyond it (M = 64 at
-            // K = N = 8192 and 16384 ended two benchmark runs with a launch failure whose cause reading has not shown)
-            // the batch is padded to a 128-token tile with two-atom stages: the configuration every mid-size batch runs
-            // (it may split K like any other: 32 tiles of 128 k-blocks are better off as 128 units).
-            if (bits == 4 && b > 16 && b <= 64 && (n_units * ((M + b - 1) / b) > 64 || kb > 32)) {
-                b = 128;
-            }
             const int64_t units = n_units * ((M + b - 1) / b);
             const double w8_single = 350.0 + 0.8 * b > 230.0 + 2.0 * b ? 350.0 + 0.8 * b : 230.0 + 2.0 * b;
-            // 4-bit, tiles of at most 128 tokens: two-atom stages (see the kernel) cost less per 128 channels
+            // 4-bit, tiles of at most 128 tokens: stages of several atoms (see the kernel) cost less per 128 channels
             const double w4 = (c == 1 && b <= 128 && K % kBlockK == 0) ? 235.0 + b : 330.0 + b;
             const double per_kb = bits == 4 ? w4 : (c == 1 ? w8_single : (2.62 * b > 545.0 ? 2.62 * b : 545.0));
-            for (int sp = 1; sp <= ((c == 1 || bits == 8) ? kMaxSplit : 1); sp *= 2) {
-                if (sp > 1 && (kb % sp != 0 || kb / sp < 2 || units * c > kMaxSplitTiles || units * c * sp > 4 * (int64_t)sms)) continue;
-                const int64_t kb_per = kb / sp;
-                const size_t scratch = sp > 1 ? kCounterBytes + (size_t)units * c * sp * kTileN * b * sizeof(int32_t) : 0;
-                if (scratch > scratch_avail) continue;
-                const int slots = sms / c;
-                const double unit_cost = (double)kb_per * per_kb + 16.0 * b + 1000.0 + (sp > 1 ? 12500.0 + 40.0 * b + 1500.0 * (sp - 1) : 0.0);
+            const int slots = sms / c;
+            auto offer = [&](int sp, bool cluster, size_t scratch, double unit_cost) {
                 const double cost = (double)((units * sp + slots - 1) / slots) * unit_cost;
                 if (best.bt == 0 || cost < best_cost * 0.98) {   // ties: the earlier candidate (larger tile, no split)
-                    best.bt = b; best.ctas = c; best.split = sp; best.scratch = scratch;
+                    best.bt = b; best.ctas = c; best.split = sp; best.cluster = cluster; best.scratch = scratch;
                     best_cost = cost;
+                }
+            };
+            offer(1, false, 0, (double)kb * per_kb + 16.0 * b + 1000.0);
+            for (int sp = 2; sp <= kMaxSplit; sp *= 2) {
+                if (kb % sp != 0 || kb / sp < 2) break;
+                const double slice = (double)(kb / sp) * per_kb + 1000.0;
+                const int atoms = atoms_per_stage(bits, c, b, K, sp);
+                const double ctas = (double)(units * sp * c);
+                if (clusters && (bits == 8 || b <= 128) && sp * c <= kMaxCluster && units <= cluster_capacity(sp * c) &&
+                    units * sp <= slots && ring_budget(cluster_sums_bytes(b, sp)) * atoms >= 4 * stage_bytes(bits, c, b, atoms))
+                    offer(sp, true, 0, slice + 16.0 * b / sp + (bits == 4 ? 2800.0 + 40.0 * ctas : 3300.0 + 18.0 * ctas) + 500.0 * (sp - 1));
+                if ((c == 1 || bits == 8) && units * c <= kMaxSplitTiles && units * c * sp <= 4 * (int64_t)sms) {
+                    const size_t scratch = kCounterBytes + (size_t)units * c * sp * kTileN * b * sizeof(int32_t);
+                    if (scratch <= scratch_avail) offer(sp, false, scratch, slice + 16.0 * b + 12500.0 + 40.0 * b + 1500.0 * (sp - 1));
                 }
             }
         }
     }
     return best;
+}
+
+int cluster_capacity(int ctas) {
+    static std::mutex mutex;
+    static int known[64][3];                         // 0: not asked yet, else capacity + 1
+    const int defaults[3] = {74, 36, 14}, i = ctas == 2 ? 0 : (ctas == 4 ? 1 : 2);
+    int dev = 0;
+    if (device_cc_major() != 10 || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+        (void)cudaGetLastError();
+        return defaults[i];
+    }
+    std::lock_guard<std::mutex> lock(mutex);
+    if (known[dev][i] == 0) {
+        const auto kern = gemm_tcgen05_kernel<8, 1, kSplitCluster, 1>;
+        const size_t smem = 224 * 1024;              // one CTA per SM
+        int n = 0;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)ctas, 1, 1);
+        cfg.blockDim = dim3((unsigned)kThreadsW8, 1, 1);
+        cfg.dynamicSmemBytes = smem;
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = (unsigned)ctas; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        if (ensure_dynamic_smem(reinterpret_cast<const void*>(kern), smem) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+            (void)cudaGetLastError();
+            n = 0;
+        }
+        known[dev][i] = n + 1;
+    }
+    return known[dev][i] - 1;
 }
 
 }  // namespace
@@ -1141,8 +1268,8 @@ Plan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t scratc
 // changes at run time.
 fq_status gemm_prepare(int64_t M, const Weights& W, void* scratch, size_t scratch_bytes, cudaStream_t stream) {
     if (M <= 0 || W.N == 0 || scratch == nullptr || gemm_stream_applies(M, W)) return FQ_OK;
-    const Plan plan = plan_gemm(M, W.N, W.K, W.bits, device_sm_count(), scratch_bytes);
-    if (plan.split <= 1) return FQ_OK;
+    const Plan plan = plan_gemm(M, W.N, W.K, W.bits, device_sm_count(), scratch_bytes, true);
+    if (plan.split <= 1 || plan.cluster) return FQ_OK;
     return cudaMemsetAsync(scratch, 0, kCounterBytes, stream) == cudaSuccess ? FQ_OK : FQ_ERR_CUDA;
 }
 
@@ -1156,7 +1283,8 @@ fq_status launch_gemm(const int8_t* a8, int64_t M, const Weights& W, int acc_shi
 
 size_t gemm_scratch_bytes(int64_t M, int64_t N, int64_t K, int bits) {
     if (M <= 0 || N <= 0 || K <= 0) return 0;
-    return plan_gemm(M, N, K, bits, device_sm_count(), (size_t)-1).scratch;
+    // (asked for whether or not this device holds the clusters that would do without: a caller sizes its workspace once)
+    return plan_gemm(M, N, K, bits, device_sm_count(), (size_t)-1, false).scratch;
 }
 
 fq_status launch_gemm_tcgen05(const int8_t* a8, int64_t M, const Weights& W, int acc_shift, const GemmOut& out,
@@ -1167,7 +1295,7 @@ fq_status launch_gemm_tcgen05(const int8_t* a8, int64_t M, const Weights& W, int
     Params p{};
     p.M = M; p.N = W.N; p.K = W.K;
     const int sms = device_sm_count();
-    const Plan plan = plan_gemm(M, W.N, W.K, W.bits, sms, scratch ? scratch_bytes : 0);
+    const Plan plan = plan_gemm(M, W.N, W.K, W.bits, sms, scratch ? scratch_bytes : 0, true);
     const int bt = plan.bt, ctas = plan.ctas, split = plan.split;
     p.split = split;
     p.counters = static_cast<uint32_t*>(scratch);            // cleared by gemm_prepare()
@@ -1185,19 +1313,16 @@ fq_status launch_gemm_tcgen05(const int8_t* a8, int64_t M, const Weights& W, int
     p.out = out;
     p.watchdog = watchdog_device_ptr();
     if (!p.watchdog) return FQ_ERR_CUDA;
-    // 4-bit weights, single CTAs, token tiles of at most 128: two 128-channel atoms per pipeline stage (the
-    // accumulators of longer tiles leave no room for TMEM slots twice as wide).  Needs whole atoms (K a multiple
-    // of 128) and, with a K split, slices of whole stages.
     const int64_t kb128 = (W.K + kBlockK - 1) / kBlockK;
-    int atoms = (W.bits == 4 && ctas == 1 && bt <= 128 && W.K % kBlockK == 0 && (split == 1 || kb128 % (2 * split) == 0)) ? 2 : 1;
-    if (atoms == 2 && bt <= 64 && kb128 >= 4 * split && (split == 1 || kb128 % (4 * split) == 0)) atoms = 4;   // four for the shortest tiles
+    const int atoms = atoms_per_stage(W.bits, ctas, bt, W.K, split);
     // 4-bit weights: every TMEM column the accumulators leave free becomes unpacked-weight ring
     int stages_w = W.bits == 4 ? (512 - kAccStages * bt) / (kColsW * atoms) : 0;
     if (stages_w > kMaxStagesW) stages_w = kMaxStagesW;
     p.tmem_cols = next_pow2(kAccStages * bt + stages_w * kColsW * atoms);
 
-    const size_t epi_bytes = (size_t)kEpiWarps * kEpiStageBytes;
-    const size_t budget = 227 * 1024 - 1024 /*alignment slack*/ - 1024 /*static*/ - epi_bytes;
+    const size_t sums_bytes = plan.cluster ? cluster_sums_bytes(bt, split) : 0;
+    const size_t epi_bytes = (size_t)kEpiWarps * kEpiStageBytes + sums_bytes;
+    const size_t budget = ring_budget(sums_bytes);
     const size_t a_bytes = (size_t)(bt / ctas) * kBlockK * atoms, w_bytes = (size_t)kTileN * kBlockK,
                  pk_bytes = w_bytes / 2 * atoms;
     size_t smem;
@@ -1216,8 +1341,8 @@ fq_status launch_gemm_tcgen05(const int8_t* a8, int64_t M, const Weights& W, int
         }
         p.stages = sa;
         p.stages_p = sp;
-        // (see the unpack warps; waiting for the slot first costs nothing measurable, and a ring one shorter is slower:
-        // 64 x 4096 x 8192 10.9 against 11.9 us, 128 x 4096 x 4096 10.5 against 11.4)
+        // (see the unpack warps; a ring one shorter is slower, one TMEM slot less no faster: 128 x 4096 x 4096 10.5, 11.3 and
+        // 10.4 us, 256 x 2048 x 4096 9.95, 10.1 and 9.9)
         p.slot_first = sp % kUnpackSets != 0 && sp < stages_w + kUnpackSets ? 1 : 0;
         if (p.slot_first && stages_w > sp) return FQ_ERR_UNSUPPORTED;      // (no tile comes here)
         smem = sa * a_bytes + sp * pk_bytes + epi_bytes + 1024;
@@ -1230,6 +1355,10 @@ fq_status launch_gemm_tcgen05(const int8_t* a8, int64_t M, const Weights& W, int
         p.stages_w = 0;
         smem = (a_bytes + w_bytes) * stages + epi_bytes + 1024;
     }
+
+    // One CTA of this kind per SM, and none of the short-batch kernel beside it: a cluster whose CTA waited for tensor memory
+    // must not be what another cluster on that SM waits for (launches of two streams).
+    if (plan.cluster && smem < 152 * 1024) smem = 152 * 1024;
 
     // each CTA of a pair loads its own half of the token tile
     CUtensorMap map_a;
@@ -1255,22 +1384,19 @@ fq_status launch_gemm_tcgen05(const int8_t* a8, int64_t M, const Weights& W, int
     p.kb_per = (int)((kb128 + atoms - 1) / atoms) / split;      // stages per unit; the planner only picks splits that divide it
     p.split_shift = split == 1 ? 0 : (split == 2 ? 1 : (split == 4 ? 2 : (split == 8 ? 3 : 4)));
 
-    if (W.bits == 4) {
-        if (ctas == 2) return launch_variant<4, 2, false>(map_a, W.tmap, map_y, p, grid, smem, 2, stream);
-        if (atoms == 4)
-            return split > 1 ? launch_variant<4, 1, true, 4>(map_a, W.tmap, map_y, p, grid, smem, 1, stream)
-                             : launch_variant<4, 1, false, 4>(map_a, W.tmap, map_y, p, grid, smem, 1, stream);
-        if (atoms == 2)
-            return split > 1 ? launch_variant<4, 1, true, 2>(map_a, W.tmap, map_y, p, grid, smem, 1, stream)
-                             : launch_variant<4, 1, false, 2>(map_a, W.tmap, map_y, p, grid, smem, 1, stream);
-        return split > 1 ? launch_variant<4, 1, true>(map_a, W.tmap, map_y, p, grid, smem, 1, stream)
-                         : launch_variant<4, 1, false>(map_a, W.tmap, map_y, p, grid, smem, 1, stream);
-    }
-    if (ctas == 2)
-        return split > 1 ? launch_variant<8, 2, true>(map_a, W.tmap, map_y, p, grid, smem, 2, stream)
-                         : launch_variant<8, 2, false>(map_a, W.tmap, map_y, p, grid, smem, 2, stream);
-    return split > 1 ? launch_variant<8, 1, true>(map_a, W.tmap, map_y, p, grid, smem, 1, stream)
-                     : launch_variant<8, 1, false>(map_a, W.tmap, map_y, p, grid, smem, 1, stream);
+    const int cluster = plan.cluster ? split * ctas : ctas;
+    auto go = [&](auto bits, auto pair, auto atoms_c) -> fq_status {
+        constexpr int B = decltype(bits)::value, C = decltype(pair)::value, A = decltype(atoms_c)::value;
+        if (split == 1) return launch_variant<B, C, kUnsplit, A>(map_a, W.tmap, map_y, p, grid, smem, cluster, stream);
+        if (plan.cluster) return launch_variant<B, C, kSplitCluster, A>(map_a, W.tmap, map_y, p, grid, smem, cluster, stream);
+        return launch_variant<B, C, kSplitScratch, A>(map_a, W.tmap, map_y, p, grid, smem, cluster, stream);
+    };
+    using I1 = std::integral_constant<int, 1>;
+    using I2 = std::integral_constant<int, 2>;
+    using I4 = std::integral_constant<int, 4>;
+    using I8 = std::integral_constant<int, 8>;
+    if (W.bits == 4) return atoms == 4 ? go(I4(), I1(), I4()) : (atoms == 2 ? go(I4(), I1(), I2()) : go(I4(), I1(), I1()));
+    return ctas == 2 ? go(I8(), I2(), I1()) : go(I8(), I1(), I1());
 }
 
 }  // namespace fq

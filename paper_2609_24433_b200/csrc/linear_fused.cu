@@ -410,8 +410,8 @@ struct FusedPlan {
 
 // At most 64 tokens, in one wave of CTAs.  In a chain of calls (graph replays, weights from memory; one launch against two):
 // 1024 x 1024: M = 8 3.8 / 4.2 us, M = 32 5.0 / 6.0, M = 50 5.8 / 6.8; K = 2048, N = 1024: M = 32 5.3 / 7.1, M = 50 6.7 / 8.1;
-// K = 4096, N = 1024: M = 16 5.4 / 6.3, M = 32 6.4 / 9.0; the largest grids are even (1024 x 4096: M = 32 6.1 / 6.2).  An
-// eager call costs the host 5.4 us instead of 7.7.  CTAs of two rounds share an SM with nobody and clusters of eight do not
+// K = 4096, N = 1024: M = 16 5.4 / 6.3, M = 32 6.4 / 9.0; the largest grids are even (1024 x 4096: M = 32 6.1 / 6.2), and
+// behind with few tokens (8 bits, M = 1 4.5 / 4.0): 96 CTAs at most there.  An eager call costs the host 5.4 us instead of 7.7.  CTAs of two rounds share an SM with nobody and clusters of eight do not
 // fill the chip, so that 128 of them would take two waves (K = 4096, N = 2048: 10.3 / 6.3): 96 at most.
 FusedPlan plan_fused(int64_t M, const Weights& W, bool mult) {
     FusedPlan f;
@@ -425,7 +425,7 @@ FusedPlan plan_fused(int64_t M, const Weights& W, bool mult) {
     while (shift < 3 && slice(shift) > round) ++shift;
     if (slice(shift) > 2 * round) return f;
     const int64_t grid = ((W.N + kTile - 1) / kTile) << shift;
-    if (grid > (slice(shift) > round ? 96 : device_sm_count())) return f;
+    if (grid > (slice(shift) > round || M <= 8 ? 96 : device_sm_count())) return f;
     f.ctas_shift = shift; f.unit = unit; f.units = units; f.slice = slice(shift); f.grid = (int)grid;
     f.rounds = f.slice > round ? 2 : 1;
     const size_t w_bytes = (size_t)kTile * f.slice * W.bits / 8;

@@ -141,3 +141,30 @@ def test_composite_prologue_at_the_edges_of_its_kernels(M, K, beta, bits, dtype,
     codes, delta = fq.quantize_act_composite(x_dev, to_dev(g), to_dev(perm), to_dev(blocks), bits, 0.9)
     assert np.array_equal(to_np(delta).view(np.uint32), want_delta.view(np.uint32))
     assert np.array_equal(to_np(codes), want_codes)
+
+
+@pytest.mark.parametrize("M,K,N,bits", [
+    (64, 16384, 2048, 4),      # clusters of four, four-atom stages
+    (16, 16384, 4096, 8),      # one token chunk: one CTA of four finishes the tile
+    (100, 16384, 256, 4),      # few tiles: clusters of eight, ragged last chunk
+    (50, 16384, 1024, 8),
+    (90, 8192, 520, 8),        # a ragged channel tile
+    (208, 16384, 136, 4),      # the longest token tiles
+    (250, 16384, 128, 8),
+    (816, 16384, 2048, 8),     # CTA pairs, clusters of two pairs
+    (790, 16384, 1960, 8),     # ... with ragged tokens and channels
+])
+def test_cluster_split_equals_the_second_witness(M, K, N, bits):
+    """int32 sums, binary32 and bf16 outputs, without any scratch in the workspace, a second call right behind the first."""
+    g = torch.Generator(device="cuda").manual_seed(M + N)
+    codes_w = torch.randint(0, 256, (N, K * bits // 8), dtype=torch.uint8, device="cuda", generator=g)
+    h = fq.weights_import(codes_w, torch.rand(N, device="cuda", generator=g) + 0.1, None, torch.randn(N, device="cuda", generator=g),
+                          K, 64, bits)
+    x = torch.randn(M, K, device="cuda", generator=g)
+    codes, delta = fq.quantize_act(x, None, 64, bits)
+    ws = torch.empty((M * K + 255) // 256 * 256 + (4 * M + 255) // 256 * 256, dtype=torch.uint8, device="cuda")
+    assert torch.equal(fq.gemm_acc_i32(codes, h, workspace=ws), fq.gemm_simt(codes, None, h, raw_acc=True))
+    for dt in (torch.float32, torch.bfloat16):
+        want = fq.gemm_simt(codes, delta, h, dt)
+        a, b = fq.linear(x, h, out_dtype=dt, workspace=ws), fq.linear(x, h, out_dtype=dt, workspace=ws)
+        assert torch.equal(a, want) and torch.equal(b, want)
