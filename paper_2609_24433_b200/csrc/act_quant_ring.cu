@@ -107,6 +107,7 @@ struct RingParams {
     uint32_t up_bytes; // gated sites: the row's up half starts so many bytes into its slot, and at this line of the row
     int up_line;
     int gate_kind;
+    int mult_ready;    // the multiplier may be read before the kernel ahead has finished
     uint32_t* watchdog;
 };
 
@@ -141,6 +142,26 @@ transform_quantize_ring_kernel(const __grid_constant__ CUtensorMap map_x, const 
         fence_proxy_async_smem();
     }
     __syncthreads();                 // barriers initialised before any copy is issued
+    auto stage_multiplier = [&]() {
+        if (p.mult == nullptr) return;
+        // Stage the multiplier in the order the registers hold a slice: inside every thread slice (E floats)
+        // the entries are interleaved as (g[q], g[q + H]) pairs, so that one 16-byte read yields two ready
+        // operands of the packed multiply (no register moves to pair them up), and the 16-byte pieces are
+        // XOR-swizzled by the slice index, so that the slice-per-thread reads are bank-conflict free.
+        for (int i = tid * 4; i < p.K; i += THREADS * 4) {
+            const float4 g4 = __ldg(reinterpret_cast<const float4*>(p.mult + i));
+            const float gv[4] = {g4.x, g4.y, g4.z, g4.w};
+            const uint32_t slice = (uint32_t)i / E;
+            const uint32_t key = (slice & 7u) << 4;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const uint32_t q = ((uint32_t)i % E) + k;                       // position inside the slice
+                const uint32_t off = q < H ? q * 8u : (q - H) * 8u + 4u;         // pair q (low half) or q - H (high half)
+                *reinterpret_cast<float*>(gen + ((slice * (E * 4u) + off) ^ key)) = gv[k];
+            }
+        }
+    };
+    if (p.mult_ready) stage_multiplier();
     griddep_wait();                  // the kernel before this one may still be writing x (or reading codes)
     griddep_launch_dependents();
 
@@ -165,24 +186,7 @@ transform_quantize_ring_kernel(const __grid_constant__ CUtensorMap map_x, const 
             }
         }
     }
-    if (p.mult != nullptr) {
-        // Stage the multiplier in the order the registers hold a slice: inside every thread slice (E floats)
-        // the entries are interleaved as (g[q], g[q + H]) pairs, so that one 16-byte read yields two ready
-        // operands of the packed multiply (no register moves to pair them up), and the 16-byte pieces are
-        // XOR-swizzled by the slice index, so that the slice-per-thread reads are bank-conflict free.
-        for (int i = tid * 4; i < p.K; i += THREADS * 4) {
-            const float4 g4 = __ldg(reinterpret_cast<const float4*>(p.mult + i));
-            const float gv[4] = {g4.x, g4.y, g4.z, g4.w};
-            const uint32_t slice = (uint32_t)i / E;
-            const uint32_t key = (slice & 7u) << 4;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const uint32_t q = ((uint32_t)i % E) + k;                       // position inside the slice
-                const uint32_t off = q < H ? q * 8u : (q - H) * 8u + 4u;         // pair q (low half) or q - H (high half)
-                *reinterpret_cast<float*>(gen + ((slice * (E * 4u) + off) ^ key)) = gv[k];
-            }
-        }
-    }
+    if (!p.mult_ready) stage_multiplier();
     __syncthreads();
 
     // swizzled starts of the (up to two) 128-byte lines of this thread's slices
@@ -437,7 +441,7 @@ cudaError_t launch_ring_e(int e, int block, const CUtensorMap& map, const RingPa
 cudaError_t launch_transform_quantize_ring(const void* x, fq_dtype xt, int64_t rows, int64_t K, int64_t ldx,
                                            const float* mult, float cnorm, bool mult_after_rotation, int block,
                                            int qmax, float clip_ratio, StoreFmt fmt, void* codes, float* delta,
-                                           cudaStream_t stream, int gate_kind) {
+                                           cudaStream_t stream, int gate_kind, bool mult_ready) {
     const bool gated = gate_kind >= 0;
     const size_t esz = xt == FQ_BF16 ? 2 : 4;
     const size_t row_bytes = (size_t)K * esz;
@@ -485,6 +489,7 @@ cudaError_t launch_transform_quantize_ring(const void* x, fq_dtype xt, int64_t r
     p.rows = rows; p.K = (int)K; p.cnorm = cnorm; p.qmax = (float)qmax; p.clip_ratio = clip_ratio;
     p.mult = mult; p.mult_after = (mult != nullptr && mult_after_rotation) ? 1 : 0; p.codes = static_cast<uint8_t*>(codes); p.delta = delta; p.gw = gw; p.depth = depth;
     p.up_bytes = (uint32_t)half; p.up_line = (int)(row_bytes / 128); p.gate_kind = gate_kind;
+    p.mult_ready = mult_ready ? 1 : 0;
     p.slot_bytes = (uint32_t)slot; p.g_bytes = (uint32_t)g_bytes;
     p.watchdog = watchdog_device_ptr();
     if (!p.watchdog) return cudaErrorUnknown;

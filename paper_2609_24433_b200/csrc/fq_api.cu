@@ -242,9 +242,9 @@ fq_status linear_impl(const void* x, fq_dtype xt, int64_t M, int64_t ldx, const 
     const float* mult = W->mult_const ? nullptr : W->mult_g;
     const cudaError_t pe =
         gate >= 0 ? launch_gated_transform_quantize(x, xt, M, W->K, ldx, gate, mult, block_norm(W->block), W->fold_after,
-                                                    W->block, qmax, clip_ratio, fmt, ws.a8, ws.delta, s)
+                                                    W->block, qmax, clip_ratio, fmt, ws.a8, ws.delta, s, true)
                   : launch_transform_quantize(x, xt, M, W->K, ldx, mult, block_norm(W->block), W->fold_after, W->block,
-                                              qmax, clip_ratio, fmt, ws.a8, ws.delta, s);
+                                              qmax, clip_ratio, fmt, ws.a8, ws.delta, s, true);
     if (pe != cudaSuccess) return FQ_ERR_CUDA;
     if (g_profile_mark != nullptr) {
         // Inside a stream capture the mark must be an external event-record node to stay readable.

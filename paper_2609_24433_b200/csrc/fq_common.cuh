@@ -76,16 +76,19 @@ enum class StoreFmt : int { Nibble = 0, Int8 = 1, Int8Perm = 2 };
 // +-qmax, store codes in `fmt`, store per-row step to delta.
 // mult_after_rotation (fold-after sites, T = D^o R): multiply by `cnorm` before the butterflies
 // and by mult[K] after them instead.
+// mult_ready: `mult` was complete before the kernel ahead in the stream was enqueued (a handle's multiplier), so it may be
+// read before that kernel has finished.
 cudaError_t launch_transform_quantize(const void* x, fq_dtype xt, int64_t rows, int64_t K, int64_t ldx,
                                       const float* mult, float cnorm, bool mult_after_rotation, int block,
                                       int qmax, float clip_ratio, StoreFmt fmt, void* codes, float* delta,
-                                      cudaStream_t stream);
+                                      cudaStream_t stream, bool mult_ready = false);
 
 // Same, for the site behind a gated MLP: x is [rows, 2K] = [gate | up] and the input is act(gate) * up
 // (gate_kind 0 = SiLU, 1 = GELU-tanh, fixed binary32 arithmetic).
 cudaError_t launch_gated_transform_quantize(const void* x, fq_dtype xt, int64_t rows, int64_t K, int64_t ldx, int gate_kind,
                                             const float* mult, float cnorm, bool mult_after_rotation, int block, int qmax,
-                                            float clip_ratio, StoreFmt fmt, void* codes, float* delta, cudaStream_t stream);
+                                            float clip_ratio, StoreFmt fmt, void* codes, float* delta, cudaStream_t stream,
+                                            bool mult_ready = false);
 
 // mult_w[c] = s_c * cnorm, mult_g[c] = (1/s_c) * cnorm (smooth == nullptr: both = cnorm).
 cudaError_t launch_multipliers(const float* smooth, int64_t K, float cnorm, float* mult_w, float* mult_g,
@@ -154,7 +157,7 @@ bool encode_tiled(CUtensorMap* map, CUtensorMapDataType dt, uint32_t rank, const
 cudaError_t launch_transform_quantize_ring(const void* x, fq_dtype xt, int64_t rows, int64_t K, int64_t ldx,
                                            const float* mult, float cnorm, bool mult_after_rotation, int block,
                                            int qmax, float clip_ratio, StoreFmt fmt, void* codes, float* delta,
-                                           cudaStream_t stream, int gate_kind = -1);
+                                           cudaStream_t stream, int gate_kind = -1, bool mult_ready = false);
 
 // Stored composite rotation: u[t][b*beta + i] = sum_j B_b[i][j] * (x (.) diag)[t][perm[b*beta + j]] in binary32,
 // u [rows, K] (pitch K).  beta in {16, 32, 64, 128, 256}; diag may be null.
