@@ -111,9 +111,11 @@ transform_quantize_kernel(const XT* __restrict__ x, int64_t rows, int K, int64_t
             for (int i = 0; i < (CACHE ? E : 1); ++i) g[i] = cnorm;
         }
     };
+    // The kernel behind may start at once: what it does ahead of its own wait touches weights only, and in a chain of short
+    // calls its pipelines fill while the kernel AHEAD of this one still runs (50 x 1024 x 3072, 4 bits: 6.97 -> 6.07 us a call).
+    griddep_launch_dependents();
     if (CACHE && mult_ready) load_g();
     griddep_wait();                   // launched with programmatic serialization: see launch_pdl
-    griddep_launch_dependents();
     if (CACHE && !mult_ready) load_g();
 
     const int64_t row_step = (int64_t)gridDim.x * rpc;
@@ -373,8 +375,8 @@ __global__ void smooth_scale_kernel(const float* __restrict__ a, const float* __
 // 16 packed bytes (32 codes) per thread -> 32 int8 holding 16*code, each group of 8 channels in the
 // (even channels, odd channels) order of StoreFmt::Int8Perm.
 __global__ void expand_nibbles_kernel(const uint4* __restrict__ packed, int64_t n_vec, uint4* __restrict__ out) {
-    griddep_wait();
     griddep_launch_dependents();
+    griddep_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_vec) return;
     const uint4 p = __ldg(packed + i);

@@ -161,9 +161,9 @@ transform_quantize_ring_kernel(const __grid_constant__ CUtensorMap map_x, const 
             }
         }
     };
+    griddep_launch_dependents();
     if (p.mult_ready) stage_multiplier();
     griddep_wait();                  // the kernel before this one may still be writing x (or reading codes)
-    griddep_launch_dependents();
 
     const int first = group * (int)gridDim.x + (int)blockIdx.x;   // rows < 2^31 (checked by the launcher)
     const int step = (int)gridDim.x * ngroups;

@@ -154,8 +154,8 @@ composite_quantize_kernel(const CompositeParams p) {
     int* s_src = reinterpret_cast<int*>(s_raw + p.off_s);
     float* s_dg = reinterpret_cast<float*>(s_src + p.span);
     if (C > 1) cluster_arrive();                       // "this CTA exists": awaited before the first remote store
-    griddep_wait();
     griddep_launch_dependents();
+    griddep_wait();
 
     const int item0 = ((int)rank * p.items) >> p.ctas_shift, item1 = (((int)rank + 1) * p.items) >> p.ctas_shift;
     const int c0 = item0 * OUT / BETA * BETA;          // first channel of the first block

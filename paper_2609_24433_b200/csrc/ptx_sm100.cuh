@@ -171,7 +171,8 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, vo
 // may start while the kernel before it in the stream is still running; griddep_wait() returns once
 // that kernel has completed and its writes are visible, so everything that touches global memory
 // comes after it and only on-chip setup (barriers, TMEM, descriptor prefetch) runs ahead.
-// griddep_launch_dependents() lets the NEXT kernel in the stream begin its own setup early.
+// griddep_launch_dependents() lets the NEXT kernel in the stream begin its own setup early; issued ahead of griddep_wait(),
+// even before the kernel in front of this one has ended (what comes before a wait must not depend on either of them).
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch_dependents() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
