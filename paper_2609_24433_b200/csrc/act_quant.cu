@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(CACHE ? 512 : kMaxThreads)
 transform_quantize_kernel(const XT* __restrict__ x, int64_t rows, int K, int64_t ldx,
                           const float* __restrict__ mult, float cnorm, int block, float qmax,
                           float clip_ratio, uint8_t* __restrict__ codes, float* __restrict__ delta,
-                          int tpr, int rpc, int mult_after, int gate_kind, int mult_ready) {
+                          int tpr, int rpc, int mult_after, int gate_kind, int mult_ready, int early) {
     __shared__ float s_part[2][32];   // per-warp partial maxima, double buffered
 
     const int tid = threadIdx.x;
@@ -111,11 +111,18 @@ transform_quantize_kernel(const XT* __restrict__ x, int64_t rows, int K, int64_t
             for (int i = 0; i < (CACHE ? E : 1); ++i) g[i] = cnorm;
         }
     };
-    // The kernel behind may start at once: what it does ahead of its own wait touches weights only, and in a chain of short
-    // calls its pipelines fill while the kernel AHEAD of this one still runs (50 x 1024 x 3072, 4 bits: 6.97 -> 6.07 us a call).
-    griddep_launch_dependents();
+    if (early) griddep_launch_dependents();
+    {   // tokens that lie in memory come as far as L2 while the kernel ahead still runs (1000 x 4096 x 4104 25.6 -> 24.4 us)
+        const int64_t row0 = (int64_t)blockIdx.x * rpc + r_in_cta;
+        if (col_ok && row0 < rows) {
+#pragma unroll
+            for (int b = 0; b < E * (int)sizeof(XT); b += 64) prefetch_l2(reinterpret_cast<const char*>(x + row0 * ldx + col0) + b);
+            if (GATED) prefetch_l2(x + row0 * ldx + K + col0);
+        }
+    }
     if (CACHE && mult_ready) load_g();
     griddep_wait();                   // launched with programmatic serialization: see launch_pdl
+    if (!early) griddep_launch_dependents();
     if (CACHE && !mult_ready) load_g();
 
     const int64_t row_step = (int64_t)gridDim.x * rpc;
@@ -284,12 +291,17 @@ cudaError_t launch_e(const XT* x, int64_t rows, int K, int64_t ldx, const float*
     const int threads = tpr * rpc;
     const int sms = device_sm_count();
     const int64_t iters = (rows + rpc - 1) / rpc;
+    // Short batches let the kernel behind start at once: what it does ahead of its own wait touches weights only, and its pipelines
+    // fill while the kernel AHEAD of this one still runs (the action expert's step 543 -> 529 us).  Otherwise behind the wait: a
+    // waiting GEMM takes issue slots and SMs from the prologues (M = 816 backbone layer 127.2 / 128.0 us, 16 x 8192 x 8192
+    // 13.8 / 14.1).
+    const int early = rows <= 64 && K <= 4096 ? 1 : 0;
     auto args = [&](auto kern) {
         const int resident = max_resident_blocks(reinterpret_cast<const void*>(kern), threads);
         int64_t grid = iters < (int64_t)sms * resident ? iters : (int64_t)sms * resident;
         if (grid < 1) grid = 1;
         launch_pdl(kern, (unsigned)grid, (unsigned)threads, 0, stream, 1u, x, rows, K, ldx, mult, cnorm, block, (float)qmax,
-                   clip_ratio, static_cast<uint8_t*>(codes), delta, tpr, rpc, mult_after, gate, ready);
+                   clip_ratio, static_cast<uint8_t*>(codes), delta, tpr, rpc, mult_after, gate, ready, early);
     };
     const bool clamp = clip_ratio < 1.0f;
     if (gate >= 0) {

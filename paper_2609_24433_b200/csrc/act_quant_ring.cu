@@ -42,6 +42,12 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
         ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
         : "memory");
 }
+// The same box as far as L2 only.
+__device__ __forceinline__ void prefetch_row(const CUtensorMap* map, int line, int row) {
+    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];"
+                 ::"l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(line), "r"(row)
+                 : "memory");
+}
 // Group barrier that also ANDs a predicate over the group (ids 1..15, count a multiple of 32).
 __device__ __forceinline__ bool group_barrier_and(int id, int count, bool pred) {
     uint32_t r;
@@ -161,9 +167,16 @@ transform_quantize_ring_kernel(const __grid_constant__ CUtensorMap map_x, const 
             }
         }
     };
-    griddep_launch_dependents();
     if (p.mult_ready) stage_multiplier();
+    if (leader) {                    // rows that lie in memory come as far as L2 while the kernel ahead still runs
+        const int r0 = group * (int)gridDim.x + (int)blockIdx.x, rs = (int)gridDim.x * ngroups;
+        for (int d = 0; d < p.depth && r0 + d * rs < (int)p.rows; ++d) {
+            prefetch_row(&map_x, 0, r0 + d * rs);
+            if (GATED) prefetch_row(&map_x, p.up_line, r0 + d * rs);
+        }
+    }
     griddep_wait();                  // the kernel before this one may still be writing x (or reading codes)
+    griddep_launch_dependents();
 
     const int first = group * (int)gridDim.x + (int)blockIdx.x;   // rows < 2^31 (checked by the launcher)
     const int step = (int)gridDim.x * ngroups;

@@ -153,6 +153,8 @@ linear_fused_kernel(const __grid_constant__ CUtensorMap map_w, const FusedParams
     if (C > 1) cluster_arrive();                           // "this CTA exists": awaited before the first remote store
     griddep_launch_dependents();
 
+    if (tid / LG < p.M && tid % LG * E < ks)               // tokens that lie in memory come as far as L2 meanwhile
+        prefetch_l2(static_cast<const XT*>(p.x) + (int64_t)(tid / LG) * p.ldx + k0 + tid % LG * E);
     if (BITS == 4) {
         mbar_wait_all(smem_u32(&s_bar_w), 0u, &s_abort, p.watchdog, kWdFusedWeights);
         // a thread owns one weight row (TMEM lane) of every fourth atom: 64 packed bytes, 64-byte TMA swizzle, to
