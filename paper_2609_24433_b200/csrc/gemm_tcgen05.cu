@@ -31,8 +31,8 @@
 // unpacked weights (unpack -> MMA, 32 TMEM columns a stage); one tcgen05.commit per k-block
 // frees both the activation stage and the k-block's TMEM slot.
 // Variants: CTAS = 2 runs CTA pairs (cta_group::2, 256 channels per MMA, each CTA staging half
-// of the token tile); SPLIT lets the CTAs of a cluster share a tile along K and exchange int32
-// partial sums through global scratch.
+// of the token tile); SPLIT lets CTAs share a tile along K and exchange int32 partial sums,
+// through the cluster's shared memory or through global scratch.
 // bf16 outputs leave through a per-warp 1 KB shared-memory transposer so that global
 // stores are 16-byte vectors of 8 consecutive channels; fp32/raw outputs store directly.
 // Every mbarrier wait is bounded by wall-clock time; on expiry the CTA records a
@@ -1173,7 +1173,14 @@ int cluster_capacity(int ctas);
 //   8-bit, one CTA:         per_kblock = max(350 + 0.8*bt, 230 + 2*bt)   (issue floor, then shared memory:
 //                                        both operands pass through it)
 //   8-bit, CTA pair:        per_kblock = max(545, 2.62*bt)   (each CTA stages half of the token tile)
-// Pairs gain nothing for 4-bit weights, which never pass through shared memory unpacked.
+//   4-bit, CTA pair:        0.95 of a single CTA's, for launches of 1.6e11 multiplications and K >= 2048.  Each CTA stages
+//                           half of the token tile, so shared memory is read half as often: no faster while the clock is
+//                           at its highest, but less power, hence a higher clock under the power cap.  Chains of calls,
+//                           pairs / single CTAs, the clock still high and after 0.2 s of load: 16384 x 8192 x 8192
+//                           (M x K x N) 773 / 804 us and 905 / 922, 16384 x 4096 x 4096 222 / 226 and 262 / 268,
+//                           4096 x 8192 x 8192 199 / 200 and 235 / 238, 12000 x 2048 x 8192 158 / 163 and 189 / 194; below
+//                           the line 7000 x 4096 x 4096 103 / 100 and 117 / 119, 4096 x 4096 x 4096 67.2 / 64.9 and 73.0 /
+//                           73.3; a short K: 16384 x 1024 x 4096 96 / 97 and 105 / 104.
 // K split: problems with fewer tiles than SMs and a long K (short batches, few output channels).
 //   By clusters of 2, 4 or 8 CTAs (one wave; at least four k-blocks of ring beside the sums, 4-bit tiles of at most 128
 //   tokens): the tail shrinks to 16*bt/split, the exchange costs 2800 + 40 per CTA of the launch at 4 bits, 3300 + 18 at 8
@@ -1189,7 +1196,8 @@ Plan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t scratc
     const int64_t kb = (K + kBlockK - 1) / kBlockK;
     Plan best;
     double best_cost = 0.0;
-    for (int c = 1; c <= ((bits == 8 && N > kTileN) ? 2 : 1); ++c) {
+    const bool pairs = N > kTileN && (bits == 8 || (K >= 2048 && (double)M * (double)N * (double)K >= 1.6e11));
+    for (int c = 1; c <= (pairs ? 2 : 1); ++c) {
         const int64_t n_units = (N + kTileN * c - 1) / (kTileN * c);
         for (int mt = (int)((M + bt_max - 1) / bt_max); mt <= (int)((M + 63) / 64); ++mt) {
             const int b = (int)(((M + mt - 1) / mt + 15) / 16 * 16);
@@ -1197,7 +1205,7 @@ Plan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t scratc
             const int64_t units = n_units * ((M + b - 1) / b);
             const double w8_single = 350.0 + 0.8 * b > 230.0 + 2.0 * b ? 350.0 + 0.8 * b : 230.0 + 2.0 * b;
             // 4-bit, tiles of at most 128 tokens: stages of several atoms (see the kernel) cost less per 128 channels
-            const double w4 = (c == 1 && b <= 128 && K % kBlockK == 0) ? 235.0 + b : 330.0 + b;
+            const double w4 = c == 2 ? 0.95 * (330.0 + b) : (b <= 128 && K % kBlockK == 0 ? 235.0 + b : 330.0 + b);
             const double per_kb = bits == 4 ? w4 : (c == 1 ? w8_single : (2.62 * b > 545.0 ? 2.62 * b : 545.0));
             const int slots = sms / c;
             auto offer = [&](int sp, bool cluster, size_t scratch, double unit_cost) {
@@ -1208,6 +1216,7 @@ Plan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t scratc
                 }
             };
             offer(1, false, 0, (double)kb * per_kb + 16.0 * b + 1000.0);
+            if (bits == 4 && c == 2) continue;           // (long launches have tiles enough: no kernel for a split of these)
             for (int sp = 2; sp <= kMaxSplit; sp *= 2) {
                 if (kb % sp != 0 || kb / sp < 2) break;
                 const double slice = (double)(kb / sp) * per_kb + 1000.0;
@@ -1395,6 +1404,7 @@ fq_status launch_gemm_tcgen05(const int8_t* a8, int64_t M, const Weights& W, int
     using I2 = std::integral_constant<int, 2>;
     using I4 = std::integral_constant<int, 4>;
     using I8 = std::integral_constant<int, 8>;
+    if (W.bits == 4 && ctas == 2) return launch_variant<4, 2, kUnsplit>(map_a, W.tmap, map_y, p, grid, smem, cluster, stream);
     if (W.bits == 4) return atoms == 4 ? go(I4(), I1(), I4()) : (atoms == 2 ? go(I4(), I1(), I2()) : go(I4(), I1(), I1()));
     return ctas == 2 ? go(I8(), I2(), I1()) : go(I8(), I1(), I1());
 }

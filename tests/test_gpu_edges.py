@@ -168,3 +168,21 @@ def test_cluster_split_equals_the_second_witness(M, K, N, bits):
         want = fq.gemm_simt(codes, delta, h, dt)
         a, b = fq.linear(x, h, out_dtype=dt, workspace=ws), fq.linear(x, h, out_dtype=dt, workspace=ws)
         assert torch.equal(a, want) and torch.equal(b, want)
+
+
+@pytest.mark.parametrize("M,K,N", [
+    (9001, 4096, 4352),        # 1.6e11 multiplications: CTA pairs, a ragged last token tile
+    (9000, 4096, 4336),        # just short of it: single CTAs
+    (60001, 2048, 1336),       # the shortest K, the last pair with no channel for its odd CTA
+    (40001, 8256, 496),        # channels past K in the last k-block, the last pair nearly full
+])
+def test_long_w4_pairs_equal_the_second_witness(M, K, N):
+    g = torch.Generator(device="cuda").manual_seed(M + N)
+    codes_w = torch.randint(0, 256, (N, K // 2), dtype=torch.uint8, device="cuda", generator=g)
+    h = fq.weights_import(codes_w, torch.rand(N, device="cuda", generator=g) + 0.1, None, torch.randn(N, device="cuda", generator=g),
+                          K, 64, 4)
+    codes = torch.randint(-7, 8, (M, K), dtype=torch.int8, device="cuda", generator=g)
+    delta = torch.rand(M, device="cuda", generator=g) + 0.1
+    for dt in (torch.float32, torch.bfloat16):
+        assert torch.equal(fq.gemm_w4a4(codes, delta, h, dt), fq.gemm_simt(codes, delta, h, dt))
+    assert torch.equal(fq.gemm_acc_i32(codes, h), fq.gemm_simt(codes, None, h, raw_acc=True))
