@@ -344,8 +344,13 @@ linear_fused_kernel(const __grid_constant__ CUtensorMap map_w, const FusedParams
     // ---- partial sums to the CTA that finishes the token: [slice][token][128 channels]
     if (const int t0 = (warp >> 2) * 16; t0 < p.M) {       // a warp: 32 channels, 16 tokens
         uint32_t a[16];
-        tmem_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)t0, a);
-        tmem_ld_wait();
+        if (atoms > 0) {
+            tmem_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)t0, a);
+            tmem_ld_wait();
+        } else {                                           // fewer units than CTAs: no channels here, nothing multiplied
+#pragma unroll
+            for (int i = 0; i < 16; ++i) a[i] = 0u;
+        }
         const uint32_t dst = base + p.off_part + (uint32_t)((warp & 3) * 32 + lane) * 4u;
 #pragma unroll
         for (int i = 0; i < 16; ++i) {

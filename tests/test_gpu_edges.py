@@ -186,3 +186,22 @@ def test_long_w4_pairs_equal_the_second_witness(M, K, N):
     for dt in (torch.float32, torch.bfloat16):
         assert torch.equal(fq.gemm_w4a4(codes, delta, h, dt), fq.gemm_simt(codes, delta, h, dt))
     assert torch.equal(fq.gemm_acc_i32(codes, h), fq.gemm_simt(codes, None, h, raw_acc=True))
+
+
+@pytest.mark.parametrize("M,K,block,bits", [
+    (9, 1536, 256, 8),         # six units of K for clusters of eight
+    (31, 1792, 256, 4),        # seven
+    (33, 384, 64, 4),          # three for clusters of four
+    (64, 896, 128, 8),
+])
+def test_one_launch_with_fewer_units_than_cluster_ctas(M, K, block, bits):
+    """CTAs without channels add nothing, whatever the launch ahead left in tensor memory."""
+    g = torch.Generator(device="cuda").manual_seed(K)
+    h = fq.weights_import(torch.randint(0, 256, (200, K * bits // 8), dtype=torch.uint8, device="cuda", generator=g),
+                          torch.rand(200, device="cuda", generator=g) + 0.1, None, None, K, block, bits)
+    x, many = (torch.randn(m, K, device="cuda", generator=g) for m in (M, 4000))
+    codes, delta = fq.quantize_act(x, None, block, bits)
+    want = fq.gemm_simt(codes, delta, h, torch.float32)
+    for _ in range(50):
+        fq.linear(many, h)     # fills tensor memory with sums
+        assert torch.equal(fq.linear(x, h), want)
