@@ -1,4 +1,4 @@
-// Streaming variant of the runtime prologue (Alg. 1 runtime half lines 1-2, Eq. 5) for long
+// Streaming variant of the runtime prologue (Alg. 1 runtime half lines 1-2, Eq. 5) for longer
 // batches: same arithmetic, bit for bit, as transform_quantize_kernel, but tokens reach the
 // SM through a TMA-fed shared-memory ring so that many rows are in flight per SM regardless
 // of register pressure, and the floating-point work is issued as packed f32x2 instructions.
@@ -16,8 +16,15 @@
 //     instruction is one IEEE binary32 operation, so the rounding is that of the scalar
 //     network); the stride-E/2 stage works inside the pairs; strides E..block/2 go across
 //     lanes (one shuffle per value, one packed FMA per pair).
+//   - A thread's 64 one-byte codes are a run of 64 bytes, so a warp-wide 16-byte store would touch 32 sectors and fill half
+//     of each.  They go through 2 KB of shared memory per warp instead and leave as one bulk store of 32 runs (64-byte
+//     swizzle: the 16-byte pieces of 8 lanes lie in different banks).  16384 x 8192, 8-bit codes, blocks of 64, 128 and 256
+//     channels: 79.6, 83.6 and 93.3 us with direct stores, 59.6 (the copy rate), 70.3 and 81.0 now.  Runs of 32 and 16 bytes
+//     (4-bit codes, 32 channels per thread) gain nothing (57.0 and 59.0 us; gated 1-5 % slower) and are stored directly.
+//     640 threads at 96 registers: 58.9, 68.4 and 81.2 us, and slower for short rows.
 #include <cuda_bf16.h>
 #include <float.h>
+#include <string.h>
 
 #include "fq_common.cuh"
 #include "ptx_sm100.cuh"
@@ -27,10 +34,9 @@ namespace fq {
 namespace {
 
 constexpr int kThreads = 512;
-// Threads of a CTA by channels per thread.  (1024 threads of 32 channels -- twice the warps at 64 registers -- measured
+// Threads of a CTA.  (1024 threads of 32 channels -- twice the warps at 64 registers -- measured
 // slower than 512 threads of 64 channels for 4-bit output: 0.65 against 0.75 of the copy rate at K = 8192, block 128;
 // the extra cross-lane butterfly stage costs more than the occupancy returns.)
-constexpr int threads_for(int) { return kThreads; }
 constexpr int kMaxSlots = 128;
 
 // 128-byte swizzle of a byte offset inside a 1024-byte aligned region.
@@ -47,6 +53,15 @@ __device__ __forceinline__ void prefetch_row(const CUtensorMap* map, int line, i
     asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];"
                  ::"l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(line), "r"(row)
                  : "memory");
+}
+// Tiled bulk STORE shared -> global; what lies beyond the tensor's extent is clipped by the copy engine.
+__device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, int c0, int c1, int c2, uint32_t src) {
+    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
+                 ::"l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void sts128(uint32_t addr, uint4 v) {
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 // Group barrier that also ANDs a predicate over the group (ids 1..15, count a multiple of 32).
 __device__ __forceinline__ bool group_barrier_and(int id, int count, bool pred) {
@@ -109,6 +124,7 @@ struct RingParams {
     int gw;            // warps per row group (power of two)
     int depth;         // ring slots per group
     uint32_t slot_bytes;
+    uint32_t stage_off; // where the codes of the warps wait for their bulk store
     uint32_t g_bytes;  // bytes of the multiplier stage (0 if no multiplier)
     uint32_t up_bytes; // gated sites: the row's up half starts so many bytes into its slot, and at this line of the row
     int up_line;
@@ -119,17 +135,19 @@ struct RingParams {
 
 // GATED: a row is [gate | up], 2K bf16 channels in one slot; the transform's input is act(gate) * up, formed as the row is
 // read from shared memory.
-template <typename XT, int FMT, bool CLAMP, int E, int BLOCK, bool AFTER, bool GATED, int THREADS = kThreads>
-__global__ void __launch_bounds__(THREADS, 1)
-transform_quantize_ring_kernel(const __grid_constant__ CUtensorMap map_x, const RingParams p) {
+template <typename XT, int FMT, bool CLAMP, int E, int BLOCK, bool AFTER, bool GATED>
+__global__ void __launch_bounds__(kThreads, 1)
+transform_quantize_ring_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_c,
+                               const RingParams p) {
     constexpr int H = E / 2;                       // channels per half: v[i] = (channel i, channel i + H)
+    constexpr bool kStaged = FMT != 0 && E == 64;  // the codes leave through bulk stores
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t s_full[kMaxSlots];
     __shared__ float s_part[2][32];
     __shared__ int s_abort;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int ngroups = (THREADS / 32) / p.gw;
+    const int ngroups = (kThreads / 32) / p.gw;
     const int group = warp / p.gw;
     const int wg = warp - group * p.gw;
     const int col0 = (wg * 32 + lane) * E;
@@ -154,7 +172,7 @@ transform_quantize_ring_kernel(const __grid_constant__ CUtensorMap map_x, const 
         // the entries are interleaved as (g[q], g[q + H]) pairs, so that one 16-byte read yields two ready
         // operands of the packed multiply (no register moves to pair them up), and the 16-byte pieces are
         // XOR-swizzled by the slice index, so that the slice-per-thread reads are bank-conflict free.
-        for (int i = tid * 4; i < p.K; i += THREADS * 4) {
+        for (int i = tid * 4; i < p.K; i += kThreads * 4) {
             const float4 g4 = __ldg(reinterpret_cast<const float4*>(p.mult + i));
             const float gv[4] = {g4.x, g4.y, g4.z, g4.w};
             const uint32_t slice = (uint32_t)i / E;
@@ -168,12 +186,11 @@ transform_quantize_ring_kernel(const __grid_constant__ CUtensorMap map_x, const 
         }
     };
     if (p.mult_ready) stage_multiplier();
-    if (leader) {                    // rows that lie in memory come as far as L2 while the kernel ahead still runs
-        const int r0 = group * (int)gridDim.x + (int)blockIdx.x, rs = (int)gridDim.x * ngroups;
-        for (int d = 0; d < p.depth && r0 + d * rs < (int)p.rows; ++d) {
-            prefetch_row(&map_x, 0, r0 + d * rs);
-            if (GATED) prefetch_row(&map_x, p.up_line, r0 + d * rs);
-        }
+    // The group's first row comes as far as L2 while the kernel ahead still runs.  (All rows of the ring: no better for short
+    // batches and slower for long ones, 2368 x 8192 13.6 us against 11.1; none: 11.5, and 816 x 2048 3.1 against 2.95.)
+    if (leader && group * (int)gridDim.x + (int)blockIdx.x < (int)p.rows) {
+        prefetch_row(&map_x, 0, group * (int)gridDim.x + (int)blockIdx.x);
+        if (GATED) prefetch_row(&map_x, p.up_line, group * (int)gridDim.x + (int)blockIdx.x);
     }
     griddep_wait();                  // the kernel before this one may still be writing x (or reading codes)
     griddep_launch_dependents();
@@ -210,6 +227,10 @@ transform_quantize_ring_kernel(const __grid_constant__ CUtensorMap map_x, const 
     const uint32_t g1 = base + (((uint32_t)col0 * 4u + 128u) ^ gkey);
     const bool warp_ok = __all_sync(0xffffffffu, col_ok);   // the usual case: no lane of the warp is past K
     const float2 neg1 = make_float2(-1.0f, -1.0f);
+
+    const uint32_t stage = base + p.stage_off + (uint32_t)(warp * 32 * E);
+    const uint32_t stage_line = stage + (uint32_t)(lane * E);
+    const uint32_t stage_key = (uint32_t)((lane >> 1) & 3);
 
     int n = 0, d = 0;
     uint32_t ph = 0;
@@ -382,11 +403,24 @@ transform_quantize_ring_kernel(const __grid_constant__ CUtensorMap map_x, const 
             wlo[j] = pack_word<FMT>(bl);
             whi[j] = pack_word<FMT>(bh);
         }
-        if (col_ok) {
-            // low-half words then high-half words are consecutive channels: one contiguous store run
-            uint32_t w[2 * kWords];
+        // low-half words then high-half words are consecutive channels: one contiguous store run
+        uint32_t w[2 * kWords];
 #pragma unroll
-            for (int j = 0; j < kWords; ++j) { w[j] = wlo[j]; w[kWords + j] = whi[j]; }
+        for (int j = 0; j < kWords; ++j) { w[j] = wlo[j]; w[kWords + j] = whi[j]; }
+        if (kStaged) {
+            if (lane == 0) bulk_wait_read<0>();          // the row before this one has left the buffer
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < 2 * kWords / 4; ++j)
+                sts128(stage_line + (((uint32_t)j ^ stage_key) << 4), make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]));
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0 && wg * 32 * E < p.K) {
+                tma_store_3d(&map_c, 0, wg * 32, row, stage);
+                bulk_commit();
+                if (wg == 0) p.delta[row] = dl;
+            }
+        } else if (col_ok) {
             const int64_t pitch = FMT == 0 ? p.K / 2 : p.K;
             uint4* dst = reinterpret_cast<uint4*>(p.codes + (int64_t)row * pitch + (FMT == 0 ? col0 / 2 : col0));
 #pragma unroll
@@ -395,6 +429,8 @@ transform_quantize_ring_kernel(const __grid_constant__ CUtensorMap map_x, const 
         }
         if (++d == p.depth) { d = 0; ph ^= 1u; }
     }
+
+    if (kStaged && lane == 0) bulk_wait_read<0>();       // (the last codes leave shared memory before the CTA does)
 
     // Winding down after an expired wait: let the copies this group still has in flight land.
     if (leader && *abort_flag) {
@@ -410,43 +446,43 @@ transform_quantize_ring_kernel(const __grid_constant__ CUtensorMap map_x, const 
 }
 
 template <typename XT, int FMT, int E, int BLOCK, bool GATED = false>
-cudaError_t launch_ring(const CUtensorMap& map, const RingParams& p, int grid, size_t smem, cudaStream_t stream) {
-    constexpr int THREADS = threads_for(E);
+cudaError_t launch_ring(const CUtensorMap& map, const CUtensorMap& map_c, const RingParams& p, int grid, size_t smem,
+                        cudaStream_t stream) {
     auto go = [&](auto kern) -> cudaError_t {
         cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), smem);
         if (e != cudaSuccess) return e;
-        return launch_pdl(kern, (unsigned)grid, (unsigned)THREADS, smem, stream, 1u, map, p);
+        return launch_pdl(kern, (unsigned)grid, (unsigned)kThreads, smem, stream, 1u, map, map_c, p);
     };
     // (the fold-after variant is its own instantiation: as a run-time branch it cost the default path registers, and spills,
     // in the 64-channels-per-thread kernels; it has no gated form, nor one for 64 channels with shuffle stages)
     if constexpr (!GATED && (E == 32 || BLOCK <= 64)) {
         if (p.mult_after) {
-            if (p.clip_ratio < 1.0f) return go(transform_quantize_ring_kernel<XT, FMT, true, E, BLOCK, true, false, THREADS>);
-            return go(transform_quantize_ring_kernel<XT, FMT, false, E, BLOCK, true, false, THREADS>);
+            if (p.clip_ratio < 1.0f) return go(transform_quantize_ring_kernel<XT, FMT, true, E, BLOCK, true, false>);
+            return go(transform_quantize_ring_kernel<XT, FMT, false, E, BLOCK, true, false>);
         }
     }
     if (p.mult_after) return cudaErrorNotSupported;
-    if (p.clip_ratio < 1.0f) return go(transform_quantize_ring_kernel<XT, FMT, true, E, BLOCK, false, GATED, THREADS>);
-    return go(transform_quantize_ring_kernel<XT, FMT, false, E, BLOCK, false, GATED, THREADS>);
+    if (p.clip_ratio < 1.0f) return go(transform_quantize_ring_kernel<XT, FMT, true, E, BLOCK, false, GATED>);
+    return go(transform_quantize_ring_kernel<XT, FMT, false, E, BLOCK, false, GATED>);
 }
 
 template <typename XT, int FMT, int E, bool GATED = false>
-cudaError_t launch_ring_block(int block, const CUtensorMap& map, const RingParams& p, int grid, size_t smem,
-                              cudaStream_t stream) {
+cudaError_t launch_ring_block(int block, const CUtensorMap& map, const CUtensorMap& map_c, const RingParams& p, int grid,
+                              size_t smem, cudaStream_t stream) {
     switch (block) {
-        case 32: return launch_ring<XT, FMT, E, 32, GATED>(map, p, grid, smem, stream);
-        case 64: return launch_ring<XT, FMT, E, 64, GATED>(map, p, grid, smem, stream);
-        case 128: return launch_ring<XT, FMT, E, 128, GATED>(map, p, grid, smem, stream);
-        case 256: return launch_ring<XT, FMT, E, 256, GATED>(map, p, grid, smem, stream);
+        case 32: return launch_ring<XT, FMT, E, 32, GATED>(map, map_c, p, grid, smem, stream);
+        case 64: return launch_ring<XT, FMT, E, 64, GATED>(map, map_c, p, grid, smem, stream);
+        case 128: return launch_ring<XT, FMT, E, 128, GATED>(map, map_c, p, grid, smem, stream);
+        case 256: return launch_ring<XT, FMT, E, 256, GATED>(map, map_c, p, grid, smem, stream);
         default: return cudaErrorNotSupported;
     }
 }
 
 template <typename XT, int FMT>
-cudaError_t launch_ring_e(int e, int block, const CUtensorMap& map, const RingParams& p, int grid, size_t smem,
-                          cudaStream_t stream) {
-    return e == 64 ? launch_ring_block<XT, FMT, 64>(block, map, p, grid, smem, stream)
-                   : launch_ring_block<XT, FMT, 32>(block, map, p, grid, smem, stream);
+cudaError_t launch_ring_e(int e, int block, const CUtensorMap& map, const CUtensorMap& map_c, const RingParams& p, int grid,
+                          size_t smem, cudaStream_t stream) {
+    return e == 64 ? launch_ring_block<XT, FMT, 64>(block, map, map_c, p, grid, smem, stream)
+                   : launch_ring_block<XT, FMT, 32>(block, map, map_c, p, grid, smem, stream);
 }
 
 }  // namespace
@@ -462,41 +498,71 @@ cudaError_t launch_transform_quantize_ring(const void* x, fq_dtype xt, int64_t r
     if (K < 1024 || row_bytes % 128 != 0 || row_bytes / 128 > 256 || rows > 0x7fffffffll || block < 32)
         return cudaErrorNotSupported;
     const int sms = device_sm_count();
-    // Short batches are latency-bound and go to the register kernel, which spreads a row over more threads: fewer
-    // than 8 rows per SM, unless the rows are long (measured at M = 816: K = 2048 6.4 us there against 7.1-7.9 us
-    // here, K = 16384 24.3 us there against 21.2 us here).
-    if (gated) {
-        // Gated sites: from two rows per SM on, or long rows.  Prologue alone, GELU, 8-bit codes, operands from memory, here /
-        // register kernel: M = 816, K = 2048 4.6 / 5.7 us, K = 8192 14.0 / 16.0, K = 16384 25.9 / 37.7 (66 before the paired
-        // gate arithmetic); M = 148, K = 8192 4.1 / 3.9, K = 16384 7.0 / 8.5.
-        if (xt != FQ_BF16 || (mult != nullptr && mult_after_rotation) || (rows < 2 * (int64_t)sms && K <= 8192))
-            return cudaErrorNotSupported;
-    } else if (rows < 2 * (int64_t)sms || (rows < 8 * (int64_t)sms && K < 8192)) return cudaErrorNotSupported;
+    // Gated sites: from two rows per SM on, or long rows.  Prologue alone, GELU, 8-bit codes, operands from memory, here /
+    // register kernel: M = 816, K = 2048 4.6 / 5.7 us, K = 8192 14.0 / 16.0, K = 16384 25.9 / 37.7 (66 before the paired
+    // gate arithmetic); M = 148, K = 8192 4.1 / 3.9, K = 16384 7.0 / 8.5.
+    if (gated && (xt != FQ_BF16 || (mult != nullptr && mult_after_rotation) || (rows < 2 * (int64_t)sms && K <= 8192)))
+        return cudaErrorNotSupported;
 
-    // channels per thread (the fold-after variant with shuffle stages does not fit 64 without spills)
-    const int e = (!gated && K >= 2048 && K % 64 == 0 && !(mult != nullptr && mult_after_rotation && block >= 128)) ? 64 : 32;
-    const int threads = threads_for(e);
-    int gw = 1;
-    while ((int64_t)gw * 32 * e < K) gw <<= 1;
-    if (gw > threads / 32) return cudaErrorNotSupported;
-    const int ngroups = (threads / 32) / gw;
-    if (gw > 1 && ngroups > 15) return cudaErrorNotSupported;      // one named barrier per group
+    // Channels per thread: 64 where at least two rows per group fit (the fold-after variant with shuffle stages would spill)
     const size_t half = (row_bytes + 1023) / 1024 * 1024;
     const size_t slot = gated ? 2 * half : half;
     const size_t g_bytes = mult ? ((size_t)K * 4 + 1023) / 1024 * 1024 : 0;
-    const size_t budget = 227 * 1024 - 2048 - 1024;
-    if (g_bytes + 2 * slot * ngroups > budget) return cudaErrorNotSupported;
-    int depth = (int)((budget - g_bytes) / (slot * ngroups));
-    if (depth > 4) depth = 4;
-    if (depth < 2 || ngroups * depth > kMaxSlots) return cudaErrorNotSupported;
+    int e = 0, gw = 0, ngroups = 0, depth = 0;
+    size_t stage_bytes = 0;
+    auto fits = [&](int channels) {
+        e = channels;
+        gw = 1;
+        while ((int64_t)gw * 32 * e < K) gw <<= 1;
+        ngroups = (kThreads / 32) / gw;
+        if (ngroups < 1 || (gw > 1 && ngroups > 15)) return false;             // one named barrier per group
+        stage_bytes = fmt != StoreFmt::Nibble && e == 64 ? (size_t)kThreads * e : 0;
+        const size_t budget = 227 * 1024 - 2048 - 1024 - stage_bytes;
+        if (g_bytes + 2 * slot * ngroups > budget) return false;
+        depth = (int)((budget - g_bytes) / (slot * ngroups));
+        if (depth > 4) depth = 4;
+        return ngroups * depth <= kMaxSlots;
+    };
+    const bool may64 = !gated && K >= 2048 && K % 64 == 0 && !(mult != nullptr && mult_after_rotation && block >= 128);
+    if (!(may64 && fits(64)) && !fits(32)) return cudaErrorNotSupported;
+    // Short batches are latency-bound and go to the register kernel, which spreads a row over more threads.  The line is drawn
+    // by channels per SM, just behind the register kernel's first full wave; it lies higher where a row leaves lanes of its
+    // group idle, most of all with a multiplier, which such lanes' warps still read.  Chains of calls, 8-bit codes, here /
+    // register kernel:
+    //   bf16     K = 1024: M = 1184 2.61 / 2.30 us, 2368 3.15 / 3.23;  K = 2048: M = 592 2.69 / 2.32, 700 2.82 / 3.11, 2368
+    //            4.38 / 5.23;  K = 4096: M = 296 2.62 / 2.36, 370 2.82 / 3.11, 2368 6.78 / 9.30;  K = 8192: M = 148 2.70 /
+    //            2.43, 370 3.62 / 4.00, 2368 11.1 / 18.0;  K = 16384: M = 74 3.14 / 3.52, 816 10.4 / 15.2
+    //   binary32 K = 1024: M = 592 2.33 / 2.16, 1184 2.69 / 3.12;  K = 4096: M = 148 2.29 / 2.13, 592 3.73 / 5.00, 4736 17.8 /
+    //            22.3;  K = 8192: M = 592 5.8 / 7.6, 4736 34.4 / 46.2
+    //   ragged   K = 2560: M = 816 3.51 / 3.27, 1184 4.15 / 4.73, 2368 6.34 / 6.77;  K = 6144: M = 296 3.15 / 2.71, 370 3.38 /
+    //            4.00;  K = 11008: M = 148 3.26 / 2.98, 220 3.96 / 4.47
+    //   ... with a multiplier   K = 2560: M = 2368 8.9 / 8.3, 4736 15.9 / 14.3;  K = 5120: M = 1184 8.8 / 8.6, 2368 15.4 / 14.0,
+    //            4736 25.6 / 25.7;  K = 3072 (three quarters of the lanes): M = 816 4.6 / 5.0, 4736 15.4 / 16.2
+    if (!gated) {
+        const int64_t width = (int64_t)gw * 32 * e;
+        int64_t line = 15000;
+        if (width == K || K < 2048) line = xt == FQ_F32 || K >= 16384 ? 8000 : 8400;
+        else if (mult != nullptr && 4 * K < 3 * width) line = 100000;
+        if (rows * K < line * sms) return cudaErrorNotSupported;
+    }
 
     CUtensorMap map;
     const uint64_t dims[3] = {128 / esz, row_bytes / 128 * (gated ? 2 : 1), (uint64_t)rows};
     const uint64_t strides[2] = {128, (uint64_t)ldx * esz};
     const uint32_t box[3] = {(uint32_t)(128 / esz), (uint32_t)(row_bytes / 128), 1};
     if (!encode_tiled(&map, xt == FQ_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, x,
-                      dims, strides, box, true))
+                      dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B))
         return cudaErrorNotSupported;
+
+    CUtensorMap map_c;
+    memset(&map_c, 0, sizeof(map_c));
+    if (stage_bytes) {
+        const uint64_t cdims[3] = {(uint64_t)e, (uint64_t)(K / e), (uint64_t)rows};
+        const uint64_t cstrides[2] = {(uint64_t)e, (uint64_t)K};
+        const uint32_t cbox[3] = {(uint32_t)e, 32, 1};
+        if (!encode_tiled(&map_c, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, codes, cdims, cstrides, cbox, CU_TENSOR_MAP_SWIZZLE_64B))
+            return cudaErrorNotSupported;
+    }
 
     RingParams p{};
     p.rows = rows; p.K = (int)K; p.cnorm = cnorm; p.qmax = (float)qmax; p.clip_ratio = clip_ratio;
@@ -506,24 +572,25 @@ cudaError_t launch_transform_quantize_ring(const void* x, fq_dtype xt, int64_t r
     p.slot_bytes = (uint32_t)slot; p.g_bytes = (uint32_t)g_bytes;
     p.watchdog = watchdog_device_ptr();
     if (!p.watchdog) return cudaErrorUnknown;
-    const size_t smem = g_bytes + slot * ngroups * depth + 1024;
+    p.stage_off = (uint32_t)(g_bytes + slot * ngroups * depth);
+    const size_t smem = p.stage_off + stage_bytes + 1024;
     // Rows are dealt to the CTAs first and to a CTA's row groups second (row r -> CTA r % grid),
     // so that a short batch spreads over all SMs instead of filling every group of a few CTAs.
     const int grid = (int)(rows < sms ? rows : sms);
     if (gated) {
-        if (fmt == StoreFmt::Nibble) return launch_ring_block<__nv_bfloat16, 0, 32, true>(block, map, p, grid, smem, stream);
-        if (fmt == StoreFmt::Int8) return launch_ring_block<__nv_bfloat16, 1, 32, true>(block, map, p, grid, smem, stream);
-        return launch_ring_block<__nv_bfloat16, 2, 32, true>(block, map, p, grid, smem, stream);
+        if (fmt == StoreFmt::Nibble) return launch_ring_block<__nv_bfloat16, 0, 32, true>(block, map, map_c, p, grid, smem, stream);
+        if (fmt == StoreFmt::Int8) return launch_ring_block<__nv_bfloat16, 1, 32, true>(block, map, map_c, p, grid, smem, stream);
+        return launch_ring_block<__nv_bfloat16, 2, 32, true>(block, map, map_c, p, grid, smem, stream);
     }
     if (xt == FQ_BF16)
     {
-        if (fmt == StoreFmt::Nibble) return launch_ring_e<__nv_bfloat16, 0>(e, block, map, p, grid, smem, stream);
-        if (fmt == StoreFmt::Int8) return launch_ring_e<__nv_bfloat16, 1>(e, block, map, p, grid, smem, stream);
-        return launch_ring_e<__nv_bfloat16, 2>(e, block, map, p, grid, smem, stream);
+        if (fmt == StoreFmt::Nibble) return launch_ring_e<__nv_bfloat16, 0>(e, block, map, map_c, p, grid, smem, stream);
+        if (fmt == StoreFmt::Int8) return launch_ring_e<__nv_bfloat16, 1>(e, block, map, map_c, p, grid, smem, stream);
+        return launch_ring_e<__nv_bfloat16, 2>(e, block, map, map_c, p, grid, smem, stream);
     }
-    if (fmt == StoreFmt::Nibble) return launch_ring_e<float, 0>(e, block, map, p, grid, smem, stream);
-    if (fmt == StoreFmt::Int8) return launch_ring_e<float, 1>(e, block, map, p, grid, smem, stream);
-    return launch_ring_e<float, 2>(e, block, map, p, grid, smem, stream);
+    if (fmt == StoreFmt::Nibble) return launch_ring_e<float, 0>(e, block, map, map_c, p, grid, smem, stream);
+    if (fmt == StoreFmt::Int8) return launch_ring_e<float, 1>(e, block, map, map_c, p, grid, smem, stream);
+    return launch_ring_e<float, 2>(e, block, map, map_c, p, grid, smem, stream);
 }
 
 }  // namespace fq

@@ -150,7 +150,7 @@ cudaError_t launch_linear_fused(const void* x, fq_dtype xt, int64_t M, int64_t l
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no link-time libcuda dependency).
 // dims/box innermost first; strides_bytes has rank-1 entries (dimension 0 is contiguous).
 bool encode_tiled(CUtensorMap* map, CUtensorMapDataType dt, uint32_t rank, const void* ptr, const uint64_t* dims,
-                  const uint64_t* strides_bytes, const uint32_t* box, bool swizzle128);
+                  const uint64_t* strides_bytes, const uint32_t* box, CUtensorMapSwizzle swizzle);
 
 // Streaming variant of the prologue (TMA-fed shared-memory ring). Returns cudaErrorNotSupported
 // when the shape does not fit it; the caller then uses the register-only kernel.

@@ -263,10 +263,6 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int c0, int
                  ::"l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(src)
                  : "memory");
 }
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-// At most N of this thread's bulk groups still read their shared-memory source.
-template <int N>
-__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory"); }
 // One channel at two adjacent tokens: y = acc * (delta_t * s_j) + b_j, rounded to bf16, token 2k in the low half.
 __device__ __forceinline__ uint32_t scale_pair_bf16(uint32_t a0, uint32_t a1, float2 d, float2 sw2, float2 bj2) {
     const float2 a2 = make_float2((float)(int)a0, (float)(int)a1);
@@ -1085,7 +1081,7 @@ bool encode_2d(CUtensorMap* map, const void* ptr, uint64_t row_bytes, uint64_t r
 }  // namespace
 
 bool encode_tiled(CUtensorMap* map, CUtensorMapDataType dt, uint32_t rank, const void* ptr, const uint64_t* dims,
-                  const uint64_t* strides_bytes, const uint32_t* box, bool swizzle128) {
+                  const uint64_t* strides_bytes, const uint32_t* box, CUtensorMapSwizzle swizzle) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
     cuuint64_t d[5], st[5];
@@ -1093,8 +1089,7 @@ bool encode_tiled(CUtensorMap* map, CUtensorMapDataType dt, uint32_t rank, const
     for (uint32_t i = 0; i < rank; ++i) { d[i] = dims[i]; b[i] = box[i]; es[i] = 1; }
     for (uint32_t i = 0; i + 1 < rank; ++i) st[i] = strides_bytes[i];
     return fn(map, dt, rank, const_cast<void*>(ptr), d, st, b, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-              swizzle128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
-              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+              swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 namespace {

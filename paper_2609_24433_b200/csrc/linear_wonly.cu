@@ -496,7 +496,7 @@ bool build_stream_tmap(Weights& W) {
     const uint64_t dims[3] = {128, (uint64_t)row_bytes / 128, (uint64_t)W.N};
     const uint64_t strides[2] = {128, (uint64_t)row_bytes};
     const uint32_t box[3] = {128, (uint32_t)kLines, (uint32_t)kRowsCta};
-    W.tmap_stream_valid = encode_tiled(&W.tmap_stream, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, W.codes, dims, strides, box, true);
+    W.tmap_stream_valid = encode_tiled(&W.tmap_stream, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, W.codes, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
     return W.tmap_stream_valid;
 }
 

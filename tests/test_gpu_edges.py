@@ -205,3 +205,40 @@ def test_one_launch_with_fewer_units_than_cluster_ctas(M, K, block, bits):
     for _ in range(50):
         fq.linear(many, h)     # fills tensor memory with sums
         assert torch.equal(fq.linear(x, h), want)
+
+
+@pytest.mark.parametrize("M,K,block,bits,dtype,form", [
+    (607, 2048, 128, 8, "bf16", "smooth"),             # 148 SMs: the longest batch of the register kernel
+    (608, 2048, 128, 8, "bf16", "smooth"),             # ... and the shortest streamed one
+    (1052, 2112, 64, 4, "bf16", "plain"),              # one lane of the row's last warp has channels
+    (269, 8256, 32, 8, "bf16", "plain"),               # warps without any
+    (73, 16384, 256, 4, "bf16", "plain"),              # the longest rows, fewer than SMs
+    (304, 4096, 128, 8, "bf16", "after"),              # 32 channels per thread
+    (810, 1536, 256, 4, "bf16", "smooth"),
+    (1157, 1024, 64, 8, "f32", "smooth"),
+    (145, 8192, 32, 4, "f32", "plain"),
+    (868, 2560, 64, 8, "f32", "plain"),                # 64 channels per thread
+    (538, 4128, 32, 8, "f32", "plain"),
+])
+def test_streamed_prologue_on_both_sides_of_its_rule(M, K, block, bits, dtype, form):
+    """Eight rows against the oracle, all of them against short batches, which never stream; codes as a caller sees them
+    (packed or int8) and, through a small layer, as the GEMM reads them."""
+    rng = np.random.default_rng(M + K)
+    x = make_x(M, K, dtype, seed=M)
+    mult = None if form == "plain" else np.exp(rng.uniform(-1, 1, K)).astype(np.float32)
+    x_dev, m_dev, after, clip = to_dev(x, dtype), to_dev(mult), form == "after", 0.9 if bits == 8 else 1.0
+    codes, delta = fq.quantize_act(x_dev, m_dev, block, bits, clip, fold_after=after)
+    rows = rng.choice(M, 8, replace=False)
+    quantize = oracle.quantize_act_after if after else oracle.quantize_act
+    want_codes, want_delta = quantize(x[rows], dtype, mult, block, bits, clip)
+    assert np.array_equal(to_np(delta)[rows].view(np.uint32), want_delta.view(np.uint32))
+    assert np.array_equal(to_np(codes)[rows], want_codes)
+    g = torch.Generator(device="cuda").manual_seed(K)
+    h = fq.weights_import(torch.randint(0, 256, (16, K * bits // 8), dtype=torch.uint8, device="cuda", generator=g),
+                          torch.rand(16, device="cuda", generator=g) + 0.1, m_dev, None, K, block, bits, fold_after=after)
+    y = fq.linear(x_dev, h, clip)
+    for r in range(0, M, 40):
+        part = x_dev[r:r + 40]
+        c, d = fq.quantize_act(part, m_dev, block, bits, clip, fold_after=after)
+        assert torch.equal(c, codes[r:r + 40]) and torch.equal(d, delta[r:r + 40])
+        assert torch.equal(fq.linear(part, h, clip), y[r:r + 40])
