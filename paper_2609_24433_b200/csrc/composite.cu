@@ -103,8 +103,8 @@ composite_rotate_kernel(const XT* __restrict__ x, int64_t rows, int K, int64_t l
 //     matrix columns that cp.async brings a step ahead.  Ascending j from 0: the defined order.
 //   - The rotated channels stay in shared memory until the cluster has exchanged the tokens' maxima; only codes and steps
 //     leave the SM.
-// M = 816, K = 2048, block 64: 22 us with cold caches (31 us for rotation and quantizer before); matrix rows read by each lane
-// straight from L2 instead of through cp.async took 52 us.
+// M = 816, K = 2048, block 64: 15.4 us in a chain of calls, 19.7 while the clusters made two waves (31 us for rotation and
+// quantizer as two kernels, cold caches); matrix rows read by each lane straight from L2 instead of through cp.async took 52 us.
 struct CompositeParams {
     const void* x;
     int64_t ldx, rows;
@@ -340,10 +340,17 @@ cudaError_t launch_quantize(CompositeParams p, cudaStream_t stream) {
         smem = at;
         return smem <= 224 * 1024;
     };
-    // as many CTAs per tile as leave half the warps an item each, fewer once the tiles alone fill the SMs; more where the
-    // rotated channels would not fit otherwise
+    // As many CTAs per tile as leave half the warps an item each and make one wave: every CTA begins by staging the tokens'
+    // rows, so a second wave costs more than longer CTAs (block 64: M = 816, K = 2048 19.7 us with clusters of four in two
+    // waves, 15.4 with pairs in one; M = 1184, K = 1024 21.0 and 9.6).  Two CTAs share an SM where shared memory allows it
+    // (816 x 1024, block 32: 7.8 us so, 10.4 with pairs); of 148 SMs clusters of four reach 144, of eight 112.  More CTAs
+    // where the rotated channels would not fit otherwise.
+    auto one_wave = [&](int shift) {
+        const int64_t sms = device_sm_count(), reach = shift == 3 ? sms * 28 / 37 : (shift == 2 ? sms * 36 / 37 : sms);
+        return fits(shift) && (tiles << shift) <= reach * (2 * (smem + 3072) <= 228 * 1024 ? 2 : 1);
+    };
     int shift = 3;
-    while (shift > 0 && (p.items >> shift < 4 || (tiles << shift) > 2ll * device_sm_count()) && fits(shift - 1)) --shift;
+    while (shift > 0 && (p.items >> shift < 4 || !one_wave(shift)) && fits(shift - 1)) --shift;
     if (!fits(shift) || p.items >> shift < 1 || (tiles << shift) > 0x7fffffffll) {
         if constexpr (TOK == 16 && BETA >= 32) return launch_quantize<XT, BETA, 8>(p, stream);
         return cudaErrorNotSupported;

@@ -128,6 +128,8 @@ def test_one_launch_path_equals_prologue_and_gemm(M, K, N, block, bits, dtype, s
     (20, 4096, 128, 8, "f32", False, 0),               # binary32 rows of which eight fit
     (9, 8192, 64, 4, "f32", False, 0),                 # ... and none: the two-kernel form
     (20, 4096, 128, 8, "bf16", False, 4),              # rows that are not 16-byte aligned
+    (576, 2048, 64, 4, "bf16", False, 0),              # 148 SMs: the most clusters of four in one wave
+    (577, 2048, 64, 4, "bf16", True, 0),               # ... and clusters of two
 ])
 def test_composite_prologue_at_the_edges_of_its_kernels(M, K, beta, bits, dtype, smooth, lead):
     rng = np.random.default_rng(M + K)
