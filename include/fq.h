@@ -134,8 +134,9 @@ fq_status fq_weights_import_after(const void* codes, const float* w_scale, const
  * Channels are rounded in index order; each rounding error (w - q s)/U_ii is spread over the channels still to
  * come along row i of the upper Cholesky factor U of (G + lambda I)^-1.  All of it runs in binary32 in a fixed
  * order, so the codes are reproducible bit for bit.  K <= 16384 (FQ_ERR_UNSUPPORTED beyond; the factorisation is
- * column-sequential and cubic in K: 0.2 s at K = 2048, minutes at K = 16384); FQ_ERR_INVALID_ARG if
- * the damped second moment is not positive definite in binary32.  Offline: allocates (about 3 K^2 + (N + Mc) K
+ * column-sequential and cubic in K: 10 ms at K = 2048, seconds beyond K = 8192); FQ_ERR_INVALID_ARG if
+ * the damped second moment is not positive definite in binary32, FQ_ERR_TIMEOUT if a bounded wait of the
+ * factorisation expired (no handle is made).  Offline: allocates (about 3 K^2 + (N + Mc) K
  * floats of temporaries) and synchronises the stream. */
 fq_status fq_fold_weights_gptq(const void* W, fq_dtype wt, int64_t N, int64_t K, int64_t ldw, const float* smooth,
                                const float* bias, const void* calib, fq_dtype ct, int64_t Mc, int64_t ldc,
@@ -155,7 +156,8 @@ fq_status fq_fold_weights_gptq(const void* W, fq_dtype wt, int64_t N, int64_t K,
  *   synchronisation); FQ_ERR_INVALID_ARG if perm has an entry outside [0, K).  The handle's runtime multiplier is
  *   1/s_c (ones without smoothing).  The handle does not keep perm and blocks.
  * fq_quantize_act_composite: the runtime prologue of such a site (rotation, then Eq. 5); workspace device, at least
- *   4*M*K bytes, 16-byte aligned (the rotated rows in binary32; two kernels).  Entries of perm outside [0, K) are
+ *   4*M*K bytes, 16-byte aligned (the rotated rows in binary32, where a row is too long for the
+ *   one-launch kernel).  Entries of perm outside [0, K) are
  *   clamped.  Then fq_gemm_w4a4 / fq_gemm_w8a8 per consumer; the one-call fq_linear_* entry points return
  *   FQ_ERR_UNSUPPORTED for a composite handle. */
 fq_status fq_fold_weights_composite(const void* W, fq_dtype wt, int64_t N, int64_t K, int64_t ldw, const float* smooth,
@@ -277,8 +279,8 @@ fq_status fq_linear_w4a4_static(const void* x, fq_dtype xt, int64_t M, int64_t l
 
 /* Bytes of workspace that fq_gemm_* / fq_linear_* want for this shape (host computation): the int8
  * activation codes and steps (M*K + 4*M bytes, each rounded up to 256), plus scratch for int32 partial
- * tiles on shapes with few output tiles and a long K, which the GEMM then splits along K.  A workspace
- * that holds only the first part is accepted; the GEMM then runs without the split.  Everything a call
+ * tiles on shapes with few output tiles and a long K, where a device that cannot hold the clusters that
+ * otherwise share such a tile splits K through memory.  A workspace that holds only the first part is accepted.  Everything a call
  * scribbles on lives in the workspace it was given (the split's tile counters included, cleared by a
  * memset node at the head of the call): a weight handle is read-only at run time, so calls on the same
  * handle may run concurrently on different streams as long as each has its own workspace. */
