@@ -283,7 +283,7 @@ transform_quantize_kernel(const XT* __restrict__ x, int64_t rows, int K, int64_t
 
 template <typename XT, int E, int FMT>
 cudaError_t launch_e(const XT* x, int64_t rows, int K, int64_t ldx, const float* mult, float cnorm, int mult_after,
-                     int block, int qmax, float clip_ratio, void* codes, float* delta, cudaStream_t stream, int ready, int gate) {
+                     int block, int qmax, float clip_ratio, void* codes, float* delta, cudaStream_t stream, int flags, int gate) {
     const int tpr = ((K / E) + 31) / 32 * 32;
     if (tpr > kMaxThreads) return cudaErrorInvalidConfiguration;
     int rpc = 256 / tpr;
@@ -293,15 +293,15 @@ cudaError_t launch_e(const XT* x, int64_t rows, int K, int64_t ldx, const float*
     const int64_t iters = (rows + rpc - 1) / rpc;
     // Short batches let the kernel behind start at once: what it does ahead of its own wait touches weights only, and its pipelines
     // fill while the kernel AHEAD of this one still runs (the action expert's step 543 -> 529 us).  Otherwise behind the wait: a
-    // waiting GEMM takes issue slots and SMs from the prologues (M = 816 backbone layer 127.2 / 128.0 us, 16 x 8192 x 8192
-    // 13.8 / 14.1).
-    const int early = rows <= 64 && K <= 4096 ? 1 : 0;
+    // waiting GEMM takes issue slots and SMs from the prologues (M = 816 backbone layer 127.2 / 128.0 us).  For rows of up to
+    // 8192 channels it depends on what follows, which the caller knows (kTriggerEarly).
+    const int early = rows <= 64 && (K <= 4096 || (K <= 8192 && (flags & kTriggerEarly))) ? 1 : 0;
     auto args = [&](auto kern) {
         const int resident = max_resident_blocks(reinterpret_cast<const void*>(kern), threads);
         int64_t grid = iters < (int64_t)sms * resident ? iters : (int64_t)sms * resident;
         if (grid < 1) grid = 1;
         launch_pdl(kern, (unsigned)grid, (unsigned)threads, 0, stream, 1u, x, rows, K, ldx, mult, cnorm, block, (float)qmax,
-                   clip_ratio, static_cast<uint8_t*>(codes), delta, tpr, rpc, mult_after, gate, ready, early);
+                   clip_ratio, static_cast<uint8_t*>(codes), delta, tpr, rpc, mult_after, gate, flags & kMultReady, early);
     };
     const bool clamp = clip_ratio < 1.0f;
     if (gate >= 0) {
@@ -319,14 +319,14 @@ cudaError_t launch_e(const XT* x, int64_t rows, int K, int64_t ldx, const float*
 
 template <typename XT, int FMT>
 cudaError_t launch_t(const XT* x, int64_t rows, int K, int64_t ldx, const float* mult, float cnorm, int mult_after,
-                     int block, int qmax, float clip_ratio, void* codes, float* delta, cudaStream_t stream, int ready, int gate) {
+                     int block, int qmax, float clip_ratio, void* codes, float* delta, cudaStream_t stream, int flags, int gate) {
     // E = 8 keeps short rows spread over a full warp; E = 16 is the streaming default;
     // E = 32 holds K = 16384 in 512 threads (cached variant) and reaches K = 32768 in 1024.
     if (K % 16 != 0 || K <= 256)
-        return launch_e<XT, 8, FMT>(x, rows, K, ldx, mult, cnorm, mult_after, block, qmax, clip_ratio, codes, delta, stream, ready, gate);
+        return launch_e<XT, 8, FMT>(x, rows, K, ldx, mult, cnorm, mult_after, block, qmax, clip_ratio, codes, delta, stream, flags, gate);
     if (K <= 8192)
-        return launch_e<XT, 16, FMT>(x, rows, K, ldx, mult, cnorm, mult_after, block, qmax, clip_ratio, codes, delta, stream, ready, gate);
-    return launch_e<XT, 32, FMT>(x, rows, K, ldx, mult, cnorm, mult_after, block, qmax, clip_ratio, codes, delta, stream, ready, gate);
+        return launch_e<XT, 16, FMT>(x, rows, K, ldx, mult, cnorm, mult_after, block, qmax, clip_ratio, codes, delta, stream, flags, gate);
+    return launch_e<XT, 32, FMT>(x, rows, K, ldx, mult, cnorm, mult_after, block, qmax, clip_ratio, codes, delta, stream, flags, gate);
 }
 
 __global__ void multipliers_kernel(const float* __restrict__ smooth, int K, float cnorm,
@@ -410,25 +410,25 @@ __global__ void expand_nibbles_kernel(const uint4* __restrict__ packed, int64_t 
 cudaError_t launch_transform_quantize(const void* x, fq_dtype xt, int64_t rows, int64_t K, int64_t ldx,
                                       const float* mult, float cnorm, bool mult_after_rotation, int block, int qmax,
                                       float clip_ratio, StoreFmt fmt, void* codes, float* delta, cudaStream_t stream,
-                                      bool mult_ready) {
+                                      int flags) {
     if (rows == 0) return cudaSuccess;
     const int mult_after = (mult != nullptr && mult_after_rotation) ? 1 : 0;
     {   // long batches stream through the TMA-fed ring; everything else stays in registers
         const cudaError_t e = launch_transform_quantize_ring(x, xt, rows, K, ldx, mult, cnorm, mult_after != 0, block, qmax,
-                                                             clip_ratio, fmt, codes, delta, stream, -1, mult_ready);
+                                                             clip_ratio, fmt, codes, delta, stream, -1, (flags & kMultReady) != 0);
         if (e != cudaErrorNotSupported) return e;
     }
-    const int k = (int)K, ready = mult_ready ? 1 : 0;
+    const int k = (int)K;
     if (xt == FQ_F32) {
         const float* p = static_cast<const float*>(x);
-            if (fmt == StoreFmt::Nibble) return launch_t<float, 0>(p, rows, k, ldx, mult, cnorm, mult_after, block, qmax, clip_ratio, codes, delta, stream, ready, -1);
-        if (fmt == StoreFmt::Int8) return launch_t<float, 1>(p, rows, k, ldx, mult, cnorm, mult_after, block, qmax, clip_ratio, codes, delta, stream, ready, -1);
-        return launch_t<float, 2>(p, rows, k, ldx, mult, cnorm, mult_after, block, qmax, clip_ratio, codes, delta, stream, ready, -1);
+            if (fmt == StoreFmt::Nibble) return launch_t<float, 0>(p, rows, k, ldx, mult, cnorm, mult_after, block, qmax, clip_ratio, codes, delta, stream, flags, -1);
+        if (fmt == StoreFmt::Int8) return launch_t<float, 1>(p, rows, k, ldx, mult, cnorm, mult_after, block, qmax, clip_ratio, codes, delta, stream, flags, -1);
+        return launch_t<float, 2>(p, rows, k, ldx, mult, cnorm, mult_after, block, qmax, clip_ratio, codes, delta, stream, flags, -1);
     }
     const __nv_bfloat16* p = static_cast<const __nv_bfloat16*>(x);
-    if (fmt == StoreFmt::Nibble) return launch_t<__nv_bfloat16, 0>(p, rows, k, ldx, mult, cnorm, mult_after, block, qmax, clip_ratio, codes, delta, stream, ready, -1);
-    if (fmt == StoreFmt::Int8) return launch_t<__nv_bfloat16, 1>(p, rows, k, ldx, mult, cnorm, mult_after, block, qmax, clip_ratio, codes, delta, stream, ready, -1);
-    return launch_t<__nv_bfloat16, 2>(p, rows, k, ldx, mult, cnorm, mult_after, block, qmax, clip_ratio, codes, delta, stream, ready, -1);
+    if (fmt == StoreFmt::Nibble) return launch_t<__nv_bfloat16, 0>(p, rows, k, ldx, mult, cnorm, mult_after, block, qmax, clip_ratio, codes, delta, stream, flags, -1);
+    if (fmt == StoreFmt::Int8) return launch_t<__nv_bfloat16, 1>(p, rows, k, ldx, mult, cnorm, mult_after, block, qmax, clip_ratio, codes, delta, stream, flags, -1);
+    return launch_t<__nv_bfloat16, 2>(p, rows, k, ldx, mult, cnorm, mult_after, block, qmax, clip_ratio, codes, delta, stream, flags, -1);
 }
 
 // The site behind a gated MLP: x is [rows, 2K] = [gate | up], the quantizer's input is act(gate) * up.
@@ -437,7 +437,7 @@ cudaError_t launch_gated_transform_quantize(const void* x, fq_dtype xt, int64_t 
                                             float clip_ratio, StoreFmt fmt, void* codes, float* delta,
                                             cudaStream_t stream, bool mult_ready) {
     if (rows == 0) return cudaSuccess;
-    const int k = (int)K, ready = mult_ready ? 1 : 0;
+    const int k = (int)K, flags = mult_ready ? kMultReady : 0;
     const int after = mult_after_rotation ? 1 : 0;
     {
         const cudaError_t e = launch_transform_quantize_ring(x, xt, rows, K, ldx, mult, cnorm, after != 0, block, qmax, clip_ratio,
@@ -446,14 +446,14 @@ cudaError_t launch_gated_transform_quantize(const void* x, fq_dtype xt, int64_t 
     }
     if (xt == FQ_F32) {
         const float* p = static_cast<const float*>(x);
-        if (fmt == StoreFmt::Nibble) return launch_t<float, 0>(p, rows, k, ldx, mult, cnorm, after, block, qmax, clip_ratio, codes, delta, stream, ready, gate_kind);
-        if (fmt == StoreFmt::Int8) return launch_t<float, 1>(p, rows, k, ldx, mult, cnorm, after, block, qmax, clip_ratio, codes, delta, stream, ready, gate_kind);
-        return launch_t<float, 2>(p, rows, k, ldx, mult, cnorm, after, block, qmax, clip_ratio, codes, delta, stream, ready, gate_kind);
+        if (fmt == StoreFmt::Nibble) return launch_t<float, 0>(p, rows, k, ldx, mult, cnorm, after, block, qmax, clip_ratio, codes, delta, stream, flags, gate_kind);
+        if (fmt == StoreFmt::Int8) return launch_t<float, 1>(p, rows, k, ldx, mult, cnorm, after, block, qmax, clip_ratio, codes, delta, stream, flags, gate_kind);
+        return launch_t<float, 2>(p, rows, k, ldx, mult, cnorm, after, block, qmax, clip_ratio, codes, delta, stream, flags, gate_kind);
     }
     const __nv_bfloat16* p = static_cast<const __nv_bfloat16*>(x);
-    if (fmt == StoreFmt::Nibble) return launch_t<__nv_bfloat16, 0>(p, rows, k, ldx, mult, cnorm, after, block, qmax, clip_ratio, codes, delta, stream, ready, gate_kind);
-    if (fmt == StoreFmt::Int8) return launch_t<__nv_bfloat16, 1>(p, rows, k, ldx, mult, cnorm, after, block, qmax, clip_ratio, codes, delta, stream, ready, gate_kind);
-    return launch_t<__nv_bfloat16, 2>(p, rows, k, ldx, mult, cnorm, after, block, qmax, clip_ratio, codes, delta, stream, ready, gate_kind);
+    if (fmt == StoreFmt::Nibble) return launch_t<__nv_bfloat16, 0>(p, rows, k, ldx, mult, cnorm, after, block, qmax, clip_ratio, codes, delta, stream, flags, gate_kind);
+    if (fmt == StoreFmt::Int8) return launch_t<__nv_bfloat16, 1>(p, rows, k, ldx, mult, cnorm, after, block, qmax, clip_ratio, codes, delta, stream, flags, gate_kind);
+    return launch_t<__nv_bfloat16, 2>(p, rows, k, ldx, mult, cnorm, after, block, qmax, clip_ratio, codes, delta, stream, flags, gate_kind);
 }
 
 cudaError_t launch_multipliers(const float* smooth, int64_t K, float cnorm, float* mult_w, float* mult_g,

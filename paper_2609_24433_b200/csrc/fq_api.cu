@@ -240,11 +240,15 @@ fq_status linear_impl(const void* x, fq_dtype xt, int64_t M, int64_t ldx, const 
     const StoreFmt fmt = bits == 4 ? StoreFmt::Int8Perm : StoreFmt::Int8;
     // a multiplier that is block^-1/2 in every channel is passed as "none": same products, no vector to stage
     const float* mult = W->mult_const ? nullptr : W->mult_g;
+    // Rows of more than 4096 channels: the GEMM gains from an early start where it has many 8-bit weights to fetch (eager
+    // calls, early / not: 64 x 8192 x 8192 18.1 / 18.6 us, 16 x 8192 x 8192 16.3 / 17.2, 16 x 6144 x 2048 9.1 / 8.75) or many
+    // four-atom stages to unpack (4 bits: 32 x 8192 x 4096 10.6 / 11.5, 50 x 6144 x 2048 9.9 / 10.6; 16 x 8192 x 8192 14.15 / 13.8).
+    const int flags = kMultReady | ((bits == 8 ? W->N >= 4096 : M > 16) ? kTriggerEarly : 0);
     const cudaError_t pe =
         gate >= 0 ? launch_gated_transform_quantize(x, xt, M, W->K, ldx, gate, mult, block_norm(W->block), W->fold_after,
                                                     W->block, qmax, clip_ratio, fmt, ws.a8, ws.delta, s, true)
                   : launch_transform_quantize(x, xt, M, W->K, ldx, mult, block_norm(W->block), W->fold_after, W->block,
-                                              qmax, clip_ratio, fmt, ws.a8, ws.delta, s, true);
+                                              qmax, clip_ratio, fmt, ws.a8, ws.delta, s, flags);
     if (pe != cudaSuccess) return FQ_ERR_CUDA;
     if (g_profile_mark != nullptr) {
         // Inside a stream capture the mark must be an external event-record node to stay readable.

@@ -76,12 +76,14 @@ enum class StoreFmt : int { Nibble = 0, Int8 = 1, Int8Perm = 2 };
 // +-qmax, store codes in `fmt`, store per-row step to delta.
 // mult_after_rotation (fold-after sites, T = D^o R): multiply by `cnorm` before the butterflies
 // and by mult[K] after them instead.
-// mult_ready: `mult` was complete before the kernel ahead in the stream was enqueued (a handle's multiplier), so it may be
-// read before that kernel has finished.
+// flags: kMultReady: `mult` was complete before the kernel ahead in the stream was enqueued (a handle's multiplier), so it
+// may be read before that kernel has finished.  kTriggerEarly: what follows gains from starting before that kernel has
+// finished, even behind long rows.
+enum : int { kMultReady = 1, kTriggerEarly = 2 };
 cudaError_t launch_transform_quantize(const void* x, fq_dtype xt, int64_t rows, int64_t K, int64_t ldx,
                                       const float* mult, float cnorm, bool mult_after_rotation, int block,
                                       int qmax, float clip_ratio, StoreFmt fmt, void* codes, float* delta,
-                                      cudaStream_t stream, bool mult_ready = false);
+                                      cudaStream_t stream, int flags = 0);
 
 // Same, for the site behind a gated MLP: x is [rows, 2K] = [gate | up] and the input is act(gate) * up
 // (gate_kind 0 = SiLU, 1 = GELU-tanh, fixed binary32 arithmetic).

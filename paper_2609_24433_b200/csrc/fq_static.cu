@@ -86,7 +86,7 @@ extern "C" fq_status fq_linear_w4a4_static(const void* x, fq_dtype xt, int64_t M
     const cudaError_t fe = launch_linear_fused(x, xt, M, ldx, *W, cnorm, 7, clip_ratio, y, yt, ldy, nullptr, nullptr, s);
     if (fe != cudaErrorNotSupported) return fe == cudaSuccess ? FQ_OK : FQ_ERR_CUDA;
     if (launch_transform_quantize(x, xt, M, W->K, ldx, W->mult_const ? nullptr : W->mult_g, cnorm, W->fold_after, W->block, 7, clip_ratio, StoreFmt::Int8Perm, a8,
-                                  delta, s, true) != cudaSuccess)
+                                  delta, s, kMultReady) != cudaSuccess)
         return FQ_ERR_CUDA;
     GemmOut out;
     out.y = y; out.yt = yt; out.ldy = ldy; out.a_delta = delta;
