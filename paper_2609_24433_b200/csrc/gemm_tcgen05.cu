@@ -1176,6 +1176,7 @@ int cluster_capacity(int ctas);
 //                           4096 x 8192 x 8192 199 / 200 and 235 / 238, 12000 x 2048 x 8192 158 / 163 and 189 / 194; below
 //                           the line 7000 x 4096 x 4096 103 / 100 and 117 / 119, 4096 x 4096 x 4096 67.2 / 64.9 and 73.0 /
 //                           73.3; a short K: 16384 x 1024 x 4096 96 / 97 and 105 / 104.
+// (A plan takes the host 0.1 to 3 us; asking for the clusters of every candidate first took up to 30.)
 // K split: problems with fewer tiles than SMs and a long K (short batches, few output channels).
 //   By clusters of 2, 4 or 8 CTAs (one wave; at least four k-blocks of ring beside the sums, 4-bit tiles of at most 128
 //   tokens): the tail shrinks to 16*bt/split, the exchange costs 2800 + 40 per CTA of the launch at 4 bits, 3300 + 18 at 8
@@ -1191,6 +1192,11 @@ Plan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t scratc
     const int64_t kb = (K + kBlockK - 1) / kBlockK;
     Plan best;
     double best_cost = 0.0;
+    int capacity[kMaxCluster + 1] = {};                  // by CTAs per cluster, asked for once per plan; 0: not yet, else + 1
+    auto held = [&](int ctas) {
+        if (capacity[ctas] == 0) capacity[ctas] = cluster_capacity(ctas) + 1;
+        return capacity[ctas] - 1;
+    };
     const bool pairs = N > kTileN && (bits == 8 || (K >= 2048 && (double)M * (double)N * (double)K >= 1.6e11));
     for (int c = 1; c <= (pairs ? 2 : 1); ++c) {
         const int64_t n_units = (N + kTileN * c - 1) / (kTileN * c);
@@ -1212,13 +1218,14 @@ Plan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t scratc
             };
             offer(1, false, 0, (double)kb * per_kb + 16.0 * b + 1000.0);
             if (bits == 4 && c == 2) continue;           // (long launches have tiles enough: no kernel for a split of these)
+            if (units * 2 > slots && units * c * 2 > 4 * (int64_t)sms) continue;       // too many tiles for any split
             for (int sp = 2; sp <= kMaxSplit; sp *= 2) {
                 if (kb % sp != 0 || kb / sp < 2) break;
                 const double slice = (double)(kb / sp) * per_kb + 1000.0;
                 const int atoms = atoms_per_stage(bits, c, b, K, sp);
                 const double ctas = (double)(units * sp * c);
-                if (clusters && (bits == 8 || b <= 128) && sp * c <= kMaxCluster && units <= cluster_capacity(sp * c) &&
-                    units * sp <= slots && ring_budget(cluster_sums_bytes(b, sp)) * atoms >= 4 * stage_bytes(bits, c, b, atoms))
+                if (clusters && (bits == 8 || b <= 128) && sp * c <= kMaxCluster && units * sp <= slots &&
+                    ring_budget(cluster_sums_bytes(b, sp)) * atoms >= 4 * stage_bytes(bits, c, b, atoms) && units <= held(sp * c))
                     offer(sp, true, 0, slice + 16.0 * b / sp + (bits == 4 ? 2800.0 + 40.0 * ctas : 3300.0 + 18.0 * ctas) + 500.0 * (sp - 1));
                 if ((c == 1 || bits == 8) && units * c <= kMaxSplitTiles && units * c * sp <= 4 * (int64_t)sms) {
                     const size_t scratch = kCounterBytes + (size_t)units * c * sp * kTileN * b * sizeof(int32_t);
