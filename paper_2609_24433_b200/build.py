@@ -33,7 +33,7 @@ def build_binding(force: bool = False) -> str:
                sysconfig.get_paths()["include"], "/usr/local/cuda/include"]
         subprocess.run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared"] + [f for d in inc for f in ("-I", d)] +
                        [src, "-o", BINDING, "-L", HERE, "-l:" + os.path.basename(LIB), "-L", os.path.join(t, "lib"), "-lc10",
-                        "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-Wl,-rpath,$ORIGIN"], check=True)
+                        "-lc10_cuda", "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python", "-Wl,-rpath,$ORIGIN"], check=True)
     return BINDING
 
 

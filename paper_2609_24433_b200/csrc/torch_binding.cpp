@@ -9,6 +9,7 @@
 #include <Python.h>
 
 #include <ATen/ATen.h>
+#include <ATen/cuda/EmptyTensor.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Dtype.h>
 #include <torch/csrc/Exceptions.h>
@@ -62,7 +63,9 @@ void* stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 bool none(PyObject* o) { return o == Py_None; }
 PyObject* status(fq_status s) { return PyLong_FromLong(s); }
 
+// (on a GPU straight from the allocator: at::empty's way through the dispatcher costs as much again)
 at::Tensor fresh(at::IntArrayRef size, at::ScalarType t, const at::Tensor& like) {
+    if (like.is_cuda()) return at::Tensor(at::detail::empty_cuda(size, t, like.device(), std::nullopt));
     return at::empty(size, at::TensorOptions().dtype(t).device(like.device()));
 }
 
