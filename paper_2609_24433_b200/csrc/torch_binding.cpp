@@ -124,27 +124,41 @@ PyObject* guarded(F f) {
     END_HANDLE_TH_ERRORS
 }
 
-// linear(x, handle, K, N, handle_bits, bits, clip_ratio, out_dtype, y, workspace, gate): gate -1 = fq_linear_w4a4 / _w8a8
-// by `bits`, else fq_linear_gated with that function
-PyObject* linear(PyObject*, PyObject* const* a, Py_ssize_t n) {
+// The arguments that the one-call entry points share: (x, handle, K, N, handle_bits, ., clip_ratio, out_dtype, y, workspace)
+template <typename F>
+PyObject* one_call(PyObject* const* a, Py_ssize_t n, F run) {
     return guarded([&]() -> PyObject* {
-        arguments(n, 11);
+        arguments(n, 10);
         const at::Tensor& x = rowmajor(a[0]);
         const fq_weights* W = static_cast<const fq_weights*>(address(a[1]));
         const int64_t K = integer(a[2]), N = integer(a[3]), M = x.size(0);
-        const int handle_bits = static_cast<int>(integer(a[4])), bits = static_cast<int>(integer(a[5]));
-        const int gate = static_cast<int>(integer(a[10]));
+        const int handle_bits = static_cast<int>(integer(a[4]));
+        const long long which = integer(a[5]);
         const float clip = real(a[6]);
         const fq_dtype xt = dtype_of(x.scalar_type());
         fq_dtype yt;
         at::Tensor y = output(a[8], a[7], M, N, x, &yt);
         const Workspace ws(a[9], none(a[9]) ? fq_workspace_bytes(M, K, N, handle_bits) : 0, x);
-        const fq_status s =
-            gate >= 0 ? fq_linear_gated(x.data_ptr(), xt, M, x.stride(0), static_cast<fq_gate_act>(gate), W, clip, y.data_ptr(),
-                                        yt, y.stride(0), ws.p, ws.bytes, stream())
-                      : (bits == 4 ? fq_linear_w4a4 : fq_linear_w8a8)(x.data_ptr(), xt, M, x.stride(0), W, clip, y.data_ptr(), yt,
-                                                                      y.stride(0), ws.p, ws.bytes, stream());
+        const fq_status s = run(which, x.data_ptr(), xt, M, x.stride(0), W, clip, y.data_ptr(), yt, y.stride(0), ws.p, ws.bytes);
         return s == FQ_OK ? THPVariable_Wrap(std::move(y)) : status(s);
+    });
+}
+
+// linear(x, handle, K, N, handle_bits, bits, clip_ratio, out_dtype, y, workspace): fq_linear_w4a4 / _w8a8 by `bits`
+PyObject* linear(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    return one_call(a, n, [](long long bits, const void* x, fq_dtype xt, int64_t M, int64_t ldx, const fq_weights* W, float clip,
+                             void* y, fq_dtype yt, int64_t ldy, void* ws, size_t ws_bytes) {
+        return (bits == 4 ? fq_linear_w4a4 : fq_linear_w8a8)(x, xt, M, ldx, W, clip, y, yt, ldy, ws, ws_bytes, stream());
+    });
+}
+
+// linear_gated(x, handle, K, N, handle_bits, act, clip_ratio, out_dtype, y, workspace): fq_linear_gated.  (`act` is the
+// caller's: whatever is neither function is refused as the library refuses it, ahead of its narrowing to the enumeration.)
+PyObject* linear_gated(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    return one_call(a, n, [](long long act, const void* x, fq_dtype xt, int64_t M, int64_t ldx, const fq_weights* W, float clip,
+                             void* y, fq_dtype yt, int64_t ldy, void* ws, size_t ws_bytes) {
+        if (act != FQ_GATE_SILU && act != FQ_GATE_GELU_TANH) return FQ_ERR_INVALID_ARG;
+        return fq_linear_gated(x, xt, M, ldx, static_cast<fq_gate_act>(act), W, clip, y, yt, ldy, ws, ws_bytes, stream());
     });
 }
 
@@ -224,7 +238,7 @@ PyObject* linear_w4a16(PyObject*, PyObject* const* a, Py_ssize_t n) {
 }
 
 #define FQ_METHOD(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(name)), METH_FASTCALL, nullptr}
-PyMethodDef methods[] = {FQ_METHOD(linear), FQ_METHOD(gemm), FQ_METHOD(quantize_act), FQ_METHOD(quantize_act_composite),
+PyMethodDef methods[] = {FQ_METHOD(linear), FQ_METHOD(linear_gated), FQ_METHOD(gemm), FQ_METHOD(quantize_act), FQ_METHOD(quantize_act_composite),
                          FQ_METHOD(linear_w4a16), {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_fq_torch", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 

@@ -308,11 +308,11 @@ def gemm_w8a8(a_codes, a_delta, W: Weights, out_dtype=torch.float32, y=None, wor
 
 
 def linear_w4a4(x, W: Weights, clip_ratio: float = 1.0, out_dtype=torch.float32, y=None, workspace=None):
-    return _result(_native().linear(x, W.address, W.K, W.N, W.bits, 4, clip_ratio, out_dtype, y, workspace, -1), "fq_linear_w4a4")
+    return _result(_native().linear(x, W.address, W.K, W.N, W.bits, 4, clip_ratio, out_dtype, y, workspace), "fq_linear_w4a4")
 
 
 def linear_w8a8(x, W: Weights, clip_ratio: float = 1.0, out_dtype=torch.float32, y=None, workspace=None):
-    return _result(_native().linear(x, W.address, W.K, W.N, W.bits, 8, clip_ratio, out_dtype, y, workspace, -1), "fq_linear_w8a8")
+    return _result(_native().linear(x, W.address, W.K, W.N, W.bits, 8, clip_ratio, out_dtype, y, workspace), "fq_linear_w8a8")
 
 
 STATIC_MAX_CODE_BYTES = 4 << 20
@@ -353,7 +353,7 @@ def quantize_act_gated(gate_up: torch.Tensor, act: int, mult_g, hadamard_block: 
 def linear_gated(gate_up: torch.Tensor, act: int, W: Weights, clip_ratio: float = 1.0, out_dtype=torch.float32, y=None,
                  workspace=None):
     """down_proj with the gate product fused into its prologue: y = linear(act(gate) * up)."""
-    return _result(_native().linear(gate_up, W.address, W.K, W.N, W.bits, W.bits, clip_ratio, out_dtype, y, workspace, act),
+    return _result(_native().linear_gated(gate_up, W.address, W.K, W.N, W.bits, act, clip_ratio, out_dtype, y, workspace),
                    "fq_linear_gated")
 
 

@@ -244,3 +244,13 @@ def test_streamed_prologue_on_both_sides_of_its_rule(M, K, block, bits, dtype, f
         c, d = fq.quantize_act(part, m_dev, block, bits, clip, fold_after=after)
         assert torch.equal(c, codes[r:r + 40]) and torch.equal(d, delta[r:r + 40])
         assert torch.equal(fq.linear(part, h, clip), y[r:r + 40])
+
+
+@pytest.mark.parametrize("act", [-1, -7, 2, 1 << 32, (1 << 32) + 1])
+def test_linear_gated_refuses_what_is_no_gate(act):
+    """No number but the two functions' own is a gate: not one that could stand for "ungated", nor one that is narrowed."""
+    h = fq.fold_weights(torch.randn(16, 64, device="cuda"), None, None, 32, 4)
+    gate_up = torch.randn(4, 128, device="cuda")
+    with pytest.raises(fq.FqError) as e:
+        fq.linear_gated(gate_up, act, h)
+    assert e.value.status == fq.ERR_INVALID_ARG
