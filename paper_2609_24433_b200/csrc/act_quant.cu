@@ -38,7 +38,7 @@ struct RawRow<float, E> {
     __device__ __forceinline__ void load(const float* p, bool pred) {
 #pragma unroll
         for (int i = 0; i < E / 4; ++i)
-            q[i] = pred ? __ldg(reinterpret_cast<const float4*>(p) + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+            q[i] = ld_global_f4(reinterpret_cast<const float4*>(p) + i, pred);
     }
     __device__ __forceinline__ void widen(float* v) const {
 #pragma unroll
@@ -57,7 +57,7 @@ struct RawRow<__nv_bfloat16, E> {
     __device__ __forceinline__ void load(const __nv_bfloat16* p, bool pred) {
 #pragma unroll
         for (int i = 0; i < E / 8; ++i)
-            q[i] = pred ? __ldg(reinterpret_cast<const uint4*>(p) + i) : make_uint4(0u, 0u, 0u, 0u);
+            q[i] = ld_global_v4(reinterpret_cast<const uint4*>(p) + i, pred);
     }
     __device__ __forceinline__ void widen(float* v) const {
 #pragma unroll
@@ -102,7 +102,7 @@ transform_quantize_kernel(const XT* __restrict__ x, int64_t rows, int K, int64_t
         if (mult != nullptr && col_ok) {
 #pragma unroll
             for (int i = 0; i < E / 4; ++i) {
-                float4 t = __ldg(reinterpret_cast<const float4*>(mult + col0) + i);
+                float4 t = ld_global_f4(reinterpret_cast<const float4*>(mult + col0) + i);
                 g[(4 * i + 0) % (CACHE ? E : 1)] = t.x; g[(4 * i + 1) % (CACHE ? E : 1)] = t.y;
                 g[(4 * i + 2) % (CACHE ? E : 1)] = t.z; g[(4 * i + 3) % (CACHE ? E : 1)] = t.w;
             }
@@ -145,17 +145,21 @@ transform_quantize_kernel(const XT* __restrict__ x, int64_t rows, int K, int64_t
             raw.load(x + row * ldx + col0, row_ok);
             raw.widen(v);
             if (GATED) {
-                RawRow<XT, E> up;
-                up.load(x + row * ldx + K + col0, row_ok);
-                float u[E];
-                up.widen(u);
+                // (binary32: eight channels at a time, sixty-four registers do not hold both halves)
+                constexpr int kUp = sizeof(XT) == 4 ? 8 : E;
+                RawRow<XT, kUp> up;
+                float u[kUp];
 #pragma unroll
                 for (int i = 0; i < E; i += 8) {
+                    if (i % kUp == 0) {
+                        up.load(x + row * ldx + K + col0 + i, row_ok);
+                        up.widen(u);
+                    }
                     float2 gp[4], upp[4];
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         gp[j] = make_float2(v[i + 2 * j], v[i + 2 * j + 1]);
-                        upp[j] = make_float2(u[i + 2 * j], u[i + 2 * j + 1]);
+                        upp[j] = make_float2(u[(i + 2 * j) % kUp], u[(i + 2 * j + 1) % kUp]);
                     }
                     gate_product<4>(gp, upp, gate_kind);
 #pragma unroll
@@ -165,7 +169,7 @@ transform_quantize_kernel(const XT* __restrict__ x, int64_t rows, int K, int64_t
             if (mult != nullptr && col_ok && !mult_after) {
 #pragma unroll
                 for (int i = 0; i < E / 4; ++i) {
-                    const float4 t = __ldg(reinterpret_cast<const float4*>(mult + col0) + i);
+                    const float4 t = ld_global_f4(reinterpret_cast<const float4*>(mult + col0) + i);
                     v[4 * i + 0] = __fmul_rn(v[4 * i + 0], t.x);
                     v[4 * i + 1] = __fmul_rn(v[4 * i + 1], t.y);
                     v[4 * i + 2] = __fmul_rn(v[4 * i + 2], t.z);
@@ -209,7 +213,7 @@ transform_quantize_kernel(const XT* __restrict__ x, int64_t rows, int K, int64_t
             } else if (col_ok) {
 #pragma unroll
                 for (int i = 0; i < E / 4; ++i) {
-                    const float4 t = __ldg(reinterpret_cast<const float4*>(mult + col0) + i);
+                    const float4 t = ld_global_f4(reinterpret_cast<const float4*>(mult + col0) + i);
                     v[4 * i + 0] = __fmul_rn(v[4 * i + 0], t.x);
                     v[4 * i + 1] = __fmul_rn(v[4 * i + 1], t.y);
                     v[4 * i + 2] = __fmul_rn(v[4 * i + 2], t.z);
@@ -391,7 +395,7 @@ __global__ void expand_nibbles_kernel(const uint4* __restrict__ packed, int64_t 
     griddep_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_vec) return;
-    const uint4 p = __ldg(packed + i);
+    const uint4 p = ld_global_v4(packed + i);
     const uint32_t w[4] = {p.x, p.y, p.z, p.w};
     uint32_t o[8];
 #pragma unroll

@@ -173,7 +173,7 @@ transform_quantize_ring_kernel(const __grid_constant__ CUtensorMap map_x, const 
         // operands of the packed multiply (no register moves to pair them up), and the 16-byte pieces are
         // XOR-swizzled by the slice index, so that the slice-per-thread reads are bank-conflict free.
         for (int i = tid * 4; i < p.K; i += kThreads * 4) {
-            const float4 g4 = __ldg(reinterpret_cast<const float4*>(p.mult + i));
+            const float4 g4 = ld_global_f4(p.mult + i);
             const float gv[4] = {g4.x, g4.y, g4.z, g4.w};
             const uint32_t slice = (uint32_t)i / E;
             const uint32_t key = (slice & 7u) << 4;

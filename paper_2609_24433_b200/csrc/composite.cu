@@ -28,10 +28,10 @@ constexpr int kChunkJ = 32;          // columns of B staged at a time
 template <typename XT>
 __device__ __forceinline__ float load_as_float(const XT* p);
 template <>
-__device__ __forceinline__ float load_as_float<float>(const float* p) { return __ldg(p); }
+__device__ __forceinline__ float load_as_float<float>(const float* p) { return ld_global_f32(p); }
 template <>
 __device__ __forceinline__ float load_as_float<__nv_bfloat16>(const __nv_bfloat16* p) {
-    return __uint_as_float((uint32_t)__ldg(reinterpret_cast<const unsigned short*>(p)) << 16);
+    return __uint_as_float(ld_global_u16(p) << 16);
 }
 
 // BETA in {16, 32, 64, 128, 256}.  Thread (group = tid / BETA, i = tid % BETA) computes output i of
@@ -54,12 +54,12 @@ composite_rotate_kernel(const XT* __restrict__ x, int64_t rows, int K, int64_t l
     // gather: p[tok][j] = x[tok][perm[b*BETA + j]] * d[perm[...]]   (an index outside [0, K) is clamped)
     for (int o = tid; o < TOK * BETA; o += kThreads) {
         const int tok = o / BETA, j = o % BETA;
-        int src = __ldg(perm + b * BETA + j);
+        int src = (int)ld_global_u32(perm + b * BETA + j);
         src = src < 0 ? 0 : (src >= K ? K - 1 : src);
         float v = 0.0f;
         if (tile0 + tok < rows) {
             v = load_as_float<XT>(x + (tile0 + tok) * ldx + src);
-            if (diag != nullptr) v = __fmul_rn(v, __ldg(diag + src));
+            if (diag != nullptr) v = __fmul_rn(v, ld_global_f32(diag + src));
         }
         s_p[j][tok] = v;
     }
@@ -73,7 +73,7 @@ composite_rotate_kernel(const XT* __restrict__ x, int64_t rows, int K, int64_t l
         constexpr int CJ = BETA < kChunkJ ? BETA : kChunkJ;
         for (int o = tid; o < BETA * CJ; o += kThreads) {
             const int row = o / CJ, jj = o % CJ;     // consecutive threads: consecutive columns of one row
-            s_b[jj][row] = __ldg(B + (size_t)row * BETA + j0 + jj);
+            s_b[jj][row] = ld_global_f32(B + (size_t)row * BETA + j0 + jj);
         }
         __syncthreads();
 #pragma unroll 8
@@ -167,7 +167,10 @@ composite_quantize_kernel(const CompositeParams p) {
             for (int c = tid * V; c < p.K; c += kThreads * V) cp_async16(smem_u32(s_x + r * p.K + c), xr + r * p.ldx + c);
     } else {
         for (int r = 0; r < mine; ++r)
-            for (int c = tid; c < p.K; c += kThreads) const_cast<XT*>(s_x)[r * p.K + c] = xr[r * p.ldx + c];
+            for (int c = tid; c < p.K; c += kThreads) {
+                if (sizeof(XT) == 2) reinterpret_cast<uint16_t*>(s_raw)[r * p.K + c] = (uint16_t)ld_global_u16(xr + r * p.ldx + c);
+                else reinterpret_cast<uint32_t*>(s_raw)[r * p.K + c] = ld_global_u32(xr + r * p.ldx + c);
+            }
     }
     cp_commit();
     // step (item, columns) of this warp: 16 columns of the item's matrix rows, 64 bytes a row, 16-byte chunks XORed by the row
@@ -184,10 +187,10 @@ composite_quantize_kernel(const CompositeParams p) {
     };
     fetch(item0 + warp, 0, 0);
     for (int i = tid; i < p.span && c0 + i < p.K; i += kThreads) {
-        int src = __ldg(p.perm + c0 + i);              // (an index outside [0, K) is clamped)
+        int src = (int)ld_global_u32(p.perm + c0 + i); // (an index outside [0, K) is clamped)
         src = src < 0 ? 0 : (src >= p.K ? p.K - 1 : src);
         s_src[i] = src;
-        s_dg[i] = p.diag != nullptr ? __ldg(p.diag + src) : 1.0f;
+        s_dg[i] = p.diag != nullptr ? ld_global_f32(p.diag + src) : 1.0f;
     }
     cp_wait<1>();                                      // the rows of x (the first matrix columns may still be on their way)
     __syncthreads();

@@ -39,8 +39,11 @@ int device_cc_major();                                              // compute-c
 cudaError_t ensure_dynamic_smem(const void* kernel, size_t bytes);  // opt a kernel in to `bytes` of dynamic shared memory
 int max_resident_blocks(const void* kernel, int threads);           // thread blocks of a kernel one SM holds (no dynamic smem)
 
-// Launch with programmatic stream serialization (the kernel must call griddep_wait() before its first
-// global-memory access) and, optionally, a thread-block cluster along x.
+// Launch with programmatic stream serialization and, optionally, a thread-block cluster along x.  The kernel may start while
+// kernels ahead of it in the stream are still running, so ahead of griddep_wait() it reads only what was complete before
+// those were enqueued (what a weight handle holds); what one of them may write -- anything else that the caller passes in,
+// the workspace -- it may at most prefetch into L2 there, and reads it behind the wait, with the ld_global_* of
+// ptx_sm100.cuh or the copy engine.  It writes no global memory ahead of the wait.
 template <typename Kern, typename... Args>
 inline cudaError_t launch_pdl(Kern kern, unsigned grid, unsigned block, size_t smem, cudaStream_t stream,
                               unsigned cluster_x, Args... args) {

@@ -424,12 +424,12 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         if (tc + 16 <= p.M && p.delta_vec) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const float4 q = __ldg(reinterpret_cast<const float4*>(p.out.a_delta + tc) + i);
+                const float4 q = ld_global_f4(p.out.a_delta + tc + 4 * i);
                 d[4 * i + 0] = q.x; d[4 * i + 1] = q.y; d[4 * i + 2] = q.z; d[4 * i + 3] = q.w;
             }
         } else {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) d[i] = tc + i < p.M ? __ldg(p.out.a_delta + tc + i) : 0.0f;
+            for (int i = 0; i < 16; ++i) d[i] = tc + i < p.M ? ld_global_f32(p.out.a_delta + tc + i) : 0.0f;
         }
         tmem_ld_wait();                          // (the sums may still be on their way)
         if (p.out.yt == FQ_BF16) {
@@ -736,10 +736,10 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                     tmem_ld_16x256b_x2(taddr + (uint32_t)c, na);                    // channels 0..15 of the quadrant
                     tmem_ld_16x256b_x2(taddr + (16u << 16) + (uint32_t)c, nb);      // channels 16..31
                     const int64_t ta = t0 + c + 2 * q, tb = ta + 8;
-                    nd0.x = ta < p.M ? __ldg(p.out.a_delta + ta) : 0.0f;
-                    nd0.y = ta + 1 < p.M ? __ldg(p.out.a_delta + ta + 1) : 0.0f;
-                    nd1.x = tb < p.M ? __ldg(p.out.a_delta + tb) : 0.0f;
-                    nd1.y = tb + 1 < p.M ? __ldg(p.out.a_delta + tb + 1) : 0.0f;
+                    nd0.x = ta < p.M ? ld_global_f32(p.out.a_delta + ta) : 0.0f;
+                    nd0.y = ta + 1 < p.M ? ld_global_f32(p.out.a_delta + ta + 1) : 0.0f;
+                    nd1.x = tb < p.M ? ld_global_f32(p.out.a_delta + tb) : 0.0f;
+                    nd1.y = tb + 1 < p.M ? ld_global_f32(p.out.a_delta + tb + 1) : 0.0f;
                 };
                 if (t0 + half * 16 < p.M) request(half * 16);
                 for (int c = half * 16; c < p.bt; c += 32) {

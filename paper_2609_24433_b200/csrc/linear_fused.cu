@@ -65,8 +65,8 @@ template <>
 struct Row<__nv_bfloat16> {
     uint4 lo, hi;
     __device__ __forceinline__ void load(const __nv_bfloat16* p, bool ok) {
-        lo = ok ? __ldg(reinterpret_cast<const uint4*>(p)) : make_uint4(0u, 0u, 0u, 0u);
-        hi = ok ? __ldg(reinterpret_cast<const uint4*>(p) + 1) : make_uint4(0u, 0u, 0u, 0u);
+        lo = ld_global_v4(p, ok);
+        hi = ld_global_v4(p + 8, ok);
     }
     __device__ __forceinline__ void widen(float2* v) const {
         const uint32_t wl[4] = {lo.x, lo.y, lo.z, lo.w}, wh[4] = {hi.x, hi.y, hi.z, hi.w};
@@ -82,7 +82,7 @@ struct Row<float> {
     float4 q[4];
     __device__ __forceinline__ void load(const float* p, bool ok) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) q[i] = ok ? __ldg(reinterpret_cast<const float4*>(p) + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int i = 0; i < 4; ++i) q[i] = ld_global_f4(p + 4 * i, ok);
     }
     __device__ __forceinline__ void widen(float2* v) const {
 #pragma unroll

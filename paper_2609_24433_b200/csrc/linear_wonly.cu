@@ -101,7 +101,7 @@ struct XFrag<kModeInt> {
     uint32_t b[1][8];
     __device__ __forceinline__ void fetch(const int8_t* p, bool ok) {
 #pragma unroll
-        for (int h = 0; h < 2; ++h) raw[h] = ok ? __ldg(reinterpret_cast<const uint4*>(p) + h) : make_uint4(0u, 0u, 0u, 0u);
+        for (int h = 0; h < 2; ++h) raw[h] = ld_global_v4(p + 16 * h, ok);
     }
     __device__ __forceinline__ void permute() {
 #pragma unroll
@@ -118,7 +118,7 @@ struct XFrag<kModeInt8> {
     uint4 raw[1];
     uint32_t b[1][4];
     __device__ __forceinline__ void fetch(const int8_t* p, bool ok) {
-        raw[0] = ok ? __ldg(reinterpret_cast<const uint4*>(p)) : make_uint4(0u, 0u, 0u, 0u);
+        raw[0] = ld_global_v4(p, ok);
     }
     __device__ __forceinline__ void permute() { b[0][0] = raw[0].x; b[0][1] = raw[0].y; b[0][2] = raw[0].z; b[0][3] = raw[0].w; }
 };
@@ -131,7 +131,7 @@ struct XFrag<kModeBf16> {
     uint32_t b[1][16];
     __device__ __forceinline__ void fetch(const __nv_bfloat16* p, bool ok) {
 #pragma unroll
-        for (int w = 0; w < 4; ++w) raw[w] = ok ? __ldg(reinterpret_cast<const uint4*>(p) + w) : make_uint4(0u, 0u, 0u, 0u);
+        for (int w = 0; w < 4; ++w) raw[w] = ld_global_v4(p + 8 * w, ok);
     }
     __device__ __forceinline__ void permute() {
 #pragma unroll
@@ -153,7 +153,7 @@ struct XFrag<kModeF32> {
     uint32_t b[3][16];
     __device__ __forceinline__ void fetch(const float* p, bool ok) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) raw[i] = ok ? __ldg(reinterpret_cast<const float4*>(p) + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int i = 0; i < 8; ++i) raw[i] = ld_global_f4(p + 4 * i, ok);
     }
     __device__ __forceinline__ void permute() {
 #pragma unroll
@@ -297,7 +297,7 @@ weight_stream_kernel(const __grid_constant__ CUtensorMap map_w, const StreamPara
                 if (has_out && (!kIntegers || p.acc_out == nullptr)) {
                     out_scale = __ldg(p.w_scale + out_j);
                     out_bias = __ldg(p.bias + out_j);
-                    if (kIntegers) out_delta = __ldg(p.a_delta + out_t);
+                    if (kIntegers) out_delta = ld_global_f32(p.a_delta + out_t);
                 }
                 [[maybe_unused]] const uint32_t minus136[4] = {0xC308C308u, 0xC308C308u, 0xC308C308u, 0xC308C308u};   // bf16 -136
                 XFrag<MODE> xf[GROUPS];

@@ -178,6 +178,39 @@ __device__ __forceinline__ void griddep_launch_dependents() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// Loads, behind griddep_wait(), of memory that a kernel ahead may have written while this one was already resident: what
+// the caller passes in (tokens, steps, codes, a multiplier of its own) and what an earlier kernel of the call left in the
+// workspace.  Not __ldg and not through `const T* __restrict__`, which become loads of the non-coherent kind: those are for
+// memory that nobody writes as long as the kernel lives, and the compiler may move them across the wait.  Three calls in a
+// row share an SM (the third one is resident before the first has ended), so a line read by the first may have been
+// rewritten when the third one reads it.  (What a complete handle holds is written by nobody: __ldg, ahead of the wait or behind.)
+__device__ __forceinline__ uint4 ld_global_v4(const void* p, bool ok = true) {      // zeros where !ok
+    uint4 v;
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "mov.b32 %0, 0;\n\tmov.b32 %1, 0;\n\tmov.b32 %2, 0;\n\tmov.b32 %3, 0;\n\t"
+        "@q ld.global.v4.b32 {%0, %1, %2, %3}, [%4];\n\t}"
+        : "=&r"(v.x), "=&r"(v.y), "=&r"(v.z), "=&r"(v.w)
+        : "l"(p), "r"((uint32_t)ok));
+    return v;
+}
+__device__ __forceinline__ float4 ld_global_f4(const void* p, bool ok = true) {
+    const uint4 v = ld_global_v4(p, ok);
+    return make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w));
+}
+__device__ __forceinline__ uint32_t ld_global_u32(const void* p) {
+    uint32_t v;
+    asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float ld_global_f32(const float* p) { return __uint_as_float(ld_global_u32(p)); }
+__device__ __forceinline__ uint32_t ld_global_u16(const void* p) {
+    uint16_t v;
+    asm volatile("ld.global.b16 %0, [%1];" : "=h"(v) : "l"(p));
+    return v;
+}
+
 // Ask for the 128-byte line at p to be brought into L2.  No value is read: allowed ahead of griddep_wait() even for memory
 // that the kernel in front is writing.
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }

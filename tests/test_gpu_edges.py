@@ -254,3 +254,47 @@ def test_linear_gated_refuses_what_is_no_gate(act):
     with pytest.raises(fq.FqError) as e:
         fq.linear_gated(gate_up, act, h)
     assert e.value.status == fq.ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("M,K,bits,call", [
+    (50, 1024, 4, "linear"),           # one launch a call
+    (64, 1024, 8, "linear"),
+    (5, 768, 4, "linear"),
+    (24, 4096, 4, "linear"),           # prologue and GEMM
+    (12, 4096, 8, "linear"),           # prologue and weight streaming
+    (300, 1024, 4, "linear"),
+    (2, 1536, 4, "linear_w4a16"),
+])
+def test_calls_that_pass_two_buffers_to_and_fro(M, K, bits, call):
+    """A -> B, B -> A, A -> B ...: kernels of three calls are resident at a time, and the third reads what the second wrote over the
+    first one's input.  As a graph and eagerly, against the same calls with a synchronisation behind each."""
+    g = torch.Generator(device="cuda").manual_seed(M + K)
+    hs = [fq.weights_import(torch.randint(0, 256, (K, K * bits // 8), dtype=torch.uint8, device="cuda", generator=g),
+                            (torch.rand(K, device="cuda", generator=g) + 0.5) / (0.3 * K ** 0.5 * (5 if bits == 4 else 74)), None,
+                            torch.randn(K, device="cuda", generator=g), K, 64 if call == "linear" else 1, bits) for _ in range(3)]
+    ws = torch.empty(fq.workspace_bytes(M, K, K, bits), dtype=torch.uint8, device="cuda")
+    a, b = (torch.empty(M, K, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    start = torch.randn(M, K, device="cuda", generator=g).to(torch.bfloat16)
+
+    def chain(sync=False):
+        a.copy_(start)
+        x, y = a, b
+        for step in range(13):
+            if call == "linear":
+                fq.linear(x, hs[step % 3], y=y, workspace=ws)
+            else:
+                fq.linear_w4a16(x, hs[step % 3], y=y)
+            if sync:
+                torch.cuda.synchronize()
+            x, y = y, x
+
+    chain(sync=True)
+    want = a.clone(), b.clone()
+    assert all(w.isfinite().all() and w.float().std() > 0.1 for w in want)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        chain()
+    for run in [graph.replay] * 40 + [chain] * 10:
+        a.fill_(7.0), b.fill_(7.0)
+        run()
+        assert torch.equal(a, want[0]) and torch.equal(b, want[1])
