@@ -7,6 +7,7 @@
 #include <unordered_map>
 
 #include "fq_common.cuh"
+#include "smem_opt_in.h"
 
 using namespace fq;
 
@@ -17,7 +18,7 @@ constexpr int kMaxDevices = 64;
 struct DeviceFacts { int sms = 0, major = -1; };
 std::mutex g_facts_mutex;
 DeviceFacts g_facts[kMaxDevices];
-std::unordered_map<const void*, size_t> g_smem_opt_in[kMaxDevices];
+SmemOptIn g_smem_opt_in[kMaxDevices];
 std::unordered_map<const void*, std::unordered_map<int, int>> g_resident[kMaxDevices];
 
 DeviceFacts device_facts() {
@@ -47,18 +48,9 @@ int device_cc_major() { return device_facts().major; }
 cudaError_t ensure_dynamic_smem(const void* kernel, size_t bytes) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return cudaGetLastError();
-    const bool cached = dev >= 0 && dev < kMaxDevices;
-    if (cached) {
-        std::lock_guard<std::mutex> lock(g_facts_mutex);
-        auto it = g_smem_opt_in[dev].find(kernel);
-        if (it != g_smem_opt_in[dev].end() && it->second >= bytes) return cudaSuccess;
-    }
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess && cached) {
-        std::lock_guard<std::mutex> lock(g_facts_mutex);
-        g_smem_opt_in[dev][kernel] = bytes;
-    }
-    return e;
+    auto set = [kernel](size_t n) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)n); };
+    if (dev < 0 || dev >= kMaxDevices) return set(bytes);
+    return g_smem_opt_in[dev].raise(kernel, bytes, set);
 }
 
 int max_resident_blocks(const void* kernel, int threads) {

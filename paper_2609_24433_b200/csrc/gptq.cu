@@ -535,18 +535,14 @@ cudaError_t launch_transform_rows(const void* x, fq_dtype xt, int64_t rows, int6
                                   float cnorm, int block, float* z, cudaStream_t stream) {
     if (rows == 0) return cudaSuccess;
     const size_t smem = sizeof(float) * (size_t)K;
-    if (xt == FQ_F32) {
-        cudaError_t e = cudaFuncSetAttribute(transform_rows_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto run = [&](auto kern, auto* p) -> cudaError_t {
+        const cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), smem);
         if (e != cudaSuccess) return e;
-        transform_rows_kernel<float><<<(unsigned)rows, 256, smem, stream>>>(static_cast<const float*>(x), (int)K, ldx, mult,
-                                                                           cnorm, block, z);
-    } else {
-        cudaError_t e = cudaFuncSetAttribute(transform_rows_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        transform_rows_kernel<__nv_bfloat16><<<(unsigned)rows, 256, smem, stream>>>(static_cast<const __nv_bfloat16*>(x),
-                                                                                   (int)K, ldx, mult, cnorm, block, z);
-    }
-    return cudaGetLastError();
+        kern<<<(unsigned)rows, 256, smem, stream>>>(p, (int)K, ldx, mult, cnorm, block, z);
+        return cudaGetLastError();
+    };
+    return xt == FQ_F32 ? run(transform_rows_kernel<float>, static_cast<const float*>(x))
+                        : run(transform_rows_kernel<__nv_bfloat16>, static_cast<const __nv_bfloat16*>(x));
 }
 
 // Whether factor and inverse of this width run in the cooperative kernel: at most 24 rows per CTA, one CTA per SM
