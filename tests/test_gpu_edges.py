@@ -1,5 +1,9 @@
 """GPU parity at the sizes where a kernel or a dispatch rule can go wrong: edges of tiles, remainders, the smallest
 and the largest of each variant's range.  Same oracle and same bounds as test_gpu_parity.py."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -298,3 +302,42 @@ def test_calls_that_pass_two_buffers_to_and_fro(M, K, bits, call):
         a.fill_(7.0), b.fill_(7.0)
         run()
         assert torch.equal(a, want[0]) and torch.equal(b, want[1])
+
+
+FIRST_CALLS = """
+import ctypes, sys, threading
+import torch
+from paper_2609_24433_b200 import fq
+torch.cuda.init()
+shapes = [(8, 256, 64), (24, 512, 128), (50, 1024, 64), (64, 2048, 64), (200, 1024, 128), (700, 2048, 128), (16, 4096, 256), (40, 1536, 128)]
+Ws = [torch.randn(N, K, device="cuda") for _, K, N in shapes]
+xs = [torch.randn(M, K, device="cuda") for M, K, _ in shapes]
+torch.cuda.synchronize()
+gate, errors, ys = threading.Barrier(len(shapes)), [], [None] * len(shapes)
+
+def work(i):
+    try:
+        gate.wait()
+        with torch.cuda.stream(torch.cuda.Stream()):
+            h = fq.fold_weights(Ws[i], None, None, 32, 4)          # the first calls of the process: folds and projections
+            for _ in range(20):
+                ys[i] = fq.linear(xs[i], h)
+            torch.cuda.current_stream().synchronize()
+    except Exception as e:
+        errors.append((i, repr(e)))
+
+threads = [threading.Thread(target=work, args=(i,)) for i in range(len(shapes))]
+[t.start() for t in threads]
+[t.join() for t in threads]
+assert not errors, errors
+for W, x, y in zip(Ws, xs, ys):
+    assert torch.equal(y, fq.linear(x, fq.fold_weights(W, None, None, 32, 4)))
+assert fq.device_status()[0] == fq.OK
+"""
+
+
+def test_first_calls_of_a_process_from_several_threads():
+    """What is looked up once (driver entry point, kernel attributes, device facts) is looked up by eight threads at a time."""
+    r = subprocess.run([sys.executable, "-c", FIRST_CALLS], cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
+                       capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
