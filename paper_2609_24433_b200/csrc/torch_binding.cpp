@@ -4,7 +4,10 @@
 // a 64-token projection take 7 us, and a call marshalled through ctypes and torch.empty took 19.4 us of host time
 // (at most 8.5 us here, its two launches included; M = 64, K = N = 1024).
 //
-// Every function returns its result, or the fq_status (an int) of a call that was refused.
+// Every function returns its result, or the fq_status (an int) of a call that was refused.  All that is read from Python
+// objects is read first; then the interpreter lock is given up for the allocations and the call into the library, as ctypes
+// and torch do: a launch waits while its stream's queue is full, and other Python threads -- a function that the stream itself
+// calls on the host among them, for which that queue may be waiting -- have to run meanwhile.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
@@ -20,6 +23,18 @@
 namespace {
 
 struct Refused {};          // a Python exception is set
+
+// The interpreter lock given up for a scope, exceptions included.
+class Unlocked {
+public:
+    Unlocked() : state_(PyEval_SaveThread()) {}
+    ~Unlocked() { PyEval_RestoreThread(state_); }
+    Unlocked(const Unlocked&) = delete;
+    Unlocked& operator=(const Unlocked&) = delete;
+
+private:
+    PyThreadState* state_;
+};
 
 const at::Tensor& tensor(PyObject* o) {
     if (!THPVariable_Check(o)) {
@@ -69,21 +84,30 @@ at::Tensor fresh(at::IntArrayRef size, at::ScalarType t, const at::Tensor& like)
     return at::empty(size, at::TensorOptions().dtype(t).device(like.device()));
 }
 
-// y as given (its own dtype decides) or a new [M, N] of `dtype` on x's device
-at::Tensor output(PyObject* y, PyObject* dtype, int64_t M, int64_t N, const at::Tensor& x, fq_dtype* yt) {
-    if (!none(y)) {
-        const at::Tensor& t = tensor(y);
-        *yt = dtype_of(t.scalar_type());
-        return t;
+// An output: the caller's tensor (its own dtype decides) or, made by make(), a new one of `dtype` on x's device.
+struct Output {
+    at::Tensor t;
+    at::ScalarType type;
+    fq_dtype dt;
+    Output(PyObject* given, PyObject* dtype) {
+        if (!none(given)) {
+            t = tensor(given);
+            type = t.scalar_type();
+        } else if (THPDtype_Check(dtype)) {
+            type = reinterpret_cast<THPDtype*>(dtype)->scalar_type;
+        } else {
+            PyErr_SetString(PyExc_TypeError, "out_dtype has to be a torch.dtype");
+            throw Refused();
+        }
+        dt = dtype_of(type);
     }
-    if (!THPDtype_Check(dtype)) {
-        PyErr_SetString(PyExc_TypeError, "out_dtype has to be a torch.dtype");
-        throw Refused();
+    Output(PyObject* given, at::ScalarType otherwise) : type(otherwise), dt(FQ_F32) {
+        if (!none(given)) t = tensor(given);
     }
-    const at::ScalarType t = reinterpret_cast<THPDtype*>(dtype)->scalar_type;
-    *yt = dtype_of(t);
-    return fresh({M, N}, t, x);
-}
+    void make(at::IntArrayRef size, const at::Tensor& like) {
+        if (!t.defined()) t = fresh(size, type, like);
+    }
+};
 
 // The caller's workspace, or one from torch's allocator for the length of the call: it is handed back when the kernels
 // are enqueued, and the allocator gives it to later work of this stream only -- what a torch.empty that goes out of
@@ -92,17 +116,23 @@ struct Workspace {
     void* p = nullptr;
     size_t bytes = 0;
     at::Tensor own;
-    Workspace(PyObject* given, size_t need, const at::Tensor& like) {
-        if (!none(given)) {
-            const at::Tensor& t = tensor(given);
-            p = t.data_ptr();
-            bytes = static_cast<size_t>(t.numel());
-        } else {
-            own = fresh({static_cast<int64_t>(need)}, at::kByte, like);
-            p = own.data_ptr();
-            bytes = need;
-        }
+    explicit Workspace(PyObject* given) {
+        if (none(given)) return;
+        const at::Tensor& t = tensor(given);
+        p = t.data_ptr();
+        bytes = static_cast<size_t>(t.numel());
+        given_ = true;
     }
+    template <typename Need>
+    void make(Need need, const at::Tensor& like) {
+        if (given_) return;
+        bytes = need();
+        own = fresh({static_cast<int64_t>(bytes)}, at::kByte, like);
+        p = own.data_ptr();
+    }
+
+private:
+    bool given_ = false;
 };
 
 PyObject* pair(at::Tensor&& a, at::Tensor&& b) {
@@ -136,11 +166,18 @@ PyObject* one_call(PyObject* const* a, Py_ssize_t n, F run) {
         const long long which = integer(a[5]);
         const float clip = real(a[6]);
         const fq_dtype xt = dtype_of(x.scalar_type());
-        fq_dtype yt;
-        at::Tensor y = output(a[8], a[7], M, N, x, &yt);
-        const Workspace ws(a[9], none(a[9]) ? fq_workspace_bytes(M, K, N, handle_bits) : 0, x);
-        const fq_status s = run(which, x.data_ptr(), xt, M, x.stride(0), W, clip, y.data_ptr(), yt, y.stride(0), ws.p, ws.bytes);
-        return s == FQ_OK ? THPVariable_Wrap(std::move(y)) : status(s);
+        const void* xp = x.data_ptr();
+        const int64_t ldx = x.stride(0);
+        Output y(a[8], a[7]);
+        Workspace ws(a[9]);
+        fq_status s;
+        {
+            const Unlocked nogil;
+            y.make({M, N}, x);
+            ws.make([&] { return fq_workspace_bytes(M, K, N, handle_bits); }, x);
+            s = run(which, xp, xt, M, ldx, W, clip, y.t.data_ptr(), y.dt, y.t.stride(0), ws.p, ws.bytes);
+        }
+        return s == FQ_OK ? THPVariable_Wrap(std::move(y.t)) : status(s);
     });
 }
 
@@ -170,12 +207,18 @@ PyObject* gemm(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const fq_weights* W = static_cast<const fq_weights*>(address(a[2]));
         const int64_t K = integer(a[3]), N = integer(a[4]), M = codes.size(0);
         const int handle_bits = static_cast<int>(integer(a[5])), bits = static_cast<int>(integer(a[6]));
-        fq_dtype yt;
-        at::Tensor y = output(a[8], a[7], M, N, codes, &yt);
-        const Workspace ws(a[9], none(a[9]) ? fq_workspace_bytes(M, K, N, handle_bits) : 0, codes);
-        const fq_status s = (bits == 4 ? fq_gemm_w4a4 : fq_gemm_w8a8)(codes.data_ptr(), static_cast<const float*>(delta.data_ptr()), M,
-                                                                      W, y.data_ptr(), yt, y.stride(0), ws.p, ws.bytes, stream());
-        return s == FQ_OK ? THPVariable_Wrap(std::move(y)) : status(s);
+        const void* cp = codes.data_ptr();
+        const float* dp = static_cast<const float*>(delta.data_ptr());
+        Output y(a[8], a[7]);
+        Workspace ws(a[9]);
+        fq_status s;
+        {
+            const Unlocked nogil;
+            y.make({M, N}, codes);
+            ws.make([&] { return fq_workspace_bytes(M, K, N, handle_bits); }, codes);
+            s = (bits == 4 ? fq_gemm_w4a4 : fq_gemm_w8a8)(cp, dp, M, W, y.t.data_ptr(), y.dt, y.t.stride(0), ws.p, ws.bytes, stream());
+        }
+        return s == FQ_OK ? THPVariable_Wrap(std::move(y.t)) : status(s);
     });
 }
 
@@ -189,11 +232,19 @@ PyObject* quantize_act(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const int block = static_cast<int>(integer(a[2])), bits = static_cast<int>(integer(a[3]));
         const float clip = real(a[4]);
         const fq_dtype xt = dtype_of(x.scalar_type());
-        at::Tensor codes = none(a[5]) ? fresh({M, K * bits / 8}, at::kByte, x) : tensor(a[5]);
-        at::Tensor delta = none(a[6]) ? fresh({M}, at::kFloat, x) : tensor(a[6]);
-        const fq_status s = (integer(a[7]) ? fq_quantize_act_after : fq_quantize_act)(
-            x.data_ptr(), xt, M, K, x.stride(0), g, block, bits, clip, codes.data_ptr(), static_cast<float*>(delta.data_ptr()), stream());
-        return s == FQ_OK ? pair(std::move(codes), std::move(delta)) : status(s);
+        const bool after = integer(a[7]) != 0;
+        const void* xp = x.data_ptr();
+        const int64_t ldx = x.stride(0);
+        Output codes(a[5], at::kByte), delta(a[6], at::kFloat);
+        fq_status s;
+        {
+            const Unlocked nogil;
+            codes.make({M, K * bits / 8}, x);
+            delta.make({M}, x);
+            s = (after ? fq_quantize_act_after : fq_quantize_act)(xp, xt, M, K, ldx, g, block, bits, clip, codes.t.data_ptr(),
+                                                                  static_cast<float*>(delta.t.data_ptr()), stream());
+        }
+        return s == FQ_OK ? pair(std::move(codes.t), std::move(delta.t)) : status(s);
     });
 }
 
@@ -212,13 +263,23 @@ PyObject* quantize_act_composite(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const int bits = static_cast<int>(integer(a[4]));
         const float clip = real(a[5]);
         const fq_dtype xt = dtype_of(x.scalar_type());
-        at::Tensor codes = none(a[6]) ? fresh({M, K * bits / 8}, at::kByte, x) : tensor(a[6]);
-        at::Tensor delta = none(a[7]) ? fresh({M}, at::kFloat, x) : tensor(a[7]);
-        const Workspace ws(a[8], static_cast<size_t>(M * K > 4 ? 4 * M * K : 16), x);
-        const fq_status s = fq_quantize_act_composite(x.data_ptr(), xt, M, K, x.stride(0), g, perm.data_ptr<int32_t>(),
-                                                      blocks.data_ptr<float>(), static_cast<int>(blocks.size(1)), bits, clip,
-                                                      codes.data_ptr(), static_cast<float*>(delta.data_ptr()), ws.p, ws.bytes, stream());
-        return s == FQ_OK ? pair(std::move(codes), std::move(delta)) : status(s);
+        const void* xp = x.data_ptr();
+        const int64_t ldx = x.stride(0);
+        const int32_t* pp = perm.data_ptr<int32_t>();
+        const float* bp = blocks.data_ptr<float>();
+        const int block = static_cast<int>(blocks.size(1));
+        Output codes(a[6], at::kByte), delta(a[7], at::kFloat);
+        Workspace ws(a[8]);
+        fq_status s;
+        {
+            const Unlocked nogil;
+            codes.make({M, K * bits / 8}, x);
+            delta.make({M}, x);
+            ws.make([&] { return static_cast<size_t>(M * K > 4 ? 4 * M * K : 16); }, x);
+            s = fq_quantize_act_composite(xp, xt, M, K, ldx, g, pp, bp, block, bits, clip, codes.t.data_ptr(),
+                                          static_cast<float*>(delta.t.data_ptr()), ws.p, ws.bytes, stream());
+        }
+        return s == FQ_OK ? pair(std::move(codes.t), std::move(delta.t)) : status(s);
     });
 }
 
@@ -230,10 +291,16 @@ PyObject* linear_w4a16(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const fq_weights* W = static_cast<const fq_weights*>(address(a[1]));
         const int64_t N = integer(a[2]), M = x.size(0);
         const fq_dtype xt = dtype_of(x.scalar_type());
-        fq_dtype yt;
-        at::Tensor y = output(a[4], a[3], M, N, x, &yt);
-        const fq_status s = fq_linear_w4a16(x.data_ptr(), xt, M, x.stride(0), W, y.data_ptr(), yt, y.stride(0), stream());
-        return s == FQ_OK ? THPVariable_Wrap(std::move(y)) : status(s);
+        const void* xp = x.data_ptr();
+        const int64_t ldx = x.stride(0);
+        Output y(a[4], a[3]);
+        fq_status s;
+        {
+            const Unlocked nogil;
+            y.make({M, N}, x);
+            s = fq_linear_w4a16(xp, xt, M, ldx, W, y.t.data_ptr(), y.dt, y.t.stride(0), stream());
+        }
+        return s == FQ_OK ? THPVariable_Wrap(std::move(y.t)) : status(s);
     });
 }
 

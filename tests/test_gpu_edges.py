@@ -3,6 +3,8 @@ and the largest of each variant's range.  Same oracle and same bounds as test_gp
 import os
 import subprocess
 import sys
+import threading
+import time
 
 import numpy as np
 import pytest
@@ -341,3 +343,39 @@ def test_first_calls_of_a_process_from_several_threads():
     r = subprocess.run([sys.executable, "-c", FIRST_CALLS], cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
                        capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr[-2000:]
+
+
+@pytest.mark.parametrize("call", ["linear", "gemm", "quantize_act", "linear_w4a16", "linear_gated", "quantize_act_composite"])
+def test_other_python_threads_run_while_a_launch_waits(call):
+    """Launches behind a busy stream wait once its queue is full; a second thread keeps counting all the while."""
+    h, x = fq.fold_weights(torch.randn(64, 256, device="cuda"), None, None, 1, 4), torch.randn(8, 256, device="cuda")
+    gate_up, ws = torch.randn(8, 512, device="cuda"), torch.empty(1 << 16, dtype=torch.uint8, device="cuda")
+    perm, blocks = (to_dev(a) for a in synth.composite_rotation(256, 32, seed=1))
+    codes, delta = fq.quantize_act(x, None, 1, 4)
+    y = torch.empty(8, 64, device="cuda")
+    run = {"linear": lambda: fq.linear(x, h, y=y, workspace=ws), "gemm": lambda: fq.gemm_w4a4(codes, delta, h, y=y, workspace=ws),
+           "quantize_act": lambda: fq.quantize_act(x, None, 1, 4, codes=codes, delta=delta),
+           "linear_w4a16": lambda: fq.linear_w4a16(x, h, y=y), "linear_gated": lambda: fq.linear_gated(gate_up, fq.GATE_SILU, h, y=y, workspace=ws),
+           "quantize_act_composite": lambda: fq.quantize_act_composite(x, None, perm, blocks, 4, codes=codes, delta=delta, workspace=ws)}[call]
+    run()
+    torch.cuda.synchronize()
+    done, ticks = threading.Event(), []
+
+    def count():
+        while not done.wait(0.002):
+            ticks.append(time.perf_counter())
+
+    torch.cuda._sleep(int(0.8 * 1.9e9))                   # the stream is busy for 0.8 s or a little more
+    thread = threading.Thread(target=count)
+    thread.start()
+    longest, start = 0.0, time.perf_counter()
+    for _ in range(4000):
+        t = time.perf_counter()
+        run()
+        longest = max(longest, time.perf_counter() - t)
+    done.set()
+    thread.join()
+    gaps = np.diff([start] + ticks)
+    torch.cuda.synchronize()
+    assert longest > 0.2, f"no launch had to wait ({longest:.3f} s): nothing was tested"
+    assert gaps.max() < 0.5 * longest, f"a launch waited {longest:.3f} s, the other thread stood still for {gaps.max():.3f} s"
