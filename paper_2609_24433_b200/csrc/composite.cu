@@ -123,8 +123,9 @@ struct CompositeParams {
     uint8_t* codes;
     float* delta;
 };
-constexpr int kCol = 16;                               // columns per step
+constexpr int kCol = kCompositeColumns;                // columns per step
 constexpr int kWarps = kThreads / 32;
+static_assert(kWarps == kCompositeWarps, "the plan sizes shared memory for these warps");
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
@@ -324,54 +325,34 @@ composite_quantize_kernel(const CompositeParams p) {
     }
 }
 
-// 16 tokens a cluster where their rows fit, else 8; *p is complete but for the sizes.
+// *p is complete but for the sizes.
 template <typename XT, int BETA, int TOK>
-cudaError_t launch_quantize(CompositeParams p, cudaStream_t stream) {
-    constexpr int OUT = BETA < 64 ? BETA : 64;
-    p.items = p.K / OUT;
-    const int64_t tiles = (p.rows + TOK - 1) / TOK;
-    size_t smem = 0;
-    auto fits = [&](int shift) {
-        const int width = ((p.items + (1 << shift) - 1) >> shift) * OUT;
-        p.u_pitch = width + 4;
-        p.span = width + (BETA > OUT ? 2 * BETA : 0);
-        size_t at = align_up((size_t)p.K * sizeof(XT) * TOK, 16);
-        p.off_u = (uint32_t)at; at += align_up((size_t)p.u_pitch * 4 * TOK, 16);
-        p.off_b = (uint32_t)at; at += (size_t)kWarps * 2 * OUT * kCol * 4;
-        p.off_p = (uint32_t)at; at += (size_t)kWarps * kCol * (TOK + 4) * 4;
-        p.off_s = (uint32_t)at; at += (size_t)p.span * 8;
-        smem = at;
-        return smem <= 224 * 1024;
-    };
-    // As many CTAs per tile as leave half the warps an item each and make one wave: every CTA begins by staging the tokens'
-    // rows, so a second wave costs more than longer CTAs (block 64: M = 816, K = 2048 19.7 us with clusters of four in two
-    // waves, 15.4 with pairs in one; M = 1184, K = 1024 21.0 and 9.6).  Two CTAs share an SM where shared memory allows it
-    // (816 x 1024, block 32: 7.8 us so, 10.4 with pairs); of 148 SMs clusters of four reach 144, of eight 112.  More CTAs
-    // where the rotated channels would not fit otherwise.
-    auto one_wave = [&](int shift) {
-        const int64_t sms = device_sm_count(), reach = shift == 3 ? sms * 28 / 37 : (shift == 2 ? sms * 36 / 37 : sms);
-        return fits(shift) && (tiles << shift) <= reach * (2 * (smem + 3072) <= 228 * 1024 ? 2 : 1);
-    };
-    int shift = 3;
-    while (shift > 0 && (p.items >> shift < 4 || !one_wave(shift)) && fits(shift - 1)) --shift;
-    if (!fits(shift) || p.items >> shift < 1 || (tiles << shift) > 0x7fffffffll) {
-        if constexpr (TOK == 16 && BETA >= 32) return launch_quantize<XT, BETA, 8>(p, stream);
-        return cudaErrorNotSupported;
-    }
-    p.ctas_shift = shift;
+cudaError_t launch_quantize_tok(const CompositeParams& p, const CompositePlan& f, cudaStream_t stream) {
     auto kern = composite_quantize_kernel<XT, BETA, TOK>;
-    const cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), smem);
+    const cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), f.smem);
     if (e != cudaSuccess) return e;
-    return launch_pdl(kern, (unsigned)(tiles << shift), (unsigned)kThreads, smem, stream, 1u << shift, p);
+    const cudaError_t launched = launch_pdl(kern, (unsigned)f.grid, (unsigned)kThreads, f.smem, stream, 1u << f.ctas_shift, p);
+    return f.ctas_shift > 0 && cluster_refused(launched) ? cudaErrorNotSupported : launched;
+}
+template <typename XT, int BETA>
+cudaError_t launch_quantize(CompositeParams p, cudaStream_t stream) {
+    const CompositePlan f = plan_composite(p.rows, p.K, (int)sizeof(XT), BETA, device_sm_count(), cluster_capacity);
+    if (f.tok == 0) return cudaErrorNotSupported;
+    p.items = f.items; p.ctas_shift = f.ctas_shift; p.u_pitch = f.u_pitch; p.span = f.span;
+    p.off_u = f.off_u; p.off_b = f.off_b; p.off_p = f.off_p; p.off_s = f.off_s;
+    if constexpr (BETA >= 32) {
+        if (f.tok == 8) return launch_quantize_tok<XT, BETA, 8>(p, f, stream);
+    }
+    return launch_quantize_tok<XT, BETA, 16>(p, f, stream);
 }
 template <typename XT>
 cudaError_t launch_quantize_beta(int beta, const CompositeParams& p, cudaStream_t stream) {
     switch (beta) {
-        case 16: return launch_quantize<XT, 16, 16>(p, stream);
-        case 32: return launch_quantize<XT, 32, 16>(p, stream);
-        case 64: return launch_quantize<XT, 64, 16>(p, stream);
-        case 128: return launch_quantize<XT, 128, 16>(p, stream);
-        case 256: return launch_quantize<XT, 256, 16>(p, stream);
+        case 16: return launch_quantize<XT, 16>(p, stream);
+        case 32: return launch_quantize<XT, 32>(p, stream);
+        case 64: return launch_quantize<XT, 64>(p, stream);
+        case 128: return launch_quantize<XT, 128>(p, stream);
+        case 256: return launch_quantize<XT, 256>(p, stream);
         default: return cudaErrorNotSupported;
     }
 }

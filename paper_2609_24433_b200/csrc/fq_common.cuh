@@ -7,6 +7,7 @@
 #include <stdint.h>
 
 #include "fq.h"
+#include "plan.h"
 
 namespace fq {
 
@@ -30,14 +31,21 @@ struct Weights {
     bool tmap_stream_valid = false;
 };
 
-inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
-
 // Facts about the current device and per-kernel launch set-up, looked up once and remembered (an eager call
 // otherwise pays several runtime queries per launch).
 int device_sm_count();                                              // multiprocessors of the current device
 int device_cc_major();                                              // compute-capability major, -1 on error
 cudaError_t ensure_dynamic_smem(const void* kernel, size_t bytes);  // opt a kernel in to `bytes` of dynamic shared memory
 int max_resident_blocks(const void* kernel, int threads);           // thread blocks of a kernel one SM holds (no dynamic smem)
+// Clusters of 2, 4 or 8 CTAs, one CTA per SM, that the device holds at a time (a whole B200: 74, 36, 14 -- its graphics
+// clusters do not divide by eight; 0 where one cannot be placed at all, on a part of a device).
+int cluster_capacity(int ctas);
+// The device would not place a cluster launch after all (a context that owns part of it): the caller takes the route without.
+inline bool cluster_refused(cudaError_t e) {
+    if (e != cudaErrorInvalidClusterSize && e != cudaErrorLaunchOutOfResources && e != cudaErrorInvalidConfiguration) return false;
+    (void)cudaGetLastError();
+    return true;
+}
 
 // Launch with programmatic stream serialization and, optionally, a thread-block cluster along x.  The kernel may start while
 // kernels ahead of it in the stream are still running, so ahead of griddep_wait() it reads only what was complete before

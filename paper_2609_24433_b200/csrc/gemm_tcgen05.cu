@@ -101,7 +101,6 @@ cudaError_t read_and_clear_watchdog(uint32_t* word) {
 
 namespace {
 
-constexpr int kTileN = 128;          // output channels per tile (MMA M)
 constexpr int kBlockK = 128;         // int8 elements (= bytes) of K per pipeline stage
 constexpr int kAccStages = 2;
 constexpr int kEpiWarps = 8;
@@ -118,7 +117,6 @@ constexpr int kMaxStagesP = 16;
 constexpr int kMaxSplit = 16;          // K slices per tile, at most
 constexpr int kMaxSplitTiles = 1024;   // tiles of a launch that splits K (one counter each, ahead of the partial sums)
 enum : int { kUnsplit = 0, kSplitScratch = 1, kSplitCluster = 2 };
-constexpr int kMaxCluster = 8;         // CTAs of a cluster that share a tile along K, at most
 constexpr size_t kCounterBytes = kMaxSplitTiles * sizeof(uint32_t);
 
 struct Params {
@@ -1117,11 +1115,13 @@ namespace {
 
 template <int BITS, int CTAS, int SPLIT, int ATOMS = 1>
 fq_status launch_variant(const CUtensorMap& map_a, const CUtensorMap& map_w, const CUtensorMap& map_y, const Params& p,
-                         int grid, size_t smem, int cluster, cudaStream_t stream) {
+                         int grid, size_t smem, int cluster, cudaStream_t stream, bool* refused) {
     auto kern = gemm_tcgen05_kernel<BITS, CTAS, SPLIT, ATOMS>;
     if (ensure_dynamic_smem(reinterpret_cast<const void*>(kern), smem) != cudaSuccess) return FQ_ERR_CUDA;
-    return launch_pdl(kern, (unsigned)grid, (unsigned)(BITS == 4 ? kThreadsW4 : kThreadsW8), smem, stream, (unsigned)cluster,
-                      map_a, map_w, map_y, p) == cudaSuccess ? FQ_OK : FQ_ERR_CUDA;
+    const cudaError_t e = launch_pdl(kern, (unsigned)grid, (unsigned)(BITS == 4 ? kThreadsW4 : kThreadsW8), smem, stream,
+                                     (unsigned)cluster, map_a, map_w, map_y, p);
+    *refused = cluster > 1 && cluster_refused(e);
+    return e == cudaSuccess ? FQ_OK : FQ_ERR_CUDA;
 }
 
 }  // namespace
@@ -1150,10 +1150,6 @@ size_t stage_bytes(int bits, int ctas, int bt, int atoms) {
     return ((size_t)(bt / ctas) * kBlockK + (size_t)kTileN * kBlockK * bits / 8) * atoms;
 }
 size_t cluster_sums_bytes(int bt, int split) { return (size_t)(split - 1) * ((bt / 16 + split - 1) / split) * 16 * kTileN * sizeof(int32_t); }
-
-// Clusters of 2, 4 or 8 CTAs, one per SM, that the device holds at a time (a B200: 74, 36, 14 -- its graphics clusters do not
-// divide by eight).
-int cluster_capacity(int ctas);
 
 // Token tile, CTA grouping and K split.  Upper bound of the tile from TMEM: two accumulator stages,
 // plus the unpacked-weight ring for 4-bit weights (2*bt + 3*32 <= 512 columns).  M is split evenly
@@ -1184,18 +1180,19 @@ int cluster_capacity(int ctas);
 //   816 x 16384 x 2048: the site 5 us faster than 96-token tiles.
 //   Through scratch, where the device cannot hold the clusters (CTA pairs on 8-bit weights, too): 12500 + 40*bt + 1500 per
 //   extra slice.
-Plan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t scratch_avail, bool clusters) {
+Plan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t scratch_avail, bool clusters, int (*capacity_of)(int)) {
     const int bt_max = bits == 4 ? 208 : 256;
     const int64_t kb = (K + kBlockK - 1) / kBlockK;
     Plan best;
     double best_cost = 0.0;
     int capacity[kMaxCluster + 1] = {};                  // by CTAs per cluster, asked for once per plan; 0: not yet, else + 1
     auto held = [&](int ctas) {
-        if (capacity[ctas] == 0) capacity[ctas] = cluster_capacity(ctas) + 1;
+        if (capacity[ctas] == 0) capacity[ctas] = capacity_of(ctas) + 1;
         return capacity[ctas] - 1;
     };
     const bool pairs = N > kTileN && (bits == 8 || (K >= 2048 && (double)M * (double)N * (double)K >= 1.6e11));
     for (int c = 1; c <= (pairs ? 2 : 1); ++c) {
+        if (c == 2 && clusters && held(2) < 1) break;
         const int64_t n_units = (N + kTileN * c - 1) / (kTileN * c);
         for (int mt = (int)((M + bt_max - 1) / bt_max); mt <= (int)((M + 63) / 64); ++mt) {
             const int b = (int)(((M + mt - 1) / mt + 15) / 16 * 16);
@@ -1234,6 +1231,8 @@ Plan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t scratc
     return best;
 }
 
+}  // namespace
+
 int cluster_capacity(int ctas) {
     static std::mutex mutex;
     static int known[64][3];                         // 0: not asked yet, else capacity + 1
@@ -1267,8 +1266,6 @@ int cluster_capacity(int ctas) {
     return known[dev][i] - 1;
 }
 
-}  // namespace
-
 // A launch that splits K counts the finished slices of every tile in counters at the head of the scratch.
 // They are cleared here, by a memset node enqueued AHEAD of the call's first kernel (between the prologue
 // and the GEMM it would break the programmatic overlap of the two): each call starts from zero whatever an
@@ -1276,7 +1273,7 @@ int cluster_capacity(int ctas) {
 // changes at run time.
 fq_status gemm_prepare(int64_t M, const Weights& W, void* scratch, size_t scratch_bytes, cudaStream_t stream) {
     if (M <= 0 || W.N == 0 || scratch == nullptr || gemm_stream_applies(M, W)) return FQ_OK;
-    const Plan plan = plan_gemm(M, W.N, W.K, W.bits, device_sm_count(), scratch_bytes, true);
+    const Plan plan = plan_gemm(M, W.N, W.K, W.bits, device_sm_count(), scratch_bytes, true, cluster_capacity);
     if (plan.split <= 1 || plan.cluster) return FQ_OK;
     return cudaMemsetAsync(scratch, 0, kCounterBytes, stream) == cudaSuccess ? FQ_OK : FQ_ERR_CUDA;
 }
@@ -1292,18 +1289,20 @@ fq_status launch_gemm(const int8_t* a8, int64_t M, const Weights& W, int acc_shi
 size_t gemm_scratch_bytes(int64_t M, int64_t N, int64_t K, int bits) {
     if (M <= 0 || N <= 0 || K <= 0) return 0;
     // (asked for whether or not this device holds the clusters that would do without: a caller sizes its workspace once)
-    return plan_gemm(M, N, K, bits, device_sm_count(), (size_t)-1, false).scratch;
+    return plan_gemm(M, N, K, bits, device_sm_count(), (size_t)-1, false, cluster_capacity).scratch;
 }
 
-fq_status launch_gemm_tcgen05(const int8_t* a8, int64_t M, const Weights& W, int acc_shift, const GemmOut& out,
-                              void* scratch, size_t scratch_bytes, cudaStream_t stream) {
-    if (M == 0 || W.N == 0) return FQ_OK;
-    if (!W.tmap_valid) return FQ_ERR_CUDA;
+namespace {
 
+int no_clusters(int) { return 0; }
+
+// *refused: the device did not take the launch's clusters, nothing was enqueued.
+fq_status launch_planned(const int8_t* a8, int64_t M, const Weights& W, int acc_shift, const GemmOut& out, void* scratch,
+                         size_t scratch_bytes, int (*held)(int), cudaStream_t stream, bool* refused) {
     Params p{};
     p.M = M; p.N = W.N; p.K = W.K;
     const int sms = device_sm_count();
-    const Plan plan = plan_gemm(M, W.N, W.K, W.bits, sms, scratch ? scratch_bytes : 0, true);
+    const Plan plan = plan_gemm(M, W.N, W.K, W.bits, sms, scratch ? scratch_bytes : 0, true, held);
     const int bt = plan.bt, ctas = plan.ctas, split = plan.split;
     p.split = split;
     p.counters = static_cast<uint32_t*>(scratch);            // cleared by gemm_prepare()
@@ -1395,17 +1394,29 @@ fq_status launch_gemm_tcgen05(const int8_t* a8, int64_t M, const Weights& W, int
     const int cluster = plan.cluster ? split * ctas : ctas;
     auto go = [&](auto bits, auto pair, auto atoms_c) -> fq_status {
         constexpr int B = decltype(bits)::value, C = decltype(pair)::value, A = decltype(atoms_c)::value;
-        if (split == 1) return launch_variant<B, C, kUnsplit, A>(map_a, W.tmap, map_y, p, grid, smem, cluster, stream);
-        if (plan.cluster) return launch_variant<B, C, kSplitCluster, A>(map_a, W.tmap, map_y, p, grid, smem, cluster, stream);
-        return launch_variant<B, C, kSplitScratch, A>(map_a, W.tmap, map_y, p, grid, smem, cluster, stream);
+        if (split == 1) return launch_variant<B, C, kUnsplit, A>(map_a, W.tmap, map_y, p, grid, smem, cluster, stream, refused);
+        if (plan.cluster) return launch_variant<B, C, kSplitCluster, A>(map_a, W.tmap, map_y, p, grid, smem, cluster, stream, refused);
+        return launch_variant<B, C, kSplitScratch, A>(map_a, W.tmap, map_y, p, grid, smem, cluster, stream, refused);
     };
     using I1 = std::integral_constant<int, 1>;
     using I2 = std::integral_constant<int, 2>;
     using I4 = std::integral_constant<int, 4>;
     using I8 = std::integral_constant<int, 8>;
-    if (W.bits == 4 && ctas == 2) return launch_variant<4, 2, kUnsplit>(map_a, W.tmap, map_y, p, grid, smem, cluster, stream);
+    if (W.bits == 4 && ctas == 2) return launch_variant<4, 2, kUnsplit>(map_a, W.tmap, map_y, p, grid, smem, cluster, stream, refused);
     if (W.bits == 4) return atoms == 4 ? go(I4(), I1(), I4()) : (atoms == 2 ? go(I4(), I1(), I2()) : go(I4(), I1(), I1()));
     return ctas == 2 ? go(I8(), I2(), I1()) : go(I8(), I1(), I1());
+}
+
+}  // namespace
+
+fq_status launch_gemm_tcgen05(const int8_t* a8, int64_t M, const Weights& W, int acc_shift, const GemmOut& out,
+                              void* scratch, size_t scratch_bytes, cudaStream_t stream) {
+    if (M == 0 || W.N == 0) return FQ_OK;
+    if (!W.tmap_valid) return FQ_ERR_CUDA;
+    bool refused = false;
+    const fq_status st = launch_planned(a8, M, W, acc_shift, out, scratch, scratch_bytes, cluster_capacity, stream, &refused);
+    // (without scratch: gemm_prepare() cleared the counters of the plan that was refused, if any)
+    return refused ? launch_planned(a8, M, W, acc_shift, out, nullptr, 0, no_clusters, stream, &refused) : st;
 }
 
 }  // namespace fq

@@ -28,10 +28,9 @@ namespace fq {
 namespace {
 
 constexpr int kThreads = 512;
-constexpr int kMaxTokens = 64;
-constexpr int kMaxCluster = 8;
-constexpr int E = 16, H = E / 2;       // channels per thread and round: v[p] = (channel p, channel p + H)
-constexpr int kTile = 128;             // output channels per MMA
+constexpr int kMaxTokens = kFusedMaxTokens;
+constexpr int E = kFusedRun, H = E / 2;       // channels per thread and round: v[p] = (channel p, channel p + H)
+constexpr int kTile = kTileN;          // output channels per MMA
 
 enum : uint32_t { kWdFusedWeights = 0x2000u, kWdFusedMma = 0x4000u };
 
@@ -403,60 +402,13 @@ linear_fused_kernel(const __grid_constant__ CUtensorMap map_w, const FusedParams
     if (s_abort && tid == 0) drain_after_abort();
 }
 
-int log2_ceil(int v) {
-    int r = 0;
-    while ((1 << r) < v) ++r;
-    return r;
-}
-
-struct FusedPlan {
-    int lanes = 0, rounds = 0, ctas_shift = 0, unit = 0, units = 0, slice = 0, grid = 0;   // lanes = 0: not for this shape
-    uint32_t off_part = 0, off_codes = 0, off_g = 0;
-    size_t smem = 0;
-};
-
-// At most 64 tokens, in one wave of CTAs.  In a chain of calls (graph replays, weights from memory; one launch against two):
-// 1024 x 1024: M = 8 3.8 / 4.2 us, M = 32 5.0 / 6.0, M = 50 5.8 / 6.8; K = 2048, N = 1024: M = 32 5.3 / 7.1, M = 50 6.7 / 8.1;
-// K = 4096, N = 1024: M = 16 5.4 / 6.3, M = 32 6.4 / 9.0; the largest grids are even (1024 x 4096: M = 32 6.1 / 6.2), and
-// behind with few tokens (8 bits, M = 1 4.5 / 4.0): 96 CTAs at most there.  An eager call costs the host 5.4 us instead of 7.7.  CTAs of two rounds share an SM with nobody and clusters of eight do not
-// fill the chip, so that 128 of them would take two waves (K = 4096, N = 2048: 10.3 / 6.3): 96 at most.
-FusedPlan plan_fused(int64_t M, const Weights& W, bool mult) {
-    FusedPlan f;
-    if (M < 1 || M > kMaxTokens || W.K % 128 != 0) return f;
-    const int lanes = M <= 32 ? 16 : 8, round = lanes * E;
-    const int unit = W.block > 128 ? W.block : 128;
-    if (W.K % unit != 0 || W.block > round || W.K > (int64_t)kMaxCluster * 2 * round) return f;
-    const int units = (int)(W.K / unit), bt = (int)((M + 15) / 16 * 16);
-    int shift = 0;
-    auto slice = [&](int s) { return (units + (1 << s) - 1) / (1 << s) * unit; };
-    while (shift < 3 && slice(shift) > round) ++shift;
-    if (slice(shift) > 2 * round) return f;
-    const int64_t grid = ((W.N + kTile - 1) / kTile) << shift;
-    if (grid > (slice(shift) > round || M <= 8 ? 96 : device_sm_count())) return f;
-    f.ctas_shift = shift; f.unit = unit; f.units = units; f.slice = slice(shift); f.grid = (int)grid;
-    f.rounds = f.slice > round ? 2 : 1;
-    const size_t w_bytes = (size_t)kTile * f.slice * W.bits / 8;
-    const size_t part_bytes = (size_t)(1 << shift) * (1 << log2_ceil((int)((M + (1 << shift) - 1) >> shift))) * kTile * 4;
-    // the partial sums take the packed 4-bit weights' place (read by then in the whole cluster: the maxima were exchanged
-    // behind the expansion); 8-bit weights are still being multiplied when another CTA's sums arrive
-    const size_t head = W.bits == 4 ? (w_bytes > part_bytes ? w_bytes : part_bytes) : w_bytes + part_bytes;
-    f.off_part = W.bits == 4 ? 0u : (uint32_t)w_bytes;
-    f.off_codes = (uint32_t)align_up(head, 1024);
-    f.off_g = (uint32_t)align_up(f.off_codes + (size_t)bt * f.slice, 1024);
-    f.smem = f.off_g + (mult ? (size_t)f.slice / E * (E + 4) * 4 : 0) + 1024;
-    // At most two CTAs per SM, whatever launches they belong to: a CTA holds up to half of tensor memory, and one that waited
-    // for columns while its cluster waited for it must not be another cluster's reason to wait (launches of two streams).
-    if (f.smem < 77 * 1024) f.smem = 77 * 1024;
-    f.lanes = lanes;
-    return f;
-}
-
 template <typename XT, int BITS, int LG, int T>
 cudaError_t launch_variant(const CUtensorMap& map, const FusedParams& p, const FusedPlan& f, cudaStream_t stream) {
     auto kern = linear_fused_kernel<XT, BITS, LG, T>;
     const cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), f.smem);
     if (e != cudaSuccess) return e;
-    return launch_pdl(kern, (unsigned)f.grid, (unsigned)kThreads, f.smem, stream, 1u << f.ctas_shift, map, p);
+    const cudaError_t launched = launch_pdl(kern, (unsigned)f.grid, (unsigned)kThreads, f.smem, stream, 1u << f.ctas_shift, map, p);
+    return f.ctas_shift > 0 && cluster_refused(launched) ? cudaErrorNotSupported : launched;
 }
 template <typename XT, int BITS>
 cudaError_t launch_bits(const CUtensorMap& map, const FusedParams& p, const FusedPlan& f, cudaStream_t stream) {
@@ -472,7 +424,7 @@ cudaError_t launch_linear_fused(const void* x, fq_dtype xt, int64_t M, int64_t l
     if (!W.tmap_valid) return cudaErrorNotSupported;
     // a multiplier that is block^-1/2 in every channel is passed as "none": same products, no vector to stage
     const float* mult = W.mult_const ? nullptr : W.mult_g;
-    const FusedPlan f = plan_fused(M, W, mult != nullptr);
+    const FusedPlan f = plan_fused(M, W.N, W.K, W.block, W.bits, mult != nullptr, device_sm_count(), cluster_capacity);
     if (f.lanes == 0) return cudaErrorNotSupported;
     FusedParams p{};
     p.x = x; p.ldx = ldx; p.ldy = ldy;
