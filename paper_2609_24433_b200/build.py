@@ -1,6 +1,7 @@
 """In-tree build of the CUDA library (sm_100a only) and of its torch binding: ``python -m paper_2609_24433_b200.build``."""
 from __future__ import annotations
 
+import importlib.metadata
 import os
 import subprocess
 import sys
@@ -14,6 +15,7 @@ SOURCES = ["fq_api.cu", "act_quant.cu", "act_quant_ring.cu", "gemm_simt.cu", "ge
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", CSRC]
 BINDING = os.path.join(HERE, "_fq_torch" + sysconfig.get_config_var("EXT_SUFFIX"))
+BINDING_TORCH = os.path.join(HERE, "_fq_torch.built")     # the torch that the binding was compiled against
 
 
 def _stale(target: str, deps) -> bool:
@@ -26,7 +28,9 @@ def _stale(target: str, deps) -> bool:
 def build_binding(force: bool = False) -> str:
     """The CPython module over the library: plain C++ against torch's headers, linked to the library next to it."""
     src = os.path.join(CSRC, "torch_binding.cpp")
-    if force or _stale(BINDING, [src, os.path.join(ROOT, "include", "fq.h")]):
+    version = importlib.metadata.version("torch")         # (its headers are part of the source: another torch, another module)
+    built = open(BINDING_TORCH).read().strip() if os.path.exists(BINDING_TORCH) else ""
+    if force or built != version or _stale(BINDING, [src, os.path.join(ROOT, "include", "fq.h")]):
         import torch
         t = os.path.dirname(torch.__file__)
         inc = [os.path.join(ROOT, "include"), os.path.join(t, "include"), os.path.join(t, "include", "torch", "csrc", "api", "include"),
@@ -34,6 +38,8 @@ def build_binding(force: bool = False) -> str:
         subprocess.run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared"] + [f for d in inc for f in ("-I", d)] +
                        [src, "-o", BINDING, "-L", HERE, "-l:" + os.path.basename(LIB), "-L", os.path.join(t, "lib"), "-lc10",
                         "-lc10_cuda", "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python", "-Wl,-rpath,$ORIGIN"], check=True)
+        with open(BINDING_TORCH, "w") as f:
+            f.write(version + "\n")
     return BINDING
 
 

@@ -73,8 +73,8 @@ def _native():
         try:
             from . import _fq_torch
         except ImportError as e:
-            raise RuntimeError("the native binding is missing: build it with `python -m paper_2609_24433_b200.build` "
-                               "(there is no fallback path)") from e
+            raise RuntimeError(f"the native binding cannot be loaded ({e}): build it with "
+                               "`python -m paper_2609_24433_b200.build` (there is no fallback path)") from e
         _torch_binding = _fq_torch
     return _torch_binding
 

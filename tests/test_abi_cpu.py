@@ -157,3 +157,30 @@ def test_missing_library_fails_loudly(monkeypatch):
     monkeypatch.setattr(fq, "LIB_PATH", "/nonexistent/libfq_b200.so")
     with pytest.raises(RuntimeError, match="no fallback"):
         fq.lib()
+
+
+def test_binding_is_rebuilt_for_another_torch(monkeypatch, tmp_path):
+    """The compiled binding belongs to one torch: another version makes it stale, the same one does not."""
+    compiled = []
+
+    def compile_(cmd, check):
+        compiled.append(cmd)
+        open(fq_build.BINDING, "w").close()
+
+    monkeypatch.setattr(fq_build, "BINDING", str(tmp_path / "_fq_torch.so"))
+    monkeypatch.setattr(fq_build, "BINDING_TORCH", str(tmp_path / "_fq_torch.built"))
+    monkeypatch.setattr(fq_build.subprocess, "run", compile_)
+    for version, total in [("2.11.0", 1), ("2.11.0", 1), ("2.12.0", 2), ("2.12.0", 2)]:
+        monkeypatch.setattr(fq_build.importlib.metadata, "version", lambda name, v=version: v)
+        fq_build.build_binding()
+        assert len(compiled) == total, version
+
+
+def test_binding_that_does_not_load_says_why(lib, monkeypatch):
+    import sys
+    monkeypatch.setattr(fq, "_torch_binding", None)
+    monkeypatch.delattr("paper_2609_24433_b200._fq_torch", raising=False)
+    monkeypatch.setitem(sys.modules, "paper_2609_24433_b200._fq_torch", None)
+    with pytest.raises(RuntimeError, match="no fallback") as e:
+        fq._native()
+    assert str(e.value.__cause__) in str(e.value) and str(e.value.__cause__)
