@@ -33,11 +33,11 @@
 namespace fq {
 namespace {
 
-constexpr int kThreads = 512;
+constexpr int kThreads = kRingThreads;
 // Threads of a CTA.  (1024 threads of 32 channels -- twice the warps at 64 registers -- measured
 // slower than 512 threads of 64 channels for 4-bit output: 0.65 against 0.75 of the copy rate at K = 8192, block 128;
 // the extra cross-lane butterfly stage costs more than the occupancy returns.)
-constexpr int kMaxSlots = 128;
+constexpr int kMaxSlots = kRingMaxSlots;
 
 // 128-byte swizzle of a byte offset inside a 1024-byte aligned region.
 __device__ __forceinline__ uint32_t swz128(uint32_t off) { return off ^ (((off >> 7) & 7u) << 4); }
@@ -494,57 +494,11 @@ cudaError_t launch_transform_quantize_ring(const void* x, fq_dtype xt, int64_t r
     const bool gated = gate_kind >= 0;
     const size_t esz = xt == FQ_BF16 ? 2 : 4;
     const size_t row_bytes = (size_t)K * esz;
-    // shape gate: whole 128-byte lines, at most 256 of them per box, blocks of 32..256 channels
-    if (K < 1024 || row_bytes % 128 != 0 || row_bytes / 128 > 256 || rows > 0x7fffffffll || block < 32)
-        return cudaErrorNotSupported;
-    const int sms = device_sm_count();
-    // Gated sites: from two rows per SM on, or long rows.  Prologue alone, GELU, 8-bit codes, operands from memory, here /
-    // register kernel: M = 816, K = 2048 4.6 / 5.7 us, K = 8192 14.0 / 16.0, K = 16384 25.9 / 37.7 (66 before the paired
-    // gate arithmetic); M = 148, K = 8192 4.1 / 3.9, K = 16384 7.0 / 8.5.
-    if (gated && (xt != FQ_BF16 || (mult != nullptr && mult_after_rotation) || (rows < 2 * (int64_t)sms && K <= 8192)))
-        return cudaErrorNotSupported;
-
-    // Channels per thread: 64 where at least two rows per group fit (the fold-after variant with shuffle stages would spill)
-    const size_t half = (row_bytes + 1023) / 1024 * 1024;
-    const size_t slot = gated ? 2 * half : half;
-    const size_t g_bytes = mult ? ((size_t)K * 4 + 1023) / 1024 * 1024 : 0;
-    int e = 0, gw = 0, ngroups = 0, depth = 0;
-    size_t stage_bytes = 0;
-    auto fits = [&](int channels) {
-        e = channels;
-        gw = 1;
-        while ((int64_t)gw * 32 * e < K) gw <<= 1;
-        ngroups = (kThreads / 32) / gw;
-        if (ngroups < 1 || (gw > 1 && ngroups > 15)) return false;             // one named barrier per group
-        stage_bytes = fmt != StoreFmt::Nibble && e == 64 ? (size_t)kThreads * e : 0;
-        const size_t budget = 227 * 1024 - 2048 - 1024 - stage_bytes;
-        if (g_bytes + 2 * slot * ngroups > budget) return false;
-        depth = (int)((budget - g_bytes) / (slot * ngroups));
-        if (depth > 4) depth = 4;
-        return ngroups * depth <= kMaxSlots;
-    };
-    const bool may64 = !gated && K >= 2048 && K % 64 == 0 && !(mult != nullptr && mult_after_rotation && block >= 128);
-    if (!(may64 && fits(64)) && !fits(32)) return cudaErrorNotSupported;
-    // Short batches are latency-bound and go to the register kernel, which spreads a row over more threads.  The line is drawn
-    // by channels per SM, just behind the register kernel's first full wave; it lies higher where a row leaves lanes of its
-    // group idle, most of all with a multiplier, which such lanes' warps still read.  Chains of calls, 8-bit codes, here /
-    // register kernel:
-    //   bf16     K = 1024: M = 1184 2.61 / 2.30 us, 2368 3.15 / 3.23;  K = 2048: M = 592 2.69 / 2.32, 700 2.82 / 3.11, 2368
-    //            4.38 / 5.23;  K = 4096: M = 296 2.62 / 2.36, 370 2.82 / 3.11, 2368 6.78 / 9.30;  K = 8192: M = 148 2.70 /
-    //            2.43, 370 3.62 / 4.00, 2368 11.1 / 18.0;  K = 16384: M = 74 3.14 / 3.52, 816 10.4 / 15.2
-    //   binary32 K = 1024: M = 592 2.33 / 2.16, 1184 2.69 / 3.12;  K = 4096: M = 148 2.29 / 2.13, 592 3.73 / 5.00, 4736 17.8 /
-    //            22.3;  K = 8192: M = 592 5.8 / 7.6, 4736 34.4 / 46.2
-    //   ragged   K = 2560: M = 816 3.51 / 3.27, 1184 4.15 / 4.73, 2368 6.34 / 6.77;  K = 6144: M = 296 3.15 / 2.71, 370 3.38 /
-    //            4.00;  K = 11008: M = 148 3.26 / 2.98, 220 3.96 / 4.47
-    //   ... with a multiplier   K = 2560: M = 2368 8.9 / 8.3, 4736 15.9 / 14.3;  K = 5120: M = 1184 8.8 / 8.6, 2368 15.4 / 14.0,
-    //            4736 25.6 / 25.7;  K = 3072 (three quarters of the lanes): M = 816 4.6 / 5.0, 4736 15.4 / 16.2
-    if (!gated) {
-        const int64_t width = (int64_t)gw * 32 * e;
-        int64_t line = 15000;
-        if (width == K || K < 2048) line = xt == FQ_F32 || K >= 16384 ? 8000 : 8400;
-        else if (mult != nullptr && 4 * K < 3 * width) line = 100000;
-        if (rows * K < line * sms) return cudaErrorNotSupported;
-    }
+    const RingPlan f = plan_ring(rows, K, (int)esz, gated, fmt != StoreFmt::Nibble, mult != nullptr, mult != nullptr && mult_after_rotation,
+                                 block, device_sm_count());
+    if (f.e == 0) return cudaErrorNotSupported;
+    const int e = f.e, gw = f.gw, ngroups = f.ngroups, depth = f.depth, sms = device_sm_count();
+    const size_t half = f.half, slot = f.slot, g_bytes = f.g_bytes, stage_bytes = f.stage_bytes;
 
     CUtensorMap map;
     const uint64_t dims[3] = {128 / esz, row_bytes / 128 * (gated ? 2 : 1), (uint64_t)rows};

@@ -101,23 +101,10 @@ cudaError_t read_and_clear_watchdog(uint32_t* word) {
 
 namespace {
 
-constexpr int kBlockK = 128;         // int8 elements (= bytes) of K per pipeline stage
-constexpr int kAccStages = 2;
-constexpr int kEpiWarps = 8;
-constexpr int kEpiBuffers = 2;                          // output buffers per epilogue warp (bulk stores in flight; four measured no faster)
-constexpr int kEpiStageBytes = kEpiBuffers * 16 * 64;   // per epilogue warp: buffers of 16 tokens x 32 channels of bf16
 constexpr int kThreadsW8 = 32 * (2 + kEpiWarps + 1);   // + one warp: TMA producer of int8 weights
 constexpr int kFirstUnpackWarp = 2 + kEpiWarps;
-constexpr int kUnpackSets = 2;          // sets of four unpack warps, one TMEM lane quadrant each
 constexpr int kThreadsW4 = 32 * (2 + kEpiWarps) + kUnpackSets * 128 + 32;
-constexpr int kMaxStagesW = 8;
-constexpr int kColsW = kBlockK / 4;     // TMEM columns of one unpacked k-block (128 int8 per lane)
-constexpr int kMaxStages = 16;
-constexpr int kMaxStagesP = 16;
-constexpr int kMaxSplit = 16;          // K slices per tile, at most
-constexpr int kMaxSplitTiles = 1024;   // tiles of a launch that splits K (one counter each, ahead of the partial sums)
 enum : int { kUnsplit = 0, kSplitScratch = 1, kSplitCluster = 2 };
-constexpr size_t kCounterBytes = kMaxSplitTiles * sizeof(uint32_t);
 
 struct Params {
     int64_t M, N, K;
@@ -1087,16 +1074,6 @@ bool encode_tiled(CUtensorMap* map, CUtensorMapDataType dt, uint32_t rank, const
               swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-namespace {
-
-int next_pow2(int v) {
-    int r = 32;
-    while (r < v) r <<= 1;
-    return r;
-}
-
-}  // namespace
-
 fq_status build_weight_tmap(Weights& W) {
     W.tmap_valid = false;
     if (W.N == 0) return FQ_OK;
@@ -1122,113 +1099,6 @@ fq_status launch_variant(const CUtensorMap& map_a, const CUtensorMap& map_w, con
                                      (unsigned)cluster, map_a, map_w, map_y, p);
     *refused = cluster > 1 && cluster_refused(e);
     return e == cudaSuccess ? FQ_OK : FQ_ERR_CUDA;
-}
-
-}  // namespace
-
-namespace {
-
-struct Plan {
-    int bt = 0;       // tokens per tile
-    int ctas = 1;     // 2: CTA pairs on 256-channel tiles (cta_group::2)
-    int split = 1;    // >1: every tile is that many work units, each on a slice of K
-    bool cluster = false; // the slices of a tile are the CTAs of a cluster (no scratch)
-    size_t scratch = 0;   // bytes of scratch the split needs: the tile counters, then the int32 partial tiles
-};
-
-// Atoms (of 128 channels) per pipeline stage.  4-bit weights, single CTAs: two for token tiles of at most 128, four for the
-// shortest (the accumulators of longer tiles leave no room for wider TMEM slots); whole atoms, slices of whole stages.
-int atoms_per_stage(int bits, int ctas, int bt, int64_t K, int split) {
-    const int64_t kb = (K + kBlockK - 1) / kBlockK;
-    if (bits != 4 || ctas != 1 || bt > 128 || K % kBlockK != 0) return 1;
-    if (bt <= 64 && kb >= 4 * split && (split == 1 || kb % (4 * split) == 0)) return 4;
-    return split == 1 || kb % (2 * split) == 0 ? 2 : 1;
-}
-// Shared memory of the pipeline rings; `sums`: bytes taken by the sums of a cluster split.
-size_t ring_budget(size_t sums) { return 227 * 1024 - 1024 /*alignment slack*/ - 1024 /*static*/ - (size_t)kEpiWarps * kEpiStageBytes - sums; }
-size_t stage_bytes(int bits, int ctas, int bt, int atoms) {
-    return ((size_t)(bt / ctas) * kBlockK + (size_t)kTileN * kBlockK * bits / 8) * atoms;
-}
-size_t cluster_sums_bytes(int bt, int split) { return (size_t)(split - 1) * ((bt / 16 + split - 1) / split) * 16 * kTileN * sizeof(int32_t); }
-
-// Token tile, CTA grouping and K split.  Upper bound of the tile from TMEM: two accumulator stages,
-// plus the unpacked-weight ring for 4-bit weights (2*bt + 3*32 <= 512 columns).  M is split evenly
-// over m_tiles so that ragged M wastes little.  Candidates are ranked by a cost model fitted to
-// measured launches (cycles): rounds of work units over the SMs, each unit costing
-//     k_blocks * per_kblock(bt) + 16*bt + 1000          (the tail: epilogue and tile hand-over)
-//   4-bit weights:          per_kblock = 330 + bt       (issue floor, then the MMAs' 2*bt); 235 + bt for tiles of at
-//                                        most 128 tokens, whose stages hold two or four k-blocks
-//   8-bit, one CTA:         per_kblock = max(350 + 0.8*bt, 230 + 2*bt)   (issue floor, then shared memory:
-//                                        both operands pass through it)
-//   8-bit, CTA pair:        per_kblock = max(545, 2.62*bt)   (each CTA stages half of the token tile)
-//   4-bit, CTA pair:        0.95 of a single CTA's, for launches of 1.6e11 multiplications and K >= 2048.  Each CTA stages
-//                           half of the token tile, so shared memory is read half as often: no faster while the clock is
-//                           at its highest, but less power, hence a higher clock under the power cap.  Chains of calls,
-//                           pairs / single CTAs, the clock still high and after 0.2 s of load: 16384 x 8192 x 8192
-//                           (M x K x N) 773 / 804 us and 905 / 922, 16384 x 4096 x 4096 222 / 226 and 262 / 268,
-//                           4096 x 8192 x 8192 199 / 200 and 235 / 238, 12000 x 2048 x 8192 158 / 163 and 189 / 194; below
-//                           the line 7000 x 4096 x 4096 103 / 100 and 117 / 119, 4096 x 4096 x 4096 67.2 / 64.9 and 73.0 /
-//                           73.3; a short K: 16384 x 1024 x 4096 96 / 97 and 105 / 104.
-// (A plan takes the host 0.1 to 3 us; asking for the clusters of every candidate first took up to 30.)
-// K split: problems with fewer tiles than SMs and a long K (short batches, few output channels).
-//   By clusters of 2, 4 or 8 CTAs (one wave; at least four k-blocks of ring beside the sums, 4-bit tiles of at most 128
-//   tokens): the tail shrinks to 16*bt/split, the exchange costs 2800 + 40 per CTA of the launch at 4 bits, 3300 + 18 at 8
-//   (the more SMs a launch takes, the less of the next one starts beside it), and 500 per extra slice.  Measured, chains of
-//   calls, split against the best unsplit tile: 64 x 16384 x 2048 (M x K x N) 14.5 / 22.5 us at 4 bits and 16.3 / 31.7 at 8;
-//   16 x 16384 x 4096 14.7 / 22.6 and 18.8 / 32.3; 64 x 4096 x 1024 8.6 / 9.9 and 8.0 / 11.1; 64 x 4096 x 4096 10.4 / 10.5
-//   and 10.2 / 11.9; 128 x 4096 x 1024 8.7 / 9.2 and 8.7 / 10.8; 256 x 4096 x 1024 10.5 / 10.1 at 4 bits; CTA pairs,
-//   816 x 16384 x 2048: the site 5 us faster than 96-token tiles.
-//   Through scratch, where the device cannot hold the clusters (CTA pairs on 8-bit weights, too): 12500 + 40*bt + 1500 per
-//   extra slice.
-Plan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t scratch_avail, bool clusters, int (*capacity_of)(int)) {
-    const int bt_max = bits == 4 ? 208 : 256;
-    const int64_t kb = (K + kBlockK - 1) / kBlockK;
-    Plan best;
-    double best_cost = 0.0;
-    int capacity[kMaxCluster + 1] = {};                  // by CTAs per cluster, asked for once per plan; 0: not yet, else + 1
-    auto held = [&](int ctas) {
-        if (capacity[ctas] == 0) capacity[ctas] = capacity_of(ctas) + 1;
-        return capacity[ctas] - 1;
-    };
-    const bool pairs = N > kTileN && (bits == 8 || (K >= 2048 && (double)M * (double)N * (double)K >= 1.6e11));
-    for (int c = 1; c <= (pairs ? 2 : 1); ++c) {
-        if (c == 2 && clusters && held(2) < 1) break;
-        const int64_t n_units = (N + kTileN * c - 1) / (kTileN * c);
-        for (int mt = (int)((M + bt_max - 1) / bt_max); mt <= (int)((M + 63) / 64); ++mt) {
-            const int b = (int)(((M + mt - 1) / mt + 15) / 16 * 16);
-            if (b > bt_max) continue;
-            const int64_t units = n_units * ((M + b - 1) / b);
-            const double w8_single = 350.0 + 0.8 * b > 230.0 + 2.0 * b ? 350.0 + 0.8 * b : 230.0 + 2.0 * b;
-            // 4-bit, tiles of at most 128 tokens: stages of several atoms (see the kernel) cost less per 128 channels
-            const double w4 = c == 2 ? 0.95 * (330.0 + b) : (b <= 128 && K % kBlockK == 0 ? 235.0 + b : 330.0 + b);
-            const double per_kb = bits == 4 ? w4 : (c == 1 ? w8_single : (2.62 * b > 545.0 ? 2.62 * b : 545.0));
-            const int slots = sms / c;
-            auto offer = [&](int sp, bool cluster, size_t scratch, double unit_cost) {
-                const double cost = (double)((units * sp + slots - 1) / slots) * unit_cost;
-                if (best.bt == 0 || cost < best_cost * 0.98) {   // ties: the earlier candidate (larger tile, no split)
-                    best.bt = b; best.ctas = c; best.split = sp; best.cluster = cluster; best.scratch = scratch;
-                    best_cost = cost;
-                }
-            };
-            offer(1, false, 0, (double)kb * per_kb + 16.0 * b + 1000.0);
-            if (bits == 4 && c == 2) continue;           // (long launches have tiles enough: no kernel for a split of these)
-            if (units * 2 > slots && units * c * 2 > 4 * (int64_t)sms) continue;       // too many tiles for any split
-            for (int sp = 2; sp <= kMaxSplit; sp *= 2) {
-                if (kb % sp != 0 || kb / sp < 2) break;
-                const double slice = (double)(kb / sp) * per_kb + 1000.0;
-                const int atoms = atoms_per_stage(bits, c, b, K, sp);
-                const double ctas = (double)(units * sp * c);
-                if (clusters && (bits == 8 || b <= 128) && sp * c <= kMaxCluster && units * sp <= slots &&
-                    ring_budget(cluster_sums_bytes(b, sp)) * atoms >= 4 * stage_bytes(bits, c, b, atoms) && units <= held(sp * c))
-                    offer(sp, true, 0, slice + 16.0 * b / sp + (bits == 4 ? 2800.0 + 40.0 * ctas : 3300.0 + 18.0 * ctas) + 500.0 * (sp - 1));
-                if ((c == 1 || bits == 8) && units * c <= kMaxSplitTiles && units * c * sp <= 4 * (int64_t)sms) {
-                    const size_t scratch = kCounterBytes + (size_t)units * c * sp * kTileN * b * sizeof(int32_t);
-                    if (scratch <= scratch_avail) offer(sp, false, scratch, slice + 16.0 * b + 12500.0 + 40.0 * b + 1500.0 * (sp - 1));
-                }
-            }
-        }
-    }
-    return best;
 }
 
 }  // namespace
@@ -1273,7 +1143,7 @@ int cluster_capacity(int ctas) {
 // changes at run time.
 fq_status gemm_prepare(int64_t M, const Weights& W, void* scratch, size_t scratch_bytes, cudaStream_t stream) {
     if (M <= 0 || W.N == 0 || scratch == nullptr || gemm_stream_applies(M, W)) return FQ_OK;
-    const Plan plan = plan_gemm(M, W.N, W.K, W.bits, device_sm_count(), scratch_bytes, true, cluster_capacity);
+    const GemmPlan plan = plan_gemm(M, W.N, W.K, W.bits, device_sm_count(), scratch_bytes, true, cluster_capacity);
     if (plan.split <= 1 || plan.cluster) return FQ_OK;
     return cudaMemsetAsync(scratch, 0, kCounterBytes, stream) == cudaSuccess ? FQ_OK : FQ_ERR_CUDA;
 }
@@ -1302,7 +1172,7 @@ fq_status launch_planned(const int8_t* a8, int64_t M, const Weights& W, int acc_
     Params p{};
     p.M = M; p.N = W.N; p.K = W.K;
     const int sms = device_sm_count();
-    const Plan plan = plan_gemm(M, W.N, W.K, W.bits, sms, scratch ? scratch_bytes : 0, true, held);
+    const GemmPlan plan = plan_gemm(M, W.N, W.K, W.bits, sms, scratch ? scratch_bytes : 0, true, held);
     const int bt = plan.bt, ctas = plan.ctas, split = plan.split;
     p.split = split;
     p.counters = static_cast<uint32_t*>(scratch);            // cleared by gemm_prepare()
@@ -1320,52 +1190,13 @@ fq_status launch_planned(const int8_t* a8, int64_t M, const Weights& W, int acc_
     p.out = out;
     p.watchdog = watchdog_device_ptr();
     if (!p.watchdog) return FQ_ERR_CUDA;
-    const int64_t kb128 = (W.K + kBlockK - 1) / kBlockK;
-    const int atoms = atoms_per_stage(W.bits, ctas, bt, W.K, split);
-    // 4-bit weights: every TMEM column the accumulators leave free becomes unpacked-weight ring
-    int stages_w = W.bits == 4 ? (512 - kAccStages * bt) / (kColsW * atoms) : 0;
-    if (stages_w > kMaxStagesW) stages_w = kMaxStagesW;
-    p.tmem_cols = next_pow2(kAccStages * bt + stages_w * kColsW * atoms);
-
-    const size_t sums_bytes = plan.cluster ? cluster_sums_bytes(bt, split) : 0;
-    const size_t epi_bytes = (size_t)kEpiWarps * kEpiStageBytes + sums_bytes;
-    const size_t budget = ring_budget(sums_bytes);
-    const size_t a_bytes = (size_t)(bt / ctas) * kBlockK * atoms, w_bytes = (size_t)kTileN * kBlockK,
-                 pk_bytes = w_bytes / 2 * atoms;
-    size_t smem;
-    if (W.bits == 4) {
-        p.stages_w = stages_w;
-        // Both TMA rings need the same look-ahead in k-blocks (their latencies are the same):
-        // split the budget evenly, then give the remainder to the cheaper packed ring.
-        int sa = (int)(budget / (a_bytes + pk_bytes));
-        if (sa > kMaxStages) sa = kMaxStages;
-        if (sa < 2) return FQ_ERR_UNSUPPORTED;
-        int sp = (int)((budget - sa * a_bytes) / pk_bytes);
-        if (sp > kMaxStagesP) sp = kMaxStagesP;
-        if (stages_w > sa) {            // the unpack warps wait on the activation ring's barriers
-            stages_w = sa;
-            p.stages_w = sa;
-        }
-        p.stages = sa;
-        p.stages_p = sp;
-        // (see the unpack warps; a ring one shorter is slower, one TMEM slot less no faster: 128 x 4096 x 4096 10.5, 11.3 and
-        // 10.4 us, 256 x 2048 x 4096 9.95, 10.1 and 9.9)
-        p.slot_first = sp % kUnpackSets != 0 && sp < stages_w + kUnpackSets ? 1 : 0;
-        if (p.slot_first && stages_w > sp) return FQ_ERR_UNSUPPORTED;      // (no tile comes here)
-        smem = sa * a_bytes + sp * pk_bytes + epi_bytes + 1024;
-    } else {
-        int stages = (int)(budget / (a_bytes + w_bytes));
-        if (stages > kMaxStages) stages = kMaxStages;
-        if (stages < 2) return FQ_ERR_UNSUPPORTED;
-        p.stages = stages;
-        p.stages_p = 0;
-        p.stages_w = 0;
-        smem = (a_bytes + w_bytes) * stages + epi_bytes + 1024;
-    }
-
-    // One CTA of this kind per SM, and none of the short-batch kernel beside it: a cluster whose CTA waited for tensor memory
-    // must not be what another cluster on that SM waits for (launches of two streams).
-    if (plan.cluster && smem < 152 * 1024) smem = 152 * 1024;
+    const GemmRings rings = gemm_rings(plan, W.bits, W.K);
+    if (!rings.fits) return FQ_ERR_UNSUPPORTED;      // (no tile comes here)
+    const int atoms = rings.atoms;
+    p.stages = rings.stages; p.stages_p = rings.stages_p; p.stages_w = rings.stages_w;
+    p.slot_first = rings.slot_first ? 1 : 0;
+    p.tmem_cols = rings.tmem_cols;
+    const size_t smem = rings.smem;
 
     // each CTA of a pair loads its own half of the token tile
     CUtensorMap map_a;
@@ -1388,7 +1219,7 @@ fq_status launch_planned(const int8_t* a8, int64_t M, const Weights& W, int acc_
     p.unit_step = clusters;
     p.units_q = num_units / clusters;
     p.units_rem = num_units % clusters;
-    p.kb_per = (int)((kb128 + atoms - 1) / atoms) / split;      // stages per unit; the planner only picks splits that divide it
+    p.kb_per = (int)(((W.K + kBlockK - 1) / kBlockK + atoms - 1) / atoms) / split;      // stages per unit; the planner only picks splits that divide it
     p.split_shift = split == 1 ? 0 : (split == 2 ? 1 : (split == 4 ? 2 : (split == 8 ? 3 : 4)));
 
     const int cluster = plan.cluster ? split * ctas : ctas;

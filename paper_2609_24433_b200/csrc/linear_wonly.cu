@@ -501,16 +501,7 @@ bool build_stream_tmap(Weights& W) {
 }
 
 bool gemm_stream_applies(int64_t M, const Weights& W) {
-    // Measured against the tcgen05 kernel, operands from memory: ahead wherever the row groups make one round over the SMs
-    // (N <= 32 x SMs: 16 x 4096 x 4096 (M x K x N) 7.0 us against 9.7), and with at most 8 tokens two rounds (8 x 4096 x 8192
-    // 9.7 / 10.1; 16 x 4096 x 8192 13.5 / 10.1) -- every row group ends with a rendezvous and a reduction --, up to
-    // 128 Mi weights for at most 8 tokens and 64 Mi for at most 16 (16 x 16384 x 8192: 23 us against 21 us).
-    if (!W.tmap_stream_valid || M < 1 || M > 16) return false;
-    // 8-bit weights (twice the bytes per row): ahead where the row groups make ONE round over the SMs, up to 64 Mi
-    // weights (16 tokens, K = 8192, N = 4096: 12.8 us against 17.5 us; K = 4096, N = 8192: 14.0 against 11.5 us)
-    if (W.bits == 8) return W.N <= 32ll * device_sm_count() && W.N * W.K <= (1ll << 26);
-    if (W.N > (M <= 8 ? 64ll : 32ll) * device_sm_count()) return false;
-    return W.N * W.K <= (M <= 8 ? (1ll << 27) : (1ll << 26));
+    return W.tmap_stream_valid && plan_stream(M, W.N, W.K, W.bits, device_sm_count());
 }
 
 cudaError_t launch_gemm_stream(const int8_t* a8, int64_t M, const Weights& W, int acc_shift, const GemmOut& out,

@@ -118,4 +118,249 @@ CompositePlan plan_composite(int64_t rows, int64_t K, int elem_bytes, int beta, 
     return f;
 }
 
+// ---- streamed prologue (act_quant_ring.cu) instead of the register one -------------------------------------------------
+constexpr int kRingThreads = 512;
+constexpr int kRingMaxSlots = 128;
+
+struct RingPlan {
+    int e = 0;                         // channels per thread; 0: the register kernel
+    int gw = 0, ngroups = 0, depth = 0;   // warps per row group, groups per CTA, ring slots per group
+    size_t half = 0, slot = 0;         // bytes of a row in shared memory, and of a slot (two rows for gated sites)
+    size_t g_bytes = 0, stage_bytes = 0;  // the multiplier's stage, the codes' stage
+};
+
+// bytes_out: one byte per code; mult: a per-channel multiplier, after: behind the rotation.
+inline RingPlan plan_ring(int64_t rows, int64_t K, int elem_bytes, bool gated, bool bytes_out, bool mult, bool after, int block, int sms) {
+    RingPlan f;
+    const size_t row_bytes = (size_t)K * elem_bytes;
+    // shape gate: whole 128-byte lines, at most 256 of them per box, blocks of 32..256 channels
+    if (K < 1024 || row_bytes % 128 != 0 || row_bytes / 128 > 256 || rows > 0x7fffffffll || block < 32)
+        return RingPlan();
+    // Gated sites: from two rows per SM on, or long rows.  Prologue alone, GELU, 8-bit codes, operands from memory, here /
+    // register kernel: M = 816, K = 2048 4.6 / 5.7 us, K = 8192 14.0 / 16.0, K = 16384 25.9 / 37.7 (66 before the paired
+    // gate arithmetic); M = 148, K = 8192 4.1 / 3.9, K = 16384 7.0 / 8.5.
+    if (gated && (elem_bytes != 2 || after || (rows < 2 * (int64_t)sms && K <= 8192)))
+        return RingPlan();
+
+    // Channels per thread: 64 where at least two rows per group fit (the fold-after variant with shuffle stages would spill)
+    f.half = (row_bytes + 1023) / 1024 * 1024;
+    f.slot = gated ? 2 * f.half : f.half;
+    f.g_bytes = mult ? ((size_t)K * 4 + 1023) / 1024 * 1024 : 0;
+    auto fits = [&](int channels) {
+        f.e = channels;
+        f.gw = 1;
+        while ((int64_t)f.gw * 32 * f.e < K) f.gw <<= 1;
+        f.ngroups = (kRingThreads / 32) / f.gw;
+        if (f.ngroups < 1 || (f.gw > 1 && f.ngroups > 15)) return false;             // one named barrier per group
+        f.stage_bytes = bytes_out && f.e == 64 ? (size_t)kRingThreads * f.e : 0;
+        const size_t budget = 227 * 1024 - 2048 - 1024 - f.stage_bytes;
+        if (f.g_bytes + 2 * f.slot * f.ngroups > budget) return false;
+        f.depth = (int)((budget - f.g_bytes) / (f.slot * f.ngroups));
+        if (f.depth > 4) f.depth = 4;
+        return f.ngroups * f.depth <= kRingMaxSlots;
+    };
+    const bool may64 = !gated && K >= 2048 && K % 64 == 0 && !(after && block >= 128);
+    if (!(may64 && fits(64)) && !fits(32)) return RingPlan();
+    // Short batches are latency-bound and go to the register kernel, which spreads a row over more threads.  The line is drawn
+    // by channels per SM, just behind the register kernel's first full wave; it lies higher where a row leaves lanes of its
+    // group idle, most of all with a multiplier, which such lanes' warps still read.  Chains of calls, 8-bit codes, here /
+    // register kernel:
+    //   bf16     K = 1024: M = 1184 2.61 / 2.30 us, 2368 3.15 / 3.23;  K = 2048: M = 592 2.69 / 2.32, 700 2.82 / 3.11, 2368
+    //            4.38 / 5.23;  K = 4096: M = 296 2.62 / 2.36, 370 2.82 / 3.11, 2368 6.78 / 9.30;  K = 8192: M = 148 2.70 /
+    //            2.43, 370 3.62 / 4.00, 2368 11.1 / 18.0;  K = 16384: M = 74 3.14 / 3.52, 816 10.4 / 15.2
+    //   binary32 K = 1024: M = 592 2.33 / 2.16, 1184 2.69 / 3.12;  K = 4096: M = 148 2.29 / 2.13, 592 3.73 / 5.00, 4736 17.8 /
+    //            22.3;  K = 8192: M = 592 5.8 / 7.6, 4736 34.4 / 46.2
+    //   ragged   K = 2560: M = 816 3.51 / 3.27, 1184 4.15 / 4.73, 2368 6.34 / 6.77;  K = 6144: M = 296 3.15 / 2.71, 370 3.38 /
+    //            4.00;  K = 11008: M = 148 3.26 / 2.98, 220 3.96 / 4.47
+    //   ... with a multiplier   K = 2560: M = 2368 8.9 / 8.3, 4736 15.9 / 14.3;  K = 5120: M = 1184 8.8 / 8.6, 2368 15.4 / 14.0,
+    //            4736 25.6 / 25.7;  K = 3072 (three quarters of the lanes): M = 816 4.6 / 5.0, 4736 15.4 / 16.2
+    if (!gated) {
+        const int64_t width = (int64_t)f.gw * 32 * f.e;
+        int64_t line = 15000;
+        if (width == K || K < 2048) line = elem_bytes == 4 || K >= 16384 ? 8000 : 8400;
+        else if (mult && 4 * K < 3 * width) line = 100000;
+        if (rows * K < line * sms) return RingPlan();
+    }
+    return f;
+}
+
+// ---- integer product of short batches: the weight-streaming kernel (linear_wonly.cu) instead of the tcgen05 one ----------
+// (Rows of whole 128-byte lines only.)
+inline bool plan_stream(int64_t M, int64_t N, int64_t K, int bits, int sms) {
+    // Measured against the tcgen05 kernel, operands from memory: ahead wherever the row groups make one round over the SMs
+    // (N <= 32 x SMs: 16 x 4096 x 4096 (M x K x N) 7.0 us against 9.7), and with at most 8 tokens two rounds (8 x 4096 x 8192
+    // 9.7 / 10.1; 16 x 4096 x 8192 13.5 / 10.1) -- every row group ends with a rendezvous and a reduction --, up to
+    // 128 Mi weights for at most 8 tokens and 64 Mi for at most 16 (16 x 16384 x 8192: 23 us against 21 us).
+    if (K % (bits == 4 ? 256 : 128) != 0 || M < 1 || M > 16) return false;
+    // 8-bit weights (twice the bytes per row): ahead where the row groups make ONE round over the SMs, up to 64 Mi
+    // weights (16 tokens, K = 8192, N = 4096: 12.8 us against 17.5 us; K = 4096, N = 8192: 14.0 against 11.5 us)
+    if (bits == 8) return N <= 32ll * sms && N * K <= (1ll << 26);
+    if (N > (M <= 8 ? 64ll : 32ll) * sms) return false;
+    return N * K <= (M <= 8 ? (1ll << 27) : (1ll << 26));
+}
+
+// ---- integer GEMM (gemm_tcgen05.cu) ------------------------------------------------------------------------------------
+constexpr int kBlockK = 128;           // int8 elements (= bytes) of K per pipeline stage
+constexpr int kAccStages = 2;
+constexpr int kUnpackSets = 2;         // sets of four unpack warps, one TMEM lane quadrant each
+constexpr int kMaxStages = 16;         // ring slots, at most: activations, packed weights, unpacked weights
+constexpr int kMaxStagesP = 16;
+constexpr int kMaxStagesW = 8;
+constexpr int kColsW = kBlockK / 4;    // TMEM columns of one unpacked k-block (128 int8 per lane)
+constexpr int kEpiWarps = 8;
+constexpr int kEpiBuffers = 2;                          // output buffers per epilogue warp (bulk stores in flight; four measured no faster)
+constexpr int kEpiStageBytes = kEpiBuffers * 16 * 64;   // per epilogue warp: buffers of 16 tokens x 32 channels of bf16
+constexpr int kMaxSplit = 16;          // K slices per tile, at most
+constexpr int kMaxSplitTiles = 1024;   // tiles of a launch that splits K (one counter each, ahead of the partial sums)
+constexpr size_t kCounterBytes = kMaxSplitTiles * sizeof(uint32_t);
+
+struct GemmPlan {
+    int bt = 0;       // tokens per tile
+    int ctas = 1;     // 2: CTA pairs on 256-channel tiles (cta_group::2)
+    int split = 1;    // >1: every tile is that many work units, each on a slice of K
+    bool cluster = false; // the slices of a tile are the CTAs of a cluster (no scratch)
+    size_t scratch = 0;   // bytes of scratch the split needs: the tile counters, then the int32 partial tiles
+};
+
+// Atoms (of 128 channels) per pipeline stage.  4-bit weights, single CTAs: two for token tiles of at most 128, four for the
+// shortest (the accumulators of longer tiles leave no room for wider TMEM slots); whole atoms, slices of whole stages.
+inline int atoms_per_stage(int bits, int ctas, int bt, int64_t K, int split) {
+    const int64_t kb = (K + kBlockK - 1) / kBlockK;
+    if (bits != 4 || ctas != 1 || bt > 128 || K % kBlockK != 0) return 1;
+    if (bt <= 64 && kb >= 4 * split && (split == 1 || kb % (4 * split) == 0)) return 4;
+    return split == 1 || kb % (2 * split) == 0 ? 2 : 1;
+}
+// Shared memory of the pipeline rings; `sums`: bytes taken by the sums of a cluster split.
+inline size_t ring_budget(size_t sums) { return 227 * 1024 - 1024 /*alignment slack*/ - 1024 /*static*/ - (size_t)kEpiWarps * kEpiStageBytes - sums; }
+inline size_t stage_bytes(int bits, int ctas, int bt, int atoms) {
+    return ((size_t)(bt / ctas) * kBlockK + (size_t)kTileN * kBlockK * bits / 8) * atoms;
+}
+inline size_t cluster_sums_bytes(int bt, int split) { return (size_t)(split - 1) * ((bt / 16 + split - 1) / split) * 16 * kTileN * sizeof(int32_t); }
+
+// Token tile, CTA grouping and K split.  Upper bound of the tile from TMEM: two accumulator stages,
+// plus the unpacked-weight ring for 4-bit weights (2*bt + 3*32 <= 512 columns).  M is split evenly
+// over m_tiles so that ragged M wastes little.  Candidates are ranked by a cost model fitted to
+// measured launches (cycles): rounds of work units over the SMs, each unit costing
+//     k_blocks * per_kblock(bt) + 16*bt + 1000          (the tail: epilogue and tile hand-over)
+//   4-bit weights:          per_kblock = 330 + bt       (issue floor, then the MMAs' 2*bt); 235 + bt for tiles of at
+//                                        most 128 tokens, whose stages hold two or four k-blocks
+//   8-bit, one CTA:         per_kblock = max(350 + 0.8*bt, 230 + 2*bt)   (issue floor, then shared memory:
+//                                        both operands pass through it)
+//   8-bit, CTA pair:        per_kblock = max(545, 2.62*bt)   (each CTA stages half of the token tile)
+//   4-bit, CTA pair:        0.95 of a single CTA's, for launches of 1.6e11 multiplications and K >= 2048.  Each CTA stages
+//                           half of the token tile, so shared memory is read half as often: no faster while the clock is
+//                           at its highest, but less power, hence a higher clock under the power cap.  Chains of calls,
+//                           pairs / single CTAs, the clock still high and after 0.2 s of load: 16384 x 8192 x 8192
+//                           (M x K x N) 773 / 804 us and 905 / 922, 16384 x 4096 x 4096 222 / 226 and 262 / 268,
+//                           4096 x 8192 x 8192 199 / 200 and 235 / 238, 12000 x 2048 x 8192 158 / 163 and 189 / 194; below
+//                           the line 7000 x 4096 x 4096 103 / 100 and 117 / 119, 4096 x 4096 x 4096 67.2 / 64.9 and 73.0 /
+//                           73.3; a short K: 16384 x 1024 x 4096 96 / 97 and 105 / 104.
+// (A plan takes the host 0.1 to 3 us; asking for the clusters of every candidate first took up to 30.)
+// K split: problems with fewer tiles than SMs and a long K (short batches, few output channels).
+//   By clusters of 2, 4 or 8 CTAs (one wave; at least four k-blocks of ring beside the sums, 4-bit tiles of at most 128
+//   tokens): the tail shrinks to 16*bt/split, the exchange costs 2800 + 40 per CTA of the launch at 4 bits, 3300 + 18 at 8
+//   (the more SMs a launch takes, the less of the next one starts beside it), and 500 per extra slice.  Measured, chains of
+//   calls, split against the best unsplit tile: 64 x 16384 x 2048 (M x K x N) 14.5 / 22.5 us at 4 bits and 16.3 / 31.7 at 8;
+//   16 x 16384 x 4096 14.7 / 22.6 and 18.8 / 32.3; 64 x 4096 x 1024 8.6 / 9.9 and 8.0 / 11.1; 64 x 4096 x 4096 10.4 / 10.5
+//   and 10.2 / 11.9; 128 x 4096 x 1024 8.7 / 9.2 and 8.7 / 10.8; 256 x 4096 x 1024 10.5 / 10.1 at 4 bits; CTA pairs,
+//   816 x 16384 x 2048: the site 5 us faster than 96-token tiles.
+//   Through scratch, where the device cannot hold the clusters (CTA pairs on 8-bit weights, too): 12500 + 40*bt + 1500 per
+//   extra slice.
+template <typename Held>
+GemmPlan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t scratch_avail, bool clusters, Held held) {
+    const int bt_max = bits == 4 ? 208 : 256;
+    const int64_t kb = (K + kBlockK - 1) / kBlockK;
+    GemmPlan best;
+    double best_cost = 0.0;
+    int capacity[kMaxCluster + 1] = {};                  // by CTAs per cluster, asked for once per plan; 0: not yet, else + 1
+    auto holds = [&](int ctas) {
+        if (capacity[ctas] == 0) capacity[ctas] = held(ctas) + 1;
+        return capacity[ctas] - 1;
+    };
+    const bool pairs = N > kTileN && (bits == 8 || (K >= 2048 && (double)M * (double)N * (double)K >= 1.6e11));
+    for (int c = 1; c <= (pairs ? 2 : 1); ++c) {
+        if (c == 2 && clusters && holds(2) < 1) break;
+        const int64_t n_units = (N + kTileN * c - 1) / (kTileN * c);
+        for (int mt = (int)((M + bt_max - 1) / bt_max); mt <= (int)((M + 63) / 64); ++mt) {
+            const int b = (int)(((M + mt - 1) / mt + 15) / 16 * 16);
+            if (b > bt_max) continue;
+            const int64_t units = n_units * ((M + b - 1) / b);
+            const double w8_single = 350.0 + 0.8 * b > 230.0 + 2.0 * b ? 350.0 + 0.8 * b : 230.0 + 2.0 * b;
+            // 4-bit, tiles of at most 128 tokens: stages of several atoms (see the kernel) cost less per 128 channels
+            const double w4 = c == 2 ? 0.95 * (330.0 + b) : (b <= 128 && K % kBlockK == 0 ? 235.0 + b : 330.0 + b);
+            const double per_kb = bits == 4 ? w4 : (c == 1 ? w8_single : (2.62 * b > 545.0 ? 2.62 * b : 545.0));
+            const int slots = sms / c;
+            auto offer = [&](int sp, bool cluster, size_t scratch, double unit_cost) {
+                const double cost = (double)((units * sp + slots - 1) / slots) * unit_cost;
+                if (best.bt == 0 || cost < best_cost * 0.98) {   // ties: the earlier candidate (larger tile, no split)
+                    best.bt = b; best.ctas = c; best.split = sp; best.cluster = cluster; best.scratch = scratch;
+                    best_cost = cost;
+                }
+            };
+            offer(1, false, 0, (double)kb * per_kb + 16.0 * b + 1000.0);
+            if (bits == 4 && c == 2) continue;           // (long launches have tiles enough: no kernel for a split of these)
+            if (units * 2 > slots && units * c * 2 > 4 * (int64_t)sms) continue;       // too many tiles for any split
+            for (int sp = 2; sp <= kMaxSplit; sp *= 2) {
+                if (kb % sp != 0 || kb / sp < 2) break;
+                const double slice = (double)(kb / sp) * per_kb + 1000.0;
+                const int atoms = atoms_per_stage(bits, c, b, K, sp);
+                const double ctas = (double)(units * sp * c);
+                if (clusters && (bits == 8 || b <= 128) && sp * c <= kMaxCluster && units * sp <= slots &&
+                    ring_budget(cluster_sums_bytes(b, sp)) * atoms >= 4 * stage_bytes(bits, c, b, atoms) && units <= holds(sp * c))
+                    offer(sp, true, 0, slice + 16.0 * b / sp + (bits == 4 ? 2800.0 + 40.0 * ctas : 3300.0 + 18.0 * ctas) + 500.0 * (sp - 1));
+                if ((c == 1 || bits == 8) && units * c <= kMaxSplitTiles && units * c * sp <= 4 * (int64_t)sms) {
+                    const size_t scratch = kCounterBytes + (size_t)units * c * sp * kTileN * b * sizeof(int32_t);
+                    if (scratch <= scratch_avail) offer(sp, false, scratch, slice + 16.0 * b + 12500.0 + 40.0 * b + 1500.0 * (sp - 1));
+                }
+            }
+        }
+    }
+    return best;
+}
+
+// The rings of a plan: slots of activations (and int8 weights, in lockstep), of packed and of unpacked 4-bit weights.
+struct GemmRings {
+    bool fits = false;
+    int atoms = 1, stages = 0, stages_p = 0, stages_w = 0, tmem_cols = 0;
+    bool slot_first = false;           // the unpack sets wait for the TMEM slot ahead of the packed stage (see the kernel)
+    size_t smem = 0;
+};
+inline GemmRings gemm_rings(const GemmPlan& plan, int bits, int64_t K) {
+    GemmRings f;
+    const int bt = plan.bt;
+    f.atoms = atoms_per_stage(bits, plan.ctas, bt, K, plan.split);
+    const size_t sums = plan.cluster ? cluster_sums_bytes(bt, plan.split) : 0, budget = ring_budget(sums);
+    const size_t epi_bytes = (size_t)kEpiWarps * kEpiStageBytes + sums;
+    const size_t a_bytes = (size_t)(bt / plan.ctas) * kBlockK * f.atoms, w_bytes = (size_t)kTileN * kBlockK, pk_bytes = w_bytes / 2 * f.atoms;
+    // 4-bit weights: every TMEM column the accumulators leave free becomes unpacked-weight ring
+    f.stages_w = bits == 4 ? (512 - kAccStages * bt) / (kColsW * f.atoms) : 0;
+    if (f.stages_w > kMaxStagesW) f.stages_w = kMaxStagesW;
+    for (f.tmem_cols = 32; f.tmem_cols < kAccStages * bt + f.stages_w * kColsW * f.atoms;) f.tmem_cols <<= 1;
+    if (bits == 4) {
+        // Both TMA rings need the same look-ahead in k-blocks (their latencies are the same): split the budget evenly, then
+        // give the remainder to the cheaper packed ring.
+        f.stages = (int)(budget / (a_bytes + pk_bytes));
+        if (f.stages > kMaxStages) f.stages = kMaxStages;
+        if (f.stages < 2) return f;
+        f.stages_p = (int)((budget - f.stages * a_bytes) / pk_bytes);
+        if (f.stages_p > kMaxStagesP) f.stages_p = kMaxStagesP;
+        if (f.stages_w > f.stages) f.stages_w = f.stages;       // the unpack warps wait on the activation ring's barriers
+        // (a ring one shorter is slower, one TMEM slot less no faster: 128 x 4096 x 4096 10.5, 11.3 and 10.4 us, 256 x 2048 x
+        // 4096 9.95, 10.1 and 9.9)
+        f.slot_first = f.stages_p % kUnpackSets != 0 && f.stages_p < f.stages_w + kUnpackSets;
+        if (f.slot_first && f.stages_w > f.stages_p) return f;
+        f.smem = f.stages * a_bytes + f.stages_p * pk_bytes + epi_bytes + 1024;
+    } else {
+        f.stages = (int)(budget / (a_bytes + w_bytes));
+        if (f.stages > kMaxStages) f.stages = kMaxStages;
+        if (f.stages < 2) return f;
+        f.smem = (a_bytes + w_bytes) * f.stages + epi_bytes + 1024;
+    }
+    // One CTA of this kind per SM, and none of the short-batch kernel beside it: a cluster whose CTA waited for tensor memory
+    // must not be what another cluster on that SM waits for (launches of two streams).
+    if (plan.cluster && f.smem < 152 * 1024) f.smem = 152 * 1024;
+    f.fits = true;
+    return f;
+}
+
 }  // namespace fq

@@ -1,5 +1,6 @@
 """GPU parity at the sizes where a kernel or a dispatch rule can go wrong: edges of tiles, remainders, the smallest
-and the largest of each variant's range.  Same oracle and same bounds as test_gpu_parity.py."""
+and the largest of each variant's range.  Same oracle and same bounds as test_gpu_parity.py.  That the sizes in the lists
+below take the routes they stand for, on a whole B200, is checked without a device in test_host_rules.py."""
 import os
 import subprocess
 import sys
@@ -43,11 +44,14 @@ def test_gptq_fold_at_the_edges_of_its_kernels(N, K, Mc, block):
     assert np.array_equal(to_np(hc), wc)
 
 
-@pytest.mark.parametrize("M,K,block,bits,act", [
+GATED = [
     (296, 2048, 32, 4, oracle.SILU),                   # the shortest batch of the streamed gated rows on 148 SMs
     (295, 2048, 128, 8, oracle.GELU_TANH),             # the longest of the register kernel
     (3, 8448, 256, 8, oracle.GELU_TANH),               # long rows are streamed at any batch size
-])
+]
+
+
+@pytest.mark.parametrize("M,K,block,bits,act", GATED)
 def test_gated_prologue_on_both_sides_of_its_rule(M, K, block, bits, act):
     rng = np.random.default_rng(M + K)
     gu = rng.standard_normal((M, 2 * K)).astype(np.float32)
@@ -62,11 +66,15 @@ def test_gated_prologue_on_both_sides_of_its_rule(M, K, block, bits, act):
     assert np.array_equal(to_np(codes), want_codes)
 
 
-@pytest.mark.parametrize("M,K,N", [
-    (64, 4096, 8192),      # 64-token tiles of four-atom stages: a packed ring of three, an odd length, for two unpack sets
-    (96, 4096, 2048),      # two-atom stages, ring of five, five TMEM slots
-    (128, 8192, 2048),     # ring of five, four TMEM slots
-])
+ODD_RINGS = [              # packed rings of an odd length, shorter than the two unpack sets' look-ahead
+    (64, 4096, 8192),      # 64-token tiles of four-atom stages: a ring of three, three TMEM slots
+    (96, 4096, 16384),     # two-atom stages: a ring of five, five TMEM slots
+    (128, 4096, 16384),    # ... four TMEM slots
+    (80, 4096, 2048),      # K split by clusters of four
+]
+
+
+@pytest.mark.parametrize("M,K,N", ODD_RINGS)
 def test_odd_packed_rings_return_the_same_bits(M, K, N):
     """400 launches on rotating weights (so that the copies come from memory and land out of order), all equal to the
     CUDA-core witness."""
@@ -91,18 +99,23 @@ def test_odd_packed_rings_return_the_same_bits(M, K, N):
             assert torch.equal(y, w)
 
 
-@pytest.mark.parametrize("M,K,N,block,bits,dtype,smooth,clip", [
+ONE_LAUNCH = [
     (1, 128, 8, 32, 4, "bf16", False, 1.0),            # one token, one slice, one CTA
     (16, 256, 136, 256, 8, "f32", True, 0.9),          # a block as wide as a slice
     (17, 640, 1032, 128, 4, "f32", True, 1.0),         # five units over four CTAs, a ragged channel tile
-    (32, 1024, 3072, 1, 8, "bf16", False, 1.0),        # identity rotation; the last batch of sixteen channels a thread
-    (33, 1024, 1024, 64, 4, "bf16", True, 1.0),        # the first of thirty-two
-    (50, 1792, 4104, 8, 4, "bf16", False, 0.8),        # fourteen units over eight CTAs
-    (64, 2304, 520, 128, 8, "bf16", True, 1.0),        # two rounds of channels in some slices, one in others
-    (64, 4096, 1024, 256, 4, "f32", False, 1.0),       # the longest rows
-    (50, 1024, 18944, 64, 4, "bf16", False, 1.0),      # two tiles per cluster, two CTAs per SM
-    (63, 512, 18952, 64, 8, "f32", False, 1.0),
-])
+    (8, 1024, 3072, 64, 4, "bf16", True, 1.0),         # the most CTAs with few tokens
+    (32, 1024, 3072, 1, 8, "bf16", False, 1.0),        # identity rotation; the last batch of sixteen lanes a token
+    (33, 1024, 1024, 64, 4, "bf16", True, 1.0),        # the first of eight
+    (50, 1792, 1032, 8, 4, "bf16", False, 0.8),        # two rounds; fourteen units over eight CTAs: one round in some slices
+    (64, 1920, 520, 128, 8, "bf16", True, 1.0),        # ... fifteen
+    (64, 2048, 1024, 128, 4, "f32", False, 1.0),       # the longest rows of more than 32 tokens
+    (32, 4096, 1024, 256, 4, "f32", False, 1.0),       # the longest rows
+    (50, 1024, 2304, 64, 4, "bf16", False, 1.0),       # the widest outputs in clusters of eight
+    (63, 512, 4736, 64, 8, "f32", False, 1.0),         # ... of four: one CTA for each of 148 SMs
+]
+
+
+@pytest.mark.parametrize("M,K,N,block,bits,dtype,smooth,clip", ONE_LAUNCH)
 def test_one_launch_path_equals_prologue_and_gemm(M, K, N, block, bits, dtype, smooth, clip):
     """Codes and steps against the oracle, outputs against the two-call route, all bit for bit, three replays of a graph
     of two calls on one workspace included."""
@@ -126,17 +139,20 @@ def test_one_launch_path_equals_prologue_and_gemm(M, K, N, block, bits, dtype, s
     assert torch.equal(ya, y) and torch.equal(yb, y.flip(0))
 
 
-@pytest.mark.parametrize("M,K,beta,bits,dtype,smooth,lead", [
+COMPOSITE = [
     (1, 64, 64, 4, "bf16", False, 0),                  # one token, one item, one CTA
     (17, 512, 16, 8, "f32", True, 0),                  # the smallest blocks, one token into the second tile
     (33, 768, 256, 4, "bf16", True, 0),                # blocks of four items, an uneven share of them
-    (700, 1024, 32, 4, "bf16", True, 8),               # more tiles than SMs, rows with a lead
+    (700, 1024, 32, 4, "bf16", True, 8),               # more CTAs than SMs, rows with a lead
     (20, 4096, 128, 8, "f32", False, 0),               # binary32 rows of which eight fit
     (9, 8192, 64, 4, "f32", False, 0),                 # ... and none: the two-kernel form
     (20, 4096, 128, 8, "bf16", False, 4),              # rows that are not 16-byte aligned
     (576, 2048, 64, 4, "bf16", False, 0),              # 148 SMs: the most clusters of four in one wave
     (577, 2048, 64, 4, "bf16", True, 0),               # ... and clusters of two
-])
+]
+
+
+@pytest.mark.parametrize("M,K,beta,bits,dtype,smooth,lead", COMPOSITE)
 def test_composite_prologue_at_the_edges_of_its_kernels(M, K, beta, bits, dtype, smooth, lead):
     rng = np.random.default_rng(M + K)
     perm, blocks = synth.composite_rotation(K, beta, seed=K)
@@ -151,17 +167,20 @@ def test_composite_prologue_at_the_edges_of_its_kernels(M, K, beta, bits, dtype,
     assert np.array_equal(to_np(codes), want_codes)
 
 
-@pytest.mark.parametrize("M,K,N,bits", [
+CLUSTER_SPLIT = [
     (64, 16384, 2048, 4),      # clusters of four, four-atom stages
-    (16, 16384, 4096, 8),      # one token chunk: one CTA of four finishes the tile
+    (16, 16384, 4608, 8),      # one token chunk: one CTA of four finishes the tile
     (100, 16384, 256, 4),      # few tiles: clusters of eight, ragged last chunk
     (50, 16384, 1024, 8),
     (90, 8192, 520, 8),        # a ragged channel tile
-    (208, 16384, 136, 4),      # the longest token tiles
+    (208, 16384, 136, 4),      # the longest batch in two tiles of 112 tokens
     (250, 16384, 128, 8),
     (816, 16384, 2048, 8),     # CTA pairs, clusters of two pairs
     (790, 16384, 1960, 8),     # ... with ragged tokens and channels
-])
+]
+
+
+@pytest.mark.parametrize("M,K,N,bits", CLUSTER_SPLIT)
 def test_cluster_split_equals_the_second_witness(M, K, N, bits):
     """int32 sums, binary32 and bf16 outputs, without any scratch in the workspace, a second call right behind the first."""
     g = torch.Generator(device="cuda").manual_seed(M + N)
@@ -178,30 +197,69 @@ def test_cluster_split_equals_the_second_witness(M, K, N, bits):
         assert torch.equal(a, want) and torch.equal(b, want)
 
 
-@pytest.mark.parametrize("M,K,N", [
+SCRATCH_SPLIT = [
+    (75, 20480, 4624, 8),      # more tiles than the clusters that a device holds: slices meet in the workspace
+    (17, 32768, 4640, 4),      # four-atom stages
+    (1562, 32768, 704, 4),     # token tiles of 144, which clusters do not take
+    (1181, 32768, 712, 8),     # CTA pairs
+]
+
+
+@pytest.mark.parametrize("M,K,N,bits", SCRATCH_SPLIT)
+def test_scratch_split_equals_the_second_witness(M, K, N, bits):
+    """Through a workspace whose scratch (counters included) holds anything, through one that has none, and on three streams
+    with a workspace each."""
+    g = torch.Generator(device="cuda").manual_seed(M + N)
+    h = fq.weights_import(torch.randint(0, 256, (N, K * bits // 8), dtype=torch.uint8, device="cuda", generator=g),
+                          torch.rand(N, device="cuda", generator=g) + 0.1, None, torch.randn(N, device="cuda", generator=g), K, 64, bits)
+    xs = [torch.randn(M, K, device="cuda", generator=g) for _ in range(3)]
+    full, base = fq.workspace_bytes(M, K, N, bits), (M * K + 255) // 256 * 256 + (4 * M + 255) // 256 * 256
+    assert full > base
+    wss = [torch.randint(0, 256, (full,), dtype=torch.uint8, device="cuda", generator=g) for _ in xs]
+    codes = [fq.quantize_act(x, None, 64, bits) for x in xs]
+    assert torch.equal(fq.gemm_acc_i32(codes[0][0], h, workspace=wss[0]), fq.gemm_simt(codes[0][0], None, h, raw_acc=True))
+    for dt in (torch.float32, torch.bfloat16):
+        want = [fq.gemm_simt(c, d, h, dt) for c, d in codes]
+        assert torch.equal(fq.linear(xs[0], h, out_dtype=dt, workspace=wss[0][:base]), want[0])
+        torch.cuda.synchronize()
+        got = []
+        for x, ws, st in zip(xs, wss, [torch.cuda.Stream() for _ in xs]):
+            with torch.cuda.stream(st):
+                got.append([fq.linear(x, h, out_dtype=dt, workspace=ws) for _ in range(3)])
+        torch.cuda.synchronize()
+        assert all(torch.equal(y, w) for ys, w in zip(got, want) for y in ys)
+
+
+W4_PAIRS = [
     (9001, 4096, 4352),        # 1.6e11 multiplications: CTA pairs, a ragged last token tile
-    (9000, 4096, 4336),        # just short of it: single CTAs
-    (60001, 2048, 1336),       # the shortest K, the last pair with no channel for its odd CTA
+    (16001, 2048, 5128),       # the shortest K, the last pair with no channel for its odd CTA
     (40001, 8256, 496),        # channels past K in the last k-block, the last pair nearly full
-])
+]
+W4_SINGLE = [(9000, 4096, 4336)]   # just short of 1.6e11: single CTAs
+
+
+@pytest.mark.parametrize("M,K,N", W4_PAIRS + W4_SINGLE)
 def test_long_w4_pairs_equal_the_second_witness(M, K, N):
     g = torch.Generator(device="cuda").manual_seed(M + N)
     codes_w = torch.randint(0, 256, (N, K // 2), dtype=torch.uint8, device="cuda", generator=g)
     h = fq.weights_import(codes_w, torch.rand(N, device="cuda", generator=g) + 0.1, None, torch.randn(N, device="cuda", generator=g),
                           K, 64, 4)
-    codes = torch.randint(-7, 8, (M, K), dtype=torch.int8, device="cuda", generator=g)
+    codes = torch.randint(0, 256, (M, K // 2), dtype=torch.uint8, device="cuda", generator=g)
     delta = torch.rand(M, device="cuda", generator=g) + 0.1
     for dt in (torch.float32, torch.bfloat16):
         assert torch.equal(fq.gemm_w4a4(codes, delta, h, dt), fq.gemm_simt(codes, delta, h, dt))
     assert torch.equal(fq.gemm_acc_i32(codes, h), fq.gemm_simt(codes, None, h, raw_acc=True))
 
 
-@pytest.mark.parametrize("M,K,block,bits", [
+FEW_UNITS = [
     (9, 1536, 256, 8),         # six units of K for clusters of eight
     (31, 1792, 256, 4),        # seven
     (33, 384, 64, 4),          # three for clusters of four
     (64, 896, 128, 8),
-])
+]
+
+
+@pytest.mark.parametrize("M,K,block,bits", FEW_UNITS)
 def test_one_launch_with_fewer_units_than_cluster_ctas(M, K, block, bits):
     """CTAs without channels add nothing, whatever the launch ahead left in tensor memory."""
     g = torch.Generator(device="cuda").manual_seed(K)
@@ -215,7 +273,7 @@ def test_one_launch_with_fewer_units_than_cluster_ctas(M, K, block, bits):
         assert torch.equal(fq.linear(x, h), want)
 
 
-@pytest.mark.parametrize("M,K,block,bits,dtype,form", [
+PROLOGUE = [
     (607, 2048, 128, 8, "bf16", "smooth"),             # 148 SMs: the longest batch of the register kernel
     (608, 2048, 128, 8, "bf16", "smooth"),             # ... and the shortest streamed one
     (1052, 2112, 64, 4, "bf16", "plain"),              # one lane of the row's last warp has channels
@@ -227,7 +285,10 @@ def test_one_launch_with_fewer_units_than_cluster_ctas(M, K, block, bits):
     (145, 8192, 32, 4, "f32", "plain"),
     (868, 2560, 64, 8, "f32", "plain"),                # 64 channels per thread
     (538, 4128, 32, 8, "f32", "plain"),
-])
+]
+
+
+@pytest.mark.parametrize("M,K,block,bits,dtype,form", PROLOGUE)
 def test_streamed_prologue_on_both_sides_of_its_rule(M, K, block, bits, dtype, form):
     """Eight rows against the oracle, all of them against short batches, which never stream; codes as a caller sees them
     (packed or int8) and, through a small layer, as the GEMM reads them."""
@@ -262,7 +323,7 @@ def test_linear_gated_refuses_what_is_no_gate(act):
     assert e.value.status == fq.ERR_INVALID_ARG
 
 
-@pytest.mark.parametrize("M,K,bits,call", [
+TO_AND_FRO = [
     (50, 1024, 4, "linear"),           # one launch a call
     (64, 1024, 8, "linear"),
     (5, 768, 4, "linear"),
@@ -270,7 +331,10 @@ def test_linear_gated_refuses_what_is_no_gate(act):
     (12, 4096, 8, "linear"),           # prologue and weight streaming
     (300, 1024, 4, "linear"),
     (2, 1536, 4, "linear_w4a16"),
-])
+]
+
+
+@pytest.mark.parametrize("M,K,bits,call", TO_AND_FRO)
 def test_calls_that_pass_two_buffers_to_and_fro(M, K, bits, call):
     """A -> B, B -> A, A -> B ...: kernels of three calls are resident at a time, and the third reads what the second wrote over the
     first one's input.  As a graph and eagerly, against the same calls with a synchronisation behind each."""

@@ -370,9 +370,10 @@ def test_accumulator_extremes_and_one_hot(bits):
 
 @pytest.mark.parametrize("M,N,K,bits", [(100, 256, 16384, 4), (208, 384, 16384, 8), (130, 128, 16384, 4), (64, 256, 16384, 8)])
 def test_k_split_equals_unsplit_and_oracle(M, N, K, bits):
-    """Few tiles and a long K: the planner splits K over a CTA cluster when the workspace has room
-    for the partial sums.  With a workspace that holds only the activation codes and steps the same
-    call runs unsplit; both must give the oracle's integer sums exactly."""
+    """Few tiles and a long K: the planner splits K.  On a device that holds the clusters the slices of a tile meet in their
+    shared memory whatever the workspace (both calls below); the scratch that the workspace is asked to hold is for devices
+    that do not (the split through it: test_scratch_split_equals_the_second_witness, at sizes that take it anywhere).  The
+    oracle's integer sums exactly."""
     rng = np.random.default_rng(M + N + K + bits)
     a, w = random_codes(rng, M, K, bits), random_codes(rng, N, K, bits)
     want = oracle.gemm_i32(a, w, K, bits)
@@ -766,7 +767,7 @@ def test_one_handle_three_streams_three_workspaces():
     """A weight handle is read-only at run time: consumers of one handle on three streams, each with its own
     workspace (K split included), give what the same calls give one after the other."""
     rng = np.random.default_rng(12)
-    M, K, N = 100, 16384, 256                   # few tiles, long K: the planner splits K when scratch is there
+    M, K, N = 100, 16384, 256                   # few tiles, long K: the planner splits K (by clusters; through scratch: test_gpu_edges.py)
     W = synth.draw_weights(rng, N, K)
     h = fq.fold_weights(to_dev(W), None, None, 128, 4)
     need = fq.workspace_bytes(M, K, N, 4)

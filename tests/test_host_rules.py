@@ -5,6 +5,8 @@ import subprocess
 
 import pytest
 
+import test_gpu_edges as edges
+
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2609_24433_b200", "csrc")
 
 
@@ -61,42 +63,138 @@ def test_shared_memory_opt_in_from_several_threads(tmp_path, threads, refuse):
 PLANS = """
 #include "plan.h"
 struct Held { int c2, c4, c8; int operator()(int ctas) const { return ctas == 2 ? c2 : (ctas == 4 ? c4 : c8); } };
-// -> CTAs per cluster, 0: two launches
-extern "C" int fused(long M, long N, long K, int block, int bits, int mult, int sms, int c2, int c4, int c8) {
+// -> 100 * rounds + CTAs per cluster, 0: two launches
+extern "C" int fused(long M, long N, long K, int block, int bits, int mult, int sms, int c2, int c4, int c8, int* grid) {
     const fq::FusedPlan f = fq::plan_fused(M, N, K, block, bits, mult != 0, sms, Held{c2, c4, c8});
-    return f.lanes ? 1 << f.ctas_shift : 0;
+    *grid = f.grid;
+    return f.lanes ? 100 * f.rounds + (1 << f.ctas_shift) : 0;
 }
 // -> 100 * tokens per cluster + CTAs per cluster, 0: two launches
-extern "C" int composite(long M, long K, int elem, int beta, int sms, int c2, int c4, int c8) {
+extern "C" int composite(long M, long K, int elem, int beta, int sms, int c2, int c4, int c8, int* grid) {
     const fq::CompositePlan f = fq::plan_composite(M, K, elem, beta, sms, Held{c2, c4, c8});
+    *grid = (int)f.grid;
     return f.tok ? 100 * f.tok + (1 << f.ctas_shift) : 0;
+}
+// -> channels per thread of the streamed prologue, 0: the register kernel
+extern "C" int ring(long M, long K, int elem, int gated, int bytes_out, int mult, int after, int block, int sms) {
+    return fq::plan_ring(M, K, elem, gated, bytes_out, mult, after, block, sms).e;
+}
+// scratch < 0: as much as the plan without clusters asks for
+extern "C" void gemm(long M, long N, long K, int bits, long scratch, int sms, int c2, int c4, int c8, int* out) {
+    const Held held{c2, c4, c8};
+    const size_t asks = fq::plan_gemm(M, N, K, bits, sms, (size_t)-1, false, held).scratch;
+    const fq::GemmPlan f = fq::plan_gemm(M, N, K, bits, sms, scratch < 0 ? asks : (size_t)scratch, true, held);
+    const fq::GemmRings r = fq::gemm_rings(f, bits, K);
+    const int v[] = {fq::plan_stream(M, N, K, bits, sms), f.bt, f.ctas, f.split, f.cluster, f.scratch > 0, r.fits, r.atoms, r.stages,
+                     r.stages_p, r.stages_w, r.slot_first, (int)r.smem, r.tmem_cols};
+    for (int i = 0; i < 14; ++i) out[i] = v[i];
 }
 """
 B200 = (148, 74, 36, 14)       # multiprocessors, clusters of 2, 4 and 8 CTAs that a whole device holds
+GEMM = "stream bt ctas split cluster scratch fits atoms stages stages_p stages_w slot_first smem tmem_cols".split()
+
+
+class Plans:
+    def __init__(self, lib):
+        self.lib, self.grid = lib, 0
+
+    def fused(self, M, K, N, block, bits, mult=False, device=B200):
+        grid = ctypes.c_int()
+        r = self.lib.fused(ctypes.c_long(M), ctypes.c_long(N), ctypes.c_long(K), block, bits, int(mult), *device, ctypes.byref(grid))
+        self.grid = grid.value
+        return r
+
+    def composite(self, M, K, dtype, beta, device=B200):
+        grid = ctypes.c_int()
+        r = self.lib.composite(ctypes.c_long(M), ctypes.c_long(K), 2 if dtype == "bf16" else 4, beta, *device, ctypes.byref(grid))
+        self.grid = grid.value
+        return r
+
+    def ring(self, M, K, dtype, block, bytes_out, form="plain", gated=False):
+        return self.lib.ring(ctypes.c_long(M), ctypes.c_long(K), 2 if dtype == "bf16" else 4, int(gated), int(bytes_out),
+                             int(form != "plain"), int(form == "after"), block, B200[0])
+
+    def gemm(self, M, K, N, bits, scratch=-1, device=B200):
+        out = (ctypes.c_int * len(GEMM))()
+        self.lib.gemm(ctypes.c_long(M), ctypes.c_long(N), ctypes.c_long(K), bits, ctypes.c_long(scratch), *device, out)
+        return dict(zip(GEMM, out))
 
 
 @pytest.fixture(scope="module")
 def plans(tmp_path_factory):
-    return compile_host(tmp_path_factory.mktemp("plans"), "plans", PLANS)
+    return Plans(compile_host(tmp_path_factory.mktemp("plans"), "plans", PLANS))
 
 
 def test_one_launch_paths_need_clusters_that_can_be_placed(plans):
-    def fused(M, N, K, block, bits, device=B200):
-        return plans.fused(M, N, K, block, bits, 0, *device)
+    assert plans.fused(50, 1024, 1024, 64, 4) == 108 and plans.fused(20, 1024, 1024, 64, 8) == 104
+    assert plans.fused(20, 512, 1024, 64, 8) == 102 and plans.fused(8, 256, 64, 64, 4) == 101
+    part, none = (16, 8, 0, 0), (16, 0, 0, 0)          # parts of a device: pairs only, and no clusters at all
+    assert plans.fused(50, 1024, 128, 64, 4, device=part) == 0 and plans.fused(20, 1024, 128, 64, 8, device=part) == 0
+    assert plans.fused(20, 512, 128, 64, 8, device=part) == 102 and plans.fused(8, 256, 64, 64, 4, device=none) == 101
 
-    assert fused(50, 1024, 1024, 64, 4) == 8 and fused(20, 1024, 1024, 64, 8) == 4 and fused(20, 1024, 512, 64, 8) == 2
-    assert fused(8, 64, 256, 64, 4) == 1
-    part = (16, 8, 0, 0)       # a part of a device: pairs only
-    assert fused(50, 128, 1024, 64, 4, part) == 0 and fused(20, 128, 1024, 64, 8, part) == 0
-    assert fused(20, 128, 512, 64, 8, part) == 2 and fused(8, 64, 256, 64, 4, (16, 0, 0, 0)) == 1
+    assert plans.composite(816, 2048, "bf16", 64) == 1602 and plans.composite(16, 2048, "bf16", 64) == 1608
+    assert plans.composite(20, 4096, "f32", 128) == 808
+    for device in (part, none):
+        for M, K, dtype, beta in [(816, 2048, "bf16", 64), (16, 2048, "bf16", 64), (20, 4096, "f32", 128), (17, 512, "f32", 16)]:
+            assert plans.composite(M, K, dtype, beta, device) % 100 <= (2 if device[1] else 1), (M, K, dtype, beta, device)
+    assert plans.composite(20, 4096, "f32", 128, none) == 0      # fits in clusters only: two launches
+    for M, K, N, bits in edges.CLUSTER_SPLIT + edges.SCRATCH_SPLIT:
+        p = plans.gemm(M, K, N, bits, scratch=0, device=none)
+        assert p["fits"] and p["ctas"] == 1 and p["split"] == 1
 
-    def composite(M, K, elem, beta, device=B200):
-        return plans.composite(M, K, elem, beta, *device)
 
-    assert composite(816, 2048, 2, 64) == 1602 and composite(576, 2048, 2, 64) == 1604 and composite(16, 2048, 2, 64) == 1608
-    assert composite(20, 4096, 4, 128) == 808                                    # binary32 rows: eight tokens, eight CTAs
-    for device in (part, (16, 0, 0, 0)):
-        for M, K, elem, beta in [(816, 2048, 2, 64), (16, 2048, 2, 64), (20, 4096, 4, 128), (17, 512, 4, 16), (9, 8192, 4, 64)]:
-            tok, ctas = divmod(composite(M, K, elem, beta, device), 100)
-            assert ctas <= (2 if device[1] else 1), (M, K, elem, beta, device)
-    assert composite(20, 4096, 4, 128, (16, 0, 0, 0)) == 0                       # fits in clusters only: two launches
+def test_sizes_of_the_device_tests_take_the_routes_they_stand_for(plans):
+    for M, K, N, block, bits, _, smooth, _ in edges.ONE_LAUNCH:
+        assert plans.fused(M, K, N, block, bits, smooth), (M, K, N)
+        assert plans.grid <= B200[0]
+    assert [plans.fused(*c[:5]) for c in edges.ONE_LAUNCH if c[1] > 1700] == [208, 208, 208, 208]       # two rounds
+    assert not plans.fused(8, 1024, 3080, 64, 4) and not plans.fused(50, 1024, 2312, 64, 4) and not plans.fused(63, 512, 4744, 64, 8)
+    assert not plans.fused(33, 2176, 128, 64, 4) and not plans.fused(32, 4224, 128, 64, 4) and not plans.fused(65, 1024, 128, 64, 4)
+    for M, K, block, bits in edges.FEW_UNITS:
+        ctas = plans.fused(M, K, 200, block, bits) % 100
+        assert K // max(block, 128) < ctas, (M, K)
+    for M, K, bits, call in edges.TO_AND_FRO[:3]:
+        assert plans.fused(M, K, K, 64, bits)
+    assert not plans.gemm(24, 4096, 4096, 4)["stream"] and not plans.fused(24, 4096, 4096, 64, 4) and plans.gemm(12, 4096, 4096, 8)["stream"]
+
+    for M, K, N in edges.ODD_RINGS:
+        p = plans.gemm(M, K, N, 4)
+        assert p["fits"] and p["slot_first"] and p["stages_p"] % 2 == 1 and not p["stream"], (M, K, N, p)
+    rings = [(p["stages_p"], p["stages_w"], p["split"]) for p in (plans.gemm(*c, 4) for c in edges.ODD_RINGS)]
+    assert rings == [(3, 3, 1), (5, 5, 1), (5, 4, 1), (5, 4, 4)]
+    for M, K, N, bits in edges.CLUSTER_SPLIT:
+        p = plans.gemm(M, K, N, bits, scratch=0)
+        assert p["fits"] and p["cluster"] and p["split"] > 1 and not p["stream"], (M, K, N, bits, p)
+        assert plans.gemm(M, K, N, bits)["cluster"]
+    for M, K, N, bits in edges.SCRATCH_SPLIT:
+        p = plans.gemm(M, K, N, bits)
+        assert p["fits"] and p["scratch"] and p["split"] > 1 and not p["cluster"] and not p["stream"], (M, K, N, bits, p)
+        assert not plans.gemm(M, K, N, bits, scratch=0)["scratch"]
+    assert plans.gemm(*edges.SCRATCH_SPLIT[-1])["ctas"] == 2
+    assert all(plans.gemm(*c, 4)["ctas"] == 2 for c in edges.W4_PAIRS) and all(plans.gemm(*c, 4)["ctas"] == 1 for c in edges.W4_SINGLE)
+
+    for M, K, beta, _, dtype, _, lead in edges.COMPOSITE:
+        assert (plans.composite(M, K, dtype, beta) == 0) == (K == 8192), (M, K, beta)
+    assert plans.composite(700, 1024, "bf16", 32) and plans.grid > B200[0]
+    assert plans.composite(576, 2048, "bf16", 64) == 1604 and plans.grid == 4 * B200[2] and plans.composite(577, 2048, "bf16", 64) == 1602
+    assert [bool(plans.ring(M, K, "bf16", block, bits == 8, gated=True)) for M, K, block, bits, _ in edges.GATED] == [True, False, True]
+    for M, K, block, bits, dtype, form in edges.PROLOGUE:
+        e = plans.ring(M, K, dtype, block, bits == 8, form)
+        assert bool(e) == (M != 607) and all(plans.ring(40, K, dtype, block, b, form) == 0 for b in (False, True)), (M, K, e)
+        assert plans.ring(M, K, dtype, block, True, form) == e                  # the one-call route writes a byte per code
+
+
+def test_rings_of_every_plan_fit(plans):
+    """Shared and tensor memory within the SM's, a ring that the unpack sets cannot misread, and room left for no second CTA of
+    the short-batch kernel (77 KB) beside a cluster."""
+    for bits in (4, 8):
+        for K in (32, 128, 160, 2048, 4096, 8192, 8256, 16384, 32768):
+            for M in (1, 16, 17, 50, 64, 65, 112, 128, 129, 208, 256, 300, 816, 1000, 4096, 20000):
+                for N in (8, 128, 136, 1024, 2048, 4104, 8192, 16384):
+                    for scratch in (0, -1):
+                        p = plans.gemm(M, K, N, bits, scratch)
+                        assert p["fits"] and p["smem"] <= 227 * 1024 and p["tmem_cols"] <= 512, (M, K, N, bits, p)
+                        assert p["smem"] + 77 * 1024 > 228 * 1024 - 2048, (M, K, N, bits, p)
+                        if bits == 4:
+                            assert p["stages_w"] <= p["stages"] and p["stages_w"] >= 2 and p["stages_p"] >= 2
+                            assert p["stages_p"] % 2 == 0 or p["stages_p"] >= p["stages_w"] + 2 or p["slot_first"]
