@@ -161,24 +161,37 @@ inline RingPlan plan_ring(int64_t rows, int64_t K, int elem_bytes, bool gated, b
     };
     const bool may64 = !gated && K >= 2048 && K % 64 == 0 && !(after && block >= 128);
     if (!(may64 && fits(64)) && !fits(32)) return RingPlan();
-    // Short batches are latency-bound and go to the register kernel, which spreads a row over more threads.  The line is drawn
-    // by channels per SM, just behind the register kernel's first full wave; it lies higher where a row leaves lanes of its
-    // group idle, most of all with a multiplier, which such lanes' warps still read.  Chains of calls, 8-bit codes, here /
-    // register kernel:
-    //   bf16     K = 1024: M = 1184 2.61 / 2.30 us, 2368 3.15 / 3.23;  K = 2048: M = 592 2.69 / 2.32, 700 2.82 / 3.11, 2368
-    //            4.38 / 5.23;  K = 4096: M = 296 2.62 / 2.36, 370 2.82 / 3.11, 2368 6.78 / 9.30;  K = 8192: M = 148 2.70 /
-    //            2.43, 370 3.62 / 4.00, 2368 11.1 / 18.0;  K = 16384: M = 74 3.14 / 3.52, 816 10.4 / 15.2
-    //   binary32 K = 1024: M = 592 2.33 / 2.16, 1184 2.69 / 3.12;  K = 4096: M = 148 2.29 / 2.13, 592 3.73 / 5.00, 4736 17.8 /
-    //            22.3;  K = 8192: M = 592 5.8 / 7.6, 4736 34.4 / 46.2
-    //   ragged   K = 2560: M = 816 3.51 / 3.27, 1184 4.15 / 4.73, 2368 6.34 / 6.77;  K = 6144: M = 296 3.15 / 2.71, 370 3.38 /
-    //            4.00;  K = 11008: M = 148 3.26 / 2.98, 220 3.96 / 4.47
-    //   ... with a multiplier   K = 2560: M = 2368 8.9 / 8.3, 4736 15.9 / 14.3;  K = 5120: M = 1184 8.8 / 8.6, 2368 15.4 / 14.0,
-    //            4736 25.6 / 25.7;  K = 3072 (three quarters of the lanes): M = 816 4.6 / 5.0, 4736 15.4 / 16.2
+    // Short batches are latency-bound and go to the register kernel, which spreads a row over more threads and leaves its SMs'
+    // shared memory to the GEMM behind it, whose CTAs set up and fetch weights beside it.  The line is drawn by what whole
+    // calls take, in channels per SM; it lies higher where a row leaves lanes of its group idle (with a multiplier such lanes'
+    // warps still read it).  Streamed minus register, us per fq_linear call (N = 2048, 8 bits; rows and channels, in brackets
+    // thousands of channels per SM), in a chain of calls / each behind a kernel that triggers nothing, where the streamed
+    // kernel's longer start does not hide:
+    //   bf16, all lanes  816 x 2048 (11) +0.43 / +1.28;  1156 x 2048 (16) +0.71 / +0.84, with a multiplier +0.35 / +0.40;  1300 x
+    //                    2048 (18) -0.69 / +0.60, -0.49 / +0.13;  614 x 4096 (17) +0.54 / +0.62;  758 x 4096 (21) -0.46 / +0.48,
+    //                    -0.36 / +0.25;  307 x 8192 (17) +0.12 / +0.46;  379 x 8192 (21) -1.01 / +0.19;  975 x 4096 (27) -0.73 /
+    //                    -0.59;  1638 x 1536 (17) +0.76 / +1.56;  1734 x 1536 (18) -0.05 / +1.19;  81 x 16384 (9) -0.43 / -0.18,
+    //                    with a multiplier -0.49 / -1.29
+    //   seven eighths    825 x 3584 (20) -0.05 / +0.97;  1238 x 3584 (30) -0.41 / +0.21, 619 x 7168 (30) -1.60 / 0.00
+    //   three quarters   1445 x 3072 (30) +0.57 / +0.70;  1927 x 3072 (40) -0.27 / +0.50;  2890 x 3072 (60) -0.57 / -0.04, with a
+    //                    multiplier -0.02 / -0.34;  963 x 6144 (40) -0.88 / -0.08, with one -0.75 / +0.09
+    //   less             1734 x 2560 (30) +1.25 / +1.24;  3468 x 2560 (60) +0.50 / +0.40;  4625 x 2560 (80) -0.84 / -0.34;  with a
+    //                    multiplier 6359 x 2560 (110) +1.23 / -0.17, 9250 x 2560 (160) -0.66 / -1.81, 3179 x 5120 (110) +0.07 / +0.03
+    //   ... past 8192    201 x 11008 (15) -0.22 / -0.02, with a multiplier -0.28 / -0.62;  1170 x 10240 with one -2.10 / -2.05
+    //   binary32         614 x 2048 (8.5) -0.29 / +0.32, with a multiplier -0.32 / -0.08;  153 x 8192 -0.70 / -0.45;  1156 x 1536
+    //                    (12) +0.22 / +0.68 (4 bits);  2167 x 1024 (15) -0.98 / +0.32;  1445 x 1536 (15) -0.33 / +0.91;  770 x 3072
+    //                    (16) -0.85 / +0.81;  with a multiplier 3121 x 2560 (54) -0.02 / +0.18, 4682 x 2560 (81) -0.95 / -1.06
+    // (Prologues alone in a chain of themselves, by which the line was drawn once, have the streamed one ahead from 9 on:
+    // 816 x 2048 3.28 / 3.46 us; behind a kernel that triggers nothing it is 3.97 / 3.46.)
     if (!gated) {
-        const int64_t width = (int64_t)f.gw * 32 * f.e;
-        int64_t line = 15000;
-        if (width == K || K < 2048) line = elem_bytes == 4 || K >= 16384 ? 8000 : 8400;
-        else if (mult && 4 * K < 3 * width) line = 100000;
+        const int64_t width = (int64_t)f.gw * 32 * f.e;          // channels that the group's lanes could hold
+        int64_t line;
+        if (elem_bytes == 4) line = K < 2048 ? 13000 : (width == K ? 8000 : (mult && 4 * K < 3 * width ? 60000 : 15000));
+        else if (K > 8192) line = width == K ? 8000 : 15000;
+        else if (width == K || K < 2048) line = 18000;
+        else if (8 * K >= 7 * width) line = 27000;
+        else if (4 * K >= 3 * width) line = 45000;
+        else line = mult ? 130000 : 80000;
         if (rows * K < line * sms) return RingPlan();
     }
     return f;

@@ -274,16 +274,21 @@ def test_one_launch_with_fewer_units_than_cluster_ctas(M, K, block, bits):
 
 
 PROLOGUE = [
-    (607, 2048, 128, 8, "bf16", "smooth"),             # 148 SMs: the longest batch of the register kernel
-    (608, 2048, 128, 8, "bf16", "smooth"),             # ... and the shortest streamed one
-    (1052, 2112, 64, 4, "bf16", "plain"),              # one lane of the row's last warp has channels
+    (1300, 2048, 128, 8, "bf16", "smooth"),            # 148 SMs: the longest batch of the register kernel
+    (1301, 2048, 128, 8, "bf16", "smooth"),            # ... and the shortest streamed one
+    (5607, 2112, 64, 4, "bf16", "plain"),              # one lane of the row's last warp has channels
     (269, 8256, 32, 8, "bf16", "plain"),               # warps without any
     (73, 16384, 256, 4, "bf16", "plain"),              # the longest rows, fewer than SMs
-    (304, 4096, 128, 8, "bf16", "after"),              # 32 channels per thread
-    (810, 1536, 256, 4, "bf16", "smooth"),
-    (1157, 1024, 64, 8, "f32", "smooth"),
+    (651, 4096, 128, 8, "bf16", "after"),              # 32 channels per thread
+    (1735, 1536, 256, 4, "bf16", "smooth"),
+    (558, 7168, 64, 4, "bf16", "plain"),               # seven eighths of the lanes
+    (2168, 3072, 128, 8, "bf16", "smooth"),            # three quarters
+    (7516, 2560, 128, 4, "bf16", "smooth"),            # less
+    (217, 10240, 128, 8, "bf16", "smooth"),            # ... behind 8192 channels
+    (1879, 1024, 64, 8, "f32", "smooth"),
     (145, 8192, 32, 4, "f32", "plain"),
     (868, 2560, 64, 8, "f32", "plain"),                # 64 channels per thread
+    (3469, 2560, 128, 4, "f32", "smooth"),
     (538, 4128, 32, 8, "f32", "plain"),
 ]
 
@@ -423,23 +428,26 @@ def test_other_python_threads_run_while_a_launch_waits(call):
            "quantize_act_composite": lambda: fq.quantize_act_composite(x, None, perm, blocks, 4, codes=codes, delta=delta, workspace=ws)}[call]
     run()
     torch.cuda.synchronize()
-    done, ticks = threading.Event(), []
+    for _ in range(5):                                    # (again where the host was held up until the stream was idle)
+        done, ticks = threading.Event(), []
 
-    def count():
-        while not done.wait(0.002):
-            ticks.append(time.perf_counter())
+        def count():
+            while not done.wait(0.002):
+                ticks.append(time.perf_counter())
 
-    torch.cuda._sleep(int(0.8 * 1.9e9))                   # the stream is busy for 0.8 s or a little more
-    thread = threading.Thread(target=count)
-    thread.start()
-    longest, start = 0.0, time.perf_counter()
-    for _ in range(4000):
-        t = time.perf_counter()
-        run()
-        longest = max(longest, time.perf_counter() - t)
-    done.set()
-    thread.join()
-    gaps = np.diff([start] + ticks)
-    torch.cuda.synchronize()
+        torch.cuda._sleep(int(0.8 * 1.9e9))               # the stream is busy for 0.8 s or a little more
+        thread = threading.Thread(target=count)
+        thread.start()
+        longest, start = 0.0, time.perf_counter()
+        while longest < 0.2 and time.perf_counter() < start + 0.6:
+            t = time.perf_counter()
+            run()
+            longest = max(longest, time.perf_counter() - t)
+        done.set()
+        thread.join()
+        gaps = np.diff([start] + ticks)
+        torch.cuda.synchronize()
+        if longest > 0.2:
+            break
     assert longest > 0.2, f"no launch had to wait ({longest:.3f} s): nothing was tested"
     assert gaps.max() < 0.5 * longest, f"a launch waited {longest:.3f} s, the other thread stood still for {gaps.max():.3f} s"

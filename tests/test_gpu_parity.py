@@ -737,7 +737,7 @@ def test_sweep_corners_sampled_rows(M, KN, block, bits):
 @pytest.mark.parametrize("clip", [1.0, 0.7])
 @pytest.mark.parametrize("M,K,block,bits,dtype", [
     (64, 2048, 128, 4, "bf16"), (816, 2048, 128, 4, "f32"),            # register kernel
-    (1184, 2048, 128, 4, "bf16"), (1500, 4096, 64, 4, "f32"),          # streaming kernel, 8 rows per SM and more
+    (1184, 2048, 128, 4, "bf16"), (1500, 4096, 64, 4, "f32"),          # the register kernel at its fullest; the streaming kernel
     (296, 8192, 256, 4, "bf16"), (400, 16384, 256, 8, "bf16"),         # streaming kernel on long rows
     (2000, 1024, 32, 8, "bf16"),
 ])

@@ -180,8 +180,13 @@ def test_sizes_of_the_device_tests_take_the_routes_they_stand_for(plans):
     assert [bool(plans.ring(M, K, "bf16", block, bits == 8, gated=True)) for M, K, block, bits, _ in edges.GATED] == [True, False, True]
     for M, K, block, bits, dtype, form in edges.PROLOGUE:
         e = plans.ring(M, K, dtype, block, bits == 8, form)
-        assert bool(e) == (M != 607) and all(plans.ring(40, K, dtype, block, b, form) == 0 for b in (False, True)), (M, K, e)
+        assert bool(e) == (M != 1300) and all(plans.ring(40, K, dtype, block, b, form) == 0 for b in (False, True)), (M, K, e)
         assert plans.ring(M, K, dtype, block, True, form) == e                  # the one-call route writes a byte per code
+        assert M == 1300 or plans.ring(M - 1, K, dtype, block, True, form) == 0
+    # prologues that are shorter in a call of their own and longer in front of a GEMM stay in the register kernel
+    assert not any(plans.ring(M, K, "bf16", 128, True, form) for M, K in ((700, 2048), (816, 2048), (1156, 2048), (320, 4096), (160, 8192))
+                   for form in ("plain", "smooth"))
+    assert plans.ring(1170, 10240, "bf16", 128, True, "smooth")
 
 
 def test_rings_of_every_plan_fit(plans):
