@@ -134,7 +134,8 @@ fq_status fq_weights_import_after(const void* codes, const float* w_scale, const
  * Channels are rounded in index order; each rounding error (w - q s)/U_ii is spread over the channels still to
  * come along row i of the upper Cholesky factor U of (G + lambda I)^-1.  All of it runs in binary32 in a fixed
  * order, so the codes are reproducible bit for bit.  K <= 16384 (FQ_ERR_UNSUPPORTED beyond; the factorisation is
- * column-sequential and cubic in K: 10 ms at K = 2048, seconds beyond K = 8192); FQ_ERR_INVALID_ARG if
+ * column-sequential and cubic in K: at K = 2048 the kernels take 9 ms and the call 10 to 31, by what its allocations cost on
+ * the host; seconds beyond K = 8192); FQ_ERR_INVALID_ARG if
  * the damped second moment is not positive definite in binary32, FQ_ERR_TIMEOUT if a bounded wait of the
  * factorisation expired (no handle is made).  Offline: allocates (about 3 K^2 + (N + Mc) K
  * floats of temporaries) and synchronises the stream. */
@@ -279,8 +280,9 @@ fq_status fq_linear_w4a4_static(const void* x, fq_dtype xt, int64_t M, int64_t l
 
 /* Bytes of workspace that fq_gemm_* / fq_linear_* want for this shape (host computation): the int8
  * activation codes and steps (M*K + 4*M bytes, each rounded up to 256), plus scratch for int32 partial
- * tiles on shapes with few output tiles and a long K, where a device that cannot hold the clusters that
- * otherwise share such a tile splits K through memory.  A workspace that holds only the first part is accepted.  Everything a call
+ * tiles on shapes with few output tiles and a long K.  The scratch is used where the device cannot hold the
+ * clusters that otherwise share such a tile (the figure does not depend on the device, so that a caller sizes
+ * its workspace once).  A workspace that holds only the first part is accepted.  Everything a call
  * scribbles on lives in the workspace it was given (the split's tile counters included, cleared by a
  * memset node at the head of the call): a weight handle is read-only at run time, so calls on the same
  * handle may run concurrently on different streams as long as each has its own workspace. */

@@ -235,6 +235,9 @@ fq_status linear_impl(const void* x, fq_dtype xt, int64_t M, int64_t ldx, const 
     // Rows of more than 4096 channels: the GEMM gains from an early start where it has many 8-bit weights to fetch (eager
     // calls, early / not: 64 x 8192 x 8192 18.1 / 18.6 us, 16 x 8192 x 8192 16.3 / 17.2, 16 x 6144 x 2048 9.1 / 8.75) or many
     // four-atom stages to unpack (4 bits: 32 x 8192 x 4096 10.6 / 11.5, 50 x 6144 x 2048 9.9 / 10.6; 16 x 8192 x 8192 14.15 / 13.8).
+    // Replayed graphs over rotating weights, K = 4608, 5120, 6144 and 8192, N = 1024 to 12288, M = 1 to 64, early minus not: where the flag
+    // is set never slower in a chain (-2.3 to -0.01 us, median -1.0; 224 points) nor behind a torch kernel (median -0.13, one point of
+    // 224 at +1.0); where it is not, -2.4 to +0.5 in a chain (slower at N <= 2048, up to 0.5; faster from N = 3072 on).
     const int flags = kMultReady | ((bits == 8 ? W->N >= 4096 : M > 16) ? kTriggerEarly : 0);
     const cudaError_t pe =
         gate >= 0 ? launch_gated_transform_quantize(x, xt, M, W->K, ldx, gate, mult, block_norm(W->block), W->fold_after,

@@ -37,8 +37,8 @@ int device_sm_count();                                              // multiproc
 int device_cc_major();                                              // compute-capability major, -1 on error
 cudaError_t ensure_dynamic_smem(const void* kernel, size_t bytes);  // opt a kernel in to `bytes` of dynamic shared memory
 int max_resident_blocks(const void* kernel, int threads);           // thread blocks of a kernel one SM holds (no dynamic smem)
-// Clusters of 2, 4 or 8 CTAs, one CTA per SM, that the device holds at a time (a whole B200: 74, 36, 14 -- its graphics
-// clusters do not divide by eight; 0 where one cannot be placed at all, on a part of a device).
+// Clusters of 2, 4 or 8 CTAs, one CTA per SM, that the device holds at a time.  B200s differ in how their 148 SMs are grouped
+// (74, 36, 14 on one, 74, 33, 15 on another); 0 where one cannot be placed at all, on a part of a device.
 int cluster_capacity(int ctas);
 // The device would not place a cluster launch after all (a context that owns part of it): the caller takes the route without.
 inline bool cluster_refused(cudaError_t e) {
@@ -142,8 +142,8 @@ cudaError_t launch_linear_wonly4(const void* x, fq_dtype xt, int64_t M, int64_t 
                                  fq_dtype yt, int64_t ldy, cudaStream_t stream);
 
 // tcgen05 integer GEMM; a8 = int8 activations [M, K] (pitch K), 16-byte aligned.  `scratch` (device,
-// 256-byte aligned, may be null) holds int32 partial tiles when the launch splits K over a cluster;
-// gemm_scratch_bytes() is what the split the planner would pick for this shape needs.
+// 256-byte aligned, may be null) holds int32 partial tiles when the launch splits K through it (slices that meet in a cluster's
+// shared memory need none); gemm_scratch_bytes() is what the split would need that the planner picks without clusters.
 fq_status launch_gemm_tcgen05(const int8_t* a8, int64_t M, const Weights& W, int acc_shift, const GemmOut& out,
                               void* scratch, size_t scratch_bytes, cudaStream_t stream);
 // The GEMM of the runtime path: the streaming kernel for short batches on 4-bit weights, else the tcgen05 kernel.

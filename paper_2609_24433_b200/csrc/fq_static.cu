@@ -1,13 +1,14 @@
 // fq_linear_w4a4_static: the fused W4A4 linear for callers that must not allocate.
 //
 // fq_linear_w4a4 keeps the quantized activations (one int8 per code) and the
-// per-token steps in a caller-supplied workspace between its two kernels.  Some
+// per-token steps in a caller-supplied workspace.  Some
 // callers have nowhere to get that workspace from: an enqueue callback of an
 // inference-engine plugin may not call cudaMalloc, a robot's control loop cannot
 // afford the device-wide synchronisation an allocation may imply, and a process
 // whose device memory was handed out once at start-up has no allocator to ask.
-// For them the same two kernels run here on a fixed scratch area that lives in
-// the library image itself.
+// For them the same kernels run here -- one launch for the shapes that
+// fq_linear_w4a4 runs in one, else two -- and what sits between two of them
+// lives in a fixed scratch area of the library image itself.
 //
 // The scratch is a file-scope __device__ array.  In host code that name is only
 // a host-side stand-in for the symbol, not an address a kernel may use, so the

@@ -11,8 +11,9 @@
 //   - the int32 partial sums meet in distributed shared memory, every CTA finishing its share of the tokens.
 // The transform is repeated by every cluster, and what is left is a chain of latencies: at M = 50, K = N = 1024, clock marks
 // behind the wait for the kernel ahead count some 600 cycles for the load, 1200 for the butterflies, 1300 for the
-// exchange of maxima, 1000 for the codes, 700 for the MMAs and 1700 for the sums' exchange and the outputs.  So a thread holds
-// no more than sixteen channels (32: 6.8 instead of 5.8 us per call) and slices are as narrow as clusters of eight allow.
+// exchange of maxima, 1000 for the codes, 700 for the MMAs and 1700 for the sums' exchange and the outputs.  So slices are as
+// narrow as clusters of eight allow, and a thread holds sixteen channels (32: 6.8 instead of 5.8 us per call); thirty-two (T = 2
+// rounds) only where rows are too long for that.
 //
 // Arithmetic: that of the prologue and GEMM kernels, operation by operation, so codes, steps, sums and outputs are
 // theirs bit for bit.  Codes and steps also go to the caller's workspace, as the two-kernel path leaves them.
@@ -179,7 +180,7 @@ linear_fused_kernel(const __grid_constant__ CUtensorMap map_w, const FusedParams
     }
     griddep_wait();                                        // the kernel ahead wrote x, and may still read y or the workspace
 
-    // ---- transform: rounds of 256 channels, LG lanes per token
+    // ---- transform: T rounds of kRoundCh channels, LG lanes per token
     const int token = tid / LG, gl = tid % LG;
     const bool tok_ok = token < p.M;
     const bool busy = warp * (32 / LG) < p.M;              // (warp-uniform) some lane of this warp has a token

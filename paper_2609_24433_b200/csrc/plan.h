@@ -277,8 +277,8 @@ inline size_t cluster_sums_bytes(int bt, int split) { return (size_t)(split - 1)
 //   16 x 16384 x 4096 14.7 / 22.6 and 18.8 / 32.3; 64 x 4096 x 1024 8.6 / 9.9 and 8.0 / 11.1; 64 x 4096 x 4096 10.4 / 10.5
 //   and 10.2 / 11.9; 128 x 4096 x 1024 8.7 / 9.2 and 8.7 / 10.8; 256 x 4096 x 1024 10.5 / 10.1 at 4 bits; CTA pairs,
 //   816 x 16384 x 2048: the site 5 us faster than 96-token tiles.
-//   Through scratch, where the device cannot hold the clusters (CTA pairs on 8-bit weights, too): 12500 + 40*bt + 1500 per
-//   extra slice.
+//   Through scratch, where the device cannot hold the clusters, their sums leave too little ring, or 4-bit tiles have more than
+//   128 tokens (CTA pairs on 8-bit weights, too; on a whole B200 rows of 20480 channels and more): 12500 + 40*bt + 1500 per extra slice.
 template <typename Held>
 GemmPlan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t scratch_avail, bool clusters, Held held) {
     const int bt_max = bits == 4 ? 208 : 256;

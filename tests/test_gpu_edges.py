@@ -1,6 +1,6 @@
 """GPU parity at the sizes where a kernel or a dispatch rule can go wrong: edges of tiles, remainders, the smallest
 and the largest of each variant's range.  Same oracle and same bounds as test_gpu_parity.py.  That the sizes in the lists
-below take the routes they stand for, on a whole B200, is checked without a device in test_host_rules.py."""
+below take the routes they stand for, on whole B200s, is checked without a device in test_host_rules.py."""
 import os
 import subprocess
 import sys
@@ -147,7 +147,7 @@ COMPOSITE = [
     (20, 4096, 128, 8, "f32", False, 0),               # binary32 rows of which eight fit
     (9, 8192, 64, 4, "f32", False, 0),                 # ... and none: the two-kernel form
     (20, 4096, 128, 8, "bf16", False, 4),              # rows that are not 16-byte aligned
-    (576, 2048, 64, 4, "bf16", False, 0),              # 148 SMs: the most clusters of four in one wave
+    (576, 2048, 64, 4, "bf16", False, 0),              # a device that holds 36 clusters of four: the most in one wave
     (577, 2048, 64, 4, "bf16", True, 0),               # ... and clusters of two
 ]
 
@@ -169,7 +169,7 @@ def test_composite_prologue_at_the_edges_of_its_kernels(M, K, beta, bits, dtype,
 
 CLUSTER_SPLIT = [
     (64, 16384, 2048, 4),      # clusters of four, four-atom stages
-    (16, 16384, 4608, 8),      # one token chunk: one CTA of four finishes the tile
+    (16, 16384, 4224, 8),      # one token chunk: one CTA of four finishes the tile
     (100, 16384, 256, 4),      # few tiles: clusters of eight, ragged last chunk
     (50, 16384, 1024, 8),
     (90, 8192, 520, 8),        # a ragged channel tile

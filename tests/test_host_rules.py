@@ -90,23 +90,27 @@ extern "C" void gemm(long M, long N, long K, int bits, long scratch, int sms, in
     for (int i = 0; i < 14; ++i) out[i] = v[i];
 }
 """
-B200 = (148, 74, 36, 14)       # multiprocessors, clusters of 2, 4 and 8 CTAs that a whole device holds
+B200 = (148, 74, 36, 14)       # multiprocessors, clusters of 2, 4 and 8 CTAs that one whole device holds
+WHOLE = [B200, (148, 74, 33, 15)]                        # ... and another, whose SMs are grouped otherwise
 GEMM = "stream bt ctas split cluster scratch fits atoms stages stages_p stages_w slot_first smem tmem_cols".split()
 
 
 class Plans:
-    def __init__(self, lib):
-        self.lib, self.grid = lib, 0
+    def __init__(self, lib, device=B200):
+        self.lib, self.device, self.grid = lib, device, 0
 
-    def fused(self, M, K, N, block, bits, mult=False, device=B200):
+    def on(self, device):
+        return Plans(self.lib, device)
+
+    def fused(self, M, K, N, block, bits, mult=False, device=None):
         grid = ctypes.c_int()
-        r = self.lib.fused(ctypes.c_long(M), ctypes.c_long(N), ctypes.c_long(K), block, bits, int(mult), *device, ctypes.byref(grid))
+        r = self.lib.fused(ctypes.c_long(M), ctypes.c_long(N), ctypes.c_long(K), block, bits, int(mult), *(device or self.device), ctypes.byref(grid))
         self.grid = grid.value
         return r
 
-    def composite(self, M, K, dtype, beta, device=B200):
+    def composite(self, M, K, dtype, beta, device=None):
         grid = ctypes.c_int()
-        r = self.lib.composite(ctypes.c_long(M), ctypes.c_long(K), 2 if dtype == "bf16" else 4, beta, *device, ctypes.byref(grid))
+        r = self.lib.composite(ctypes.c_long(M), ctypes.c_long(K), 2 if dtype == "bf16" else 4, beta, *(device or self.device), ctypes.byref(grid))
         self.grid = grid.value
         return r
 
@@ -114,9 +118,9 @@ class Plans:
         return self.lib.ring(ctypes.c_long(M), ctypes.c_long(K), 2 if dtype == "bf16" else 4, int(gated), int(bytes_out),
                              int(form != "plain"), int(form == "after"), block, B200[0])
 
-    def gemm(self, M, K, N, bits, scratch=-1, device=B200):
+    def gemm(self, M, K, N, bits, scratch=-1, device=None):
         out = (ctypes.c_int * len(GEMM))()
-        self.lib.gemm(ctypes.c_long(M), ctypes.c_long(N), ctypes.c_long(K), bits, ctypes.c_long(scratch), *device, out)
+        self.lib.gemm(ctypes.c_long(M), ctypes.c_long(N), ctypes.c_long(K), bits, ctypes.c_long(scratch), *(device or self.device), out)
         return dict(zip(GEMM, out))
 
 
@@ -143,7 +147,9 @@ def test_one_launch_paths_need_clusters_that_can_be_placed(plans):
         assert p["fits"] and p["ctas"] == 1 and p["split"] == 1
 
 
-def test_sizes_of_the_device_tests_take_the_routes_they_stand_for(plans):
+@pytest.mark.parametrize("device", WHOLE)
+def test_sizes_of_the_device_tests_take_the_routes_they_stand_for(plans, device):
+    plans = plans.on(device)
     for M, K, N, block, bits, _, smooth, _ in edges.ONE_LAUNCH:
         assert plans.fused(M, K, N, block, bits, smooth), (M, K, N)
         assert plans.grid <= B200[0]
@@ -176,7 +182,8 @@ def test_sizes_of_the_device_tests_take_the_routes_they_stand_for(plans):
     for M, K, beta, _, dtype, _, lead in edges.COMPOSITE:
         assert (plans.composite(M, K, dtype, beta) == 0) == (K == 8192), (M, K, beta)
     assert plans.composite(700, 1024, "bf16", 32) and plans.grid > B200[0]
-    assert plans.composite(576, 2048, "bf16", 64) == 1604 and plans.grid == 4 * B200[2] and plans.composite(577, 2048, "bf16", 64) == 1602
+    assert plans.composite(16 * device[2], 2048, "bf16", 64) == 1604 and plans.grid == 4 * device[2]
+    assert plans.composite(16 * device[2] + 1, 2048, "bf16", 64) == 1602
     assert [bool(plans.ring(M, K, "bf16", block, bits == 8, gated=True)) for M, K, block, bits, _ in edges.GATED] == [True, False, True]
     for M, K, block, bits, dtype, form in edges.PROLOGUE:
         e = plans.ring(M, K, dtype, block, bits == 8, form)
@@ -189,7 +196,8 @@ def test_sizes_of_the_device_tests_take_the_routes_they_stand_for(plans):
     assert plans.ring(1170, 10240, "bf16", 128, True, "smooth")
 
 
-def test_rings_of_every_plan_fit(plans):
+@pytest.mark.parametrize("device", WHOLE + [(16, 8, 0, 0)])
+def test_rings_of_every_plan_fit(plans, device):
     """Shared and tensor memory within the SM's, a ring that the unpack sets cannot misread, and room left for no second CTA of
     the short-batch kernel (77 KB) beside a cluster."""
     for bits in (4, 8):
@@ -197,7 +205,7 @@ def test_rings_of_every_plan_fit(plans):
             for M in (1, 16, 17, 50, 64, 65, 112, 128, 129, 208, 256, 300, 816, 1000, 4096, 20000):
                 for N in (8, 128, 136, 1024, 2048, 4104, 8192, 16384):
                     for scratch in (0, -1):
-                        p = plans.gemm(M, K, N, bits, scratch)
+                        p = plans.gemm(M, K, N, bits, scratch, device)
                         assert p["fits"] and p["smem"] <= 227 * 1024 and p["tmem_cols"] <= 512, (M, K, N, bits, p)
                         assert p["smem"] + 77 * 1024 > 228 * 1024 - 2048, (M, K, N, bits, p)
                         if bits == 4:
