@@ -30,12 +30,25 @@ struct FusedPlan {
     size_t smem = 0;
 };
 
-// At most 64 tokens, in one wave of CTAs.  In a chain of calls (graph replays, weights from memory; one launch against two):
-// 1024 x 1024: M = 8 3.8 / 4.2 us, M = 32 5.0 / 6.0, M = 50 5.8 / 6.8; K = 2048, N = 1024: M = 32 5.3 / 7.1, M = 50 6.7 / 8.1;
-// K = 4096, N = 1024: M = 16 5.4 / 6.3, M = 32 6.4 / 9.0; the largest grids are even (1024 x 4096: M = 32 6.1 / 6.2), and
-// behind with few tokens (8 bits, M = 1 4.5 / 4.0): 96 CTAs at most there.  An eager call costs the host 5.4 us instead of 7.7.
-// CTAs of two rounds share an SM with nobody and clusters of eight do not fill the chip, so that 128 of them would take two
-// waves (K = 4096, N = 2048: 10.3 / 6.3): 96 at most.  Two launches where the device cannot place the clusters.
+// At most 64 tokens, in one wave of CTAs.  One launch minus two, us per call (bf16, 4 / 8 bits, weights from memory): in a chain
+// of graph nodes, of calls made eagerly (bound by the host, which one launch saves), and in a graph behind a kernel that triggers
+// nothing, where the launch's start does not hide:
+//                                  chain          eager          behind another kernel
+//   K x N = 1024 x 1024   M = 8    -0.2 / +0.2    -1.1 / -1.1    +1.4 / +1.5
+//                         M = 16   -0.8 / -0.2    -1.0 / -0.6    +0.7 / +1.1
+//                         M = 24   -0.9 / -1.2    -1.3 / -1.6    -0.3 / -0.1
+//                         M = 50   -0.2 / -0.4    -0.3 / -0.7    -0.2 / +0.3
+//   2048 x 1024           M = 24   -1.2 / -2.3    -1.6 / -2.5    -1.2 / -1.6
+//                         M = 50   -0.3 / -0.3    -0.9 / -1.1    -0.4 / +0.5
+//   4096 x 1024           M = 24   -1.2 / -1.6    -1.8 / -2.3    -1.4 / -0.6
+//   1024 x 4096 (128 CTAs) M = 17  -0.1 / -0.4    -0.3 / -0.5    -0.3 / +0.1;   x 4736 (148) +0.2 / -0.1, -0.4 / -0.7, +1.1 / +1.2
+//   512 x 1024 (32)       M = 50   -0.1 / -0.2    -0.5 / -0.7    +0.2 / +0.8;   x 2048 (64) +0.3 / +0.4, +0.3 / +0.2, +0.2 / +0.8
+//   1024 x 1280 (80)      M = 50   +0.4 / +0.2    +0.6 / +0.2    -0.1 / +0.4;   x 2304 (144) +1.1 / +0.9, +0.6 / +0.5, +1.5 / +2.0
+//   256 x 1024            M = 50   +0.3 / +0.5    -0.2 / -0.4    +0.4 / +1.2
+// So at most 128 CTAs, and of more than 32 tokens (whose transform every channel tile repeats over twice the CTAs) 64 CTAs, 12
+// channel tiles and no rows below 384 channels.  With at most 8 tokens the largest grids are behind in a chain, too (8 bits, M = 1
+// 4.5 / 4.0): 96 CTAs.  CTAs of two rounds share an SM with nobody and clusters of eight do not fill the chip, so that 128 of them
+// would take two waves (K = 4096, N = 2048: 10.3 / 6.3): 96 as well.  Two launches where the device cannot place the clusters.
 template <typename Held>
 FusedPlan plan_fused(int64_t M, int64_t N, int64_t K, int block, int bits, bool mult, int sms, Held held) {
     FusedPlan f;
@@ -49,7 +62,9 @@ FusedPlan plan_fused(int64_t M, int64_t N, int64_t K, int block, int bits, bool 
     while (shift < 3 && slice(shift) > round) ++shift;
     if (slice(shift) > 2 * round) return f;
     const int64_t grid = ((N + kTileN - 1) / kTileN) << shift;
-    if (grid > (slice(shift) > round || M <= 8 ? 96 : sms)) return f;
+    const bool two_rounds = slice(shift) > round;
+    if (grid > sms || grid > (two_rounds || M <= 8 ? 96 : (M <= 32 ? 128 : 64))) return f;
+    if (M > 32 && !two_rounds && (K < 384 || N > 12 * kTileN)) return f;
     if (shift > 0 && held(1 << shift) < 1) return f;
     f.ctas_shift = shift; f.unit = unit; f.units = units; f.slice = slice(shift); f.grid = (int)grid;
     f.rounds = f.slice > round ? 2 : 1;

@@ -105,13 +105,15 @@ ONE_LAUNCH = [
     (17, 640, 1032, 128, 4, "f32", True, 1.0),         # five units over four CTAs, a ragged channel tile
     (8, 1024, 3072, 64, 4, "bf16", True, 1.0),         # the most CTAs with few tokens
     (32, 1024, 3072, 1, 8, "bf16", False, 1.0),        # identity rotation; the last batch of sixteen lanes a token
+    (24, 1024, 4096, 64, 4, "bf16", True, 1.0),        # the most CTAs with up to 32 tokens
     (33, 1024, 1024, 64, 4, "bf16", True, 1.0),        # the first of eight
     (50, 1792, 1032, 8, 4, "bf16", False, 0.8),        # two rounds; fourteen units over eight CTAs: one round in some slices
     (64, 1920, 520, 128, 8, "bf16", True, 1.0),        # ... fifteen
     (64, 2048, 1024, 128, 4, "f32", False, 1.0),       # the longest rows of more than 32 tokens
     (32, 4096, 1024, 256, 4, "f32", False, 1.0),       # the longest rows
-    (50, 1024, 2304, 64, 4, "bf16", False, 1.0),       # the widest outputs in clusters of eight
-    (63, 512, 4736, 64, 8, "f32", False, 1.0),         # ... of four: one CTA for each of 148 SMs
+    (50, 896, 1024, 64, 4, "bf16", False, 1.0),        # the widest outputs in clusters of eight
+    (63, 512, 1536, 64, 8, "f32", False, 1.0),         # ... of four
+    (40, 384, 136, 128, 8, "bf16", True, 0.9),         # the shortest rows of more than 32 tokens
 ]
 
 

@@ -154,7 +154,8 @@ def test_sizes_of_the_device_tests_take_the_routes_they_stand_for(plans, device)
         assert plans.fused(M, K, N, block, bits, smooth), (M, K, N)
         assert plans.grid <= B200[0]
     assert [plans.fused(*c[:5]) for c in edges.ONE_LAUNCH if c[1] > 1700] == [208, 208, 208, 208]       # two rounds
-    assert not plans.fused(8, 1024, 3080, 64, 4) and not plans.fused(50, 1024, 2312, 64, 4) and not plans.fused(63, 512, 4744, 64, 8)
+    assert not plans.fused(8, 1024, 3080, 64, 4) and not plans.fused(32, 1024, 4104, 64, 4) and not plans.fused(33, 1024, 1032, 64, 4)
+    assert not plans.fused(33, 512, 1544, 64, 8) and not plans.fused(33, 256, 128, 64, 4)
     assert not plans.fused(33, 2176, 128, 64, 4) and not plans.fused(32, 4224, 128, 64, 4) and not plans.fused(65, 1024, 128, 64, 4)
     for M, K, block, bits in edges.FEW_UNITS:
         ctas = plans.fused(M, K, 200, block, bits) % 100
