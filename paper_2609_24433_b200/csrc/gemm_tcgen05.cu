@@ -21,9 +21,10 @@
 //
 // Roles (warp specialised, persistent over tiles):
 //   warp 0       TMA producer          warp 1  MMA issuer + TMEM allocator
-//   warps 2-9    epilogue (two warps per TMEM lane quadrant, alternating 16-token chunks)
-//   warps 10-17  nibble unpack (two sets of four, alternating k-blocks), warp 18 TMA producer
-//                of packed weights (4-bit weights); warp 10 TMA producer of int8 weights (8-bit)
+//   4-bit weights: warps 2-9 epilogue (two warps per TMEM lane quadrant, alternating 16-token chunks),
+//                warps 10-17 nibble unpack (two sets of four, alternating k-blocks), warp 18 TMA producer
+//                of packed weights
+//   8-bit weights: warps 2-17 epilogue (four per quadrant), warp 18 TMA producer of int8 weights
 // Every role runs its loop with the whole warp converged and elects one lane (elect.sync) for
 // the issue itself; a k-block of the MMA warp is one block of PTX that also tests the next
 // k-block's barriers (see issue_kblock_*).  With 4-bit weights three rings are decoupled:
@@ -101,9 +102,9 @@ cudaError_t read_and_clear_watchdog(uint32_t* word) {
 
 namespace {
 
-constexpr int kThreadsW8 = 32 * (2 + kEpiWarps + 1);   // + one warp: TMA producer of int8 weights
-constexpr int kFirstUnpackWarp = 2 + kEpiWarps;
-constexpr int kThreadsW4 = 32 * (2 + kEpiWarps) + kUnpackSets * 128 + 32;
+constexpr int kThreadsW8 = 32 * (2 + kEpiWarpsW8 + 1);   // + one warp: TMA producer of int8 weights
+constexpr int kFirstUnpackWarp = 2 + kEpiWarpsW4;
+constexpr int kThreadsW4 = 32 * (2 + kEpiWarpsW4) + kUnpackSets * 128 + 32;
 enum : int { kUnsplit = 0, kSplitScratch = 1, kSplitCluster = 2 };
 
 struct Params {
@@ -129,7 +130,6 @@ struct Params {
     int32_t* partials;   // [tile][slice][bt tokens][128 channels] int32 raw sums of the slices (K split)
     uint32_t* counters;  // [tile] slices finished so far; zeroed by the host before the launch (K split)
     int slot_first;      // 1: the unpack sets wait for the TMEM slot ahead of the packed stage (see there)
-    int delta_vec;       // a_delta is 16-byte aligned: the epilogue may read four steps per load
     uint32_t zero;       // 0, as a run-time value (see the unpack warps' release of a packed stage)
 };
 
@@ -257,6 +257,8 @@ __device__ __forceinline__ uint32_t scale_pair_bf16(uint32_t a0, uint32_t a1, fl
     return w;
 }
 
+constexpr int kSumBytes = 16 * 32 * 4;                   // cluster split: a warp's sums of one token chunk
+
 enum : uint32_t {
     kWdProducer = 1u, kWdMmaFull = 2u, kWdMmaAcc = 4u, kWdEpilogue = 8u, kWdUnpackFull = 16u,
     kWdUnpackEmpty = 32u, kWdDrain = 64u, kWdPartials = 128u
@@ -285,6 +287,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     __shared__ uint64_t s_full_w8[kMaxStagesW];     // unpacked weights written
     __shared__ uint64_t s_acc_full[kAccStages];
     __shared__ uint64_t s_acc_empty[kAccStages];
+    __shared__ uint64_t s_sums;                     // cluster split: the other slices' sums are here
     __shared__ uint64_t s_epi_sync;                 // K split: rendezvous of the eight epilogue warps (bounded, unlike bar.sync)
     __shared__ int s_last[2];                       // K split: this CTA counted the last slice of its tile (alternating slots)
     __shared__ uint32_t s_tmem_base;
@@ -304,6 +307,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     const uint32_t cta_rank = CTAS == 2 ? cluster_ctarank() & 1u : 0u;
     const bool leader = cta_rank == 0;
     constexpr bool kCluster = SPLIT == kSplitCluster;
+    constexpr int kEpiWarps = BITS == 4 ? kEpiWarpsW4 : kEpiWarpsW8, kEpiSets = kEpiWarps / 4;    // warps per TMEM lane quadrant: every kEpiSets-th chunk
     // K split: a tile is `split` work units, unit = tile * split + slice, slice s
     // covering k-blocks [s * k_blocks, (s + 1) * k_blocks).  Any CTA takes any unit; the CTA that
     // finishes a tile's last slice adds up the slices' partial sums and runs the epilogue.
@@ -323,7 +327,8 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     const uint32_t smem_w = smem_a + (uint32_t)p.stages * a_bytes;
     const uint32_t smem_p = smem_w + (BITS == 4 ? 0u : (uint32_t)p.stages * w_bytes);
     const uint32_t smem_e = smem_p + (BITS == 4 ? (uint32_t)p.stages_p * pk_bytes : 0u);
-    const uint32_t smem_sums = smem_e + (uint32_t)(kEpiWarps * kEpiStageBytes);    // cluster split: the other slices' sums
+    constexpr int kEpiBytes = BITS == 8 && SPLIT != kUnsplit ? kEpiStageBytes / kEpiBuffers : kEpiStageBytes;
+    const uint32_t smem_sums = smem_e + (uint32_t)(kEpiWarps * kEpiBytes);    // cluster split: the other slices' sums
     uint8_t* gen_base = smem_raw + (base - smem_u32(smem_raw));   // generic pointer to `base`
 
     if (threadIdx.x == 0) {
@@ -346,6 +351,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             mbar_init(smem_u32(&s_acc_empty[a]), kEpiWarps * CTAS);
         }
         mbar_init(smem_u32(&s_epi_sync), kEpiWarps);
+        mbar_init(smem_u32(&s_sums), 1);
         fence_mbarrier_init();
         fence_proxy_async_smem();
     }
@@ -353,7 +359,28 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     tc_fence_before();
     __syncthreads();
     if (CTAS == 2) cluster_sync_all();              // the peer's barriers exist before anyone signals them
-    if (kCluster) cluster_arrive();                 // "this CTA exists": awaited before the first remote store
+    // Tile order.  Consecutive tile numbers -- the tiles the SMs work on at the same time -- cover a compact block of
+    // the output: the token tiles are cut into bands of p.band, a band is walked channel tile by channel tile with
+    // its token tiles fastest.  What one wave of CTAs pulls through L2 is then band activation tiles plus SMs/band
+    // weight tiles instead of every activation tile of the batch (long batches: the int8 activations alone exceed
+    // L2, and in channel-major order every wave streamed all of them from HBM again).
+    auto m_of = [&](int tile) {
+        if (p.band >= p.m_tiles) return tile % p.m_tiles;
+        const int b = tile / (p.band * p.n_tiles);
+        const int r = tile - b * (p.band * p.n_tiles);
+        const int rows = max(1, min(p.band, p.m_tiles - b * p.band));   // (a producer also maps the unit past its last one)
+        return b * p.band + r % rows;
+    };
+    if (kCluster) {
+        // what the other slices will send: the chunks of 16 tokens that this one finishes
+        const int unit = (int)blockIdx.x >> p.cluster_shift, tile = unit >> split_shift, slice = unit & (split - 1);
+        if (threadIdx.x == 0) {
+            const int64_t left = p.M - (int64_t)m_of(tile) * p.bt;
+            const int chunks = min(p.bt / 16, (int)min((left + 15) / 16, (int64_t)16));
+            mbar_arrive_expect_tx(smem_u32(&s_sums), (uint32_t)((split - 1) * ((chunks - slice + split - 1) >> split_shift) * 4 * kSumBytes));
+        }
+        cluster_arrive();                           // "this CTA exists": awaited before the first copy to another
+    }
     tc_fence_after();
     const uint32_t tmem_base = s_tmem_base;
     // Everything above is on-chip setup; from here on global memory is touched (activations written
@@ -373,18 +400,6 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     const int my_units = p.units_q + (unit0 < p.units_rem ? 1 : 0);
     const int k_blocks = p.kb_per;
     auto tile_of = [&](int unit) { return unit >> split_shift; };
-    // Tile order.  Consecutive tile numbers -- the tiles the SMs work on at the same time -- cover a compact block of
-    // the output: the token tiles are cut into bands of p.band, a band is walked channel tile by channel tile with
-    // its token tiles fastest.  What one wave of CTAs pulls through L2 is then band activation tiles plus SMs/band
-    // weight tiles instead of every activation tile of the batch (long batches: the int8 activations alone exceed
-    // L2, and in channel-major order every wave streamed all of them from HBM again).
-    auto m_of = [&](int tile) {
-        if (p.band >= p.m_tiles) return tile % p.m_tiles;
-        const int b = tile / (p.band * p.n_tiles);
-        const int r = tile - b * (p.band * p.n_tiles);
-        const int rows = max(1, min(p.band, p.m_tiles - b * p.band));   // (a producer also maps the unit past its last one)
-        return b * p.band + r % rows;
-    };
     auto n_of = [&](int tile) {
         if (p.band >= p.m_tiles) return tile / p.m_tiles;
         const int b = tile / (p.band * p.n_tiles);
@@ -393,9 +408,20 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     };
     auto kb0_of = [&](int unit) { return (unit & (split - 1)) * k_blocks; };   // first k-block of the unit's slice
 
+    // Steps of the 16 tokens of this warp's next chunk: lanes 16 (n & 1) ... of the first register; requested ahead of the sums,
+    // so that their trip through L2 is over when those are complete.
+    constexpr int kStepRegs = (16 / kEpiSets + 1) / 2;          // tiles have at most sixteen chunks
+    [[maybe_unused]] float steps[kStepRegs] = {};
+    auto next_steps = [&](int n) {
+        if ((n & 1) != 0) {
+#pragma unroll
+            for (int i = 0; i + 1 < kStepRegs; ++i) steps[i] = steps[i + 1];
+        }
+    };
+    [[maybe_unused]] float2 tail = make_float2(0.0f, 0.0f);   // (cluster split: scale and bias of this lane's channel)
     [[maybe_unused]] bool ok = true, waited = false;   // (ok: of the epilogue warps; the other roles have their own)
-    // ---- output of 16 tokens from t on, lane = channel j of this warp's 32 (jq ..): r = integer sums
-    auto emit = [&](uint32_t* r, int64_t tc, int64_t jq, float sw, float bj, uint8_t* xpose) {
+    // ---- output of 16 tokens from tc on (this warp's n-th chunk), lane = channel j of this warp's 32 (jq ..): r = integer sums
+    auto emit = [&](uint32_t* r, int n, int64_t tc, int64_t jq, float sw, float bj, uint8_t* xpose) {
         const int64_t j = jq + lane;
         const bool j_ok = j < p.N;
         if (p.out.acc != nullptr) {
@@ -406,16 +432,9 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             return;
         }
         float d[16];
-        if (tc + 16 <= p.M && p.delta_vec) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float4 q = ld_global_f4(p.out.a_delta + tc + 4 * i);
-                d[4 * i + 0] = q.x; d[4 * i + 1] = q.y; d[4 * i + 2] = q.z; d[4 * i + 3] = q.w;
-            }
-        } else {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) d[i] = tc + i < p.M ? ld_global_f32(p.out.a_delta + tc + i) : 0.0f;
-        }
+        for (int i = 0; i < 16; ++i) d[i] = __shfl_sync(0xffffffffu, steps[0], 16 * (n & 1) + i);
+        next_steps(n);
         tmem_ld_wait();                          // (the sums may still be on their way)
         if (p.out.yt == FQ_BF16) {
             // Transpose 32 channels x 16 tokens through shared memory, then 16-byte stores.  Tokens
@@ -584,9 +603,14 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         // ---------------------------------------------------------------- epilogue
         const int quad = warp & 3;                       // TMEM lanes [32*quad, 32*quad + 32)
         const int half = (warp - 2) >> 2;                // which of the alternating 16-token chunks
-        uint8_t* xpose = gen_base + (smem_e - base) + (warp - 2) * kEpiStageBytes;
+        uint8_t* xpose = gen_base + (smem_e - base) + (warp - 2) * kEpiBytes;
         const bool staged = p.out.acc == nullptr && p.out.yt == FQ_BF16;
         const float unshift = 1.0f / (float)(1 << p.acc_shift);   // exact power of two
+        auto constants = [&](int64_t j) {                // of channel j: scale and bias
+            const bool j_ok = j < p.N && p.out.acc == nullptr;
+            // ((float)acc * 2^-shift is exact: the shift is folded into the scale)
+            return j_ok ? make_float2(__ldg(p.w_scale + j) * unshift, __ldg(p.bias + j)) : make_float2(0.0f, 0.0f);
+        };
         int acc_stage = 0;
         uint32_t acc_phase = 0;
         [[maybe_unused]] uint32_t epi_phase = 0;
@@ -594,44 +618,82 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         [[maybe_unused]] int store_use = 0;             // bulk stores issued by this warp so far (buffer = parity)
         for (int unit = unit0; unit < num_units && ok; unit += unit_step) {
             const int tile = tile_of(unit);
-            const int64_t jq = (int64_t)n_of(tile) * (kTileN * CTAS) + (int64_t)cta_rank * kTileN + quad * 32;   // first channel of this warp
-            const int64_t j = jq + lane;
+            // first channel of this warp
+            const int64_t jq = (int64_t)n_of(tile) * (kTileN * CTAS) + (int64_t)cta_rank * kTileN + quad * 32;
             const int64_t t0 = (int64_t)m_of(tile) * p.bt;
-            const bool j_ok = j < p.N;
-            float sw = 0.0f, bj = 0.0f;
-            if (j_ok && p.out.acc == nullptr) {
-                sw = __ldg(p.w_scale + j) * unshift;     // (float)acc * 2^-shift is exact: fold the shift here
-                bj = __ldg(p.bias + j);
+            const float2 cj = constants(jq + lane);
+            const float sw = cj.x, bj = cj.y;
+            if (SPLIT != kUnsplit || !staged) {            // the steps of this warp's chunks
+                const int sh = kCluster ? split_shift : 0;
+                const int off = kCluster ? unit & (split - 1) : 0;
+#pragma unroll
+                for (int i = 0; i < kStepRegs; ++i) {
+                    const int t = (((half + (2 * i + (lane >> 4)) * kEpiSets) << sh) + off) * 16 + (lane & 15);
+                    steps[i] = p.out.acc == nullptr && t < p.bt && t0 + t < p.M ? ld_global_f32(p.out.a_delta + t0 + t) : 0.0f;
+                }
             }
+            // bf16 outputs of an unsplit launch: the four channels of this thread's accumulator fragments
+            [[maybe_unused]] float2 sw4[4], bj4[4], nd0, nd1;
+            auto request_steps = [&](int c) {                // ... and the steps of its four tokens
+                const int64_t ta = t0 + c + 2 * (lane & 3), tb = ta + 8;
+                nd0.x = ta < p.M ? ld_global_f32(p.out.a_delta + ta) : 0.0f;
+                nd0.y = ta + 1 < p.M ? ld_global_f32(p.out.a_delta + ta + 1) : 0.0f;
+                nd1.x = tb < p.M ? ld_global_f32(p.out.a_delta + tb) : 0.0f;
+                nd1.y = tb + 1 < p.M ? ld_global_f32(p.out.a_delta + tb + 1) : 0.0f;
+            };
+            auto request_constants = [&]() {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float2 ci = constants(jq + (lane >> 2) + 8 * i);
+                    sw4[i] = make_float2(ci.x, ci.x);
+                    bj4[i] = make_float2(ci.y, ci.y);
+                }
+                request_steps(half * 16);
+            };
+            // Ahead of the sums for the last tile, whose epilogue hides behind nothing: their trip through L2 is over when the
+            // sums are complete.  (Not for the others, beside whose epilogue the next tile is multiplied: 816 x 2048 x 32768 47.8 us
+            // instead of 48.1; the pairs of 4-bit weights have no registers for it.)
+            const bool ahead = !(BITS == 4 && CTAS == 2) && unit + unit_step >= num_units;
+            if (SPLIT == kUnsplit && staged && ahead) request_constants();
             // a tile takes at least ~0.2 us per k-block: sleep through a quarter of that before the first look,
             // so that eight idle warps do not spend issue slots polling while a long tile is being accumulated
             if (k_blocks * ATOMS >= 32) __nanosleep(k_blocks * ATOMS >= 400 ? 20000u : (unsigned)(k_blocks * ATOMS) * 50u);
             ok = mbar_wait_warp_relaxed(smem_u32(&s_acc_full[acc_stage]), acc_phase, abort_flag, p.watchdog, kWdEpilogue);
             if (!ok) break;
             if (kCluster) {
-                // Token chunk c (16 tokens) is finished by slice c % split of the cluster: the others send it their sums,
-                // [sender][chunk / split][token][channel] there, and all meet at the end of the role code.  (CTA pairs: each
-                // CTA has 128 channels of its own, and exchanges with the CTA of the same parity.)
-                cluster_wait();                  // the cluster's CTAs exist
+                // Token chunk c (16 tokens) is finished by slice c % split of the cluster: the others send it their sums, a
+                // bulk copy of [16 tokens][32 channels] per warp and chunk, counted on the finisher's barrier.  (CTA pairs: each
+                // CTA has 128 channels of its own, and exchanges with the CTA of the same parity.)  The copies' sources are the
+                // ring's memory: everything in it has been multiplied.
+                // Four-byte stores into the other CTAs went out at 17 bytes per cycle, and the cluster barrier behind them, whose
+                // arrivals wait for them, took 2750 cycles: 816 x 16384 x 2048 (8 bits) 35.8 us, so 34.6.
+                cluster_wait();                  // the cluster's CTAs exist, their barriers are armed
                 waited = true;
                 tc_fence_after();
                 const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16);
                 const int slice = unit & (split - 1), per = (p.bt / 16 + split - 1) >> split_shift;
-                const uint32_t dst = smem_sums + (uint32_t)(quad * 32 + lane) * 4u;
-                for (int c = half; c < p.bt / 16; c += 2) {
+                for (int c = half, sent = 0; c < p.bt / 16; c += kEpiSets) {
                     const int owner = c & (split - 1);
                     if (t0 + c * 16 >= p.M) break;
                     if (owner == slice) continue;
                     uint32_t r[16];
                     tmem_ld16(taddr + (uint32_t)(c * 16), r);
                     tmem_ld_wait();
-                    const int from = slice - (slice > owner ? 1 : 0);
-                    const uint32_t to = cluster_address(dst + (uint32_t)((from * per + (c >> split_shift)) * 16 * kTileN) * 4u,
-                                                        (uint32_t)owner * CTAS + cta_rank);
+                    const uint32_t from = base + (uint32_t)((sent * kEpiWarps + warp - 2) * kSumBytes);
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) st_cluster(to + (uint32_t)(i * kTileN) * 4u, r[i]);
+                    for (int i = 0; i < 16; ++i) sts32(from + (uint32_t)(i * 32 + lane) * 4u, r[i]);
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    const int sender = slice - (slice > owner ? 1 : 0);
+                    const uint32_t to = (uint32_t)owner * CTAS + cta_rank;
+                    if (lane == 0)
+                        bulk_copy_cluster(cluster_address(smem_sums + (uint32_t)(((sender * per + (c >> split_shift)) * 4 + quad) * kSumBytes), to),
+                                          from, (uint32_t)kSumBytes, cluster_address(smem_u32(&s_sums), to));
+                    __syncwarp();
+                    ++sent;
                 }
                 tc_fence_before();
+                tail = cj;
                 break;                           // one tile per cluster
             }
             // K split.  Every slice writes its raw int32 sums to its own block of scratch
@@ -647,7 +709,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                 const int ctile = tile * CTAS + (int)cta_rank;
                 int32_t* tile_part = p.partials + (size_t)ctile * (size_t)split * kTileN * (size_t)p.bt + (size_t)(quad * 32 + lane);
                 int32_t* mine = tile_part + (size_t)slice * kTileN * (size_t)p.bt;
-                for (int c = half * 16; c < p.bt; c += 32) {
+                for (int c = half * 16; c < p.bt; c += 16 * kEpiSets) {
                     if (t0 + c >= p.M) break;
                     uint32_t r[16];
                     tmem_ld16(taddr + (uint32_t)c, r);
@@ -695,39 +757,24 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                 // tokens of each 8-token group), scaled in packed pairs, stored token-major into a 1 KB buffer of
                 // [16 tokens][32 channels] with two transposing matrix stores, and leave as one tiled bulk store; two
                 // buffers alternate so that a chunk is written while the previous one is on its way out.
-                const int g = lane >> 2, q = lane & 3;
-                float2 sw4[4], bj4[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int64_t ji = jq + g + 8 * i;
-                    float swv = 0.0f, bv = 0.0f;
-                    if (ji < p.N) { swv = __ldg(p.w_scale + ji) * unshift; bv = __ldg(p.bias + ji); }
-                    sw4[i] = make_float2(swv, swv);
-                    bj4[i] = make_float2(bv, bv);
-                }
                 // address of "matrix lane>>3, row lane&7" inside a buffer: token (lane>>4)*8 + (lane&7), 16-byte
                 // chunk ((lane>>3)&1) [+2 for channels 16..31], chunk index XORed with (token>>1)&3 (64-byte swizzle)
                 const uint32_t tok = (uint32_t)((lane >> 4) * 8 + (lane & 7));
                 const uint32_t ch = (uint32_t)((lane >> 3) & 1);
                 const uint32_t off_a = tok * 64u + ((ch ^ ((tok >> 1) & 3u)) << 4);
                 const uint32_t off_b = tok * 64u + (((ch + 2u) ^ ((tok >> 1) & 3u)) << 4);
-                const uint32_t buf0 = smem_e + (uint32_t)(warp - 2) * kEpiStageBytes;
+                const uint32_t buf0 = smem_e + (uint32_t)(warp - 2) * kEpiBytes;
                 const bool any_channel = jq < p.N;        // warp-uniform
-                // The accumulators and steps of a chunk are requested as soon as the chunk before it has been handed to the
-                // copy engine.
+                if (!ahead) request_constants();
+                // The accumulators and steps of a chunk are requested as soon as the chunk before it has been handed to the copy
+                // engine.
                 uint32_t na[8], nb[8];
-                float2 nd0, nd1;
                 auto request = [&](int c) {
                     tmem_ld_16x256b_x2(taddr + (uint32_t)c, na);                    // channels 0..15 of the quadrant
                     tmem_ld_16x256b_x2(taddr + (16u << 16) + (uint32_t)c, nb);      // channels 16..31
-                    const int64_t ta = t0 + c + 2 * q, tb = ta + 8;
-                    nd0.x = ta < p.M ? ld_global_f32(p.out.a_delta + ta) : 0.0f;
-                    nd0.y = ta + 1 < p.M ? ld_global_f32(p.out.a_delta + ta + 1) : 0.0f;
-                    nd1.x = tb < p.M ? ld_global_f32(p.out.a_delta + tb) : 0.0f;
-                    nd1.y = tb + 1 < p.M ? ld_global_f32(p.out.a_delta + tb + 1) : 0.0f;
                 };
-                if (t0 + half * 16 < p.M) request(half * 16);
-                for (int c = half * 16; c < p.bt; c += 32) {
+                if (half * 16 < p.bt && t0 + half * 16 < p.M) request(half * 16);
+                for (int c = half * 16; c < p.bt; c += 16 * kEpiSets) {
                     const int64_t tc = t0 + c;
                     if (tc >= p.M) break;                // tokens beyond M: nothing to store (warp-uniform)
                     tmem_ld_wait();
@@ -759,7 +806,10 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                     ++store_use;
                     // (requested only now: with the next chunk's TMEM loads in flight during the arithmetic above, the
                     // main loop beside this epilogue ran slower -- gate/up 46.5 against 44.9 us)
-                    if (c + 32 < p.bt && tc + 32 < p.M) request(c + 32);
+                    if (c + 16 * kEpiSets < p.bt && tc + 16 * kEpiSets < p.M) {
+                        request(c + 16 * kEpiSets);
+                        request_steps(c + 16 * kEpiSets);
+                    }
                 }
                 tmem_ld_wait();                          // (nothing outstanding unless the loop broke early)
             } else {
@@ -776,8 +826,8 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                     for (int i = 0; i < 16; ++i) pv_next[i] += __ldcg(src + (size_t)i * kTileN);
                 }
             };
-            if (split > 1 && t0 + half * 16 < p.M) fetch_partials(half * 16);
-            for (int c = half * 16; c < p.bt; c += 32) {
+            if (split > 1 && half * 16 < p.bt && t0 + half * 16 < p.M) fetch_partials(half * 16);
+            for (int c = half * 16, n = 0; c < p.bt; c += 16 * kEpiSets, ++n) {
                 const int64_t tc = t0 + c;
                 if (tc >= p.M) break;                    // tokens beyond M: nothing to store (warp-uniform)
                 uint32_t r[16];
@@ -786,12 +836,12 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                     int32_t pv[16];
 #pragma unroll
                     for (int i = 0; i < 16; ++i) pv[i] = pv_next[i];
-                    if (c + 32 < p.bt && tc + 32 < p.M) fetch_partials(c + 32);
+                    if (c + 16 * kEpiSets < p.bt && tc + 16 * kEpiSets < p.M) fetch_partials(c + 16 * kEpiSets);
                     tmem_ld_wait();
 #pragma unroll
                     for (int i = 0; i < 16; ++i) r[i] += (uint32_t)pv[i];
                 }
-                emit(r, tc, jq, sw, bj, xpose);
+                emit(r, n, tc, jq, sw, bj, xpose);
             }
             }
             tc_fence_before();
@@ -987,23 +1037,20 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     if (kCluster) {
         __syncwarp();
         if (!waited) cluster_wait();
-        cluster_arrive();
-        cluster_wait();                              // every CTA's sums are where they belong
-        if (warp >= 2 && warp < 2 + kEpiWarps && ok && unit0 < num_units) {
+        const bool finishes = warp >= 2 && warp < 2 + kEpiWarps && ok && unit0 < num_units;
+        if (finishes) ok = mbar_wait_all(smem_u32(&s_sums), 0u, abort_flag, p.watchdog, kWdPartials);
+        __syncwarp();
+        cluster_arrive_relaxed();                    // "this CTA has its sums": no copy is under way when everybody has said so
+        if (finishes && ok) {
             const int quad = warp & 3, half = (warp - 2) >> 2, slice = unit0 & (split - 1);
             const int tile = tile_of(unit0);
             const int64_t jq = (int64_t)n_of(tile) * (kTileN * CTAS) + (int64_t)cta_rank * kTileN + quad * 32;
             const int64_t t0 = (int64_t)m_of(tile) * p.bt;
-            float sw = 0.0f, bj = 0.0f;
-            if (jq + lane < p.N && p.out.acc == nullptr) {
-                sw = __ldg(p.w_scale + jq + lane) * (1.0f / (float)(1 << p.acc_shift));
-                bj = __ldg(p.bias + jq + lane);
-            }
             const int per = (p.bt / 16 + split - 1) >> split_shift;
-            const int32_t* sums = reinterpret_cast<const int32_t*>(gen_base + (smem_sums - base)) + quad * 32 + lane;
-            uint8_t* xpose = gen_base + (smem_e - base) + (warp - 2) * kEpiStageBytes;
+            const int32_t* sums = reinterpret_cast<const int32_t*>(gen_base + (smem_sums - base)) + lane;
+            uint8_t* xpose = gen_base + (smem_e - base) + (warp - 2) * kEpiBytes;
             tc_fence_after();
-            for (int i = half; i < per; i += 2) {
+            for (int i = half, n = 0; i < per; i += kEpiSets, ++n) {
                 const int c = (i << split_shift) + slice;
                 const int64_t tc = t0 + c * 16;
                 if (c * 16 >= p.bt || tc >= p.M) break;
@@ -1011,11 +1058,11 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                 tmem_ld16(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(c * 16), r);
                 tmem_ld_wait();
                 for (int k = 0; k < split - 1; ++k) {
-                    const int32_t* q = sums + (size_t)(k * per + i) * 16 * kTileN;
+                    const int32_t* q = sums + (size_t)((k * per + i) * 4 + quad) * (kSumBytes / 4);
 #pragma unroll
-                    for (int t = 0; t < 16; ++t) r[t] += (uint32_t)q[t * kTileN];
+                    for (int t = 0; t < 16; ++t) r[t] += (uint32_t)q[t * 32];
                 }
-                emit(r, tc, jq, sw, bj, xpose);
+                emit(r, n, tc, jq, tail.x, tail.y, xpose);
             }
         }
     }
@@ -1023,7 +1070,8 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     // ------------------------------------------------------------------ teardown
     tc_fence_before();
     __syncthreads();
-    if (CTAS == 2) cluster_sync_all();              // neither CTA leaves while the other may still signal it
+    if (kCluster) cluster_wait();                   // nobody leaves while its own copies may still be under way
+    else if (CTAS == 2) cluster_sync_all();         // neither CTA leaves while the other may still signal it
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc<CTAS>(tmem_base, (uint32_t)p.tmem_cols);
@@ -1177,7 +1225,6 @@ fq_status launch_planned(const int8_t* a8, int64_t M, const Weights& W, int acc_
     p.split = split;
     p.counters = static_cast<uint32_t*>(scratch);            // cleared by gemm_prepare()
     p.partials = reinterpret_cast<int32_t*>(static_cast<uint8_t*>(scratch) + kCounterBytes);
-    p.delta_vec = (reinterpret_cast<uintptr_t>(out.a_delta) & 15u) == 0 ? 1 : 0;
     p.bt = bt;
     p.m_tiles = (int)((M + bt - 1) / bt);
     p.n_tiles = (int)((W.N + kTileN * ctas - 1) / (kTileN * ctas));

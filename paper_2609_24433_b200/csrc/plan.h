@@ -235,7 +235,11 @@ constexpr int kMaxStages = 16;         // ring slots, at most: activations, pack
 constexpr int kMaxStagesP = 16;
 constexpr int kMaxStagesW = 8;
 constexpr int kColsW = kBlockK / 4;    // TMEM columns of one unpacked k-block (128 int8 per lane)
-constexpr int kEpiWarps = 8;
+// Epilogue warps: the launch's last tile has nothing to hide its epilogue behind, a chain of TMEM load, arithmetic and store per 16
+// tokens, some 500 cycles each; twice the warps halve it (8 bits, 1000 x 4096 x 4104 21.7 -> 19.8 us; at 4 bits the unpack warps leave no
+// registers for them).
+constexpr int kEpiWarpsW4 = 8, kEpiWarpsW8 = 16;
+inline int epi_warps(int bits) { return bits == 4 ? kEpiWarpsW4 : kEpiWarpsW8; }
 constexpr int kEpiBuffers = 2;                          // output buffers per epilogue warp (bulk stores in flight; four measured no faster)
 constexpr int kEpiStageBytes = kEpiBuffers * 16 * 64;   // per epilogue warp: buffers of 16 tokens x 32 channels of bf16
 constexpr int kMaxSplit = 16;          // K slices per tile, at most
@@ -259,7 +263,11 @@ inline int atoms_per_stage(int bits, int ctas, int bt, int64_t K, int split) {
     return split == 1 || kb % (2 * split) == 0 ? 2 : 1;
 }
 // Shared memory of the pipeline rings; `sums`: bytes taken by the sums of a cluster split.
-inline size_t ring_budget(size_t sums) { return 227 * 1024 - 1024 /*alignment slack*/ - 1024 /*static*/ - (size_t)kEpiWarps * kEpiStageBytes - sums; }
+// Output buffers of the epilogue warps (8-bit launches that split K have one per warp: its ring is worth more).
+inline int epi_stage_bytes(int bits, bool split) { return bits == 8 && split ? kEpiStageBytes / kEpiBuffers : kEpiStageBytes; }
+inline size_t ring_budget(int bits, bool split, size_t sums) {
+    return 227 * 1024 - 1024 /*alignment slack*/ - 1024 /*static*/ - (size_t)epi_warps(bits) * epi_stage_bytes(bits, split) - sums;
+}
 inline size_t stage_bytes(int bits, int ctas, int bt, int atoms) {
     return ((size_t)(bt / ctas) * kBlockK + (size_t)kTileN * kBlockK * bits / 8) * atoms;
 }
@@ -334,7 +342,7 @@ GemmPlan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t sc
                 const int atoms = atoms_per_stage(bits, c, b, K, sp);
                 const double ctas = (double)(units * sp * c);
                 if (clusters && (bits == 8 || b <= 128) && sp * c <= kMaxCluster && units * sp <= slots &&
-                    ring_budget(cluster_sums_bytes(b, sp)) * atoms >= 4 * stage_bytes(bits, c, b, atoms) && units <= holds(sp * c))
+                    ring_budget(bits, true, cluster_sums_bytes(b, sp)) * atoms >= 4 * stage_bytes(bits, c, b, atoms) && units <= holds(sp * c))
                     offer(sp, true, 0, slice + 16.0 * b / sp + (bits == 4 ? 2800.0 + 40.0 * ctas : 3300.0 + 18.0 * ctas) + 500.0 * (sp - 1));
                 if ((c == 1 || bits == 8) && units * c <= kMaxSplitTiles && units * c * sp <= 4 * (int64_t)sms) {
                     const size_t scratch = kCounterBytes + (size_t)units * c * sp * kTileN * b * sizeof(int32_t);
@@ -356,9 +364,10 @@ struct GemmRings {
 inline GemmRings gemm_rings(const GemmPlan& plan, int bits, int64_t K) {
     GemmRings f;
     const int bt = plan.bt;
+    const bool split = plan.split > 1;
     f.atoms = atoms_per_stage(bits, plan.ctas, bt, K, plan.split);
-    const size_t sums = plan.cluster ? cluster_sums_bytes(bt, plan.split) : 0, budget = ring_budget(sums);
-    const size_t epi_bytes = (size_t)kEpiWarps * kEpiStageBytes + sums;
+    const size_t sums = plan.cluster ? cluster_sums_bytes(bt, plan.split) : 0, budget = ring_budget(bits, split, sums);
+    const size_t epi_bytes = (size_t)epi_warps(bits) * epi_stage_bytes(bits, split) + sums;
     const size_t a_bytes = (size_t)(bt / plan.ctas) * kBlockK * f.atoms, w_bytes = (size_t)kTileN * kBlockK, pk_bytes = w_bytes / 2 * f.atoms;
     // 4-bit weights: every TMEM column the accumulators leave free becomes unpacked-weight ring
     f.stages_w = bits == 4 ? (512 - kAccStages * bt) / (kColsW * f.atoms) : 0;
@@ -384,6 +393,9 @@ inline GemmRings gemm_rings(const GemmPlan& plan, int bits, int64_t K) {
         if (f.stages < 2) return f;
         f.smem = (a_bytes + w_bytes) * f.stages + epi_bytes + 1024;
     }
+    // (The sums that a cluster split sends on are staged in the ring's memory, 2 KB per epilogue warp and chunk.)
+    const int warps = epi_warps(bits);
+    if (plan.cluster && (size_t)((bt / 16 + warps / 4 - 1) / (warps / 4)) * warps * 2048 > f.smem - epi_bytes - 1024) return f;
     // One CTA of this kind per SM, and none of the short-batch kernel beside it: a cluster whose CTA waited for tensor memory
     // must not be what another cluster on that SM waits for (launches of two streams).
     if (plan.cluster && f.smem < 152 * 1024) f.smem = 152 * 1024;
