@@ -33,7 +33,7 @@
 // frees both the activation stage and the k-block's TMEM slot.
 // Variants: CTAS = 2 runs CTA pairs (cta_group::2, 256 channels per MMA, each CTA staging half
 // of the token tile); SPLIT lets CTAs share a tile along K and exchange int32 partial sums,
-// through the cluster's shared memory or through global scratch.
+// through the cluster's shared memory or through global scratch, or stacks two slices of K in one tile.
 // bf16 outputs leave through a per-warp 1 KB shared-memory transposer so that global
 // stores are 16-byte vectors of 8 consecutive channels; fp32/raw outputs store directly.
 // Every mbarrier wait is bounded by wall-clock time; on expiry the CTA records a
@@ -105,11 +105,13 @@ namespace {
 constexpr int kThreadsW8 = 32 * (2 + kEpiWarpsW8 + 1);   // + one warp: TMA producer of int8 weights
 constexpr int kFirstUnpackWarp = 2 + kEpiWarpsW4;
 constexpr int kThreadsW4 = 32 * (2 + kEpiWarpsW4) + kUnpackSets * 128 + 32;
-enum : int { kUnsplit = 0, kSplitScratch = 1, kSplitCluster = 2 };
+constexpr int kStackRows = kTileN / kStackSlices;        // channels of a stacked tile
+enum : int { kUnsplit = 0, kSplitScratch = 1, kSplitCluster = 2, kStacked = 3 };
 
 struct Params {
     int64_t M, N, K;
-    int bt;              // tokens per tile (MMA N), multiple of 16, <= 256
+    int bt;              // columns per tile (MMA N): tokens, times the K slices of a stacked tile; multiple of 16, <= 256
+    int tok;             // tokens per tile
     int stages;          // activation ring (and int8 weight ring, in lockstep, for 8-bit weights)
     int stages_p;        // packed-weight ring (4-bit weights)
     int stages_w;        // unpacked-weight ring (4-bit weights)
@@ -307,12 +309,14 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     const uint32_t cta_rank = CTAS == 2 ? cluster_ctarank() & 1u : 0u;
     const bool leader = cta_rank == 0;
     constexpr bool kCluster = SPLIT == kSplitCluster;
+    constexpr bool kStack = SPLIT == kStacked;
+    constexpr bool kBox = ATOMS > 1;                // the copy maps are [atom][row][byte]: a stage is one copy
     constexpr int kEpiWarps = BITS == 4 ? kEpiWarpsW4 : kEpiWarpsW8, kEpiSets = kEpiWarps / 4;    // warps per TMEM lane quadrant: every kEpiSets-th chunk
     // K split: a tile is `split` work units, unit = tile * split + slice, slice s
     // covering k-blocks [s * k_blocks, (s + 1) * k_blocks).  Any CTA takes any unit; the CTA that
     // finishes a tile's last slice adds up the slices' partial sums and runs the epilogue.
-    const int split = SPLIT != kUnsplit ? p.split : 1;   // compile-time 1 in the common instantiation
-    const int split_shift = SPLIT != kUnsplit ? p.split_shift : 0;
+    const int split = SPLIT != kUnsplit && !kStack ? p.split : 1;   // compile-time 1 in the common instantiation
+    const int split_shift = SPLIT != kUnsplit && !kStack ? p.split_shift : 0;
     const int bt_cta = p.bt / CTAS;                 // token rows this CTA loads
 
     // carve dynamic shared memory: [A8 stages][W8 stages][packed stages][epilogue transposers], 1024-byte aligned
@@ -488,7 +492,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             bool ok = true;
             int stage = 0, kb = 0, unit = unit0;
             uint32_t phase = 0;
-            int t0 = m_of(tile_of(unit)) * p.bt + (int)cta_rank * bt_cta;
+            int t0 = m_of(tile_of(unit)) * p.tok + (int)cta_rank * bt_cta;
             int kb0 = kb0_of(unit);
             bool peek = false;
             for (int n = 0; n < total_kb; ++n) {
@@ -503,9 +507,9 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                     const uint32_t bar = smem_u32(&s_full_tma[stage]);
                     if (CTAS == 1) {
                         mbar_arrive_expect_tx(bar, tx);
-#pragma unroll
-                        for (int h = 0; h < ATOMS; ++h)     // channels past K arrive as zeros
-                            tma_load_2d(smem_a + stage * a_bytes + h * a_atom, &map_a, ((kb0 + kb) * ATOMS + h) * kBlockK, t0, bar);
+                        if constexpr (kStack) tma_load_4d(smem_a + stage * a_bytes, &map_a, 0, t0, 0, (kb0 + kb) * ATOMS, bar);
+                        else if constexpr (kBox) tma_load_3d(smem_a + stage * a_bytes, &map_a, 0, t0, (kb0 + kb) * ATOMS, bar);
+                        else tma_load_2d(smem_a + stage * a_bytes, &map_a, (kb0 + kb) * kBlockK, t0, bar);    // channels past K arrive as zeros
                     } else {
                         // the pair's bytes are all counted on the even CTA's barrier, which it arms for both
                         if (leader) mbar_arrive_expect_tx(bar, tx * CTAS);
@@ -516,7 +520,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                 if (++kb == k_blocks) {
                     kb = 0;
                     unit += unit_step;
-                    t0 = m_of(tile_of(unit)) * p.bt + (int)cta_rank * bt_cta;
+                    t0 = m_of(tile_of(unit)) * p.tok + (int)cta_rank * bt_cta;
                     kb0 = kb0_of(unit);
                 }
             }
@@ -619,17 +623,18 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         for (int unit = unit0; unit < num_units && ok; unit += unit_step) {
             const int tile = tile_of(unit);
             // first channel of this warp
-            const int64_t jq = (int64_t)n_of(tile) * (kTileN * CTAS) + (int64_t)cta_rank * kTileN + quad * 32;
-            const int64_t t0 = (int64_t)m_of(tile) * p.bt;
+            const int64_t jq = kStack ? (int64_t)n_of(tile) * kStackRows + (quad & 1) * 32
+                                      : (int64_t)n_of(tile) * (kTileN * CTAS) + (int64_t)cta_rank * kTileN + quad * 32;
+            const int64_t t0 = (int64_t)m_of(tile) * p.tok;
             const float2 cj = constants(jq + lane);
             const float sw = cj.x, bj = cj.y;
             if (SPLIT != kUnsplit || !staged) {            // the steps of this warp's chunks
-                const int sh = kCluster ? split_shift : 0;
-                const int off = kCluster ? unit & (split - 1) : 0;
+                const int sh = kStack ? 1 : (kCluster ? split_shift : 0);
+                const int off = kStack ? quad >> 1 : (kCluster ? unit & (split - 1) : 0);
 #pragma unroll
                 for (int i = 0; i < kStepRegs; ++i) {
                     const int t = (((half + (2 * i + (lane >> 4)) * kEpiSets) << sh) + off) * 16 + (lane & 15);
-                    steps[i] = p.out.acc == nullptr && t < p.bt && t0 + t < p.M ? ld_global_f32(p.out.a_delta + t0 + t) : 0.0f;
+                    steps[i] = p.out.acc == nullptr && t < p.tok && t0 + t < p.M ? ld_global_f32(p.out.a_delta + t0 + t) : 0.0f;
                 }
             }
             // bf16 outputs of an unsplit launch: the four channels of this thread's accumulator fragments
@@ -695,6 +700,51 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                 tc_fence_before();
                 tail = cj;
                 break;                           // one tile per cluster
+            }
+            if constexpr (kStack) {
+                // Half g of the tile's lanes holds K slice g of the tile's 64 channels, and only that slice's columns count.  Token
+                // chunk c is finished by half c % 2: the other half's warps hand it their sums through shared memory,
+                // [finisher][chunk / 2][token][channel].
+                tc_fence_after();
+                const int g = quad >> 1, chunks = p.tok / 16, per = (chunks + 1) / 2;
+                const uint32_t mine = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc_stage * p.bt + g * p.tok);
+                int32_t* sums = reinterpret_cast<int32_t*>(gen_base + (smem_sums - base)) + (quad & 1) * 32 + lane;
+                for (int c = half; c < chunks; c += kEpiSets) {
+                    if (t0 + c * 16 >= p.M) break;
+                    if ((c & 1) == g) continue;
+                    uint32_t r[16];
+                    tmem_ld16(mine + (uint32_t)(c * 16), r);
+                    tmem_ld_wait();
+                    int32_t* q = sums + (((c & 1) * per + c / 2) * 16) * kStackRows;
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) q[i * kStackRows] = (int)r[i];
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&s_epi_sync));
+                ok = mbar_wait_all(smem_u32(&s_epi_sync), epi_phase, abort_flag, p.watchdog, kWdPartials);
+                epi_phase ^= 1u;
+                if (!ok) break;
+                for (int i = half, n = 0; i < per; i += kEpiSets, ++n) {
+                    const int c = 2 * i + g;
+                    if (c >= chunks || t0 + c * 16 >= p.M) break;
+                    uint32_t r[16];
+                    tmem_ld16(mine + (uint32_t)(c * 16), r);
+                    tmem_ld_wait();
+                    const int32_t* q = sums + ((g * per + i) * 16) * kStackRows;
+#pragma unroll
+                    for (int t = 0; t < 16; ++t) r[t] += (uint32_t)q[t * kStackRows];
+                    emit(r, n, t0 + c * 16, jq, sw, bj, xpose);
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(smem_u32(&s_acc_empty[acc_stage]));
+                    mbar_arrive(smem_u32(&s_epi_sync));              // the sums have been read
+                }
+                ok = mbar_wait_all(smem_u32(&s_epi_sync), epi_phase, abort_flag, p.watchdog, kWdPartials);
+                epi_phase ^= 1u;
+                if (++acc_stage == kAccStages) { acc_stage = 0; acc_phase ^= 1u; }
+                continue;
             }
             // K split.  Every slice writes its raw int32 sums to its own block of scratch
             // ([tile][slice][bt tokens][128 channels]: a warp's 32 channels of one token are one 128-byte
@@ -863,7 +913,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             bool ok = true;
             int stage = 0, kb = 0, unit = unit0;
             uint32_t phase = 0;
-            int n0 = n_of(tile_of(unit)) * (kTileN * CTAS) + (int)cta_rank * kTileN;
+            int n0 = n_of(tile_of(unit)) * (kStack ? kStackRows : kTileN * CTAS) + (int)cta_rank * kTileN;
             int kb0 = kb0_of(unit);
             bool peek = false;
             for (int n = 0; n < total_kb; ++n) {
@@ -888,7 +938,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                 if (++kb == k_blocks) {
                     kb = 0;
                     unit += unit_step;
-                    n0 = n_of(tile_of(unit)) * (kTileN * CTAS) + (int)cta_rank * kTileN;
+                    n0 = n_of(tile_of(unit)) * (kStack ? kStackRows : kTileN * CTAS) + (int)cta_rank * kTileN;
                     kb0 = kb0_of(unit);
                 }
             }
@@ -1004,7 +1054,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             bool ok = true;
             int ps = 0, kb = 0, unit = unit0;
             uint32_t pph = 0;
-            int n0 = n_of(tile_of(unit)) * (kTileN * CTAS) + (int)cta_rank * kTileN;
+            int n0 = n_of(tile_of(unit)) * (kStack ? kStackRows : kTileN * CTAS) + (int)cta_rank * kTileN;
             int kb0 = kb0_of(unit);
             bool peek = false;
             for (int n = 0; n < total_kb; ++n) {
@@ -1018,15 +1068,15 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                 if (elect_one()) {
                     const uint32_t bar = smem_u32(&s_full_p[ps]);
                     mbar_arrive_expect_tx(bar, pk_bytes);
-#pragma unroll
-                    for (int h = 0; h < ATOMS; ++h)
-                        tma_load_2d(smem_p + ps * pk_bytes + h * pk_atom, &map_w, ((kb0 + kb) * ATOMS + h) * (kBlockK / 2), n0, bar);
+                    if constexpr (kStack) tma_load_4d(smem_p + ps * pk_bytes, &map_w, 0, n0, 0, (kb0 + kb) * ATOMS, bar);
+                    else if constexpr (kBox) tma_load_3d(smem_p + ps * pk_bytes, &map_w, 0, n0, (kb0 + kb) * ATOMS, bar);
+                    else tma_load_2d(smem_p + ps * pk_bytes, &map_w, (kb0 + kb) * (kBlockK / 2), n0, bar);
                 }
                 if (++ps == p.stages_p) { ps = 0; pph ^= 1u; }
                 if (++kb == k_blocks) {
                     kb = 0;
                     unit += unit_step;
-                    n0 = n_of(tile_of(unit)) * (kTileN * CTAS) + (int)cta_rank * kTileN;
+                    n0 = n_of(tile_of(unit)) * (kStack ? kStackRows : kTileN * CTAS) + (int)cta_rank * kTileN;
                     kb0 = kb0_of(unit);
                 }
             }
@@ -1122,6 +1172,24 @@ bool encode_tiled(CUtensorMap* map, CUtensorMapDataType dt, uint32_t rank, const
               swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+namespace {
+// Rows of whole atoms as [atom][row][byte], so that a stage of several atoms is one copy.
+bool encode_atoms(CUtensorMap* map, const void* ptr, uint64_t row_bytes, uint64_t rows, uint32_t atom_bytes, uint32_t box_rows, uint32_t atoms,
+                  CUtensorMapSwizzle swizzle) {
+    const uint64_t dims[3] = {atom_bytes, rows, row_bytes / atom_bytes}, strides[2] = {row_bytes, atom_bytes};
+    const uint32_t box[3] = {atom_bytes, box_rows, atoms};
+    return encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, ptr, dims, strides, box, swizzle);
+}
+// ... and as [atom][K slice][row][byte]: a stacked tile's stage is one copy.
+bool encode_stacked(CUtensorMap* map, const void* ptr, uint64_t row_bytes, uint64_t rows, uint32_t atom_bytes, uint32_t box_rows, uint32_t atoms,
+                    CUtensorMapSwizzle swizzle) {
+    const uint64_t slice_bytes = row_bytes / kStackSlices;
+    const uint64_t dims[4] = {atom_bytes, rows, kStackSlices, slice_bytes / atom_bytes}, strides[3] = {row_bytes, slice_bytes, atom_bytes};
+    const uint32_t box[4] = {atom_bytes, box_rows, kStackSlices, atoms};
+    return encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, ptr, dims, strides, box, swizzle);
+}
+}  // namespace
+
 fq_status build_weight_tmap(Weights& W) {
     W.tmap_valid = false;
     if (W.N == 0) return FQ_OK;
@@ -1131,6 +1199,11 @@ fq_status build_weight_tmap(Weights& W) {
                         : encode_2d(&W.tmap, W.codes, (uint64_t)W.K, (uint64_t)W.N, kBlockK, kTileN,
                                     CU_TENSOR_MAP_SWIZZLE_128B);
     if (!ok) return FQ_ERR_CUDA;
+    if (W.bits == 4 && W.K % kBlockK == 0)
+        for (int i = 0; i < 2; ++i)
+            if (!encode_atoms(&W.tmap_atoms[i], W.codes, (uint64_t)W.K / 2, (uint64_t)W.N, kBlockK / 2, kTileN, 2u << i,
+                              CU_TENSOR_MAP_SWIZZLE_64B))
+                return FQ_ERR_CUDA;
     W.tmap_valid = true;
     build_stream_tmap(W);       // optional second view (short batches); shapes it does not fit go without
     return FQ_OK;
@@ -1191,7 +1264,7 @@ int cluster_capacity(int ctas) {
 // changes at run time.
 fq_status gemm_prepare(int64_t M, const Weights& W, void* scratch, size_t scratch_bytes, cudaStream_t stream) {
     if (M <= 0 || W.N == 0 || scratch == nullptr || gemm_stream_applies(M, W)) return FQ_OK;
-    const GemmPlan plan = plan_gemm(M, W.N, W.K, W.bits, device_sm_count(), scratch_bytes, true, cluster_capacity);
+    const GemmPlan plan = plan_call(M, W.N, W.K, W.bits, device_sm_count(), scratch_bytes, cluster_capacity);
     if (plan.split <= 1 || plan.cluster) return FQ_OK;
     return cudaMemsetAsync(scratch, 0, kCounterBytes, stream) == cudaSuccess ? FQ_OK : FQ_ERR_CUDA;
 }
@@ -1220,14 +1293,16 @@ fq_status launch_planned(const int8_t* a8, int64_t M, const Weights& W, int acc_
     Params p{};
     p.M = M; p.N = W.N; p.K = W.K;
     const int sms = device_sm_count();
-    const GemmPlan plan = plan_gemm(M, W.N, W.K, W.bits, sms, scratch ? scratch_bytes : 0, true, held);
-    const int bt = plan.bt, ctas = plan.ctas, split = plan.split;
+    const GemmPlan plan = plan_call(M, W.N, W.K, W.bits, sms, scratch ? scratch_bytes : 0, held);
+    const int bt = plan.bt, tok = bt / plan.stack, ctas = plan.ctas, split = plan.split;
     p.split = split;
     p.counters = static_cast<uint32_t*>(scratch);            // cleared by gemm_prepare()
     p.partials = reinterpret_cast<int32_t*>(static_cast<uint8_t*>(scratch) + kCounterBytes);
     p.bt = bt;
-    p.m_tiles = (int)((M + bt - 1) / bt);
-    p.n_tiles = (int)((W.N + kTileN * ctas - 1) / (kTileN * ctas));
+    p.tok = tok;
+    p.m_tiles = (int)((M + tok - 1) / tok);
+    const int n_step = plan.stack > 1 ? kStackRows : kTileN * ctas;
+    p.n_tiles = (int)((W.N + n_step - 1) / n_step);
     // Bands of 8 token tiles once the batch is long enough for the order to matter: a wave of 148 CTAs (74 pairs)
     // then covers 8 token tiles x 18 (9) channel tiles, close to the square that minimises the bytes it shares.
     p.band = p.m_tiles >= 16 ? 8 : p.m_tiles;
@@ -1247,14 +1322,22 @@ fq_status launch_planned(const int8_t* a8, int64_t M, const Weights& W, int acc_
 
     // each CTA of a pair loads its own half of the token tile
     CUtensorMap map_a;
-    if (!encode_2d(&map_a, a8, (uint64_t)W.K, (uint64_t)M, kBlockK, (uint32_t)(bt / ctas), CU_TENSOR_MAP_SWIZZLE_128B))
+    CUtensorMap map_stacked;
+    if (plan.stack > 1) {
+        if (!encode_stacked(&map_stacked, W.codes, (uint64_t)W.K / 2, (uint64_t)W.N, kBlockK / 2, kStackRows, (uint32_t)atoms, CU_TENSOR_MAP_SWIZZLE_64B) ||
+            !encode_stacked(&map_a, a8, (uint64_t)W.K, (uint64_t)M, kBlockK, (uint32_t)tok, (uint32_t)atoms, CU_TENSOR_MAP_SWIZZLE_128B))
+            return FQ_ERR_CUDA;
+    } else if (!(atoms > 1 ? encode_atoms(&map_a, a8, (uint64_t)W.K, (uint64_t)M, kBlockK, (uint32_t)bt, (uint32_t)atoms, CU_TENSOR_MAP_SWIZZLE_128B)
+                           : encode_2d(&map_a, a8, (uint64_t)W.K, (uint64_t)M, kBlockK, (uint32_t)(bt / ctas), CU_TENSOR_MAP_SWIZZLE_128B))) {
         return FQ_ERR_CUDA;
+    }
+    const CUtensorMap& map_w = plan.stack > 1 ? map_stacked : (atoms > 1 ? W.tmap_atoms[atoms == 4 ? 1 : 0] : W.tmap);
 
     // bf16 outputs of an unsplit launch leave through tiled bulk stores of [16 tokens x 32 channels] (64-byte rows,
     // 64-byte swizzle in shared memory); the copy engine clips what lies beyond M tokens or N channels
     CUtensorMap map_y;
     memset(&map_y, 0, sizeof(map_y));
-    if (out.acc == nullptr && out.yt == FQ_BF16 && split == 1 &&
+    if (out.acc == nullptr && out.yt == FQ_BF16 && split == 1 && plan.stack == 1 &&
         !encode_2d(&map_y, out.y, (uint64_t)W.N * 2, (uint64_t)M, 64, 16, CU_TENSOR_MAP_SWIZZLE_64B, (uint64_t)out.ldy * 2))
         return FQ_ERR_CUDA;
 
@@ -1266,21 +1349,23 @@ fq_status launch_planned(const int8_t* a8, int64_t M, const Weights& W, int acc_
     p.unit_step = clusters;
     p.units_q = num_units / clusters;
     p.units_rem = num_units % clusters;
-    p.kb_per = (int)(((W.K + kBlockK - 1) / kBlockK + atoms - 1) / atoms) / split;      // stages per unit; the planner only picks splits that divide it
+    p.kb_per = (int)(((W.K / plan.stack + kBlockK - 1) / kBlockK + atoms - 1) / atoms) / split;      // stages per unit; the planner only picks splits that divide it
     p.split_shift = split == 1 ? 0 : (split == 2 ? 1 : (split == 4 ? 2 : (split == 8 ? 3 : 4)));
 
     const int cluster = plan.cluster ? split * ctas : ctas;
     auto go = [&](auto bits, auto pair, auto atoms_c) -> fq_status {
         constexpr int B = decltype(bits)::value, C = decltype(pair)::value, A = decltype(atoms_c)::value;
-        if (split == 1) return launch_variant<B, C, kUnsplit, A>(map_a, W.tmap, map_y, p, grid, smem, cluster, stream, refused);
-        if (plan.cluster) return launch_variant<B, C, kSplitCluster, A>(map_a, W.tmap, map_y, p, grid, smem, cluster, stream, refused);
-        return launch_variant<B, C, kSplitScratch, A>(map_a, W.tmap, map_y, p, grid, smem, cluster, stream, refused);
+        if constexpr (B == 4 && A > 1)
+            if (plan.stack > 1) return launch_variant<B, C, kStacked, A>(map_a, map_w, map_y, p, grid, smem, cluster, stream, refused);
+        if (split == 1) return launch_variant<B, C, kUnsplit, A>(map_a, map_w, map_y, p, grid, smem, cluster, stream, refused);
+        if (plan.cluster) return launch_variant<B, C, kSplitCluster, A>(map_a, map_w, map_y, p, grid, smem, cluster, stream, refused);
+        return launch_variant<B, C, kSplitScratch, A>(map_a, map_w, map_y, p, grid, smem, cluster, stream, refused);
     };
     using I1 = std::integral_constant<int, 1>;
     using I2 = std::integral_constant<int, 2>;
     using I4 = std::integral_constant<int, 4>;
     using I8 = std::integral_constant<int, 8>;
-    if (W.bits == 4 && ctas == 2) return launch_variant<4, 2, kUnsplit>(map_a, W.tmap, map_y, p, grid, smem, cluster, stream, refused);
+    if (W.bits == 4 && ctas == 2) return launch_variant<4, 2, kUnsplit>(map_a, map_w, map_y, p, grid, smem, cluster, stream, refused);
     if (W.bits == 4) return atoms == 4 ? go(I4(), I1(), I4()) : (atoms == 2 ? go(I4(), I1(), I2()) : go(I4(), I1(), I1()));
     return ctas == 2 ? go(I8(), I2(), I1()) : go(I8(), I1(), I1());
 }

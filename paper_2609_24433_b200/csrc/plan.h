@@ -212,6 +212,29 @@ inline RingPlan plan_ring(int64_t rows, int64_t K, int elem_bytes, bool gated, b
     return f;
 }
 
+// ---- stacked tiles of the integer GEMM (gemm_tcgen05.cu) -----------------------------------------------------------------
+// Short batches on 4-bit matrices of too few channels leave SMs idle, and a split of K over CTAs pays for the exchange of sums.
+// A stacked tile splits K inside one MMA tile: its 128 rows are 64 channels at two slices of K, its columns the tokens at those
+// two slices; every row is multiplied with all columns, and only its own slice's count.  Twice the CTAs, each with half the
+// k-blocks, and the sums meet in the CTA.  Chains of calls, stacked / the best of the others, us:
+//   M <= 32   24 x 3072 x 2048 (M x K x N) 6.5 / 7.2;  32 x 3072 x 6144 6.6 / 7.4;  32 x 4096 x 2048 7.0 / 8.2;  16 x 4096 x 8192
+//             7.5 / 8.5;  32 x 4096 x 8192 8.0 / 8.3;  32 x 5120 x 4096 7.6 / 9.2;  32 x 6144 x 6144 8.5 / 10.5;  16 x 6144 x 8704
+//             10.1 / 11.6;  16 x 8192 x 8192 11.5 / 13.6;  32 x 8192 x 9472 12.2 / 12.8;  16 x 16384 x 8192 16.0 / 17.4
+//   behind    fewer channels, where clusters split K: 32 x 5120 x 2048 7.5 / 6.9, 32 x 8192 x 4096 9.7 / 8.9;  a short K: 32 x 2048
+//             x 8192 6.7 / 6.6;  a launch on all SMs, which leaves none to the next one: 16 x 4096 x 9472 8.9 / 8.1
+//   M <= 48   3072 x 4096 7.1 / 7.7, 4096 x 6144 8.1 / 9.0, 6144 x 6144 9.5 / 11.2;  behind 4096 x 2048 7.8 / 7.4, 6144 x 4096 9.3 / 8.8
+//   M <= 64   3072 x 4096 7.5 / 8.0, 4096 x 4096 8.2 / 9.1, 4096 x 6144 8.6 / 9.1;  behind 5120 x 4096 9.1 / 8.8, 6144 x 6144 10.7 / 10.0
+// (Four slices of 32 channels, 8-bit weights, whose operands pass through shared memory twice then, and longer batches are behind.)
+constexpr int kStackSlices = 2;
+inline bool stacked_applies(int64_t M, int64_t N, int64_t K, int bits, int sms) {
+    if (bits != 4 || M < 1 || M > 64 || K % 256 != 0 || K < 3072) return false;
+    if (M <= 32) {
+        const int64_t least = K <= 4096 ? 2048 : (2 * K / 3 < 5120 ? 2 * K / 3 : 5120);
+        return N >= least && N <= 64ll * (K >= 8192 ? sms : sms - 12);
+    }
+    return K <= (M <= 48 ? 6144 : 4096) && 4 * N >= 3 * K && N <= 7168 && N <= 64ll * (sms - 12);
+}
+
 // ---- integer product of short batches: the weight-streaming kernel (linear_wonly.cu) instead of the tcgen05 one ----------
 // (Rows of whole 128-byte lines only.)
 inline bool plan_stream(int64_t M, int64_t N, int64_t K, int bits, int sms) {
@@ -219,7 +242,13 @@ inline bool plan_stream(int64_t M, int64_t N, int64_t K, int bits, int sms) {
     // (N <= 32 x SMs: 16 x 4096 x 4096 (M x K x N) 7.0 us against 9.7), and with at most 8 tokens two rounds (8 x 4096 x 8192
     // 9.7 / 10.1; 16 x 4096 x 8192 13.5 / 10.1) -- every row group ends with a rendezvous and a reduction --, up to
     // 128 Mi weights for at most 8 tokens and 64 Mi for at most 16 (16 x 16384 x 8192: 23 us against 21 us).
+    // Long rows: the split of K by clusters is ahead with more than 8 tokens (4 / 8 bits, stream / clusters: 16 x 8192 x 2048 8.4 /
+    // 8.8 us and 9.5 / 9.8, 16 x 10240 x 2048 9.95 / 9.4 and 10.8 / 10.7, 16 x 16384 x 4096 15.1 / 12.7 and 18.3 / 16.7), and on few
+    // channels of 8 bits (1 x 10240 x 1024 9.6 / 8.9, x 2048 9.8 / 10.5; 8 x 16384 x 1024 14.2 / 11.3).  Two rounds of row groups:
+    // stacked tiles, where they apply (4 x 8192 x 8192 12.1 / 11.6, 8 x 6144 x 9472 11.5 / 10.8).
     if (K % (bits == 4 ? 256 : 128) != 0 || M < 1 || M > 16) return false;
+    if (K >= 10240 && (M > 8 || (bits == 8 && N <= 1024))) return false;
+    if (N > 32ll * sms && stacked_applies(M, N, K, bits, sms)) return false;
     // 8-bit weights (twice the bytes per row): ahead where the row groups make ONE round over the SMs, up to 64 Mi
     // weights (16 tokens, K = 8192, N = 4096: 12.8 us against 17.5 us; K = 4096, N = 8192: 14.0 against 11.5 us)
     if (bits == 8) return N <= 32ll * sms && N * K <= (1ll << 26);
@@ -251,6 +280,7 @@ struct GemmPlan {
     int ctas = 1;     // 2: CTA pairs on 256-channel tiles (cta_group::2)
     int split = 1;    // >1: every tile is that many work units, each on a slice of K
     bool cluster = false; // the slices of a tile are the CTAs of a cluster (no scratch)
+    int stack = 1;        // 2: a stacked tile, 64 channels at two slices of K (see stacked_applies); bt counts its columns
     size_t scratch = 0;   // bytes of scratch the split needs: the tile counters, then the int32 partial tiles
 };
 
@@ -354,6 +384,18 @@ GemmPlan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t sc
     return best;
 }
 
+inline size_t stacked_sums_bytes(int tok) { return (size_t)((tok / 16 + 1) / 2) * 16 * kTileN * sizeof(int32_t); }
+
+// The plan of a call: a stacked tile where they are the faster ones, else plan_gemm's.
+template <typename Held>
+GemmPlan plan_call(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t scratch_avail, Held held) {
+    if (!stacked_applies(M, N, K, bits, sms)) return plan_gemm(M, N, K, bits, sms, scratch_avail, true, held);
+    GemmPlan plan;
+    plan.bt = kStackSlices * (int)((M + 15) / 16 * 16);
+    plan.stack = kStackSlices;
+    return plan;
+}
+
 // The rings of a plan: slots of activations (and int8 weights, in lockstep), of packed and of unpacked 4-bit weights.
 struct GemmRings {
     bool fits = false;
@@ -364,9 +406,9 @@ struct GemmRings {
 inline GemmRings gemm_rings(const GemmPlan& plan, int bits, int64_t K) {
     GemmRings f;
     const int bt = plan.bt;
-    const bool split = plan.split > 1;
-    f.atoms = atoms_per_stage(bits, plan.ctas, bt, K, plan.split);
-    const size_t sums = plan.cluster ? cluster_sums_bytes(bt, plan.split) : 0, budget = ring_budget(bits, split, sums);
+    const bool split = plan.split > 1 || plan.stack > 1;
+    f.atoms = atoms_per_stage(bits, plan.ctas, bt, K / plan.stack, plan.split);
+    const size_t sums = plan.cluster ? cluster_sums_bytes(bt, plan.split) : (plan.stack > 1 ? stacked_sums_bytes(bt / plan.stack) : 0), budget = ring_budget(bits, split, sums);
     const size_t epi_bytes = (size_t)epi_warps(bits) * epi_stage_bytes(bits, split) + sums;
     const size_t a_bytes = (size_t)(bt / plan.ctas) * kBlockK * f.atoms, w_bytes = (size_t)kTileN * kBlockK, pk_bytes = w_bytes / 2 * f.atoms;
     // 4-bit weights: every TMEM column the accumulators leave free becomes unpacked-weight ring

@@ -199,6 +199,44 @@ def test_cluster_split_equals_the_second_witness(M, K, N, bits):
         assert torch.equal(a, want) and torch.equal(b, want)
 
 
+STACKED = [                # two K slices of 64 channels in one tile
+    (5, 3072, 4744),       # the shortest rows, two rounds of the streaming kernel's row groups, a ragged channel tile
+    (17, 3328, 2056),      # thirteen k-blocks per slice: a last stage of one
+    (32, 8192, 9472),      # a tile per SM
+    (30, 16384, 5120),     # two chunks of tokens, the last one ragged
+    (48, 6144, 7168),      # three: an uneven share
+    (64, 3328, 2504),      # the longest batch
+]
+
+
+@pytest.mark.parametrize("M,K,N", STACKED)
+def test_stacked_tiles_equal_the_second_witness(M, K, N):
+    """int32 sums, binary32 and bf16 outputs bit for bit, in a workspace of codes and steps only; a second call right behind the
+    first, and twenty replays over rotating weights, whose copies come from memory."""
+    g = torch.Generator(device="cuda").manual_seed(M + N)
+    hs = [fq.weights_import(torch.randint(0, 256, (N, K // 2), dtype=torch.uint8, device="cuda", generator=g),
+                            torch.rand(N, device="cuda", generator=g) + 0.1, None, torch.randn(N, device="cuda", generator=g), K, 64, 4)
+          for _ in range(8)]
+    h, x = hs[0], torch.randn(M, K, device="cuda", generator=g)
+    codes, delta = fq.quantize_act(x, None, 64, 4)
+    ws = torch.empty((M * K + 255) // 256 * 256 + (4 * M + 255) // 256 * 256, dtype=torch.uint8, device="cuda")
+    assert torch.equal(fq.gemm_acc_i32(codes, h, workspace=ws), fq.gemm_simt(codes, None, h, raw_acc=True))
+    for dt in (torch.float32, torch.bfloat16):
+        want = fq.gemm_simt(codes, delta, h, dt)
+        a, b = fq.linear(x, h, out_dtype=dt, workspace=ws), fq.linear(x, h, out_dtype=dt, workspace=ws)
+        assert torch.equal(a, want) and torch.equal(b, want)
+    want = [fq.gemm_simt(codes, delta, h, torch.bfloat16) for h in hs]
+    ys = [torch.empty_like(w) for w in want]
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for h, y in zip(hs, ys):
+            fq.linear(x, h, y=y, workspace=ws)
+    for _ in range(20):
+        graph.replay()
+        for y, w in zip(ys, want):
+            assert torch.equal(y, w)
+
+
 SCRATCH_SPLIT = [
     (75, 20480, 4624, 8),      # more tiles than the clusters that a device holds: slices meet in the workspace
     (17, 32768, 4640, 4),      # four-atom stages

@@ -212,3 +212,32 @@ def test_rings_of_every_plan_fit(plans, device):
                         if bits == 4:
                             assert p["stages_w"] <= p["stages"] and p["stages_w"] >= 2 and p["stages_p"] >= 2
                             assert p["stages_p"] % 2 == 0 or p["stages_p"] >= p["stages_w"] + 2 or p["slot_first"]
+
+
+CALLS = """
+#include "plan.h"
+struct Held { int operator()(int ctas) const { return ctas == 2 ? 74 : (ctas == 4 ? 33 : 14); } };
+// -> 100 * K slices of a stacked tile + atoms per stage, 0: another plan; -1: a plan that does not fit the SM
+extern "C" int stacked(long M, long N, long K, int bits, int sms) {
+    const fq::GemmPlan f = fq::plan_call(M, N, K, bits, sms, (size_t)-1, Held());
+    const fq::GemmRings r = fq::gemm_rings(f, bits, K);
+    if (!r.fits || r.smem > 227 * 1024 || r.tmem_cols > 512) return -1;
+    if (f.stack > 1 && (f.split > 1 || f.ctas > 1 || f.bt > 128 || fq::plan_stream(M, N, K, bits, sms))) return -2;
+    return f.stack > 1 ? 100 * f.stack + r.atoms : 0;
+}
+"""
+
+
+def test_stacked_tiles_and_their_lines(tmp_path):
+    lib = compile_host(tmp_path, "calls", CALLS)
+    call = lambda M, K, N, bits=4, sms=148: lib.stacked(ctypes.c_long(M), ctypes.c_long(N), ctypes.c_long(K), bits, sms)
+    assert [call(*c) for c in edges.STACKED] == [204, 204, 204, 204, 202, 202]
+    for inside, outside in [((32, 3072, 2048), (32, 2816, 2048)), ((32, 4096, 2048), (32, 4096, 2040)), ((32, 4096, 8704), (32, 4096, 8712)),
+                            ((32, 6144, 4096), (32, 6144, 4088)), ((16, 16384, 5120), (16, 16384, 5112)), ((32, 8192, 9472), (32, 8192, 9480)),
+                            ((48, 6144, 4608), (49, 6144, 4608)), ((64, 4096, 7168), (64, 4096, 7176)), ((64, 4096, 3072), (65, 4096, 3072))]:
+        assert call(*inside) > 200 and call(*outside) == 0, (inside, outside)
+    for M in (1, 16, 17, 32, 33, 48, 49, 64):
+        for K in (3072, 3328, 4096, 8448, 16384):
+            for N in (8, 136, 2048, 4744, 7168, 8704, 9472):
+                for sms in (16, 148):
+                    assert call(M, K, N, 8, sms) == 0 and (call(M, K, N, 4, sms) >= 0 or N <= 32 * sms), (M, K, N, sms)
