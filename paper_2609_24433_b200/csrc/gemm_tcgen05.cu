@@ -259,8 +259,6 @@ __device__ __forceinline__ uint32_t scale_pair_bf16(uint32_t a0, uint32_t a1, fl
     return w;
 }
 
-constexpr int kSumBytes = 16 * 32 * 4;                   // cluster split: a warp's sums of one token chunk
-
 enum : uint32_t {
     kWdProducer = 1u, kWdMmaFull = 2u, kWdMmaAcc = 4u, kWdEpilogue = 8u, kWdUnpackFull = 16u,
     kWdUnpackEmpty = 32u, kWdDrain = 64u, kWdPartials = 128u

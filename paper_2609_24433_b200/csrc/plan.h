@@ -283,6 +283,11 @@ struct GemmPlan {
     int stack = 1;        // 2: a stacked tile, 64 channels at two slices of K (see stacked_applies); bt counts its columns
     size_t scratch = 0;   // bytes of scratch the split needs: the tile counters, then the int32 partial tiles
 };
+inline GemmPlan cluster_plan(int bt, int ctas, int split) {
+    GemmPlan plan;
+    plan.bt = bt; plan.ctas = ctas; plan.split = split; plan.cluster = true;
+    return plan;
+}
 
 // Atoms (of 128 channels) per pipeline stage.  4-bit weights, single CTAs: two for token tiles of at most 128, four for the
 // shortest (the accumulators of longer tiles leave no room for wider TMEM slots); whole atoms, slices of whole stages.
@@ -302,6 +307,69 @@ inline size_t stage_bytes(int bits, int ctas, int bt, int atoms) {
     return ((size_t)(bt / ctas) * kBlockK + (size_t)kTileN * kBlockK * bits / 8) * atoms;
 }
 inline size_t cluster_sums_bytes(int bt, int split) { return (size_t)(split - 1) * ((bt / 16 + split - 1) / split) * 16 * kTileN * sizeof(int32_t); }
+
+inline size_t stacked_sums_bytes(int tok) { return (size_t)((tok / 16 + 1) / 2) * 16 * kTileN * sizeof(int32_t); }
+// Bytes of the ring's memory that a CTA of a cluster split stages the sums in which it sends: the n-th chunk that a warp sends lies at
+// [n][warp], and a warp sends every (warps / 4)-th chunk of 16 tokens but those that its own slice finishes.
+constexpr int kSumBytes = 16 * 32 * 4;                   // a warp's sums of one token chunk
+inline size_t staged_sums_bytes(int bits, int bt, int split) {
+    const int warps = epi_warps(bits), sets = warps / 4;
+    int top = 0;
+    for (int slice = 0; slice < split; ++slice)
+        for (int set = 0; set < sets; ++set) {
+            int sent = 0;
+            for (int c = set; c < bt / 16; c += sets) sent += (c & (split - 1)) != slice;
+            if (sent > 0 && (sent - 1) * warps + 4 * (set + 1) > top) top = (sent - 1) * warps + 4 * (set + 1);
+        }
+    return (size_t)top * kSumBytes;
+}
+
+// The rings of a plan: slots of activations (and int8 weights, in lockstep), of packed and of unpacked 4-bit weights.
+struct GemmRings {
+    bool fits = false;
+    int atoms = 1, stages = 0, stages_p = 0, stages_w = 0, tmem_cols = 0;
+    bool slot_first = false;           // the unpack sets wait for the TMEM slot ahead of the packed stage (see the kernel)
+    size_t smem = 0;
+};
+inline GemmRings gemm_rings(const GemmPlan& plan, int bits, int64_t K) {
+    GemmRings f;
+    const int bt = plan.bt;
+    const bool split = plan.split > 1 || plan.stack > 1;
+    f.atoms = atoms_per_stage(bits, plan.ctas, bt, K / plan.stack, plan.split);
+    const size_t sums = plan.cluster ? cluster_sums_bytes(bt, plan.split) : (plan.stack > 1 ? stacked_sums_bytes(bt / plan.stack) : 0), budget = ring_budget(bits, split, sums);
+    const size_t epi_bytes = (size_t)epi_warps(bits) * epi_stage_bytes(bits, split) + sums;
+    const size_t a_bytes = (size_t)(bt / plan.ctas) * kBlockK * f.atoms, w_bytes = (size_t)kTileN * kBlockK, pk_bytes = w_bytes / 2 * f.atoms;
+    // 4-bit weights: every TMEM column the accumulators leave free becomes unpacked-weight ring
+    f.stages_w = bits == 4 ? (512 - kAccStages * bt) / (kColsW * f.atoms) : 0;
+    if (f.stages_w > kMaxStagesW) f.stages_w = kMaxStagesW;
+    for (f.tmem_cols = 32; f.tmem_cols < kAccStages * bt + f.stages_w * kColsW * f.atoms;) f.tmem_cols <<= 1;
+    if (bits == 4) {
+        // Both TMA rings need the same look-ahead in k-blocks (their latencies are the same): split the budget evenly, then
+        // give the remainder to the cheaper packed ring.
+        f.stages = (int)(budget / (a_bytes + pk_bytes));
+        if (f.stages > kMaxStages) f.stages = kMaxStages;
+        if (f.stages < 2) return f;
+        f.stages_p = (int)((budget - f.stages * a_bytes) / pk_bytes);
+        if (f.stages_p > kMaxStagesP) f.stages_p = kMaxStagesP;
+        if (f.stages_w > f.stages) f.stages_w = f.stages;       // the unpack warps wait on the activation ring's barriers
+        // (a ring one shorter is slower, one TMEM slot less no faster: 128 x 4096 x 4096 10.5, 11.3 and 10.4 us, 256 x 2048 x
+        // 4096 9.95, 10.1 and 9.9)
+        f.slot_first = f.stages_p % kUnpackSets != 0 && f.stages_p < f.stages_w + kUnpackSets;
+        if (f.slot_first && f.stages_w > f.stages_p) return f;
+        f.smem = f.stages * a_bytes + f.stages_p * pk_bytes + epi_bytes + 1024;
+    } else {
+        f.stages = (int)(budget / (a_bytes + w_bytes));
+        if (f.stages > kMaxStages) f.stages = kMaxStages;
+        if (f.stages < 2) return f;
+        f.smem = (a_bytes + w_bytes) * f.stages + epi_bytes + 1024;
+    }
+    if (plan.cluster && staged_sums_bytes(bits, bt, plan.split) > f.smem - epi_bytes - 1024) return f;
+    // One CTA of this kind per SM, and none of the short-batch kernel beside it: a cluster whose CTA waited for tensor memory
+    // must not be what another cluster on that SM waits for (launches of two streams).
+    if (plan.cluster && f.smem < 152 * 1024) f.smem = 152 * 1024;
+    f.fits = true;
+    return f;
+}
 
 // Token tile, CTA grouping and K split.  Upper bound of the tile from TMEM: two accumulator stages,
 // plus the unpacked-weight ring for 4-bit weights (2*bt + 3*32 <= 512 columns).  M is split evenly
@@ -372,7 +440,8 @@ GemmPlan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t sc
                 const int atoms = atoms_per_stage(bits, c, b, K, sp);
                 const double ctas = (double)(units * sp * c);
                 if (clusters && (bits == 8 || b <= 128) && sp * c <= kMaxCluster && units * sp <= slots &&
-                    ring_budget(bits, true, cluster_sums_bytes(b, sp)) * atoms >= 4 * stage_bytes(bits, c, b, atoms) && units <= holds(sp * c))
+                    ring_budget(bits, true, cluster_sums_bytes(b, sp)) * atoms >= 4 * stage_bytes(bits, c, b, atoms) &&
+                    gemm_rings(cluster_plan(b, c, sp), bits, K).fits && units <= holds(sp * c))
                     offer(sp, true, 0, slice + 16.0 * b / sp + (bits == 4 ? 2800.0 + 40.0 * ctas : 3300.0 + 18.0 * ctas) + 500.0 * (sp - 1));
                 if ((c == 1 || bits == 8) && units * c <= kMaxSplitTiles && units * c * sp <= 4 * (int64_t)sms) {
                     const size_t scratch = kCounterBytes + (size_t)units * c * sp * kTileN * b * sizeof(int32_t);
@@ -384,8 +453,6 @@ GemmPlan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t sc
     return best;
 }
 
-inline size_t stacked_sums_bytes(int tok) { return (size_t)((tok / 16 + 1) / 2) * 16 * kTileN * sizeof(int32_t); }
-
 // The plan of a call: a stacked tile where they are the faster ones, else plan_gemm's.
 template <typename Held>
 GemmPlan plan_call(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t scratch_avail, Held held) {
@@ -394,55 +461,6 @@ GemmPlan plan_call(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t sc
     plan.bt = kStackSlices * (int)((M + 15) / 16 * 16);
     plan.stack = kStackSlices;
     return plan;
-}
-
-// The rings of a plan: slots of activations (and int8 weights, in lockstep), of packed and of unpacked 4-bit weights.
-struct GemmRings {
-    bool fits = false;
-    int atoms = 1, stages = 0, stages_p = 0, stages_w = 0, tmem_cols = 0;
-    bool slot_first = false;           // the unpack sets wait for the TMEM slot ahead of the packed stage (see the kernel)
-    size_t smem = 0;
-};
-inline GemmRings gemm_rings(const GemmPlan& plan, int bits, int64_t K) {
-    GemmRings f;
-    const int bt = plan.bt;
-    const bool split = plan.split > 1 || plan.stack > 1;
-    f.atoms = atoms_per_stage(bits, plan.ctas, bt, K / plan.stack, plan.split);
-    const size_t sums = plan.cluster ? cluster_sums_bytes(bt, plan.split) : (plan.stack > 1 ? stacked_sums_bytes(bt / plan.stack) : 0), budget = ring_budget(bits, split, sums);
-    const size_t epi_bytes = (size_t)epi_warps(bits) * epi_stage_bytes(bits, split) + sums;
-    const size_t a_bytes = (size_t)(bt / plan.ctas) * kBlockK * f.atoms, w_bytes = (size_t)kTileN * kBlockK, pk_bytes = w_bytes / 2 * f.atoms;
-    // 4-bit weights: every TMEM column the accumulators leave free becomes unpacked-weight ring
-    f.stages_w = bits == 4 ? (512 - kAccStages * bt) / (kColsW * f.atoms) : 0;
-    if (f.stages_w > kMaxStagesW) f.stages_w = kMaxStagesW;
-    for (f.tmem_cols = 32; f.tmem_cols < kAccStages * bt + f.stages_w * kColsW * f.atoms;) f.tmem_cols <<= 1;
-    if (bits == 4) {
-        // Both TMA rings need the same look-ahead in k-blocks (their latencies are the same): split the budget evenly, then
-        // give the remainder to the cheaper packed ring.
-        f.stages = (int)(budget / (a_bytes + pk_bytes));
-        if (f.stages > kMaxStages) f.stages = kMaxStages;
-        if (f.stages < 2) return f;
-        f.stages_p = (int)((budget - f.stages * a_bytes) / pk_bytes);
-        if (f.stages_p > kMaxStagesP) f.stages_p = kMaxStagesP;
-        if (f.stages_w > f.stages) f.stages_w = f.stages;       // the unpack warps wait on the activation ring's barriers
-        // (a ring one shorter is slower, one TMEM slot less no faster: 128 x 4096 x 4096 10.5, 11.3 and 10.4 us, 256 x 2048 x
-        // 4096 9.95, 10.1 and 9.9)
-        f.slot_first = f.stages_p % kUnpackSets != 0 && f.stages_p < f.stages_w + kUnpackSets;
-        if (f.slot_first && f.stages_w > f.stages_p) return f;
-        f.smem = f.stages * a_bytes + f.stages_p * pk_bytes + epi_bytes + 1024;
-    } else {
-        f.stages = (int)(budget / (a_bytes + w_bytes));
-        if (f.stages > kMaxStages) f.stages = kMaxStages;
-        if (f.stages < 2) return f;
-        f.smem = (a_bytes + w_bytes) * f.stages + epi_bytes + 1024;
-    }
-    // (The sums that a cluster split sends on are staged in the ring's memory, 2 KB per epilogue warp and chunk.)
-    const int warps = epi_warps(bits);
-    if (plan.cluster && (size_t)((bt / 16 + warps / 4 - 1) / (warps / 4)) * warps * 2048 > f.smem - epi_bytes - 1024) return f;
-    // One CTA of this kind per SM, and none of the short-batch kernel beside it: a cluster whose CTA waited for tensor memory
-    // must not be what another cluster on that SM waits for (launches of two streams).
-    if (plan.cluster && f.smem < 152 * 1024) f.smem = 152 * 1024;
-    f.fits = true;
-    return f;
 }
 
 }  // namespace fq

@@ -179,6 +179,8 @@ CLUSTER_SPLIT = [
     (250, 16384, 128, 8),
     (816, 16384, 2048, 8),     # CTA pairs, clusters of two pairs
     (790, 16384, 1960, 8),     # ... with ragged tokens and channels
+    (900, 16384, 2048, 8),     # ... tiles of 240 tokens: fifteen chunks, the most that a pair stages beside a ring of four
+    (240, 8192, 8192, 8),
 ]
 
 

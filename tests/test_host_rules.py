@@ -83,16 +83,16 @@ extern "C" int ring(long M, long K, int elem, int gated, int bytes_out, int mult
 extern "C" void gemm(long M, long N, long K, int bits, long scratch, int sms, int c2, int c4, int c8, int* out) {
     const Held held{c2, c4, c8};
     const size_t asks = fq::plan_gemm(M, N, K, bits, sms, (size_t)-1, false, held).scratch;
-    const fq::GemmPlan f = fq::plan_gemm(M, N, K, bits, sms, scratch < 0 ? asks : (size_t)scratch, true, held);
+    const fq::GemmPlan f = fq::plan_call(M, N, K, bits, sms, scratch < 0 ? asks : (size_t)scratch, held);
     const fq::GemmRings r = fq::gemm_rings(f, bits, K);
     const int v[] = {fq::plan_stream(M, N, K, bits, sms), f.bt, f.ctas, f.split, f.cluster, f.scratch > 0, r.fits, r.atoms, r.stages,
-                     r.stages_p, r.stages_w, r.slot_first, (int)r.smem, r.tmem_cols};
-    for (int i = 0; i < 14; ++i) out[i] = v[i];
+                     r.stages_p, r.stages_w, r.slot_first, (int)r.smem, r.tmem_cols, f.stack};
+    for (int i = 0; i < 15; ++i) out[i] = v[i];
 }
 """
 B200 = (148, 74, 36, 14)       # multiprocessors, clusters of 2, 4 and 8 CTAs that one whole device holds
 WHOLE = [B200, (148, 74, 33, 15)]                        # ... and another, whose SMs are grouped otherwise
-GEMM = "stream bt ctas split cluster scratch fits atoms stages stages_p stages_w slot_first smem tmem_cols".split()
+GEMM = "stream bt ctas split cluster scratch fits atoms stages stages_p stages_w slot_first smem tmem_cols stack".split()
 
 
 class Plans:
@@ -212,6 +212,17 @@ def test_rings_of_every_plan_fit(plans, device):
                         if bits == 4:
                             assert p["stages_w"] <= p["stages"] and p["stages_w"] >= 2 and p["stages_p"] >= 2
                             assert p["stages_p"] % 2 == 0 or p["stages_p"] >= p["stages_w"] + 2 or p["slot_first"]
+
+
+@pytest.mark.parametrize("device", WHOLE + [(16, 8, 0, 0)])
+def test_every_token_count_has_a_plan_that_fits(plans, device):
+    """Each tile height there is, 16 to 256 tokens, with the last token of a tile and the first of the next one."""
+    for bits in (4, 8):
+        for K in (2048, 5120, 8192, 10496, 16384):
+            for N in (1024, 2048, 2560, 4096, 6400, 8192):
+                for M in [m for t in range(16, 1041, 16) for m in (t - 15, t - 1, t, t + 1)]:
+                    p = plans.gemm(M, K, N, bits, device=device)
+                    assert p["fits"] and p["smem"] <= 227 * 1024 and p["tmem_cols"] <= 512, (M, K, N, bits, p)
 
 
 CALLS = """
