@@ -381,6 +381,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             const int chunks = min(p.bt / 16, (int)min((left + 15) / 16, (int64_t)16));
             mbar_arrive_expect_tx(smem_u32(&s_sums), (uint32_t)((split - 1) * ((chunks - slice + split - 1) >> split_shift) * 4 * kSumBytes));
         }
+        __syncwarp();                               // (the arrival is the converged warp's)
         cluster_arrive();                           // "this CTA exists": awaited before the first copy to another
     }
     tc_fence_after();
@@ -1088,7 +1089,9 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         const bool finishes = warp >= 2 && warp < 2 + kEpiWarps && ok && unit0 < num_units;
         if (finishes) ok = mbar_wait_all(smem_u32(&s_sums), 0u, abort_flag, p.watchdog, kWdPartials);
         __syncwarp();
-        cluster_arrive_relaxed();                    // "this CTA has its sums": no copy is under way when everybody has said so
+        // "this CTA has its sums": no copy is under way when everybody has said so.  (Pairs say it at the end, behind their last read
+        // of tensor memory.)
+        if (CTAS == 1) cluster_arrive_relaxed();
         if (finishes && ok) {
             const int quad = warp & 3, half = (warp - 2) >> 2, slice = unit0 & (split - 1);
             const int tile = tile_of(unit0);
@@ -1118,8 +1121,10 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     // ------------------------------------------------------------------ teardown
     tc_fence_before();
     __syncthreads();
-    if (kCluster) cluster_wait();                   // nobody leaves while its own copies may still be under way
-    else if (CTAS == 2) cluster_sync_all();         // neither CTA leaves while the other may still signal it
+    // Nobody leaves while its own copies may still be under way.  Pairs free their tensor memory together, with both CTAs present and
+    // neither reading it any more, and neither leaves while the other may still signal it.
+    if (CTAS == 2) cluster_sync_all();
+    else if (kCluster) cluster_wait();
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc<CTAS>(tmem_base, (uint32_t)p.tmem_cols);

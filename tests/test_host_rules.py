@@ -225,6 +225,18 @@ def test_every_token_count_has_a_plan_that_fits(plans, device):
                     assert p["fits"] and p["smem"] <= 227 * 1024 and p["tmem_cols"] <= 512, (M, K, N, bits, p)
 
 
+def test_ctas_of_a_pair_meet_between_their_last_read_of_tensor_memory_and_its_deallocation():
+    """A pair's allocation is given back by both CTAs together: whatever else the kernel's end does, a barrier of the whole cluster,
+    arrival and wait, lies between the outputs and the deallocation.  Its aligned arrivals are made by converged warps."""
+    with open(os.path.join(CSRC, "gemm_tcgen05.cu")) as f:
+        kernel = f.read().split("gemm_tcgen05_kernel(", 1)[1].split("// ---- host side", 1)[0]
+    end = [line.split("//")[0].strip() for line in kernel[kernel.rindex("emit("):kernel.index("tmem_dealloc<CTAS>")].splitlines()]
+    assert "if (CTAS == 2) cluster_sync_all();" in end and end.index("__syncthreads();") < end.index("if (CTAS == 2) cluster_sync_all();")
+    lines = [line.split("//")[0].strip() for line in kernel.splitlines()]
+    lines = [line for line in lines if line]
+    assert lines[lines.index("cluster_arrive();") - 1] == "__syncwarp();" == lines[lines.index("if (CTAS == 1) cluster_arrive_relaxed();") - 1]
+
+
 CALLS = """
 #include "plan.h"
 struct Held { int operator()(int ctas) const { return ctas == 2 ? 74 : (ctas == 4 ? 33 : 14); } };
