@@ -136,7 +136,8 @@ cudaError_t launch_gemm_simt(const int8_t* a8, int64_t M, const Weights& W, int 
 //  - launch_linear_wonly4: weight-only projection of float activations, y = s^W (qW x) + b;
 //  - launch_gemm_stream: the integer product + epilogue of the GEMM for batches gemm_stream_applies() accepts.
 bool build_stream_tmap(Weights& W);
-bool gemm_stream_applies(int64_t M, const Weights& W);
+// (`held`: clusters that the device holds, by CTAs per cluster.)
+bool gemm_stream_applies(int64_t M, const Weights& W, int (*held)(int) = cluster_capacity);
 cudaError_t launch_gemm_stream(const int8_t* a8, int64_t M, const Weights& W, int acc_shift, const GemmOut& out,
                                cudaStream_t stream);
 cudaError_t launch_linear_wonly4(const void* x, fq_dtype xt, int64_t M, int64_t ldx, const Weights& W, void* y,

@@ -1382,6 +1382,8 @@ fq_status launch_gemm_tcgen05(const int8_t* a8, int64_t M, const Weights& W, int
     bool refused = false;
     const fq_status st = launch_planned(a8, M, W, acc_shift, out, scratch, scratch_bytes, cluster_capacity, stream, &refused);
     // (without scratch: gemm_prepare() cleared the counters of the plan that was refused, if any)
+    if (refused && gemm_stream_applies(M, W, no_clusters))
+        return launch_gemm_stream(a8, M, W, acc_shift, out, stream) == cudaSuccess ? FQ_OK : FQ_ERR_CUDA;
     return refused ? launch_planned(a8, M, W, acc_shift, out, nullptr, 0, no_clusters, stream, &refused) : st;
 }
 

@@ -500,8 +500,8 @@ bool build_stream_tmap(Weights& W) {
     return W.tmap_stream_valid;
 }
 
-bool gemm_stream_applies(int64_t M, const Weights& W) {
-    return W.tmap_stream_valid && plan_stream(M, W.N, W.K, W.bits, device_sm_count());
+bool gemm_stream_applies(int64_t M, const Weights& W, int (*held)(int)) {
+    return W.tmap_stream_valid && plan_stream(M, W.N, W.K, W.bits, device_sm_count(), held);
 }
 
 cudaError_t launch_gemm_stream(const int8_t* a8, int64_t M, const Weights& W, int acc_shift, const GemmOut& out,

@@ -235,27 +235,6 @@ inline bool stacked_applies(int64_t M, int64_t N, int64_t K, int bits, int sms) 
     return K <= (M <= 48 ? 6144 : 4096) && 4 * N >= 3 * K && N <= 7168 && N <= 64ll * (sms - 12);
 }
 
-// ---- integer product of short batches: the weight-streaming kernel (linear_wonly.cu) instead of the tcgen05 one ----------
-// (Rows of whole 128-byte lines only.)
-inline bool plan_stream(int64_t M, int64_t N, int64_t K, int bits, int sms) {
-    // Measured against the tcgen05 kernel, operands from memory: ahead wherever the row groups make one round over the SMs
-    // (N <= 32 x SMs: 16 x 4096 x 4096 (M x K x N) 7.0 us against 9.7), and with at most 8 tokens two rounds (8 x 4096 x 8192
-    // 9.7 / 10.1; 16 x 4096 x 8192 13.5 / 10.1) -- every row group ends with a rendezvous and a reduction --, up to
-    // 128 Mi weights for at most 8 tokens and 64 Mi for at most 16 (16 x 16384 x 8192: 23 us against 21 us).
-    // Long rows: the split of K by clusters is ahead with more than 8 tokens (4 / 8 bits, stream / clusters: 16 x 8192 x 2048 8.4 /
-    // 8.8 us and 9.5 / 9.8, 16 x 10240 x 2048 9.95 / 9.4 and 10.8 / 10.7, 16 x 16384 x 4096 15.1 / 12.7 and 18.3 / 16.7), and on few
-    // channels of 8 bits (1 x 10240 x 1024 9.6 / 8.9, x 2048 9.8 / 10.5; 8 x 16384 x 1024 14.2 / 11.3).  Two rounds of row groups:
-    // stacked tiles, where they apply (4 x 8192 x 8192 12.1 / 11.6, 8 x 6144 x 9472 11.5 / 10.8).
-    if (K % (bits == 4 ? 256 : 128) != 0 || M < 1 || M > 16) return false;
-    if (K >= 10240 && (M > 8 || (bits == 8 && N <= 1024))) return false;
-    if (N > 32ll * sms && stacked_applies(M, N, K, bits, sms)) return false;
-    // 8-bit weights (twice the bytes per row): ahead where the row groups make ONE round over the SMs, up to 64 Mi
-    // weights (16 tokens, K = 8192, N = 4096: 12.8 us against 17.5 us; K = 4096, N = 8192: 14.0 against 11.5 us)
-    if (bits == 8) return N <= 32ll * sms && N * K <= (1ll << 26);
-    if (N > (M <= 8 ? 64ll : 32ll) * sms) return false;
-    return N * K <= (M <= 8 ? (1ll << 27) : (1ll << 26));
-}
-
 // ---- integer GEMM (gemm_tcgen05.cu) ------------------------------------------------------------------------------------
 constexpr int kBlockK = 128;           // int8 elements (= bytes) of K per pipeline stage
 constexpr int kAccStages = 2;
@@ -451,6 +430,41 @@ GemmPlan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t sc
         }
     }
     return best;
+}
+
+// ---- integer product of short batches: the weight-streaming kernel (linear_wonly.cu) instead of the tcgen05 one ----------
+// (Rows of whole 128-byte lines only.)  Chains of calls, operands from memory, stream / the other kernel, M x K x N, us.
+// One round of row groups over the SMs (N <= 32 x SMs): ahead (16 x 4096 x 4096 7.0 / 9.7), up to 64 Mi weights.  8-bit weights:
+// 16 x 8192 x 4096 10.4 / 10.3 in a chain, and 0.55 us ahead between unrelated calls; 16 x 4096 x 8192, two rounds, 14.0 / 11.5.
+//   Long rows: behind a split of K into four or more slices by clusters -- where the plan has one: 16 x 16384 x 4096 15.2 / 12.6 at 4 bits
+//   and 18.5 / 16.9 at 8, 16 x 10240 x 2048 10.0 / 9.4 and 10.9 / 10.9, 16 x 10752 x 2048 at 8 bits 11.4 / 11.0.  Ahead of everything
+//   else, which is what widths with fewer factors of two get: 16 x 10496 x 4096 (two slices) 12.1 / 16.7 and 13.6 / 15.1, 16 x 16256 x
+//   4096 (none) at 8 bits 18.1 / 32.0.  At 4 bits the slices have to be whole stages of two atoms (16 x 10752 x 4096 11.9 / 12.5),
+//   and up to 12 tokens the rows 12288 channels (12 x 10240 x 2048 9.2 / 9.5, 12 x 12288 x 4096 11.75 / 11.3).  At most 8 tokens: on 8 bits
+//   and eight slices only (8 x 10240 x 1024 10.0 / 9.2, 8 x 16384 x 1024 14.2 / 11.3; four: 8 x 16384 x 2048 14.3 / 14.2).
+// Two rounds, at most 8 tokens on 4 bits, up to 128 Mi weights: ahead of plain tiles (8 x 4096 x 8192 9.7 / 10.1; 16 x 4096 x 8192
+//   13.5 / 10.1: every row group ends with a rendezvous and a reduction), behind stacked ones with 5 tokens and more
+//   (8 x 4096 x 8192 8.5 / 7.4, 5 x 8704 x 9216 13.7 / 13.1).  With fewer the streamed calls are shorter, and ahead (1 x 4096 x
+//   8192 7.05 / 7.7, 2 x 6144 x 8192 10.2 / 10.5, 1 x 12288 x 9472 15.2 / 15.4) but for long rows (1 x 7168 x 7168 11.0 / 10.4,
+//   4 x 8192 x 8192 12.3 / 11.8, 1 x 16384 x 5120 16.8 / 14.7) and where a stacked tile has few stages (4 x 3072 x 5120 6.3 / 5.95, 3 x 4096 x
+//   7168 7.55 / 7.1).
+inline bool stacked_beats_stream(int64_t M, int64_t N, int64_t K) {
+    if (M > 4) return true;
+    if (K >= 7168) return N <= (K >= 8192 ? 8192 : 7168);
+    return K == 3072 ? N <= 6144 : (M >= 3 && K >= 3840 && K <= 4096 && N <= 7168);
+}
+// `held`: as for plan_gemm.
+template <typename Held>
+bool plan_stream(int64_t M, int64_t N, int64_t K, int bits, int sms, Held held) {
+    if (K % (bits == 4 ? 256 : 128) != 0 || M < 1 || M > 16) return false;
+    const int64_t rounds = (N + 32ll * sms - 1) / (32ll * sms);
+    if (rounds > (bits == 4 && M <= 8 ? 2 : 1) || N * K > (bits == 4 && M <= 8 ? 1ll << 27 : 1ll << 26)) return false;
+    if (rounds == 2) return !(stacked_applies(M, N, K, bits, sms) && stacked_beats_stream(M, N, K));
+    // (no plan is made where its answer would change nothing: it is the host's time)
+    const bool ask = K >= 10240 && (bits == 8 ? (M > 8 || N <= 1024) : (M > 8 && K % 1024 == 0 && (M > 12 || K >= 12288)));
+    if (!ask) return true;
+    const GemmPlan plan = plan_gemm(M, N, K, bits, sms, 0, true, held);
+    return !(plan.cluster && plan.split >= (M > 8 ? 4 : 8));
 }
 
 // The plan of a call: a stacked tile where they are the faster ones, else plan_gemm's.

@@ -85,7 +85,7 @@ extern "C" void gemm(long M, long N, long K, int bits, long scratch, int sms, in
     const size_t asks = fq::plan_gemm(M, N, K, bits, sms, (size_t)-1, false, held).scratch;
     const fq::GemmPlan f = fq::plan_call(M, N, K, bits, sms, scratch < 0 ? asks : (size_t)scratch, held);
     const fq::GemmRings r = fq::gemm_rings(f, bits, K);
-    const int v[] = {fq::plan_stream(M, N, K, bits, sms), f.bt, f.ctas, f.split, f.cluster, f.scratch > 0, r.fits, r.atoms, r.stages,
+    const int v[] = {fq::plan_stream(M, N, K, bits, sms, held), f.bt, f.ctas, f.split, f.cluster, f.scratch > 0, r.fits, r.atoms, r.stages,
                      r.stages_p, r.stages_w, r.slot_first, (int)r.smem, r.tmem_cols, f.stack};
     for (int i = 0; i < 15; ++i) out[i] = v[i];
 }
@@ -237,30 +237,56 @@ def test_ctas_of_a_pair_meet_between_their_last_read_of_tensor_memory_and_its_de
     assert lines[lines.index("cluster_arrive();") - 1] == "__syncwarp();" == lines[lines.index("if (CTAS == 1) cluster_arrive_relaxed();") - 1]
 
 
-CALLS = """
-#include "plan.h"
-struct Held { int operator()(int ctas) const { return ctas == 2 ? 74 : (ctas == 4 ? 33 : 14); } };
-// -> 100 * K slices of a stacked tile + atoms per stage, 0: another plan; -1: a plan that does not fit the SM
-extern "C" int stacked(long M, long N, long K, int bits, int sms) {
-    const fq::GemmPlan f = fq::plan_call(M, N, K, bits, sms, (size_t)-1, Held());
-    const fq::GemmRings r = fq::gemm_rings(f, bits, K);
-    if (!r.fits || r.smem > 227 * 1024 || r.tmem_cols > 512) return -1;
-    if (f.stack > 1 && (f.split > 1 || f.ctas > 1 || f.bt > 128 || fq::plan_stream(M, N, K, bits, sms))) return -2;
-    return f.stack > 1 ? 100 * f.stack + r.atoms : 0;
-}
-"""
+def route(plans, M, K, N, bits, device=None):
+    """What runs the integer product of a call: the streaming kernel, a stacked tile, else how K is split."""
+    p = plans.gemm(M, K, N, bits, device=device)
+    assert p["fits"] and p["smem"] <= 227 * 1024 and p["tmem_cols"] <= 512, (M, K, N, bits, p)
+    if p["stream"]:
+        return "stream"
+    if p["stack"] > 1:
+        # one tile per CTA, and no second one behind it
+        assert p["split"] == 1 and p["ctas"] == 1 and p["bt"] <= 128 and M <= p["bt"] // p["stack"] and N <= 64 * (device or plans.device)[0]
+        return "stacked, %d atoms" % p["atoms"]
+    return "%d %s" % (p["split"], "by clusters" if p["cluster"] else "tiles") if p["split"] > 1 else "tiles"
 
 
-def test_stacked_tiles_and_their_lines(tmp_path):
-    lib = compile_host(tmp_path, "calls", CALLS)
-    call = lambda M, K, N, bits=4, sms=148: lib.stacked(ctypes.c_long(M), ctypes.c_long(N), ctypes.c_long(K), bits, sms)
-    assert [call(*c) for c in edges.STACKED] == [204, 204, 204, 204, 202, 202]
+def test_stacked_tiles_and_their_lines(plans):
+    call = lambda M, K, N, bits=4, device=None: route(plans, M, K, N, bits, device)
+    assert [call(*c)[-7:] for c in edges.STACKED] == ["4 atoms"] * 4 + ["2 atoms"] * 2
     for inside, outside in [((32, 3072, 2048), (32, 2816, 2048)), ((32, 4096, 2048), (32, 4096, 2040)), ((32, 4096, 8704), (32, 4096, 8712)),
                             ((32, 6144, 4096), (32, 6144, 4088)), ((16, 16384, 5120), (16, 16384, 5112)), ((32, 8192, 9472), (32, 8192, 9480)),
-                            ((48, 6144, 4608), (49, 6144, 4608)), ((64, 4096, 7168), (64, 4096, 7176)), ((64, 4096, 3072), (65, 4096, 3072))]:
-        assert call(*inside) > 200 and call(*outside) == 0, (inside, outside)
-    for M in (1, 16, 17, 32, 33, 48, 49, 64):
+                            ((48, 6144, 4608), (49, 6144, 4608)), ((64, 4096, 7168), (64, 4096, 7176)), ((64, 4096, 3072), (65, 4096, 3072)),
+                            ((5, 4096, 8192), (4, 4096, 8192)), ((4, 4096, 7168), (2, 4096, 7168)), ((1, 7168, 7168), (1, 6912, 7168)),
+                            ((1, 7168, 7168), (1, 7168, 7176)), ((2, 8192, 8192), (2, 8192, 8200)), ((1, 3072, 6144), (1, 3072, 6152))]:
+        assert call(*inside).startswith("stacked") and not call(*outside).startswith("stacked"), (inside, outside)
+    for M in (1, 4, 5, 16, 17, 32, 33, 48, 49, 64):
         for K in (3072, 3328, 4096, 8448, 16384):
             for N in (8, 136, 2048, 4744, 7168, 8704, 9472):
                 for sms in (16, 148):
-                    assert call(M, K, N, 8, sms) == 0 and (call(M, K, N, 4, sms) >= 0 or N <= 32 * sms), (M, K, N, sms)
+                    assert not call(M, K, N, 8, (sms, 74, 33, 14)).startswith("stacked")
+                    got = call(M, K, N, 4, (sms, 74, 33, 14))
+                    assert M > 4 or N <= 32 * sms or N > 64 * sms or got == "stream" or got.startswith("stacked"), (M, K, N, sms, got)
+
+
+@pytest.mark.parametrize("device", WHOLE + [(148, 16, 0, 0)])
+def test_short_batches_on_long_rows_leave_the_streaming_kernel_for_enough_slices_only(plans, device):
+    """Every width from 9216 to 16384 channels: a call that the streaming kernel could take (one round of row groups, at most 64 Mi
+    weights) runs there, or in clusters of four slices and more.  Without clusters of four it always runs there."""
+    left = set()
+    for bits in (4, 8):
+        for K in range(9216, 16385, 256 if bits == 4 else 128):
+            for M in (1, 8, 9, 12, 13, 16):
+                for N in (8, 512, 1024, 1032, 2048, 4096, 4104, 4736):
+                    if N * K > 1 << 26:
+                        continue
+                    got = route(plans, M, K, N, bits, device)
+                    if got != "stream":
+                        assert device[2] and got in ("4 by clusters", "8 by clusters") and K >= 10240, (M, K, N, bits, got)
+                        assert M > 8 or (bits == 8 and N <= 1024 and got[0] == "8"), (M, K, N, bits, got)
+                        left.add((M, K, N, bits))
+    if device[2]:
+        assert {(16, 10240, 2048, 4), (16, 16384, 4096, 4), (12, 12288, 4096, 4), (9, 10240, 2048, 8), (16, 10752, 2048, 8),
+                (1, 10240, 1024, 8), (8, 16384, 512, 8)} <= left
+    for M, K, N, bits in [(16, 9984, 2048, 4), (16, 10496, 4096, 4), (16, 10752, 4096, 4), (12, 10240, 2048, 4), (8, 16384, 1024, 4),
+                          (1, 10368, 1024, 8), (8, 14464, 512, 8), (16, 16256, 4096, 8), (16, 10496, 4096, 8), (8, 16384, 1032, 8), (8, 10752, 512, 8)]:
+        assert route(plans, M, K, N, bits, device) == "stream", (M, K, N, bits)
