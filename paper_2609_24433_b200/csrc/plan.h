@@ -444,7 +444,7 @@ GemmPlan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t sc
 //   and eight slices only (8 x 10240 x 1024 10.0 / 9.2, 8 x 16384 x 1024 14.2 / 11.3; four: 8 x 16384 x 2048 14.3 / 14.2).
 // Two rounds, at most 8 tokens on 4 bits, up to 128 Mi weights: ahead of plain tiles (8 x 4096 x 8192 9.7 / 10.1; 16 x 4096 x 8192
 //   13.5 / 10.1: every row group ends with a rendezvous and a reduction), behind stacked ones with 5 tokens and more
-//   (8 x 4096 x 8192 8.5 / 7.4, 5 x 8704 x 9216 13.7 / 13.1).  With fewer the streamed calls are shorter, and ahead (1 x 4096 x
+//   (8 x 4096 x 8192 8.5 / 7.4, 5 x 9216 x 8704 13.7 / 13.1).  With fewer the streamed calls are shorter, and ahead (1 x 4096 x
 //   8192 7.05 / 7.7, 2 x 6144 x 8192 10.2 / 10.5, 1 x 12288 x 9472 15.2 / 15.4) but for long rows (1 x 7168 x 7168 11.0 / 10.4,
 //   4 x 8192 x 8192 12.3 / 11.8, 1 x 16384 x 5120 16.8 / 14.7) and where a stacked tile has few stages (4 x 3072 x 5120 6.3 / 5.95, 3 x 4096 x
 //   7168 7.55 / 7.1).
