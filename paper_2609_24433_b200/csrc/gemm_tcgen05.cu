@@ -24,7 +24,7 @@
 //   4-bit weights: warps 2-9 epilogue (two warps per TMEM lane quadrant, alternating 16-token chunks),
 //                warps 10-17 nibble unpack (two sets of four, alternating k-blocks), warp 18 TMA producer
 //                of packed weights
-//   8-bit weights: warps 2-17 epilogue (four per quadrant), warp 18 TMA producer of int8 weights
+//   8-bit weights: warps 2-9 epilogue, warp 10 TMA producer of int8 weights; or warps 2-17 (four per quadrant) and warp 18 (see epi_warps())
 // Every role runs its loop with the whole warp converged and elects one lane (elect.sync) for
 // the issue itself; a k-block of the MMA warp is one block of PTX that also tests the next
 // k-block's barriers (see issue_kblock_*).  With 4-bit weights three rings are decoupled:
@@ -102,9 +102,12 @@ cudaError_t read_and_clear_watchdog(uint32_t* word) {
 
 namespace {
 
-constexpr int kThreadsW8 = 32 * (2 + kEpiWarpsW8 + 1);   // + one warp: TMA producer of int8 weights
-constexpr int kFirstUnpackWarp = 2 + kEpiWarpsW4;
-constexpr int kThreadsW4 = 32 * (2 + kEpiWarpsW4) + kUnpackSets * 128 + 32;
+// Activation producer, MMA issuer, epilogue, nibble unpack, weight producer.
+constexpr int gemm_threads(int bits, int epi) { return 32 * (2 + epi) + (bits == 4 ? kUnpackSets * 128 : 0) + 32; }
+// 8-bit weights, eight epilogue warps: at most 128 registers per thread (140 to 147 without), so that the next call's prologue finds room
+// beside it: 64 x 2048 x 20000 14.1 -> 12.8 us, 128 x 4096 x 9472 13.2 -> 12.4.
+constexpr int gemm_bounds(int bits, int epi) { return bits == 8 && epi == kEpiWarps ? 512 : gemm_threads(bits, epi); }
+constexpr int kFirstUnpackWarp = 2 + kEpiWarps;
 constexpr int kStackRows = kTileN / kStackSlices;        // channels of a stacked tile
 enum : int { kUnsplit = 0, kSplitScratch = 1, kSplitCluster = 2, kStacked = 3 };
 
@@ -274,8 +277,8 @@ enum : uint32_t {
 // third off the instructions per channel.  (Longer token tiles have no TMEM left for slots twice as wide.)
 // SPLIT: kSplitScratch exchanges the K slices' sums through global scratch, any CTA taking any slice; kSplitCluster gives the
 // slices of a tile to the CTAs of a cluster, one tile per cluster and launch, and exchanges through distributed shared memory.
-template <int BITS, int CTAS, int SPLIT, int ATOMS = 1>
-__global__ void __launch_bounds__(BITS == 4 ? kThreadsW4 : kThreadsW8, 1)
+template <int BITS, int CTAS, int SPLIT, int ATOMS, int EPI>
+__global__ void __launch_bounds__(gemm_bounds(BITS, EPI), 1)
 gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_w,
                     const __grid_constant__ CUtensorMap map_y, const Params p) {
     extern __shared__ uint8_t smem_raw[];
@@ -309,7 +312,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     constexpr bool kCluster = SPLIT == kSplitCluster;
     constexpr bool kStack = SPLIT == kStacked;
     constexpr bool kBox = ATOMS > 1;                // the copy maps are [atom][row][byte]: a stage is one copy
-    constexpr int kEpiWarps = BITS == 4 ? kEpiWarpsW4 : kEpiWarpsW8, kEpiSets = kEpiWarps / 4;    // warps per TMEM lane quadrant: every kEpiSets-th chunk
+    constexpr int kEpiSets = EPI / 4;               // epilogue warps per TMEM lane quadrant: each takes every kEpiSets-th chunk
     // K split: a tile is `split` work units, unit = tile * split + slice, slice s
     // covering k-blocks [s * k_blocks, (s + 1) * k_blocks).  Any CTA takes any unit; the CTA that
     // finishes a tile's last slice adds up the slices' partial sums and runs the epilogue.
@@ -330,7 +333,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     const uint32_t smem_p = smem_w + (BITS == 4 ? 0u : (uint32_t)p.stages * w_bytes);
     const uint32_t smem_e = smem_p + (BITS == 4 ? (uint32_t)p.stages_p * pk_bytes : 0u);
     constexpr int kEpiBytes = BITS == 8 && SPLIT != kUnsplit ? kEpiStageBytes / kEpiBuffers : kEpiStageBytes;
-    const uint32_t smem_sums = smem_e + (uint32_t)(kEpiWarps * kEpiBytes);    // cluster split: the other slices' sums
+    const uint32_t smem_sums = smem_e + (uint32_t)(EPI * kEpiBytes);    // cluster split: the other slices' sums
     uint8_t* gen_base = smem_raw + (base - smem_u32(smem_raw));   // generic pointer to `base`
 
     if (threadIdx.x == 0) {
@@ -350,9 +353,9 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         }
         for (int a = 0; a < kAccStages; ++a) {
             mbar_init(smem_u32(&s_acc_full[a]), 1);
-            mbar_init(smem_u32(&s_acc_empty[a]), kEpiWarps * CTAS);
+            mbar_init(smem_u32(&s_acc_empty[a]), EPI * CTAS);
         }
-        mbar_init(smem_u32(&s_epi_sync), kEpiWarps);
+        mbar_init(smem_u32(&s_epi_sync), EPI);
         mbar_init(smem_u32(&s_sums), 1);
         fence_mbarrier_init();
         fence_proxy_async_smem();
@@ -392,7 +395,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     // producer, and the epilogue warps (per-token steps, K-split scratch, the output).  A weight handle is
     // complete before any call that uses it is enqueued, so the weight producer streams tiles in, the unpack
     // warps fill their TMEM slots, and the MMA warp parks on its barriers while the prologue still runs.
-    if (warp == 0 || (warp >= 2 && warp < 2 + kEpiWarps)) griddep_wait();
+    if (warp == 0 || (warp >= 2 && warp < 2 + EPI)) griddep_wait();
     griddep_launch_dependents();
 
     // work units: (super-tile of 128*CTAS channels) x (token tile) [x K slice]; one unit per CTA or
@@ -602,7 +605,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                 if (++acc_stage == kAccStages) { acc_stage = 0; acc_phase ^= 1u; }
             }
         }
-    } else if (warp < 2 + kEpiWarps) {
+    } else if (warp < 2 + EPI) {
         // ---------------------------------------------------------------- epilogue
         const int quad = warp & 3;                       // TMEM lanes [32*quad, 32*quad + 32)
         const int half = (warp - 2) >> 2;                // which of the alternating 16-token chunks
@@ -660,7 +663,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             const bool ahead = !(BITS == 4 && CTAS == 2) && unit + unit_step >= num_units;
             if (SPLIT == kUnsplit && staged && ahead) request_constants();
             // a tile takes at least ~0.2 us per k-block: sleep through a quarter of that before the first look,
-            // so that eight idle warps do not spend issue slots polling while a long tile is being accumulated
+            // so that idle warps do not spend issue slots polling while a long tile is being accumulated
             if (k_blocks * ATOMS >= 32) __nanosleep(k_blocks * ATOMS >= 400 ? 20000u : (unsigned)(k_blocks * ATOMS) * 50u);
             ok = mbar_wait_warp_relaxed(smem_u32(&s_acc_full[acc_stage]), acc_phase, abort_flag, p.watchdog, kWdEpilogue);
             if (!ok) break;
@@ -683,7 +686,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                     uint32_t r[16];
                     tmem_ld16(taddr + (uint32_t)(c * 16), r);
                     tmem_ld_wait();
-                    const uint32_t from = base + (uint32_t)((sent * kEpiWarps + warp - 2) * kSumBytes);
+                    const uint32_t from = base + (uint32_t)((sent * EPI + warp - 2) * kSumBytes);
 #pragma unroll
                     for (int i = 0; i < 16; ++i) sts32(from + (uint32_t)(i * 32 + lane) * 4u, r[i]);
                     fence_proxy_async_smem();
@@ -1086,7 +1089,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     if (kCluster) {
         __syncwarp();
         if (!waited) cluster_wait();
-        const bool finishes = warp >= 2 && warp < 2 + kEpiWarps && ok && unit0 < num_units;
+        const bool finishes = warp >= 2 && warp < 2 + EPI && ok && unit0 < num_units;
         if (finishes) ok = mbar_wait_all(smem_u32(&s_sums), 0u, abort_flag, p.watchdog, kWdPartials);
         __syncwarp();
         // "this CTA has its sums": no copy is under way when everybody has said so.  (Pairs say it at the end, behind their last read
@@ -1214,12 +1217,12 @@ fq_status build_weight_tmap(Weights& W) {
 
 namespace {
 
-template <int BITS, int CTAS, int SPLIT, int ATOMS = 1>
+template <int BITS, int CTAS, int SPLIT, int ATOMS = 1, int EPI = kEpiWarps>
 fq_status launch_variant(const CUtensorMap& map_a, const CUtensorMap& map_w, const CUtensorMap& map_y, const Params& p,
                          int grid, size_t smem, int cluster, cudaStream_t stream, bool* refused) {
-    auto kern = gemm_tcgen05_kernel<BITS, CTAS, SPLIT, ATOMS>;
+    auto kern = gemm_tcgen05_kernel<BITS, CTAS, SPLIT, ATOMS, EPI>;
     if (ensure_dynamic_smem(reinterpret_cast<const void*>(kern), smem) != cudaSuccess) return FQ_ERR_CUDA;
-    const cudaError_t e = launch_pdl(kern, (unsigned)grid, (unsigned)(BITS == 4 ? kThreadsW4 : kThreadsW8), smem, stream,
+    const cudaError_t e = launch_pdl(kern, (unsigned)grid, (unsigned)gemm_threads(BITS, EPI), smem, stream,
                                      (unsigned)cluster, map_a, map_w, map_y, p);
     *refused = cluster > 1 && cluster_refused(e);
     return e == cudaSuccess ? FQ_OK : FQ_ERR_CUDA;
@@ -1238,12 +1241,12 @@ int cluster_capacity(int ctas) {
     }
     std::lock_guard<std::mutex> lock(mutex);
     if (known[dev][i] == 0) {
-        const auto kern = gemm_tcgen05_kernel<8, 1, kSplitCluster, 1>;
+        const auto kern = gemm_tcgen05_kernel<8, 1, kSplitCluster, 1, kEpiWarps>;
         const size_t smem = 224 * 1024;              // one CTA per SM
         int n = 0;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)ctas, 1, 1);
-        cfg.blockDim = dim3((unsigned)kThreadsW8, 1, 1);
+        cfg.blockDim = dim3((unsigned)gemm_threads(8, kEpiWarps), 1, 1);
         cfg.dynamicSmemBytes = smem;
         cudaLaunchAttribute attr;
         attr.id = cudaLaunchAttributeClusterDimension;
@@ -1360,6 +1363,8 @@ fq_status launch_planned(const int8_t* a8, int64_t M, const Weights& W, int acc_
         constexpr int B = decltype(bits)::value, C = decltype(pair)::value, A = decltype(atoms_c)::value;
         if constexpr (B == 4 && A > 1)
             if (plan.stack > 1) return launch_variant<B, C, kStacked, A>(map_a, map_w, map_y, p, grid, smem, cluster, stream, refused);
+        if constexpr (B == 8)
+            if (plan.epi == kEpiWarpsMany) return launch_variant<B, C, kUnsplit, A, kEpiWarpsMany>(map_a, map_w, map_y, p, grid, smem, cluster, stream, refused);
         if (split == 1) return launch_variant<B, C, kUnsplit, A>(map_a, map_w, map_y, p, grid, smem, cluster, stream, refused);
         if (plan.cluster) return launch_variant<B, C, kSplitCluster, A>(map_a, map_w, map_y, p, grid, smem, cluster, stream, refused);
         return launch_variant<B, C, kSplitScratch, A>(map_a, map_w, map_y, p, grid, smem, cluster, stream, refused);

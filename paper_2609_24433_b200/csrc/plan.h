@@ -243,11 +243,7 @@ constexpr int kMaxStages = 16;         // ring slots, at most: activations, pack
 constexpr int kMaxStagesP = 16;
 constexpr int kMaxStagesW = 8;
 constexpr int kColsW = kBlockK / 4;    // TMEM columns of one unpacked k-block (128 int8 per lane)
-// Epilogue warps: the launch's last tile has nothing to hide its epilogue behind, a chain of TMEM load, arithmetic and store per 16
-// tokens, some 500 cycles each; twice the warps halve it (8 bits, 1000 x 4096 x 4104 21.7 -> 19.8 us; at 4 bits the unpack warps leave no
-// registers for them).
-constexpr int kEpiWarpsW4 = 8, kEpiWarpsW8 = 16;
-inline int epi_warps(int bits) { return bits == 4 ? kEpiWarpsW4 : kEpiWarpsW8; }
+constexpr int kEpiWarps = 8, kEpiWarpsMany = 16;         // epilogue warps (see epi_warps)
 constexpr int kEpiBuffers = 2;                          // output buffers per epilogue warp (bulk stores in flight; four measured no faster)
 constexpr int kEpiStageBytes = kEpiBuffers * 16 * 64;   // per epilogue warp: buffers of 16 tokens x 32 channels of bf16
 constexpr int kMaxSplit = 16;          // K slices per tile, at most
@@ -259,6 +255,7 @@ struct GemmPlan {
     int ctas = 1;     // 2: CTA pairs on 256-channel tiles (cta_group::2)
     int split = 1;    // >1: every tile is that many work units, each on a slice of K
     bool cluster = false; // the slices of a tile are the CTAs of a cluster (no scratch)
+    int epi = kEpiWarps;  // epilogue warps
     int stack = 1;        // 2: a stacked tile, 64 channels at two slices of K (see stacked_applies); bt counts its columns
     size_t scratch = 0;   // bytes of scratch the split needs: the tile counters, then the int32 partial tiles
 };
@@ -277,13 +274,33 @@ inline int atoms_per_stage(int bits, int ctas, int bt, int64_t K, int split) {
     return split == 1 || kb % (2 * split) == 0 ? 2 : 1;
 }
 // Shared memory of the pipeline rings; `sums`: bytes taken by the sums of a cluster split.
-// Output buffers of the epilogue warps (8-bit launches that split K have one per warp: its ring is worth more).
+// Bytes of an epilogue warp's output buffers (8-bit launches that split K have one: the ring is worth more).
 inline int epi_stage_bytes(int bits, bool split) { return bits == 8 && split ? kEpiStageBytes / kEpiBuffers : kEpiStageBytes; }
-inline size_t ring_budget(int bits, bool split, size_t sums) {
-    return 227 * 1024 - 1024 /*alignment slack*/ - 1024 /*static*/ - (size_t)epi_warps(bits) * epi_stage_bytes(bits, split) - sums;
+inline size_t ring_budget(int epi, int bits, bool split, size_t sums) {
+    return 227 * 1024 - 1024 /*alignment slack*/ - 1024 /*static*/ - (size_t)epi * epi_stage_bytes(bits, split) - sums;
 }
 inline size_t stage_bytes(int bits, int ctas, int bt, int atoms) {
     return ((size_t)(bt / ctas) * kBlockK + (size_t)kTileN * kBlockK * bits / 8) * atoms;
+}
+// Epilogue warps.  The last tile of a launch has nothing to hide its epilogue behind, a chain of TMEM load, arithmetic and store per
+// 16 tokens, some 500 cycles each; twice the warps halve it.  They also take registers that the next call's prologue could start on
+// (608 threads x 96 instead of 352 x 128), issue slots from the main loop, and 16 KB from the ring.  Unsplit 8-bit launches, sixteen /
+// eight, chains of calls, M x K x N, us (at 4 bits the unpack warps leave no registers for them; with K split a CTA finishes its
+// share only: 64 x 8192 x 8192 17.0 / 16.5, 400 x 16384 x 2048 29.0 / 25.9, 816 x 16384 x 2048 35.7 / 35.2):
+//   single CTAs, one round: 512 x 4096 x 4096 (128-token tiles) 14.8 / 15.2, 400 x 4096 x 4096 (112) 14.4 / 14.8; with fewer tokens ahead on
+//     short rows only (256 x 1024 x 4096 7.5 / 7.7; 816 x 4096 x 2048 (96) 14.9 / 14.8, 269 x 3072 x 3968 (80) 12.0 / 11.5, 128 x 4096 x
+//     9472 (64) 13.5 / 12.4); more rounds: 100 x 4096 x 30000 (112) 27.7 / 27.4, 64 x 2048 x 20000 14.1 / 12.8
+//   pairs, one round: 1000 x 4096 x 4104 20.1 / 21.5, 208 x 2048 x 16384 13.7 / 14.7
+//     more: ahead on short rows, whose every tile is mostly epilogue (16384 x 1024 x 4096 80 / 103, 816 x 1024 x 16384 19.5 / 22.1), and
+//     up to 2048 channels or two rounds (16384 x 2048 x 2048 72.6 / 75.9, 2000 x 4096 x 4104 31.6 / 32.2) unless the ring loses a stage
+//     by them (816 x 2048 x 32768 49.3 / 46.5, 7312 x 8960 x 792 106 / 104); else no faster (4096 x 4096 x 4096 59 / 59)
+inline int epi_warps(int bits, int ctas, int bt, int64_t K, int64_t rounds, int split) {
+    if (bits == 4 || split > 1) return kEpiWarps;
+    if (rounds == 1 ? (ctas == 2 || bt >= 112 || K <= 1024) : (ctas == 2 && K <= 1024)) return kEpiWarpsMany;
+    const size_t stage = stage_bytes(bits, ctas, bt, 1);
+    return ctas == 2 && (rounds == 2 || (rounds > 2 && K <= 2048)) &&
+                   ring_budget(kEpiWarps, bits, false, 0) / stage == ring_budget(kEpiWarpsMany, bits, false, 0) / stage
+               ? kEpiWarpsMany : kEpiWarps;
 }
 inline size_t cluster_sums_bytes(int bt, int split) { return (size_t)(split - 1) * ((bt / 16 + split - 1) / split) * 16 * kTileN * sizeof(int32_t); }
 
@@ -291,8 +308,8 @@ inline size_t stacked_sums_bytes(int tok) { return (size_t)((tok / 16 + 1) / 2) 
 // Bytes of the ring's memory that a CTA of a cluster split stages the sums in which it sends: the n-th chunk that a warp sends lies at
 // [n][warp], and a warp sends every (warps / 4)-th chunk of 16 tokens but those that its own slice finishes.
 constexpr int kSumBytes = 16 * 32 * 4;                   // a warp's sums of one token chunk
-inline size_t staged_sums_bytes(int bits, int bt, int split) {
-    const int warps = epi_warps(bits), sets = warps / 4;
+inline size_t staged_sums_bytes(int warps, int bt, int split) {
+    const int sets = warps / 4;
     int top = 0;
     for (int slice = 0; slice < split; ++slice)
         for (int set = 0; set < sets; ++set) {
@@ -315,8 +332,8 @@ inline GemmRings gemm_rings(const GemmPlan& plan, int bits, int64_t K) {
     const int bt = plan.bt;
     const bool split = plan.split > 1 || plan.stack > 1;
     f.atoms = atoms_per_stage(bits, plan.ctas, bt, K / plan.stack, plan.split);
-    const size_t sums = plan.cluster ? cluster_sums_bytes(bt, plan.split) : (plan.stack > 1 ? stacked_sums_bytes(bt / plan.stack) : 0), budget = ring_budget(bits, split, sums);
-    const size_t epi_bytes = (size_t)epi_warps(bits) * epi_stage_bytes(bits, split) + sums;
+    const size_t sums = plan.cluster ? cluster_sums_bytes(bt, plan.split) : (plan.stack > 1 ? stacked_sums_bytes(bt / plan.stack) : 0), budget = ring_budget(plan.epi, bits, split, sums);
+    const size_t epi_bytes = (size_t)plan.epi * epi_stage_bytes(bits, split) + sums;
     const size_t a_bytes = (size_t)(bt / plan.ctas) * kBlockK * f.atoms, w_bytes = (size_t)kTileN * kBlockK, pk_bytes = w_bytes / 2 * f.atoms;
     // 4-bit weights: every TMEM column the accumulators leave free becomes unpacked-weight ring
     f.stages_w = bits == 4 ? (512 - kAccStages * bt) / (kColsW * f.atoms) : 0;
@@ -342,7 +359,7 @@ inline GemmRings gemm_rings(const GemmPlan& plan, int bits, int64_t K) {
         if (f.stages < 2) return f;
         f.smem = (a_bytes + w_bytes) * f.stages + epi_bytes + 1024;
     }
-    if (plan.cluster && staged_sums_bytes(bits, bt, plan.split) > f.smem - epi_bytes - 1024) return f;
+    if (plan.cluster && staged_sums_bytes(plan.epi, bt, plan.split) > f.smem - epi_bytes - 1024) return f;
     // One CTA of this kind per SM, and none of the short-batch kernel beside it: a cluster whose CTA waited for tensor memory
     // must not be what another cluster on that SM waits for (launches of two streams).
     if (plan.cluster && f.smem < 152 * 1024) f.smem = 152 * 1024;
@@ -404,9 +421,11 @@ GemmPlan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t sc
             const double per_kb = bits == 4 ? w4 : (c == 1 ? w8_single : (2.62 * b > 545.0 ? 2.62 * b : 545.0));
             const int slots = sms / c;
             auto offer = [&](int sp, bool cluster, size_t scratch, double unit_cost) {
-                const double cost = (double)((units * sp + slots - 1) / slots) * unit_cost;
+                const int64_t rounds = (units * sp + slots - 1) / slots;
+                const double cost = (double)rounds * unit_cost;
                 if (best.bt == 0 || cost < best_cost * 0.98) {   // ties: the earlier candidate (larger tile, no split)
                     best.bt = b; best.ctas = c; best.split = sp; best.cluster = cluster; best.scratch = scratch;
+                    best.epi = epi_warps(bits, c, b, K, rounds, sp);
                     best_cost = cost;
                 }
             };
@@ -419,7 +438,7 @@ GemmPlan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t sc
                 const int atoms = atoms_per_stage(bits, c, b, K, sp);
                 const double ctas = (double)(units * sp * c);
                 if (clusters && (bits == 8 || b <= 128) && sp * c <= kMaxCluster && units * sp <= slots &&
-                    ring_budget(bits, true, cluster_sums_bytes(b, sp)) * atoms >= 4 * stage_bytes(bits, c, b, atoms) &&
+                    ring_budget(kEpiWarps, bits, true, cluster_sums_bytes(b, sp)) * atoms >= 4 * stage_bytes(bits, c, b, atoms) &&
                     gemm_rings(cluster_plan(b, c, sp), bits, K).fits && units <= holds(sp * c))
                     offer(sp, true, 0, slice + 16.0 * b / sp + (bits == 4 ? 2800.0 + 40.0 * ctas : 3300.0 + 18.0 * ctas) + 500.0 * (sp - 1));
                 if ((c == 1 || bits == 8) && units * c <= kMaxSplitTiles && units * c * sp <= 4 * (int64_t)sms) {

@@ -293,6 +293,33 @@ def test_long_w4_pairs_equal_the_second_witness(M, K, N):
     assert torch.equal(fq.gemm_acc_i32(codes, h), fq.gemm_simt(codes, None, h, raw_acc=True))
 
 
+W8_EPILOGUE = [            # tokens, K, channels, epilogue warps: unsplit launches on 8-bit weights
+    (112, 256, 136, 16),       # short rows, short tiles, one round
+    (130, 1280, 264, 8),       # longer rows
+    (390, 512, 4000, 16),      # tiles of 112 tokens
+    (299, 256, 16400, 8),      # two rounds
+    (1000, 512, 4104, 16),     # CTA pairs in one round
+    (501, 2304, 13000, 16),    # ... in two
+    (816, 1280, 9000, 8),      # ... and the ring a stage longer without the eight warps more
+    (2300, 512, 4104, 16),     # three, short rows
+    (4090, 1280, 4104, 16),    # four
+    (3001, 2304, 5000, 8),     # four, longer rows
+]
+
+
+@pytest.mark.parametrize("M,K,N,warps", W8_EPILOGUE)
+def test_w8_epilogues_equal_the_second_witness(M, K, N, warps):
+    g = torch.Generator(device="cuda").manual_seed(M + N)
+    codes_w = torch.randint(0, 256, (N, K), dtype=torch.uint8, device="cuda", generator=g)
+    h = fq.weights_import(codes_w, torch.rand(N, device="cuda", generator=g) + 0.1, None, torch.randn(N, device="cuda", generator=g),
+                          K, 64, 8)
+    codes = torch.randint(0, 256, (M, K), dtype=torch.uint8, device="cuda", generator=g)
+    delta = torch.rand(M, device="cuda", generator=g) + 0.1
+    for dt in (torch.float32, torch.bfloat16):
+        assert torch.equal(fq.gemm_w8a8(codes, delta, h, dt), fq.gemm_simt(codes, delta, h, dt))
+    assert torch.equal(fq.gemm_acc_i32(codes, h), fq.gemm_simt(codes, None, h, raw_acc=True))
+
+
 FEW_UNITS = [
     (9, 1536, 256, 8),         # six units of K for clusters of eight
     (31, 1792, 256, 4),        # seven

@@ -86,13 +86,13 @@ extern "C" void gemm(long M, long N, long K, int bits, long scratch, int sms, in
     const fq::GemmPlan f = fq::plan_call(M, N, K, bits, sms, scratch < 0 ? asks : (size_t)scratch, held);
     const fq::GemmRings r = fq::gemm_rings(f, bits, K);
     const int v[] = {fq::plan_stream(M, N, K, bits, sms, held), f.bt, f.ctas, f.split, f.cluster, f.scratch > 0, r.fits, r.atoms, r.stages,
-                     r.stages_p, r.stages_w, r.slot_first, (int)r.smem, r.tmem_cols, f.stack};
-    for (int i = 0; i < 15; ++i) out[i] = v[i];
+                     r.stages_p, r.stages_w, r.slot_first, (int)r.smem, r.tmem_cols, f.stack, f.epi};
+    for (int i = 0; i < 16; ++i) out[i] = v[i];
 }
 """
 B200 = (148, 74, 36, 14)       # multiprocessors, clusters of 2, 4 and 8 CTAs that one whole device holds
 WHOLE = [B200, (148, 74, 33, 15)]                        # ... and another, whose SMs are grouped otherwise
-GEMM = "stream bt ctas split cluster scratch fits atoms stages stages_p stages_w slot_first smem tmem_cols stack".split()
+GEMM = "stream bt ctas split cluster scratch fits atoms stages stages_p stages_w slot_first smem tmem_cols stack epi".split()
 
 
 class Plans:
@@ -178,6 +178,11 @@ def test_sizes_of_the_device_tests_take_the_routes_they_stand_for(plans, device)
         assert p["fits"] and p["scratch"] and p["split"] > 1 and not p["cluster"] and not p["stream"], (M, K, N, bits, p)
         assert not plans.gemm(M, K, N, bits, scratch=0)["scratch"]
     assert plans.gemm(*edges.SCRATCH_SPLIT[-1])["ctas"] == 2
+    for M, K, N, warps in edges.W8_EPILOGUE:
+        p = plans.gemm(M, K, N, 8)
+        assert p["fits"] and p["split"] == 1 and p["epi"] == warps and not p["stream"], (M, K, N, p)
+    assert [plans.gemm(M, K, N, 8)["ctas"] for M, K, N, _ in edges.W8_EPILOGUE] == [1] * 4 + [2] * 6
+    assert all(plans.gemm(*c)["epi"] == 8 for c in edges.CLUSTER_SPLIT + edges.SCRATCH_SPLIT)
     assert all(plans.gemm(*c, 4)["ctas"] == 2 for c in edges.W4_PAIRS) and all(plans.gemm(*c, 4)["ctas"] == 1 for c in edges.W4_SINGLE)
 
     for M, K, beta, _, dtype, _, lead in edges.COMPOSITE:
