@@ -134,6 +134,7 @@ struct Params {
     int split, split_shift;   // K split: a tile is `split` (power of two) work units, each on a slice of K
     int32_t* partials;   // [tile][slice][bt tokens][128 channels] int32 raw sums of the slices (K split)
     uint32_t* counters;  // [tile] slices finished so far; zeroed by the host before the launch (K split)
+    int delta_vec;       // a_delta is 16-byte aligned: the epilogue may read four steps per load
     int slot_first;      // 1: the unpack sets wait for the TMEM slot ahead of the packed stage (see there)
     uint32_t zero;       // 0, as a run-time value (see the unpack warps' release of a packed stage)
 };
@@ -415,7 +416,10 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     auto kb0_of = [&](int unit) { return (unit & (split - 1)) * k_blocks; };   // first k-block of the unit's slice
 
     // Steps of the 16 tokens of this warp's next chunk: lanes 16 (n & 1) ... of the first register; requested ahead of the sums,
-    // so that their trip through L2 is over when those are complete.
+    // so that their trip through L2 is over when those are complete.  (Not in unsplit launches on 4-bit weights, whose epilogue
+    // takes its issue slots from the nibble unpack: with the exchange between lanes binary32 outputs took 2048 x 4096 x 4096 42.0 us
+    // instead of 40.6, 6819 x 5120 x 2176 82.1 instead of 80.2.)
+    constexpr bool kStepsAhead = BITS == 8 || SPLIT != kUnsplit;
     constexpr int kStepRegs = (16 / kEpiSets + 1) / 2;          // tiles have at most sixteen chunks
     [[maybe_unused]] float steps[kStepRegs] = {};
     auto next_steps = [&](int n) {
@@ -438,9 +442,20 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             return;
         }
         float d[16];
+        if constexpr (kStepsAhead) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) d[i] = __shfl_sync(0xffffffffu, steps[0], 16 * (n & 1) + i);
-        next_steps(n);
+            for (int i = 0; i < 16; ++i) d[i] = __shfl_sync(0xffffffffu, steps[0], 16 * (n & 1) + i);
+            next_steps(n);
+        } else if (tc + 16 <= p.M && p.delta_vec) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float4 q = ld_global_f4(p.out.a_delta + tc + 4 * i);
+                d[4 * i + 0] = q.x; d[4 * i + 1] = q.y; d[4 * i + 2] = q.z; d[4 * i + 3] = q.w;
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) d[i] = tc + i < p.M ? ld_global_f32(p.out.a_delta + tc + i) : 0.0f;
+        }
         tmem_ld_wait();                          // (the sums may still be on their way)
         if (p.out.yt == FQ_BF16) {
             // Transpose 32 channels x 16 tokens through shared memory, then 16-byte stores.  Tokens
@@ -630,7 +645,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             const int64_t t0 = (int64_t)m_of(tile) * p.tok;
             const float2 cj = constants(jq + lane);
             const float sw = cj.x, bj = cj.y;
-            if (SPLIT != kUnsplit || !staged) {            // the steps of this warp's chunks
+            if (kStepsAhead && (SPLIT != kUnsplit || !staged)) {   // the steps of this warp's chunks
                 const int sh = kStack ? 1 : (kCluster ? split_shift : 0);
                 const int off = kStack ? quad >> 1 : (kCluster ? unit & (split - 1) : 0);
 #pragma unroll
@@ -1304,6 +1319,7 @@ fq_status launch_planned(const int8_t* a8, int64_t M, const Weights& W, int acc_
     p.split = split;
     p.counters = static_cast<uint32_t*>(scratch);            // cleared by gemm_prepare()
     p.partials = reinterpret_cast<int32_t*>(static_cast<uint8_t*>(scratch) + kCounterBytes);
+    p.delta_vec = (reinterpret_cast<uintptr_t>(out.a_delta) & 15u) == 0 ? 1 : 0;
     p.bt = bt;
     p.tok = tok;
     p.m_tiles = (int)((M + tok - 1) / tok);
