@@ -26,7 +26,6 @@ struct Weights {
     bool mult_const = false;    // mult_g holds the constant block^-1/2 in every entry (no smoothing, or the diagonal absorbed
                                 // upstream): the fused calls then run the prologue without the per-channel vector
     CUtensorMap tmap;           // TMA view of `codes` for the GEMM's weight operand
-    CUtensorMap tmap_atoms[2];  // 4-bit weights of whole atoms (128 channels): the same for stages of 2 and 4 atoms
     bool tmap_valid = false;
     CUtensorMap tmap_stream;    // 4-bit weights: view for the short-batch streaming kernel (32 rows x 128 bytes)
     bool tmap_stream_valid = false;

@@ -312,7 +312,6 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     const bool leader = cta_rank == 0;
     constexpr bool kCluster = SPLIT == kSplitCluster;
     constexpr bool kStack = SPLIT == kStacked;
-    constexpr bool kBox = ATOMS > 1;                // the copy maps are [atom][row][byte]: a stage is one copy
     constexpr int kEpiSets = EPI / 4;               // epilogue warps per TMEM lane quadrant: each takes every kEpiSets-th chunk
     // K split: a tile is `split` work units, unit = tile * split + slice, slice s
     // covering k-blocks [s * k_blocks, (s + 1) * k_blocks).  Any CTA takes any unit; the CTA that
@@ -525,8 +524,11 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                     if (CTAS == 1) {
                         mbar_arrive_expect_tx(bar, tx);
                         if constexpr (kStack) tma_load_4d(smem_a + stage * a_bytes, &map_a, 0, t0, 0, (kb0 + kb) * ATOMS, bar);
-                        else if constexpr (kBox) tma_load_3d(smem_a + stage * a_bytes, &map_a, 0, t0, (kb0 + kb) * ATOMS, bar);
-                        else tma_load_2d(smem_a + stage * a_bytes, &map_a, (kb0 + kb) * kBlockK, t0, bar);    // channels past K arrive as zeros
+                        else {
+#pragma unroll
+                            for (int h = 0; h < ATOMS; ++h)     // channels past K arrive as zeros
+                                tma_load_2d(smem_a + stage * a_bytes + h * a_atom, &map_a, ((kb0 + kb) * ATOMS + h) * kBlockK, t0, bar);
+                        }
                     } else {
                         // the pair's bytes are all counted on the even CTA's barrier, which it arms for both
                         if (leader) mbar_arrive_expect_tx(bar, tx * CTAS);
@@ -1086,8 +1088,11 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                     const uint32_t bar = smem_u32(&s_full_p[ps]);
                     mbar_arrive_expect_tx(bar, pk_bytes);
                     if constexpr (kStack) tma_load_4d(smem_p + ps * pk_bytes, &map_w, 0, n0, 0, (kb0 + kb) * ATOMS, bar);
-                    else if constexpr (kBox) tma_load_3d(smem_p + ps * pk_bytes, &map_w, 0, n0, (kb0 + kb) * ATOMS, bar);
-                    else tma_load_2d(smem_p + ps * pk_bytes, &map_w, (kb0 + kb) * (kBlockK / 2), n0, bar);
+                    else {
+#pragma unroll
+                        for (int h = 0; h < ATOMS; ++h)
+                            tma_load_2d(smem_p + ps * pk_bytes + h * pk_atom, &map_w, ((kb0 + kb) * ATOMS + h) * (kBlockK / 2), n0, bar);
+                    }
                 }
                 if (++ps == p.stages_p) { ps = 0; pph ^= 1u; }
                 if (++kb == k_blocks) {
@@ -1194,14 +1199,7 @@ bool encode_tiled(CUtensorMap* map, CUtensorMapDataType dt, uint32_t rank, const
 }
 
 namespace {
-// Rows of whole atoms as [atom][row][byte], so that a stage of several atoms is one copy.
-bool encode_atoms(CUtensorMap* map, const void* ptr, uint64_t row_bytes, uint64_t rows, uint32_t atom_bytes, uint32_t box_rows, uint32_t atoms,
-                  CUtensorMapSwizzle swizzle) {
-    const uint64_t dims[3] = {atom_bytes, rows, row_bytes / atom_bytes}, strides[2] = {row_bytes, atom_bytes};
-    const uint32_t box[3] = {atom_bytes, box_rows, atoms};
-    return encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, ptr, dims, strides, box, swizzle);
-}
-// ... and as [atom][K slice][row][byte]: a stacked tile's stage is one copy.
+// Rows of whole atoms as [atom][K slice][row][byte]: a stacked tile's stage is one copy.
 bool encode_stacked(CUtensorMap* map, const void* ptr, uint64_t row_bytes, uint64_t rows, uint32_t atom_bytes, uint32_t box_rows, uint32_t atoms,
                     CUtensorMapSwizzle swizzle) {
     const uint64_t slice_bytes = row_bytes / kStackSlices;
@@ -1220,11 +1218,6 @@ fq_status build_weight_tmap(Weights& W) {
                         : encode_2d(&W.tmap, W.codes, (uint64_t)W.K, (uint64_t)W.N, kBlockK, kTileN,
                                     CU_TENSOR_MAP_SWIZZLE_128B);
     if (!ok) return FQ_ERR_CUDA;
-    if (W.bits == 4 && W.K % kBlockK == 0)
-        for (int i = 0; i < 2; ++i)
-            if (!encode_atoms(&W.tmap_atoms[i], W.codes, (uint64_t)W.K / 2, (uint64_t)W.N, kBlockK / 2, kTileN, 2u << i,
-                              CU_TENSOR_MAP_SWIZZLE_64B))
-                return FQ_ERR_CUDA;
     W.tmap_valid = true;
     build_stream_tmap(W);       // optional second view (short batches); shapes it does not fit go without
     return FQ_OK;
@@ -1349,11 +1342,10 @@ fq_status launch_planned(const int8_t* a8, int64_t M, const Weights& W, int acc_
         if (!encode_stacked(&map_stacked, W.codes, (uint64_t)W.K / 2, (uint64_t)W.N, kBlockK / 2, kStackRows, (uint32_t)atoms, CU_TENSOR_MAP_SWIZZLE_64B) ||
             !encode_stacked(&map_a, a8, (uint64_t)W.K, (uint64_t)M, kBlockK, (uint32_t)tok, (uint32_t)atoms, CU_TENSOR_MAP_SWIZZLE_128B))
             return FQ_ERR_CUDA;
-    } else if (!(atoms > 1 ? encode_atoms(&map_a, a8, (uint64_t)W.K, (uint64_t)M, kBlockK, (uint32_t)bt, (uint32_t)atoms, CU_TENSOR_MAP_SWIZZLE_128B)
-                           : encode_2d(&map_a, a8, (uint64_t)W.K, (uint64_t)M, kBlockK, (uint32_t)(bt / ctas), CU_TENSOR_MAP_SWIZZLE_128B))) {
+    } else if (!encode_2d(&map_a, a8, (uint64_t)W.K, (uint64_t)M, kBlockK, (uint32_t)(bt / ctas), CU_TENSOR_MAP_SWIZZLE_128B)) {
         return FQ_ERR_CUDA;
     }
-    const CUtensorMap& map_w = plan.stack > 1 ? map_stacked : (atoms > 1 ? W.tmap_atoms[atoms == 4 ? 1 : 0] : W.tmap);
+    const CUtensorMap& map_w = plan.stack > 1 ? map_stacked : W.tmap;
 
     // bf16 outputs of an unsplit launch leave through tiled bulk stores of [16 tokens x 32 channels] (64-byte rows,
     // 64-byte swizzle in shared memory); the copy engine clips what lies beyond M tokens or N channels
