@@ -741,7 +741,6 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&s_epi_sync));
                 ok = mbar_wait_all(smem_u32(&s_epi_sync), epi_phase, abort_flag, p.watchdog, kWdPartials);
-                epi_phase ^= 1u;
                 if (!ok) break;
                 for (int i = half, n = 0; i < per; i += kEpiSets, ++n) {
                     const int c = 2 * i + g;
@@ -755,15 +754,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                     emit(r, n, t0 + c * 16, jq, sw, bj, xpose);
                 }
                 tc_fence_before();
-                __syncwarp();
-                if (lane == 0) {
-                    mbar_arrive(smem_u32(&s_acc_empty[acc_stage]));
-                    mbar_arrive(smem_u32(&s_epi_sync));              // the sums have been read
-                }
-                ok = mbar_wait_all(smem_u32(&s_epi_sync), epi_phase, abort_flag, p.watchdog, kWdPartials);
-                epi_phase ^= 1u;
-                if (++acc_stage == kAccStages) { acc_stage = 0; acc_phase ^= 1u; }
-                continue;
+                break;                           // one tile per CTA (see stacked_applies())
             }
             // K split.  Every slice writes its raw int32 sums to its own block of scratch
             // ([tile][slice][bt tokens][128 channels]: a warp's 32 channels of one token are one 128-byte
@@ -932,7 +923,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             bool ok = true;
             int stage = 0, kb = 0, unit = unit0;
             uint32_t phase = 0;
-            int n0 = n_of(tile_of(unit)) * (kStack ? kStackRows : kTileN * CTAS) + (int)cta_rank * kTileN;
+            int n0 = n_of(tile_of(unit)) * (kTileN * CTAS) + (int)cta_rank * kTileN;
             int kb0 = kb0_of(unit);
             bool peek = false;
             for (int n = 0; n < total_kb; ++n) {
@@ -957,7 +948,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                 if (++kb == k_blocks) {
                     kb = 0;
                     unit += unit_step;
-                    n0 = n_of(tile_of(unit)) * (kStack ? kStackRows : kTileN * CTAS) + (int)cta_rank * kTileN;
+                    n0 = n_of(tile_of(unit)) * (kTileN * CTAS) + (int)cta_rank * kTileN;
                     kb0 = kb0_of(unit);
                 }
             }

@@ -225,6 +225,7 @@ inline RingPlan plan_ring(int64_t rows, int64_t K, int elem_bytes, bool gated, b
 //   M <= 48   3072 x 4096 7.1 / 7.7, 4096 x 6144 8.1 / 9.0, 6144 x 6144 9.5 / 11.2;  behind 4096 x 2048 7.8 / 7.4, 6144 x 4096 9.3 / 8.8
 //   M <= 64   3072 x 4096 7.5 / 8.0, 4096 x 4096 8.2 / 9.1, 4096 x 6144 8.6 / 9.1;  behind 5120 x 4096 9.1 / 8.8, 6144 x 6144 10.7 / 10.0
 // (Four slices of 32 channels, 8-bit weights, whose operands pass through shared memory twice then, and longer batches are behind.)
+// (One tile of tokens and at most 64 x SMs channels: a CTA has one tile.)
 constexpr int kStackSlices = 2;
 inline bool stacked_applies(int64_t M, int64_t N, int64_t K, int bits, int sms) {
     if (bits != 4 || M < 1 || M > 64 || K % 256 != 0 || K < 3072) return false;
