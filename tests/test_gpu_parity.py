@@ -467,11 +467,15 @@ def test_random_shapes_against_the_second_witness():
         assert st == fq.OK, (M, N, K, bits, hex(word))
 
 
-@pytest.mark.parametrize("M,N,K", [(1, 72, 1152), (9, 136, 640), (16, 1032, 2176), (5, 8, 128), (16, 4096, 16384)])
+# (M, N, K) at 8 bits
+STREAM_W8 = [(1, 72, 1152), (9, 136, 640), (16, 1032, 2176), (5, 8, 128), (16, 4096, 16256), (8, 4096, 16384)]
+
+
+@pytest.mark.parametrize("M,N,K", STREAM_W8 + [(16, 4096, 16384)])
 def test_short_batches_on_8bit_weights_take_the_streaming_kernel_bit_exact(M, N, K):
     """At most 16 tokens on 8-bit weights of at most 32 x SMs rows: rows that end inside a stage (K not a multiple of
     1024), row groups that end inside the matrix (N not a multiple of 32), one and two token groups, and the longest
-    rows it is given -- integer sums against the oracle, outputs against its epilogue."""
+    rows it is given (the last size, the longest of all with more than 8 tokens, is split by clusters) -- integer sums against the oracle, outputs against its epilogue."""
     rng = np.random.default_rng(M + N + K)
     a, w = random_codes(rng, M, K, 8), random_codes(rng, N, K, 8)
     ws = np.exp2(rng.uniform(-10, -6, size=N)).astype(np.float32)
@@ -486,13 +490,18 @@ def test_short_batches_on_8bit_weights_take_the_streaming_kernel_bit_exact(M, N,
     assert st == fq.OK, hex(word)
 
 
-@pytest.mark.parametrize("M,K,N,bits", [(816, 2048, 4096, 4), (50, 4096, 1024, 4), (256, 4096, 4096, 4), (64, 8192, 2048, 8),
-                                        (16, 16384, 1024, 4), (100, 16384, 256, 4)])
+REPEATED_STREAM = [(16, 8192, 2048, 4), (8, 16384, 1024, 4), (8, 2048, 8192, 4), (16, 8192, 2048, 8)]     # the third: two rounds of row groups
+REPEATED_STACKED = [(16, 8192, 8192, 4), (48, 6144, 6144, 4)]
+REPEATED_CLUSTERS = [(50, 4096, 1024, 4), (64, 8192, 2048, 8), (16, 16384, 1024, 4), (100, 16384, 256, 4)]
+REPEATED_TILES = [(816, 2048, 4096, 4), (256, 4096, 4096, 4)]
+
+
+@pytest.mark.parametrize("M,K,N,bits", REPEATED_TILES + REPEATED_CLUSTERS + REPEATED_STACKED + REPEATED_STREAM)
 def test_repeated_launches_return_the_same_bits(M, K, N, bits):
     """Rings that are full all the time (weights prefetched far ahead) hand their stages over thousands of times per
     launch: a stage given back an instant too early shows up as a rare wrong output, not as a failure.  Six hundred
-    launches per configuration (one-, two- and four-atom stages, 8-bit operands, the streaming kernel, a K split)
-    must return the bits of the first, which match the dp4a witness."""
+    launches per configuration (one-, two- and four-atom stages, 8-bit operands, K splits by clusters, stacked tiles, the
+    streaming kernel) must return the bits of the first, which match the dp4a witness."""
     q = 7 if bits == 4 else 127
     gen = torch.Generator(device="cuda").manual_seed(M + K + N)
     wc = torch.randint(-q, q + 1, (N, K), dtype=torch.int8, device="cuda", generator=gen)
@@ -700,7 +709,8 @@ SWEEP_SAMPLE = [
     # M, K=N, block, bits  (a sample of the throughput-sweep grid; outputs checked on sampled token rows)
     (1, 1024, 32, 4), (1, 4096, 256, 8), (16, 2048, 64, 4), (64, 1024, 128, 8), (256, 4096, 32, 8),
     (256, 2048, 256, 4), (1024, 1024, 64, 4), (1024, 4096, 128, 8), (4096, 2048, 128, 4),
-    (8, 8192, 128, 4), (16, 8192, 64, 4),      # the weight-streaming kernel at its largest square (64 Mi weights)
+    (8, 8192, 128, 4), (16, 8192, 64, 4),      # stacked tiles
+    (4, 6144, 64, 4), (16, 4096, 128, 4),      # the weight-streaming kernel at its largest squares
     (3, 1024, 32, 8), (16, 4096, 64, 8), (9, 2048, 256, 8),   # ... and on 8-bit weights
 ]
 

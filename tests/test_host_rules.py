@@ -6,6 +6,7 @@ import subprocess
 import pytest
 
 import test_gpu_edges as edges
+import test_gpu_parity as parity
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2609_24433_b200", "csrc")
 
@@ -271,6 +272,20 @@ def test_stacked_tiles_and_their_lines(plans):
                     assert not call(M, K, N, 8, (sms, 74, 33, 14)).startswith("stacked")
                     got = call(M, K, N, 4, (sms, 74, 33, 14))
                     assert M > 4 or N <= 32 * sms or N > 64 * sms or got == "stream" or got.startswith("stacked"), (M, K, N, sms, got)
+
+
+@pytest.mark.parametrize("device", WHOLE)
+def test_sizes_of_the_parity_tests_take_the_routes_they_stand_for(plans, device):
+    assert all(route(plans, M, K, N, 8, device) == "stream" for M, N, K in parity.STREAM_W8)
+    assert route(plans, 16, 16384, 4096, 8, device) == "4 by clusters"
+    assert all(route(plans, *c, device) == "stream" for c in parity.REPEATED_STREAM)
+    assert all(route(plans, *c, device).startswith("stacked") for c in parity.REPEATED_STACKED)
+    assert all(route(plans, *c, device).endswith("by clusters") for c in parity.REPEATED_CLUSTERS)
+    assert all(route(plans, *c, device) == "tiles" for c in parity.REPEATED_TILES)
+    sweep = {(M, KN, bits): route(plans, M, KN, KN, bits, device) for M, KN, _, bits in parity.SWEEP_SAMPLE}
+    assert all(sweep[c] == "stream" for c in [(4, 6144, 4), (16, 4096, 4), (3, 1024, 8), (16, 4096, 8), (9, 2048, 8)])
+    assert all(sweep[c].startswith("stacked") for c in [(8, 8192, 4), (16, 8192, 4)])
+    assert all(route(plans, 16, K, N, bits, device) == "stream" for K, N, bits in [(4096, 4096, 4), (4096, 4096, 8), (8192, 1024, 4), (1024, 4096, 8)])
 
 
 @pytest.mark.parametrize("device", WHOLE + [(148, 16, 0, 0)])
