@@ -388,13 +388,14 @@ inline GemmRings gemm_rings(const GemmPlan& plan, int bits, int64_t K) {
 //                           73.3; a short K: 16384 x 1024 x 4096 96 / 97 and 105 / 104.
 // (A plan takes the host 0.1 to 3 us; asking for the clusters of every candidate first took up to 30.)
 // K split: problems with fewer tiles than SMs and a long K (short batches, few output channels).
-//   By clusters of 2, 4 or 8 CTAs (one wave; at least four k-blocks of ring beside the sums, 4-bit tiles of at most 128
-//   tokens): the tail shrinks to 16*bt/split, the exchange costs 2800 + 40 per CTA of the launch at 4 bits, 3300 + 18 at 8
+//   By clusters of 2, 4 or 8 CTAs (one wave; at least four k-blocks of ring beside the sums and two output buffers per warp -- with
+//   one, as 8-bit splits have, pairs of long tiles come in that are behind: 644 x 3584 x 1280 (M x K x N) 13.8 / 12.4 us,
+//   203 x 11264 x 3008 20.0 / 19.4 --, 4-bit tiles of at most 128 tokens): the tail shrinks to 16*bt/split, the exchange costs 2800 + 40 per CTA of the launch at 4 bits, 3300 + 18 at 8
 //   (the more SMs a launch takes, the less of the next one starts beside it), and 500 per extra slice.  Measured, chains of
-//   calls, split against the best unsplit tile: 64 x 16384 x 2048 (M x K x N) 14.5 / 22.5 us at 4 bits and 16.3 / 31.7 at 8;
-//   16 x 16384 x 4096 14.7 / 22.6 and 18.8 / 32.3; 64 x 4096 x 1024 8.6 / 9.9 and 8.0 / 11.1; 64 x 4096 x 4096 10.4 / 10.5
-//   and 10.2 / 11.9; 128 x 4096 x 1024 8.7 / 9.2 and 8.7 / 10.8; 256 x 4096 x 1024 10.5 / 10.1 at 4 bits; CTA pairs,
-//   816 x 16384 x 2048: the site 5 us faster than 96-token tiles.
+//   calls, split against the best unsplit tile: 64 x 16384 x 2048 (M x K x N) 12.8 / 22.1 us at 4 bits and 14.1 / 31.3 at 8;
+//   16 x 16384 x 4096 12.8 / 21.6 and 16.2 / 30.1; 64 x 4096 x 1024 7.5 / 8.9 and 7.5 / 10.8; 64 x 4096 x 4096 8.75 / 11.0
+//   at 8 bits; 128 x 4096 x 1024 9.2 / 9.7 and 7.9 / 11.3; 256 x 4096 x 1024 9.9 / 9.7 and 9.9 / 11.5; CTA pairs,
+//   816 x 16384 x 2048 34.9 / 39.3.
 //   Through scratch, where the device cannot hold the clusters, their sums leave too little ring, or 4-bit tiles have more than
 //   128 tokens (CTA pairs on 8-bit weights, too; on a whole B200 rows of 20480 channels and more): 12500 + 40*bt + 1500 per extra slice.
 template <typename Held>
@@ -439,7 +440,7 @@ GemmPlan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t sc
                 const int atoms = atoms_per_stage(bits, c, b, K, sp);
                 const double ctas = (double)(units * sp * c);
                 if (clusters && (bits == 8 || b <= 128) && sp * c <= kMaxCluster && units * sp <= slots &&
-                    ring_budget(kEpiWarps, bits, true, cluster_sums_bytes(b, sp)) * atoms >= 4 * stage_bytes(bits, c, b, atoms) &&
+                    ring_budget(kEpiWarps, bits, false, cluster_sums_bytes(b, sp)) * atoms >= 4 * stage_bytes(bits, c, b, atoms) &&
                     gemm_rings(cluster_plan(b, c, sp), bits, K).fits && units <= holds(sp * c))
                     offer(sp, true, 0, slice + 16.0 * b / sp + (bits == 4 ? 2800.0 + 40.0 * ctas : 3300.0 + 18.0 * ctas) + 500.0 * (sp - 1));
                 if ((c == 1 || bits == 8) && units * c <= kMaxSplitTiles && units * c * sp <= 4 * (int64_t)sms) {
