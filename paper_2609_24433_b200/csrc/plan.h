@@ -290,14 +290,16 @@ inline size_t stage_bytes(int bits, int ctas, int bt, int atoms) {
 // share only: 64 x 8192 x 8192 17.0 / 16.5, 400 x 16384 x 2048 29.0 / 25.9, 816 x 16384 x 2048 35.7 / 35.2):
 //   single CTAs, one round: 512 x 4096 x 4096 (128-token tiles) 14.8 / 15.2, 400 x 4096 x 4096 (112) 14.4 / 14.8; with fewer tokens ahead on
 //     short rows only (256 x 1024 x 4096 7.5 / 7.7; 816 x 4096 x 2048 (96) 14.9 / 14.8, 269 x 3072 x 3968 (80) 12.0 / 11.5, 128 x 4096 x
-//     9472 (64) 13.5 / 12.4); more rounds: 100 x 4096 x 30000 (112) 27.7 / 27.4, 64 x 2048 x 20000 14.1 / 12.8
+//     9472 (64) 13.5 / 12.4); more rounds: 783 x 1408 x 6368 (160) 13.95 / 14.6, 300 x 256 x 16384 (160) 9.4 / 10.2, 100 x 1024 x 30000
+//     (112) 11.5 / 11.6, 600 x 1536 x 8192 (160) 14.2 / 14.3; 1200 x 2048 x 4104 (160) 18.1 / 17.0, 100 x 2048 x 30000 (112) 17.3 / 16.7,
+//     64 x 1024 x 20000 9.7 / 9.3
 //   pairs, one round: 1000 x 4096 x 4104 20.1 / 21.5, 208 x 2048 x 16384 13.7 / 14.7
 //     more: ahead on short rows, whose every tile is mostly epilogue (16384 x 1024 x 4096 80 / 103, 816 x 1024 x 16384 19.5 / 22.1), and
 //     up to 2048 channels or two rounds (16384 x 2048 x 2048 72.6 / 75.9, 2000 x 4096 x 4104 31.6 / 32.2) unless the ring loses a stage
 //     by them (816 x 2048 x 32768 49.3 / 46.5, 7312 x 8960 x 792 106 / 104); else no faster (4096 x 4096 x 4096 59 / 59)
 inline int epi_warps(int bits, int ctas, int bt, int64_t K, int64_t rounds, int split) {
     if (bits == 4 || split > 1) return kEpiWarps;
-    if (rounds == 1 ? (ctas == 2 || bt >= 112 || K <= 1024) : (ctas == 2 && K <= 1024)) return kEpiWarpsMany;
+    if (rounds == 1 ? (ctas == 2 || bt >= 112 || K <= 1024) : (ctas == 2 ? K <= 1024 : bt >= 112 && K <= 1536)) return kEpiWarpsMany;
     const size_t stage = stage_bytes(bits, ctas, bt, 1);
     return ctas == 2 && (rounds == 2 || (rounds > 2 && K <= 2048)) &&
                    ring_budget(kEpiWarps, bits, false, 0) / stage == ring_budget(kEpiWarpsMany, bits, false, 0) / stage

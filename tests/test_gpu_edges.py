@@ -297,7 +297,8 @@ W8_EPILOGUE = [            # tokens, K, channels, epilogue warps: unsplit launch
     (112, 256, 136, 16),       # short rows, short tiles, one round
     (130, 1280, 264, 8),       # longer rows
     (390, 512, 4000, 16),      # tiles of 112 tokens
-    (299, 256, 16400, 8),      # two rounds
+    (299, 256, 16400, 16),     # two rounds, short rows
+    (450, 2304, 12296, 8),     # two rounds, longer rows
     (1000, 512, 4104, 16),     # CTA pairs in one round
     (501, 2304, 13000, 16),    # ... in two
     (816, 1280, 9000, 8),      # ... and the ring a stage longer without the eight warps more

@@ -182,7 +182,7 @@ def test_sizes_of_the_device_tests_take_the_routes_they_stand_for(plans, device)
     for M, K, N, warps in edges.W8_EPILOGUE:
         p = plans.gemm(M, K, N, 8)
         assert p["fits"] and p["split"] == 1 and p["epi"] == warps and not p["stream"], (M, K, N, p)
-    assert [plans.gemm(M, K, N, 8)["ctas"] for M, K, N, _ in edges.W8_EPILOGUE] == [1] * 4 + [2] * 6
+    assert [plans.gemm(M, K, N, 8)["ctas"] for M, K, N, _ in edges.W8_EPILOGUE] == [1] * 5 + [2] * 6
     assert all(plans.gemm(*c)["epi"] == 8 for c in edges.CLUSTER_SPLIT + edges.SCRATCH_SPLIT)
     assert all(plans.gemm(*c, 4)["ctas"] == 2 for c in edges.W4_PAIRS) and all(plans.gemm(*c, 4)["ctas"] == 1 for c in edges.W4_SINGLE)
 
