@@ -362,7 +362,9 @@ inline GemmRings gemm_rings(const GemmPlan& plan, int bits, int64_t K) {
         if (f.stages < 2) return f;
         f.smem = (a_bytes + w_bytes) * f.stages + epi_bytes + 1024;
     }
-    if (plan.cluster && staged_sums_bytes(plan.epi, bt, plan.split) > f.smem - epi_bytes - 1024) return f;
+    // (mostly there is room for every chunk of the tile: no need to count those that are sent)
+    const size_t ring = f.smem - epi_bytes - 1024;
+    if (plan.cluster && (size_t)(bt / 16 + 3) * 4 * kSumBytes > ring && staged_sums_bytes(plan.epi, bt, plan.split) > ring) return f;
     // One CTA of this kind per SM, and none of the short-batch kernel beside it: a cluster whose CTA waited for tensor memory
     // must not be what another cluster on that SM waits for (launches of two streams).
     if (plan.cluster && f.smem < 152 * 1024) f.smem = 152 * 1024;
@@ -406,6 +408,7 @@ GemmPlan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t sc
     const int64_t kb = (K + kBlockK - 1) / kBlockK;
     GemmPlan best;
     double best_cost = 0.0;
+    int64_t best_rounds = 0;
     int capacity[kMaxCluster + 1] = {};                  // by CTAs per cluster, asked for once per plan; 0: not yet, else + 1
     auto holds = [&](int ctas) {
         if (capacity[ctas] == 0) capacity[ctas] = held(ctas) + 1;
@@ -427,9 +430,10 @@ GemmPlan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t sc
             auto offer = [&](int sp, bool cluster, size_t scratch, double unit_cost) {
                 const int64_t rounds = (units * sp + slots - 1) / slots;
                 const double cost = (double)rounds * unit_cost;
-                if (best.bt == 0 || cost < best_cost * 0.98) {   // ties: the earlier candidate (larger tile, no split)
+                // ties: the earlier candidate (larger tile, no split)
+                if (best.bt == 0 || (cost < best_cost * 0.98 && (!cluster || gemm_rings(cluster_plan(b, c, sp), bits, K).fits))) {
                     best.bt = b; best.ctas = c; best.split = sp; best.cluster = cluster; best.scratch = scratch;
-                    best.epi = epi_warps(bits, c, b, K, rounds, sp);
+                    best_rounds = rounds;
                     best_cost = cost;
                 }
             };
@@ -442,8 +446,7 @@ GemmPlan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t sc
                 const int atoms = atoms_per_stage(bits, c, b, K, sp);
                 const double ctas = (double)(units * sp * c);
                 if (clusters && (bits == 8 || b <= 128) && sp * c <= kMaxCluster && units * sp <= slots &&
-                    ring_budget(kEpiWarps, bits, false, cluster_sums_bytes(b, sp)) * atoms >= 4 * stage_bytes(bits, c, b, atoms) &&
-                    gemm_rings(cluster_plan(b, c, sp), bits, K).fits && units <= holds(sp * c))
+                    ring_budget(kEpiWarps, bits, false, cluster_sums_bytes(b, sp)) * atoms >= 4 * stage_bytes(bits, c, b, atoms) && units <= holds(sp * c))
                     offer(sp, true, 0, slice + 16.0 * b / sp + (bits == 4 ? 2800.0 + 40.0 * ctas : 3300.0 + 18.0 * ctas) + 500.0 * (sp - 1));
                 if ((c == 1 || bits == 8) && units * c <= kMaxSplitTiles && units * c * sp <= 4 * (int64_t)sms) {
                     const size_t scratch = kCounterBytes + (size_t)units * c * sp * kTileN * b * sizeof(int32_t);
@@ -452,6 +455,7 @@ GemmPlan plan_gemm(int64_t M, int64_t N, int64_t K, int bits, int sms, size_t sc
             }
         }
     }
+    if (best.bt != 0) best.epi = epi_warps(bits, best.ctas, best.bt, K, best_rounds, best.split);
     return best;
 }
 
